@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(1024) k_jacobi_block(double *H, double *V, int
     const int np = kp / 2;
     int *pp = reinterpret_cast<int *>(smem_raw);             // p of pair t (p < q)
     int *pq = pp + np;                                        // q of pair t
-    double *pc = reinterpret_cast<double *>(pq + np + (np & 1));
+    double *pc = reinterpret_cast<double *>(pq + np);        // 2 np ints: 8-byte aligned for every np
     double *ps = pc + np;
     __shared__ double red_off[32], red_all[32];
     __shared__ int s_stop;
