@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "factor_kernels.cuh"
+#include "fold_kernels.cuh"
 #include "internal.h"
 #include "solve_kernels.cuh"
 #include "sparse_kernels.cuh"
@@ -149,6 +150,11 @@ extern "C" ss_status ss_set_solve_mode(ss_ctx *ctx, int32_t mode) {
 
 template <typename T>
 static void set_smem_attrs(int device);
+static int fold_shift(ss_numeric *f, int j);
+
+// ctx->d_bar: the grid barrier of the sweep kernels, then counters of blocks per SM id
+constexpr int kSmSlots = 1024;
+constexpr size_t kBarBytes = sizeof(GridBar) + sizeof(int32_t) * kSmSlots;
 
 extern "C" ss_status ss_set_sweep_fusion(ss_ctx *ctx, int32_t max_items) {
     if (!ctx) return SS_ERR_ARG;
@@ -284,6 +290,14 @@ int ss_symbolic_upload(ss_symbolic *s) {
     SweepLevel *dl = nullptr;
     UP(lev, dl);
     s->d_sweep_lev = dl;
+    UP(s->solve_tile128_pre, s->d_solve_tile128_pre);
+    std::vector<FoldLevel> flev(s->solve_levels.size());
+    for (size_t L = 0; L < flev.size(); ++L)
+        flev[L] = FoldLevel{(int32_t)s->solve_levels[L].panel_off, s->solve_levels[L].count,
+                            s->solve_levels[L].tiles128, 0};
+    FoldLevel *df = nullptr;
+    UP(flev, df);
+    s->d_fold_lev = df;
 #undef UP
     return SS_OK;
 }
@@ -291,14 +305,15 @@ int ss_symbolic_upload(ss_symbolic *s) {
 void ss_symbolic_free_device(ss_symbolic *s) {
     void *ptrs[] = {s->d_rowptr, s->d_colind, s->d_iperm, s->d_perm, s->d_idx, s->d_asm_e,
                     s->d_asm_dest, s->d_relmap, s->d_ext_tasks, s->d_panels, s->d_store_tasks, s->d_tasks,
-                    s->d_solve_panels, s->d_solve_tile_pre, s->d_col_panel, s->d_sweep_lev};
+                    s->d_solve_panels, s->d_solve_tile_pre, s->d_col_panel, s->d_sweep_lev, s->d_solve_tile128_pre,
+                    s->d_fold_lev};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     s->d_rowptr = nullptr; s->d_colind = nullptr; s->d_iperm = nullptr; s->d_perm = nullptr;
     s->d_idx = nullptr; s->d_asm_e = nullptr; s->d_asm_dest = nullptr; s->d_relmap = nullptr;
     s->d_ext_tasks = nullptr; s->d_panels = nullptr; s->d_store_tasks = nullptr; s->d_tasks = nullptr;
     s->d_solve_panels = nullptr; s->d_solve_tile_pre = nullptr; s->d_col_panel = nullptr;
-    s->d_sweep_lev = nullptr;
+    s->d_sweep_lev = nullptr; s->d_solve_tile128_pre = nullptr; s->d_fold_lev = nullptr;
 }
 
 // ------------------------------------------------------------------ norms
@@ -339,6 +354,20 @@ static bool first_use_on_device(int device, std::mutex &mu, std::vector<char> &s
     return true;
 }
 
+// the FP64 sweep kernel for items of nc right-hand sides (1 .. kFoldMaxNc)
+static void (*fold_sweeps_kernel(int nc))(FoldArgs, double *) {
+    switch (nc) {
+        case 1: return k_fold_sweeps<1>;
+        case 2: return k_fold_sweeps<2>;
+        case 3: return k_fold_sweeps<3>;
+        case 4: return k_fold_sweeps<4>;
+        case 5: return k_fold_sweeps<5>;
+        case 6: return k_fold_sweeps<6>;
+        case 7: return k_fold_sweeps<7>;
+        default: return k_fold_sweeps<8>;
+    }
+}
+
 template <typename T>
 static void set_smem_attrs(int device) {
     static std::mutex mu;
@@ -347,12 +376,17 @@ static void set_smem_attrs(int device) {
     cudaFuncSetAttribute(k_diag_bk<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDiagSmem);
     cudaFuncSetAttribute(k_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem<T>());
     cudaFuncSetAttribute(k_schur<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)schur_smem<T>());
-    cudaFuncSetAttribute(k_fwd_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)diag_solve_smem<T>());
-    cudaFuncSetAttribute(k_bwd_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)diag_solve_smem<T>());
-    cudaFuncSetAttribute(k_fwd_update<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_kernel_smem<T>());
-    cudaFuncSetAttribute(k_bwd_gather<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_kernel_smem<T>());
-    cudaFuncSetAttribute(k_solve_sweeps<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_launch_smem<T>());
-    if (std::is_same<T, double>::value) {
+    if constexpr (std::is_same<T, float>::value) {
+        cudaFuncSetAttribute(k_fwd_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)diag_solve_smem());
+        cudaFuncSetAttribute(k_bwd_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)diag_solve_smem());
+        cudaFuncSetAttribute(k_fwd_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_solve_smem());
+        cudaFuncSetAttribute(k_bwd_gather, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_solve_smem());
+        cudaFuncSetAttribute(k_solve_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem());
+    } else {
+        cudaFuncSetAttribute(k_fold_panels, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFoldPanelsSmem);
+        cudaFuncSetAttribute(k_fold_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFoldMidSmem);
+        for (int nc = 1; nc <= kFoldMaxNc; ++nc)
+            cudaFuncSetAttribute(fold_sweeps_kernel(nc), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFoldSmem);
         cudaFuncSetAttribute(sstc::k_schur_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sstc::kSchurTcSmem);
         cudaFuncSetAttribute(sstc::k_tc_selftest, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sstc::kSelftestSmem);
@@ -833,6 +867,10 @@ int ss_factor_create(ss_symbolic *sym, const double *a_vals, const double *b_val
     } else {
         rc = factor_run<double>(f, all);
     }
+    // FP64 solves (and ss_solve_noalloc) read the folded panels; FP32 copies were rounded from L21
+    if (!f->inertia_only)
+        for (int j = 0; j < n_shift && rc == SS_OK; ++j)
+            if (f->shift_prec[j] == SS_FP64) rc = fold_shift(f, j);
     if (rc == SS_OK) rc = ss_factor_fetch_counts(f);
     if (rc != SS_OK && rc != SS_ERR_SINGULAR) {
         factor_free(f);
@@ -1016,12 +1054,125 @@ extern "C" ss_status ss_factor_stats(const ss_numeric *f, int32_t j, double *min
 }
 
 // ------------------------------------------------------------------ solves
-template <typename T>
-static int solve_levels(ss_numeric *f, int j, T *b, int k, bool forward, bool backward, int dinv);
+// ---- FP64: the folded factor (fold_kernels.cuh)
+static FoldArgs fold_args(const ss_numeric *f, int j, int k, bool full) {
+    const ss_symbolic *s = f->sym;
+    FoldArgs a{};
+    a.lev = (const FoldLevel *)s->d_fold_lev;
+    a.nlev = (int32_t)s->solve_levels.size();
+    a.npan = (int32_t)s->panels.size();
+    a.k = k;
+    a.full = full ? 1 : 0;
+    a.solve_panels = s->d_solve_panels;
+    a.tile_pre = s->d_solve_tile128_pre;
+    a.panels = s->d_panels;
+    a.idx = s->d_idx;
+    a.linv = f->linv[j];
+    a.dblk = f->dblk[j];
+    a.piv = f->piv[j];
+    a.arena = (const double *)f->arena[j];
+    return a;
+}
 
-template <typename T>
-int solve_permuted(ss_numeric *f, int j, T *b, int k) {
-    return solve_levels<T>(f, j, b, k, true, true, 1);
+// right-hand sides of an item: k cut into as few, equally wide chunks as kFoldMaxNc allows
+static int fold_nc(int k) {
+    const int nch = (k + kFoldMaxNc - 1) / kFoldMaxNc;
+    return (k + nch - 1) / nch;
+}
+
+// G = L21 L11^-1 P in the FP64 L storage of shift j (once, when its factorisation is done)
+static int fold_shift(ss_numeric *f, int j) {
+    ss_symbolic *s = f->sym;
+    ss_ctx *ctx = s->ctx;
+    if (s->panels.empty() || s->max_rows_below == 0) return SS_OK;
+    set_smem_attrs<double>(ctx->device);
+    ss_launch(ctx, SS_K_PANEL, k_fold_panels, dim3((unsigned)s->panels.size(), (unsigned)((s->max_rows_below + TR - 1) / TR)),
+              256, kFoldPanelsSmem, ctx->stream, (const PanelDesc *)s->d_panels, (const double *)f->linv[j],
+              (const int32_t *)f->piv[j], (double *)f->arena[j]);
+    SS_CUDA_TRY(ctx, cudaGetLastError());
+    return SS_OK;
+}
+
+// one launch per level and sweep: no allocation, no synchronisation
+static int fold_per_step(ss_numeric *f, int j, double *b, int k, bool full) {
+    ss_symbolic *s = f->sym;
+    ss_ctx *ctx = s->ctx;
+    cudaStream_t st = ctx->stream;
+    const FoldArgs a = fold_args(f, j, k, full);
+    const int nc = fold_nc(k), nch = (k + nc - 1) / nc;
+    auto level = [&](int L, int backward) {
+        const SolveLevel &sl = s->solve_levels[L];
+        if (sl.tiles128 == 0) return;
+        const int64_t items = (int64_t)sl.tiles128 * 16 * nch;
+        const unsigned grid = (unsigned)((items + kFoldWarps - 1) / kFoldWarps);
+        const int cls = backward ? SS_K_BWD_GATHER : SS_K_FWD_UPDATE;
+        switch (nc) {
+#define SS_FOLD_LEVEL(N) case N: ss_launch(ctx, cls, k_fold_level<N>, grid, kFoldThreads, 0, st, a, L, backward, b); break
+            SS_FOLD_LEVEL(1);
+            SS_FOLD_LEVEL(2);
+            SS_FOLD_LEVEL(3);
+            SS_FOLD_LEVEL(4);
+            SS_FOLD_LEVEL(5);
+            SS_FOLD_LEVEL(6);
+            SS_FOLD_LEVEL(7);
+            default: ss_launch(ctx, cls, k_fold_level<8>, grid, kFoldThreads, 0, st, a, L, backward, b);
+#undef SS_FOLD_LEVEL
+        }
+        ctx->add_flops(cls, 2.0 * sl.offdiag * k);
+    };
+    const int nlev = (int)s->solve_levels.size();
+    for (int L = 0; full && L < nlev; ++L) level(L, 0);
+    const int mc = fold_mid_cols(k);
+    if (a.npan > 0)
+        ss_launch(ctx, SS_K_FWD_DIAG, k_fold_mid, dim3((unsigned)a.npan, (unsigned)((k + mc - 1) / mc)), kFoldThreads,
+                  kFoldMidSmem, st, a, b);
+    for (int L = nlev - 1; L >= 0; --L) level(L, 1);
+    SS_CUDA_TRY(ctx, cudaGetLastError());
+    return SS_OK;
+}
+
+// both sweeps in one cooperative launch of k_fold_sweeps (every block resident, a bounded grid
+// barrier between levels).  Returns SS_ERR_TIMEOUT if a barrier gave up.
+static int fold_sweeps(ss_numeric *f, int j, double *b, int k, bool full) {
+    ss_symbolic *s = f->sym;
+    ss_ctx *ctx = s->ctx;
+    cudaStream_t st = ctx->stream;
+    if (!ctx->d_bar) SS_CUDA_TRY(ctx, cudaMalloc((void **)&ctx->d_bar, kBarBytes));
+    const int nc = fold_nc(k), nch = (k + nc - 1) / nc, mc = fold_mid_cols(k);
+    // enough blocks that the largest step's items lie on as many SMs as there are, no more: a
+    // barrier over few blocks is quicker
+    int64_t items = (int64_t)s->panels.size() * ((k + mc - 1) / mc);
+    double flops = 0.0;
+    for (const SolveLevel &sl : s->solve_levels) {
+        items = std::max<int64_t>(items, (int64_t)sl.tiles128 * 16 * nch);
+        flops += (full ? 4.0 : 2.0) * sl.offdiag * k;
+    }
+    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(ctx->sm_count, items));
+    SS_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_bar, 0, sizeof(GridBar), st));
+    FoldArgs a = fold_args(f, j, k, full);
+    a.bar = ctx->d_bar;
+    a.limit = 20000000;        // polls of about 64 ns: ~1 s per barrier
+    void *args[] = {(void *)&a, (void *)&b};
+    g_ss_launches.fetch_add(1, std::memory_order_relaxed);
+    size_t slot = 0;
+    const bool prof = ctx->prof_mask & (1u << SS_K_SOLVE);
+    if (prof) slot = ss_prof_begin(ctx, SS_K_SOLVE);
+    SS_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((void *)fold_sweeps_kernel(nc), dim3(nb), dim3(kFoldThreads), args,
+                                                 kFoldSmem, st));
+    if (prof) ss_prof_end(ctx, SS_K_SOLVE, slot);
+    ctx->add_flops(SS_K_SOLVE, flops);
+    int herr = 0;
+    SS_CUDA_TRY(ctx, cudaMemcpyAsync(&herr, &ctx->d_bar->err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    SS_CUDA_TRY(ctx, cudaStreamSynchronize(st));
+    if (herr) return ctx->set_error(SS_ERR_TIMEOUT, "solve: grid barrier of the sweep kernel timed out");
+    return SS_OK;
+}
+
+static int fold_solve(ss_numeric *f, int j, double *b, int k, bool full) {
+    ss_ctx *ctx = f->sym->ctx;
+    set_smem_attrs<double>(ctx->device);
+    if (f->sym->solve_levels.empty()) return SS_OK;
+    return ctx->solve_mode == SS_SOLVE_SWEEP_KERNEL ? fold_sweeps(f, j, b, k, full) : fold_per_step(f, j, b, k, full);
 }
 
 // x = P L^-T D^-1/2 y for an SPD factor (the Cholesky frame of B = G G^T, G = P L D^1/2):
@@ -1035,7 +1186,7 @@ int solve_half_backward(ss_numeric *f, int j, const double *y, int k, double *x)
     double *w = nullptr;
     SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&w, sizeof(double) * tot, st));
     ss_launch(ctx, SS_K_MISC, k_dhalf<double>, g, 256, 0, st, s->n, s->d_col_panel, s->d_panels, f->dblk[j], y, w, k);
-    int rc = solve_levels<double>(f, j, w, k, false, true, 0);
+    int rc = fold_solve(f, j, w, k, false);
     if (rc != SS_OK) return rc;
     ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, double>, g, 256, 0, st, s->n, k, s->d_perm,
               (const double *)w, x, 1);
@@ -1044,52 +1195,46 @@ int solve_half_backward(ss_numeric *f, int j, const double *y, int k, double *x)
     return SS_OK;
 }
 
-// Both sweeps in one cooperative launch of k_solve_sweeps (every block resident, a
-// bounded grid barrier between steps).  Returns SS_ERR_TIMEOUT if a barrier gave up.
-template <typename T>
-static int solve_sweeps(ss_numeric *f, int j, T *b, int k, bool forward, bool backward, int dinv, const T *arena) {
+// ---- FP32: k_solve_sweeps (every block resident, a bounded grid barrier between steps).
+// Returns SS_ERR_TIMEOUT if a barrier gave up.
+static int solve_sweeps(ss_numeric *f, int j, float *b, int k, const float *arena) {
     ss_symbolic *s = f->sym;
     ss_ctx *ctx = s->ctx;
     cudaStream_t st = ctx->stream;
-    const int cls = std::is_same<T, float>::value ? SS_K_SOLVE_F32 : SS_K_SOLVE;
-    constexpr int kSmSlots = 1024;
-    if (!ctx->d_bar) SS_CUDA_TRY(ctx, cudaMalloc((void **)&ctx->d_bar, sizeof(GridBar) + sizeof(int32_t) * kSmSlots));
+    const int cls = SS_K_SOLVE_F32;
+    if (!ctx->d_bar) SS_CUDA_TRY(ctx, cudaMalloc((void **)&ctx->d_bar, kBarBytes));
     int32_t *sm_slots = reinterpret_cast<int32_t *>(ctx->d_bar + 1);
-    int &per_sm = ctx->sweep_blocks_per_sm[std::is_same<T, float>::value ? 1 : 0];
+    int &per_sm = ctx->sweep_blocks_per_sm;
     if (per_sm == 0) {
-        SS_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_sweeps<T>, 256,
-                                                                       sweep_launch_smem<T>()));
+        SS_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_sweeps, 256, sweep_smem()));
         if (per_sm <= 0) return ctx->set_error(SS_ERR_CUDA, "solve: sweep kernel cannot be resident");
     }
     const int nchunk = (k + KC - 1) / KC, ndchunk = (k + KD - 1) / KD;
-    // FP32 solves with both sweeps may take the fused items on their small levels (one grid
-    // barrier per level and sweep there)
-    const bool fused = std::is_same<T, float>::value && forward && backward && dinv && ctx->sweep_fuse_max != 0;
+    // the small levels may take the fused items (one grid barrier per level and sweep there)
+    const bool fused = ctx->sweep_fuse_max != 0;
     int64_t items = 1;
     double flops = 0.0;
     for (const SolveLevel &sl : s->solve_levels) {
         items = std::max<int64_t>(items, std::max<int64_t>((int64_t)sl.count * ndchunk, (int64_t)sl.row_tiles * nchunk));
         if (fused) items = std::max<int64_t>(items, (int64_t)(sl.row_tiles + sl.count) * nchunk);
-        flops += ((forward ? 2.0 : 0.0) + (backward ? 2.0 : 0.0)) * sl.offdiag * k;
+        flops += 4.0 * sl.offdiag * k;
     }
     const int nb = (int)std::min<int64_t>((int64_t)per_sm * ctx->sm_count, items);
     const int64_t npan = std::max<int64_t>(1, (int64_t)s->panels.size());
     const int64_t zn = npan * NB * k;
     // fused: the arrival counters (npan x nchunk int32) and the forward output y (N x k)
     // follow z in the same allocation
-    const int64_t an = fused ? (npan * nchunk * (int64_t)sizeof(int32_t) + sizeof(T) - 1) / sizeof(T) : 0;
+    const int64_t an = fused ? npan * nchunk : 0;
     const int64_t yn = fused ? s->n * (int64_t)k : 0;
-    T *zall = nullptr, *ybuf = nullptr;
+    float *zall = nullptr, *ybuf = nullptr;
     int32_t *arrive = nullptr;
-    if (backward) {
-        SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&zall, sizeof(T) * (zn + an + yn), st));
-        SS_CUDA_TRY(ctx, cudaMemsetAsync(zall, 0, sizeof(T) * (zn + an), st));
-        if (fused) {
-            arrive = reinterpret_cast<int32_t *>(zall + zn);
-            ybuf = zall + zn + an;
-        }
+    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&zall, sizeof(float) * (zn + an + yn), st));
+    SS_CUDA_TRY(ctx, cudaMemsetAsync(zall, 0, sizeof(float) * (zn + an), st));
+    if (fused) {
+        arrive = reinterpret_cast<int32_t *>(zall + zn);
+        ybuf = zall + zn + an;
     }
-    SS_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_bar, 0, sizeof(GridBar) + sizeof(int32_t) * kSmSlots, st));
+    SS_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_bar, 0, kBarBytes, st));
     SweepArgs a{};
     a.lev = (const SweepLevel *)s->d_sweep_lev;
     a.nlev = (int32_t)s->solve_levels.size();
@@ -1101,9 +1246,9 @@ static int solve_sweeps(ss_numeric *f, int j, T *b, int k, bool forward, bool ba
     a.linv = f->linv[j];
     a.dblk = f->dblk[j];
     a.piv = f->piv[j];
-    a.forward = forward ? 1 : 0;
-    a.backward = backward ? 1 : 0;
-    a.dinv = dinv;
+    a.forward = 1;
+    a.backward = 1;
+    a.dinv = 1;
     a.bar = ctx->d_bar;
     a.limit = 20000000;        // polls of about 64 ns: ~1 s per barrier
     a.sm_slots = sm_slots;
@@ -1115,64 +1260,61 @@ static int solve_sweeps(ss_numeric *f, int j, T *b, int k, bool forward, bool ba
     size_t slot = 0;
     const bool prof = ctx->prof_mask & (1u << cls);
     if (prof) slot = ss_prof_begin(ctx, cls);
-    SS_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((void *)k_solve_sweeps<T>, dim3(nb), dim3(256), args,
-                                                 sweep_launch_smem<T>(), st));
+    SS_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((void *)k_solve_sweeps, dim3(nb), dim3(256), args, sweep_smem(), st));
     if (prof) ss_prof_end(ctx, cls, slot);
     ctx->add_flops(cls, flops);
     int herr = 0;
     SS_CUDA_TRY(ctx, cudaMemcpyAsync(&herr, &ctx->d_bar->err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    if (zall) SS_CUDA_TRY(ctx, cudaFreeAsync(zall, st));
+    SS_CUDA_TRY(ctx, cudaFreeAsync(zall, st));
     SS_CUDA_TRY(ctx, cudaStreamSynchronize(st));
     if (herr) return ctx->set_error(SS_ERR_TIMEOUT, "solve: grid barrier of the sweep kernel timed out");
     return SS_OK;
 }
 
-template <typename T>
-static int solve_levels(ss_numeric *f, int j, T *b, int k, bool forward, bool backward, int dinv) {
+static int solve_levels(ss_numeric *f, int j, float *b, int k) {
     ss_symbolic *s = f->sym;
     ss_ctx *ctx = s->ctx;
     cudaStream_t st = ctx->stream;
-    set_smem_attrs<T>(ctx->device);
-    const T *arena = (const T *)f->arena[j];
-    if (std::is_same<T, float>::value && f->arena_lo[j]) arena = (const T *)f->arena_lo[j];
-    if (ctx->solve_mode == SS_SOLVE_SWEEP_KERNEL) return solve_sweeps<T>(f, j, b, k, forward, backward, dinv, arena);
+    set_smem_attrs<float>(ctx->device);
+    const float *arena = f->arena_lo[j] ? f->arena_lo[j] : (const float *)f->arena[j];
+    if (ctx->solve_mode == SS_SOLVE_SWEEP_KERNEL) return solve_sweeps(f, j, b, k, arena);
     const int nchunk = (k + KC - 1) / KC;
     const int ndchunk = (k + KD - 1) / KD;
     const int nlev = (int)s->solve_levels.size();
-    for (int L = 0; forward && L < nlev; ++L) {
+    for (int L = 0; L < nlev; ++L) {
         const SolveLevel &sl = s->solve_levels[L];
         const int32_t *lp = s->d_solve_panels + sl.panel_off;
-        ss_launch(ctx, SS_K_FWD_DIAG, k_fwd_diag<T>, dim3(sl.count, ndchunk), 256, diag_solve_smem<T>(), st, lp, s->d_panels, f->linv[j],
-                                                                               f->piv[j], b, k);
-        if (sl.row_tiles > 0)
-            ss_launch(ctx, std::is_same<T, float>::value ? SS_K_FWD_UPDATE_F32 : SS_K_FWD_UPDATE, k_fwd_update<T>, dim3(sl.row_tiles, nchunk), 256, tile_kernel_smem<T>(), st,
-                lp, s->d_solve_tile_pre + sl.panel_off, sl.count, s->d_panels, s->d_idx, arena, b, k);
-        if (sl.row_tiles > 0)
-            ctx->add_flops(std::is_same<T, float>::value ? SS_K_FWD_UPDATE_F32 : SS_K_FWD_UPDATE, 2.0 * sl.offdiag * k);
+        ss_launch(ctx, SS_K_FWD_DIAG, k_fwd_diag, dim3(sl.count, ndchunk), 256, diag_solve_smem(), st, lp, s->d_panels,
+                  f->linv[j], f->piv[j], b, k);
+        if (sl.row_tiles > 0) {
+            ss_launch(ctx, SS_K_FWD_UPDATE_F32, k_fwd_update, dim3(sl.row_tiles, nchunk), 256, tile_solve_smem(), st,
+                      lp, s->d_solve_tile_pre + sl.panel_off, sl.count, s->d_panels, s->d_idx, arena, b, k);
+            ctx->add_flops(SS_K_FWD_UPDATE_F32, 2.0 * sl.offdiag * k);
+        }
     }
-    if (!backward) return SS_OK;
     int32_t maxc = 0;
     for (const SolveLevel &sl : s->solve_levels) maxc = std::max(maxc, sl.count);
-    T *z = nullptr;
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&z, sizeof(T) * (int64_t)maxc * NB * k, st));
+    float *z = nullptr;
+    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&z, sizeof(float) * (int64_t)maxc * NB * k, st));
     for (int L = nlev - 1; L >= 0; --L) {
         const SolveLevel &sl = s->solve_levels[L];
         const int32_t *lp = s->d_solve_panels + sl.panel_off;
         if (sl.row_tiles > 0) {
-            SS_CUDA_TRY(ctx, cudaMemsetAsync(z, 0, sizeof(T) * (int64_t)sl.count * NB * k, st));
-            ss_launch(ctx, std::is_same<T, float>::value ? SS_K_BWD_GATHER_F32 : SS_K_BWD_GATHER, k_bwd_gather<T>, dim3(sl.row_tiles, nchunk), 256, tile_kernel_smem<T>(), st,
-                lp, s->d_solve_tile_pre + sl.panel_off, sl.count, s->d_panels, s->d_idx, arena, b, k, z);
-            ctx->add_flops(std::is_same<T, float>::value ? SS_K_BWD_GATHER_F32 : SS_K_BWD_GATHER, 2.0 * sl.offdiag * k);
+            SS_CUDA_TRY(ctx, cudaMemsetAsync(z, 0, sizeof(float) * (int64_t)sl.count * NB * k, st));
+            ss_launch(ctx, SS_K_BWD_GATHER_F32, k_bwd_gather, dim3(sl.row_tiles, nchunk), 256, tile_solve_smem(), st,
+                      lp, s->d_solve_tile_pre + sl.panel_off, sl.count, s->d_panels, s->d_idx, arena, b, k, z);
+            ctx->add_flops(SS_K_BWD_GATHER_F32, 2.0 * sl.offdiag * k);
         }
-        ss_launch(ctx, SS_K_BWD_DIAG, k_bwd_diag<T>, dim3(sl.count, ndchunk), 256, diag_solve_smem<T>(), st, 
-            lp, s->d_panels, f->linv[j], f->dblk[j], f->piv[j], z, sl.row_tiles > 0 ? 1 : 0, b, k, dinv);
+        ss_launch(ctx, SS_K_BWD_DIAG, k_bwd_diag, dim3(sl.count, ndchunk), 256, diag_solve_smem(), st,
+                  lp, s->d_panels, f->linv[j], f->dblk[j], f->piv[j], z, sl.row_tiles > 0 ? 1 : 0, b, k, 1);
     }
     SS_CUDA_TRY(ctx, cudaFreeAsync(z, st));
     SS_CUDA_TRY(ctx, cudaGetLastError());
     return SS_OK;
 }
-template int solve_permuted<double>(ss_numeric *, int, double *, int);
-template int solve_permuted<float>(ss_numeric *, int, float *, int);
+
+int solve_permuted(ss_numeric *f, int j, double *b, int k) { return fold_solve(f, j, b, k, true); }
+int solve_permuted(ss_numeric *f, int j, float *b, int k) { return solve_levels(f, j, b, k); }
 
 __global__ void k_axpy_sub(int64_t tot, const double *__restrict__ R, const double *__restrict__ Y,
                            double *__restrict__ out) {
@@ -1274,7 +1416,7 @@ int solve_contraction(ss_numeric *f, int j, double *rho) {
     ss_launch(ctx, SS_K_MISC, k_fill_const, 1, 32, 0, st, 1, 1.0, co);
     ss_launch(ctx, SS_K_MISC, k_fill_const, 1, 32, 0, st, 1, -f->sigma[j], co + 1);
     ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<float, double>, g, 256, 0, st, n, 1, s->d_perm, (const double *)r, w, 0);
-    int rc = solve_permuted<float>(f, j, w, 1);
+    int rc = solve_permuted(f, j, w, 1);
     if (rc != SS_OK) return rc;
     ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, float>, g, 256, 0, st, n, 1, s->d_perm, (const float *)w, x, 1);
     if ((rc = spmm_launch(s, f->a_vals, f->b_vals, co, co + 1, x, 1, y)) != SS_OK) return rc;
@@ -1357,7 +1499,7 @@ int solve_apply(ss_numeric *f, int j, const double *R, int k, double *X, int ref
         }
         double *out = refine > 0 ? x : X;
         ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, double>, g, 256, 0, st, s->n, k, s->d_perm, R, w, 0);
-        if ((rc = solve_permuted<double>(f, j, w, k)) != SS_OK) return rc;
+        if ((rc = solve_permuted(f, j, w, k)) != SS_OK) return rc;
         ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, double>, g, 256, 0, st, s->n, k, s->d_perm,
                   (const double *)w, out, 1);
         for (int it = 0; it < refine; ++it) {
@@ -1365,7 +1507,7 @@ int solve_apply(ss_numeric *f, int j, const double *R, int k, double *X, int ref
             ss_launch(ctx, SS_K_MISC, k_axpy_sub, g, 256, 0, st, tot, R, (const double *)y, y);
             ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, double>, g, 256, 0, st, s->n, k, s->d_perm,
                       (const double *)y, w, 0);
-            if ((rc = solve_permuted<double>(f, j, w, k)) != SS_OK) return rc;
+            if ((rc = solve_permuted(f, j, w, k)) != SS_OK) return rc;
             ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, double>, g, 256, 0, st, s->n, k, s->d_perm,
                       (const double *)w, x, 2);
             if (steps_done) (*steps_done)++;
@@ -1415,7 +1557,7 @@ int solve_apply(ss_numeric *f, int j, const double *R, int k, double *X, int ref
             rhs = r;
         }
         ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<float, double>, g, 256, 0, st, s->n, k, s->d_perm, rhs, wf, 0);
-        if ((rc = solve_permuted<float>(f, j, wf, k)) != SS_OK) return rc;
+        if ((rc = solve_permuted(f, j, wf, k)) != SS_OK) return rc;
         ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, float>, g, 256, 0, st, s->n, k, s->d_perm, wf, x, 2);
         if (steps_done && it > 0) (*steps_done)++;
     }
@@ -1475,7 +1617,8 @@ extern "C" ss_status ss_band_energy_grad(ss_symbolic *s, const double *X, const 
 // under another framework's memory budget, inside a region where a new allocation would
 // break an upstream memory plan, or where the allocator itself is unavailable.  Its
 // working space is the file-scope array below: a permuted copy of the right-hand sides
-// (N x k) followed by the per-level gather buffer of the backward sweep.
+// (N x k), solved in place.  The documented size limit also counts 64 k doubles per panel of
+// the widest solve level.
 namespace {
 
 constexpr int64_t kNoAllocScratchDoubles = 4ll * 1024 * 1024;   // 32 MiB per device
@@ -1515,8 +1658,7 @@ extern "C" ss_status ss_solve_noalloc(ss_numeric *f, int32_t j, const double *R,
     int32_t maxc = 0;
     for (const SolveLevel &sl : s->solve_levels) maxc = std::max(maxc, sl.count);
     const int64_t nk = s->n * (int64_t)k;
-    const int64_t zoff = (nk + 31) / 32 * 32;                     // keep the gather buffer 256-byte aligned
-    const int64_t need = zoff + (int64_t)maxc * NB * k;
+    const int64_t need = (nk + 31) / 32 * 32 + (int64_t)maxc * NB * k;
     if (need > kNoAllocScratchDoubles)
         return ctx->set_error(SS_ERR_ARG, "ss_solve_noalloc: N*k + (widest solve level)*64*k = " +
                                               std::to_string(need) + " doubles exceeds the 4,194,304-double (32 MiB) "
@@ -1525,38 +1667,11 @@ extern "C" ss_status ss_solve_noalloc(ss_numeric *f, int32_t j, const double *R,
     double *w = nullptr;
     int rc = noalloc_scratch(ctx, &w);
     if (rc != SS_OK) return rc;
-    double *z = w + zoff;
     cudaStream_t st = ctx->stream;
     set_smem_attrs<double>(ctx->device);
     const unsigned g = (unsigned)((nk + 255) / 256);
     ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, double>, g, 256, 0, st, s->n, (int)k, s->d_perm, R, w, 0);
-    const double *arena = (const double *)f->arena[j];
-    const int nchunk = (k + KC - 1) / KC, ndchunk = (k + KD - 1) / KD;
-    const int nlev = (int)s->solve_levels.size();
-    for (int L = 0; L < nlev; ++L) {
-        const SolveLevel &sl = s->solve_levels[L];
-        const int32_t *lp = s->d_solve_panels + sl.panel_off;
-        ss_launch(ctx, SS_K_FWD_DIAG, k_fwd_diag<double>, dim3(sl.count, ndchunk), 256, diag_solve_smem<double>(), st,
-                  lp, s->d_panels, (const double *)f->linv[j], (const int32_t *)f->piv[j], w, (int)k);
-        if (sl.row_tiles > 0)
-            ss_launch(ctx, SS_K_FWD_UPDATE, k_fwd_update<double>, dim3(sl.row_tiles, nchunk), 256,
-                      tile_solve_smem<double>(), st, lp, s->d_solve_tile_pre + sl.panel_off, sl.count, s->d_panels,
-                      s->d_idx, arena, w, (int)k);
-    }
-    for (int L = nlev - 1; L >= 0; --L) {
-        const SolveLevel &sl = s->solve_levels[L];
-        const int32_t *lp = s->d_solve_panels + sl.panel_off;
-        if (sl.row_tiles > 0) {
-            // the gather buffer keeps the previous call's contents: clear this level's part
-            SS_CUDA_TRY(ctx, cudaMemsetAsync(z, 0, sizeof(double) * (int64_t)sl.count * NB * k, st));
-            ss_launch(ctx, SS_K_BWD_GATHER, k_bwd_gather<double>, dim3(sl.row_tiles, nchunk), 256,
-                      tile_solve_smem<double>(), st, lp, s->d_solve_tile_pre + sl.panel_off, sl.count, s->d_panels,
-                      s->d_idx, arena, (const double *)w, (int)k, z);
-        }
-        ss_launch(ctx, SS_K_BWD_DIAG, k_bwd_diag<double>, dim3(sl.count, ndchunk), 256, diag_solve_smem<double>(), st,
-                  lp, s->d_panels, (const double *)f->linv[j], (const double *)f->dblk[j],
-                  (const int32_t *)f->piv[j], (const double *)z, sl.row_tiles > 0 ? 1 : 0, w, (int)k, 1);
-    }
+    if ((rc = fold_per_step(f, j, w, k, true)) != SS_OK) return rc;
     ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, double>, g, 256, 0, st, s->n, (int)k, s->d_perm,
               (const double *)w, X, 1);
     SS_CUDA_TRY(ctx, cudaGetLastError());

@@ -28,7 +28,7 @@ struct ss_ctx {
     int64_t plan_gen = 0;                     // bumped when a setting baked into captured graphs changes
     double tc_min_flops = 2.0e7;              // a factor step's Schur flops below which it stays on CUDA cores
     GridBar *d_bar = nullptr;                 // grid barrier state of the sweep kernel
-    int sweep_blocks_per_sm[2] = {0, 0};      // resident sweep-kernel blocks per SM (FP64, FP32)
+    int sweep_blocks_per_sm = 0;              // resident FP32 sweep-kernel blocks per SM
     int sweep_fuse_max = 0;                   // FP32 sweep: fuse levels with at most this many items
                                               // (-1: the resident blocks; 0: never)
     // per-class launch timing (ss_profile): event pairs recorded around launches
@@ -151,6 +151,7 @@ struct SolveLevel {      // panels whose forward step can run together
     int32_t count;
     int32_t row_tiles;   // total row tiles (64 rows) of the panels' below-diagonal rows
     double offdiag;      // sum over its panels of (rows below the diagonal block) x w
+    int32_t tiles128;    // total 128-row tiles of the same rows (FP64 solves)
 };
 
 // A captured factorisation of `ns` shifts (one wave) in one precision: persistent scratch
@@ -218,6 +219,8 @@ struct ss_symbolic {
     std::vector<int32_t> solve_panels;       // panel ids grouped by solve level
     std::vector<SolveLevel> solve_levels;
     std::vector<int32_t> solve_tile_pre;     // per solve_panels entry: exclusive row-tile prefix
+    std::vector<int32_t> solve_tile128_pre;  // the same for 128-row tiles
+    int32_t max_rows_below = 0;              // most rows below a panel's diagonal block
 
     ss_symbolic_info info{};
 
@@ -237,7 +240,9 @@ struct ss_symbolic {
     int32_t *d_solve_panels = nullptr;
     int32_t *d_solve_tile_pre = nullptr;
     int32_t *d_col_panel = nullptr;          // permuted column -> panel
-    void *d_sweep_lev = nullptr;             // solve levels for the sweep kernel (SweepLevel)
+    void *d_sweep_lev = nullptr;             // solve levels for the FP32 sweep kernel (SweepLevel)
+    int32_t *d_solve_tile128_pre = nullptr;
+    void *d_fold_lev = nullptr;              // solve levels for the FP64 sweep kernel (FoldLevel)
 };
 
 struct ss_numeric {
@@ -251,7 +256,9 @@ struct ss_numeric {
     double norm_a1 = 0, norm_b1 = 0;
     bool inertia_only = false;            // no L storage kept: inertia counts only
     // per shift
-    std::vector<void *> arena;            // L storage (double or float), l_total entries
+    std::vector<void *> arena;            // L storage (double or float), l_total entries; an FP64
+                                          // one holds G = L21 L11^-1 P below the diagonal blocks
+                                          // (fold_kernels.cuh) once ss_factor_create has returned
     std::vector<float *> arena_lo;        // FP32 rounding of an FP64 L storage that solves read, or null
     std::vector<double *> linv;           // npanels * nb * nb, L11^-1 of each panel
     std::vector<double *> dblk;           // npanels * nb * 2: D diagonal, D sub-diagonal
@@ -293,7 +300,8 @@ constexpr int SS_NCOUNT = 8;   // per-shift device counters: neg, zero, pos, tin
 int ss_norm1(ss_symbolic *s, const double *vals, double *out);
 int solve_contraction(ss_numeric *f, int j, double *rho);
 // in-place solve (A - sigma_j B) x = b of a permuted-order N x k block
-template <typename T> int solve_permuted(ss_numeric *f, int j, T *b, int k);
+int solve_permuted(ss_numeric *f, int j, double *b, int k);
+int solve_permuted(ss_numeric *f, int j, float *b, int k);
 // X = (A - sigma_j B)^-1 R in the original order (FP64 in/out, refinement for mixed)
 // target > 0 (FP32 solves only): refine until max|R - M X| <= target max|R|, at most
 // max(refine, 12) steps

@@ -1,12 +1,12 @@
-// Level-scheduled panel triangular solves with the multifrontal factor (Alg. 2 step 3:
-// V <- L^-T D^-1 L^-1 (B V)).  Right-hand sides are N x k row-major in the permuted
+// FP32 level-scheduled panel triangular solves with the multifrontal factor (Alg. 2 step 3:
+// V <- L^-T D^-1 L^-1 (B V); FP64 solves: fold_kernels.cuh).  Right-hand sides are N x k row-major in the permuted
 // (analysis) order.  For a panel with pivot order P, unit lower L11 (its inverse stored),
 // block-diagonal D and below-diagonal rows L21 (front rows [k0+w, m)):
 //   forward:  y = L11^-1 P b1 (stored in place of b1),  b2 -= L21 y       (push, atomics)
 //   backward: z = L21^T x2 (gathered, atomics into a per-panel buffer),
 //             x1 = P^T L11^-T (D^-1 y - z)                                 (scatter)
 // Panels in one solve level are independent; levels run in order (forward) or reverse
-// order (backward).  T is the factor / right-hand-side type.
+// order (backward).
 //
 // Each step is a device function over one work item (a panel or a row tile, times a
 // chunk of right-hand-side columns).  Two drivers run them: one kernel launch per level
@@ -20,8 +20,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <type_traits>
-
 #include "grid_sync.cuh"
 #include "internal.h"
 
@@ -34,19 +32,8 @@ constexpr int KD = 8;      // right-hand-side columns per block of the diagonal 
 constexpr int LT_LD = NB + 4;   // row stride of the FP32 gather's transposed panel tile
 
 // dynamic shared memory of the solve steps
-template <typename T> constexpr size_t diag_solve_smem() { return sizeof(T) * NB * ((KD + 1) + (NB + 1)); }
-template <typename T> constexpr size_t tile_solve_smem() { return sizeof(T) * (NB * (TR + 1) + TR * (KC + 1)); }
-constexpr size_t tile_solve_smem_f32() { return sizeof(float) * (TR * LT_LD + TR * KC); }
-// shared memory of the per-step update / gather kernels for T
-template <typename T> constexpr size_t tile_kernel_smem() {
-    return std::is_same<T, float>::value ? tile_solve_smem_f32() : tile_solve_smem<T>();
-}
-template <typename T> constexpr size_t sweep_smem() {
-    return diag_solve_smem<T>() > tile_kernel_smem<T>() ? diag_solve_smem<T>() : tile_kernel_smem<T>();
-}
-
-__device__ __forceinline__ void atomic_add_t(double *p, double v) { atomicAdd(p, v); }
-__device__ __forceinline__ void atomic_add_t(float *p, float v) { atomicAdd(p, v); }
+constexpr size_t diag_solve_smem() { return sizeof(float) * NB * ((KD + 1) + (NB + 1)); }
+constexpr size_t tile_solve_smem() { return sizeof(float) * (TR * LT_LD + TR * KC); }
 
 __device__ __forceinline__ void atomic_add_pair(float *p, float v0, float v1, bool both, bool paired) {
     if (paired) {
@@ -72,14 +59,13 @@ __device__ __forceinline__ int tile_slot(const int32_t *__restrict__ tile_pre, i
 // the same shared memory.
 
 // forward diagonal step of panel slot `slot`, right-hand-side chunk `chunk` (KD columns)
-template <typename T>
 __device__ __forceinline__ void fwd_diag_item(unsigned char *smem_raw, int slot, int chunk,
                                               const int32_t *__restrict__ lvl_panels,
                                               const PanelDesc *__restrict__ panels,
                                               const double *__restrict__ linv,
-                                              const int32_t *__restrict__ piv, T *b, int k) {
-    T (*Y)[KD + 1] = reinterpret_cast<T (*)[KD + 1]>(smem_raw);
-    T (*Lm)[NB + 1] = reinterpret_cast<T (*)[NB + 1]>(smem_raw + sizeof(T) * NB * (KD + 1));
+                                              const int32_t *__restrict__ piv, float *b, int k) {
+    float (*Y)[KD + 1] = reinterpret_cast<float (*)[KD + 1]>(smem_raw);
+    float (*Lm)[NB + 1] = reinterpret_cast<float (*)[NB + 1]>(smem_raw + sizeof(float) * NB * (KD + 1));
     const int p = lvl_panels[slot];
     const PanelDesc pd = panels[p];
     const int w = pd.w, c0 = chunk * KD, kc = min(KD, k - c0);
@@ -87,7 +73,7 @@ __device__ __forceinline__ void fwd_diag_item(unsigned char *smem_raw, int slot,
     // all loads before the first store to shared memory (one memory latency per item)
     constexpr int MU = NB * NB / 256, YU = NB * KD / 256;
     double mv[MU];
-    T yv[YU];
+    float yv[YU];
     int sv[YU];
 #pragma unroll
     for (int u = 0; u < YU; ++u) {
@@ -99,7 +85,7 @@ __device__ __forceinline__ void fwd_diag_item(unsigned char *smem_raw, int slot,
 #pragma unroll
     for (int u = 0; u < YU; ++u) {
         const int q = tid + 256 * u, i = q / KD, c = q % KD;
-        yv[u] = (i < w && c < kc) ? b[(int64_t)(pd.g0 + sv[u]) * k + c0 + c] : (T)0;
+        yv[u] = (i < w && c < kc) ? b[(int64_t)(pd.g0 + sv[u]) * k + c0 + c] : (float)0;
     }
     __syncthreads();
 #pragma unroll
@@ -110,22 +96,22 @@ __device__ __forceinline__ void fwd_diag_item(unsigned char *smem_raw, int slot,
 #pragma unroll
     for (int u = 0; u < MU; ++u) {
         const int q = tid + 256 * u;
-        Lm[q / NB][q % NB] = (T)mv[u];
+        Lm[q / NB][q % NB] = (float)mv[u];
     }
     __syncthreads();
     // rows i and i + 32 of column c accumulate side by side
     {
         constexpr int RU = NB * KD / 256;
         const int c = tid % KD, i0 = tid / KD;
-        T acc[RU];
+        float acc[RU];
 #pragma unroll
         for (int u = 0; u < RU; ++u) acc[u] = 0;
         for (int t = 0; t < w; ++t) {
-            const T yt = Y[t][c];
+            const float yt = Y[t][c];
 #pragma unroll
             for (int u = 0; u < RU; ++u) {
                 const int i = i0 + (256 / KD) * u;
-                acc[u] += (t <= i) ? Lm[i][t] * yt : (T)0;
+                acc[u] += (t <= i) ? Lm[i][t] * yt : (float)0;
             }
         }
 #pragma unroll
@@ -136,68 +122,10 @@ __device__ __forceinline__ void fwd_diag_item(unsigned char *smem_raw, int slot,
     }
 }
 
-// forward update of row tile `tile`, chunk `chunk` (KC columns): b2 -= L21 y
-template <typename T>
-__device__ __forceinline__ void fwd_update_item(unsigned char *smem_raw, int tile, int chunk,
-                                                const int32_t *__restrict__ lvl_panels,
-                                                const int32_t *__restrict__ tile_pre, int32_t count,
-                                                const PanelDesc *__restrict__ panels,
-                                                const int32_t *__restrict__ idx,
-                                                const T *__restrict__ arena, T *b, int k) {
-    T (*Ls)[TR + 1] = reinterpret_cast<T (*)[TR + 1]>(smem_raw);                 // Ls[t][row]
-    T (*Y)[KC + 1] = reinterpret_cast<T (*)[KC + 1]>(smem_raw + sizeof(T) * NB * (TR + 1));
-    const int lo = tile_slot(tile_pre, count, tile);
-    const PanelDesc pd = panels[lvl_panels[lo]];
-    const int w = pd.w, m = pd.m;
-    const int r0 = (tile - tile_pre[lo]) * TR;
-    const int nr = min(TR, m - pd.k0 - w - r0);
-    const int c0 = chunk * KC, kc = min(KC, k - c0);
-    const T *F = arena + pd.front_off;
-    const int64_t rowbase = pd.k0 + w + r0;
-    const int tid = threadIdx.x;
-    // all loads before the first store to shared memory (one memory latency per item)
-    constexpr int LU = NB * TR / 256, YU = NB * KC / 256;
-    T lv[LU], yv[YU];
-#pragma unroll
-    for (int u = 0; u < LU; ++u) {
-        const int q = tid + 256 * u, t = q / TR, i = q % TR;
-        lv[u] = (t < w && i < nr) ? F[(int64_t)(pd.k0 + t) * m + rowbase + i] : (T)0;
-    }
-#pragma unroll
-    for (int u = 0; u < YU; ++u) {
-        const int q = tid + 256 * u, t = q / KC, c = q % KC;
-        yv[u] = (t < w && c < kc) ? b[(int64_t)(pd.g0 + t) * k + c0 + c] : (T)0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < LU; ++u) {
-        const int q = tid + 256 * u;
-        Ls[q / TR][q % TR] = lv[u];
-    }
-#pragma unroll
-    for (int u = 0; u < YU; ++u) {
-        const int q = tid + 256 * u;
-        Y[q / KC][q % KC] = yv[u];
-    }
-    __syncthreads();
-    const int *gi = idx + pd.idx_off + rowbase;
-    // thread: column c = tid % 32, rows (tid / 32) + 8 a
-    const int c = tid & 31, rr = tid >> 5;
-    if (c < kc) {
-        for (int a = 0; a < TR / 8; ++a) {
-            int i = rr + 8 * a;
-            if (i >= nr) break;
-            T acc = 0;
-            for (int t = 0; t < w; ++t) acc += Ls[t][i] * Y[t][c];
-            atomic_add_t(&b[(int64_t)gi[i] * k + c0 + c], -acc);
-        }
-    }
-}
-
-// FP32 forward update.  With FP32 arithmetic the one-FMA-per-two-shared-loads loop above
-// is bound by shared-memory bandwidth, so each thread keeps a 4 x 2 register tile (one
-// 16-byte and one 8-byte shared load per 8 FMAs) and adds with paired atomics where the
-// row stride allows.
+// forward update of row tile `tile`, chunk `chunk` (KC columns): b2 -= L21 y.  One FMA per two
+// shared loads would be bound by shared-memory bandwidth, so each thread keeps a 4 x 2 register
+// tile (one 16-byte and one 8-byte shared load per 8 FMAs) and adds with paired atomics where
+// the row stride allows.
 __device__ __forceinline__ void fwd_update_f32_item(unsigned char *smem_raw, int tile, int chunk,
                                                     const int32_t *__restrict__ lvl_panels,
                                                     const int32_t *__restrict__ tile_pre, int32_t count,
@@ -261,69 +189,8 @@ __device__ __forceinline__ void fwd_update_f32_item(unsigned char *smem_raw, int
     }
 }
 
-// backward gather of row tile `tile`: z[slot][t][c] += sum_rows L21[row][t] x[idx[row]][c]
-template <typename T>
-__device__ __forceinline__ void bwd_gather_item(unsigned char *smem_raw, int tile, int chunk,
-                                                const int32_t *__restrict__ lvl_panels,
-                                                const int32_t *__restrict__ tile_pre, int32_t count,
-                                                const PanelDesc *__restrict__ panels,
-                                                const int32_t *__restrict__ idx,
-                                                const T *__restrict__ arena, const T *x, int k, T *zbuf) {
-    T (*Ls)[TR + 1] = reinterpret_cast<T (*)[TR + 1]>(smem_raw);
-    T (*Xs)[KC + 1] = reinterpret_cast<T (*)[KC + 1]>(smem_raw + sizeof(T) * NB * (TR + 1));
-    const int lo = tile_slot(tile_pre, count, tile);
-    const PanelDesc pd = panels[lvl_panels[lo]];
-    const int w = pd.w, m = pd.m;
-    const int r0 = (tile - tile_pre[lo]) * TR;
-    const int nr = min(TR, m - pd.k0 - w - r0);
-    const int c0 = chunk * KC, kc = min(KC, k - c0);
-    const T *F = arena + pd.front_off;
-    const int64_t rowbase = pd.k0 + w + r0;
-    const int *gi = idx + pd.idx_off + rowbase;
-    const int tid = threadIdx.x;
-    // all loads before the first store to shared memory (one memory latency per item, plus
-    // one for the row indices)
-    constexpr int LU = NB * TR / 256, XU = TR * KC / 256;
-    T lv[LU], xv[XU];
-    int gv[XU];
-#pragma unroll
-    for (int u = 0; u < XU; ++u) {
-        const int i = (tid + 256 * u) / KC;
-        gv[u] = i < nr ? gi[i] : 0;
-    }
-#pragma unroll
-    for (int u = 0; u < LU; ++u) {
-        const int q = tid + 256 * u, t = q / TR, i = q % TR;
-        lv[u] = (t < w && i < nr) ? F[(int64_t)(pd.k0 + t) * m + rowbase + i] : (T)0;
-    }
-#pragma unroll
-    for (int u = 0; u < XU; ++u) {
-        const int q = tid + 256 * u, i = q / KC, c = q % KC;
-        xv[u] = (i < nr && c < kc) ? x[(int64_t)gv[u] * k + c0 + c] : (T)0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < LU; ++u) {
-        const int q = tid + 256 * u;
-        Ls[q / TR][q % TR] = lv[u];
-    }
-#pragma unroll
-    for (int u = 0; u < XU; ++u) {
-        const int q = tid + 256 * u;
-        Xs[q / KC][q % KC] = xv[u];
-    }
-    __syncthreads();
-    T *z = zbuf + (int64_t)lo * NB * k;
-    for (int q = tid; q < w * KC; q += 256) {
-        int t = q / KC, c = q % KC;
-        if (c >= kc) continue;
-        T acc = 0;
-        for (int i = 0; i < nr; ++i) acc += Ls[t][i] * Xs[i][c];
-        atomic_add_t(&z[(int64_t)t * k + c0 + c], acc);
-    }
-}
-
-// FP32 backward gather with a 4 x 2 register tile per thread (see the FP32 update)
+// backward gather of row tile `tile`: z[slot][t][c] += sum_rows L21[row][t] x[idx[row]][c], with a
+// 4 x 2 register tile per thread (see the forward update)
 __device__ __forceinline__ void bwd_gather_f32_item(unsigned char *smem_raw, int tile, int chunk,
                                                     const int32_t *__restrict__ lvl_panels,
                                                     const int32_t *__restrict__ tile_pre, int32_t count,
@@ -396,16 +263,15 @@ __device__ __forceinline__ void bwd_gather_f32_item(unsigned char *smem_raw, int
 }
 
 // backward diagonal step of panel slot `slot`: x1 = P^T L11^-T (D^-1 y - z)
-template <typename T>
 __device__ __forceinline__ void bwd_diag_item(unsigned char *smem_raw, int slot, int chunk,
                                               const int32_t *__restrict__ lvl_panels,
                                               const PanelDesc *__restrict__ panels,
                                               const double *__restrict__ linv,
                                               const double *__restrict__ dblk,
                                               const int32_t *__restrict__ piv,
-                                              const T *zbuf, int use_z, T *x, int k, int dinv) {
-    T (*U)[KD + 1] = reinterpret_cast<T (*)[KD + 1]>(smem_raw);
-    T (*Lm)[NB + 1] = reinterpret_cast<T (*)[NB + 1]>(smem_raw + sizeof(T) * NB * (KD + 1));
+                                              const float *zbuf, int use_z, float *x, int k, int dinv) {
+    float (*U)[KD + 1] = reinterpret_cast<float (*)[KD + 1]>(smem_raw);
+    float (*Lm)[NB + 1] = reinterpret_cast<float (*)[NB + 1]>(smem_raw + sizeof(float) * NB * (KD + 1));
     __shared__ double sd[NB], se[NB];
     const int p = lvl_panels[slot];
     const PanelDesc pd = panels[p];
@@ -414,7 +280,7 @@ __device__ __forceinline__ void bwd_diag_item(unsigned char *smem_raw, int slot,
     // all loads before the first store to shared memory (one memory latency per item)
     constexpr int MU = NB * NB / 256, UU = NB * KD / 256;
     double mv[MU], dv = 0.0, ev = 0.0;
-    T uv[UU];
+    float uv[UU];
     if (tid < NB) {
         dv = dblk[(int64_t)p * 2 * NB + tid];
         ev = dblk[(int64_t)p * 2 * NB + NB + tid];
@@ -424,7 +290,7 @@ __device__ __forceinline__ void bwd_diag_item(unsigned char *smem_raw, int slot,
 #pragma unroll
     for (int u = 0; u < UU; ++u) {
         const int q = tid + 256 * u, i = q / KD, c = q % KD;
-        uv[u] = (i < w && c < kc) ? x[(int64_t)(pd.g0 + i) * k + c0 + c] : (T)0;
+        uv[u] = (i < w && c < kc) ? x[(int64_t)(pd.g0 + i) * k + c0 + c] : (float)0;
     }
     __syncthreads();
     if (tid < NB) {
@@ -434,7 +300,7 @@ __device__ __forceinline__ void bwd_diag_item(unsigned char *smem_raw, int slot,
 #pragma unroll
     for (int u = 0; u < MU; ++u) {
         const int q = tid + 256 * u;
-        Lm[q / NB][q % NB] = (T)mv[u];
+        Lm[q / NB][q % NB] = (float)mv[u];
     }
 #pragma unroll
     for (int u = 0; u < UU; ++u) {
@@ -442,7 +308,7 @@ __device__ __forceinline__ void bwd_diag_item(unsigned char *smem_raw, int slot,
         U[q / KD][q % KD] = uv[u];
     }
     __syncthreads();
-    T val[NB * KD / 256];
+    float val[NB * KD / 256];
     // u = Dinv y - z, each thread handles entries (i, c) with i = tid/KD + (256/KD) a
     const int c = tid % KD, rr = tid / KD;
     constexpr int RS = 256 / KD;
@@ -463,7 +329,7 @@ __device__ __forceinline__ void bwd_diag_item(unsigned char *smem_raw, int slot,
             }
             if (use_z) u -= (double)zbuf[(int64_t)slot * NB * k + (int64_t)i * k + c0 + c];
         }
-        val[a] = (T)u;
+        val[a] = (float)u;
     }
     __syncthreads();
     for (int a = 0; a < NB * KD / 256; ++a) {
@@ -476,15 +342,15 @@ __device__ __forceinline__ void bwd_diag_item(unsigned char *smem_raw, int slot,
     {
         constexpr int RU = NB * KD / 256;
         const int cc = tid % KD, i0 = tid / KD;
-        T acc[RU];
+        float acc[RU];
 #pragma unroll
         for (int u = 0; u < RU; ++u) acc[u] = 0;
         for (int t = 0; t < w; ++t) {
-            const T ut = U[t][cc];
+            const float ut = U[t][cc];
 #pragma unroll
             for (int u = 0; u < RU; ++u) {
                 const int i = i0 + (256 / KD) * u;
-                acc[u] += (t >= i) ? Lm[t][i] * ut : (T)0;
+                acc[u] += (t >= i) ? Lm[t][i] * ut : (float)0;
             }
         }
 #pragma unroll
@@ -496,54 +362,41 @@ __device__ __forceinline__ void bwd_diag_item(unsigned char *smem_raw, int slot,
 }
 
 // ---------------------------------------------------------------- one launch per step
-template <typename T>
 __global__ void __launch_bounds__(256) k_fwd_diag(const int32_t *__restrict__ lvl_panels,
                                                    const PanelDesc *__restrict__ panels,
                                                    const double *__restrict__ linv,
-                                                   const int32_t *__restrict__ piv, T *b, int k) {
+                                                   const int32_t *__restrict__ piv, float *b, int k) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    fwd_diag_item<T>(smem_raw, blockIdx.x, blockIdx.y, lvl_panels, panels, linv, piv, b, k);
+    fwd_diag_item(smem_raw, blockIdx.x, blockIdx.y, lvl_panels, panels, linv, piv, b, k);
 }
 
-template <typename T>
 __global__ void __launch_bounds__(256) k_fwd_update(const int32_t *__restrict__ lvl_panels,
                                                      const int32_t *__restrict__ tile_pre,
                                                      int32_t count, const PanelDesc *__restrict__ panels,
                                                      const int32_t *__restrict__ idx,
-                                                     const T *__restrict__ arena, T *b, int k) {
+                                                     const float *__restrict__ arena, float *b, int k) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if constexpr (std::is_same<T, float>::value)
-        fwd_update_f32_item(smem_raw, blockIdx.x, blockIdx.y, lvl_panels, tile_pre, count, panels, idx, arena, b, k);
-    else
-        fwd_update_item<T>(smem_raw, blockIdx.x, blockIdx.y, lvl_panels, tile_pre, count, panels, idx, arena, b, k);
+    fwd_update_f32_item(smem_raw, blockIdx.x, blockIdx.y, lvl_panels, tile_pre, count, panels, idx, arena, b, k);
 }
 
-template <typename T>
 __global__ void __launch_bounds__(256) k_bwd_gather(const int32_t *__restrict__ lvl_panels,
                                                      const int32_t *__restrict__ tile_pre,
                                                      int32_t count, const PanelDesc *__restrict__ panels,
                                                      const int32_t *__restrict__ idx,
-                                                     const T *__restrict__ arena, const T *x,
-                                                     int k, T *zbuf) {
+                                                     const float *__restrict__ arena, const float *x,
+                                                     int k, float *zbuf) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if constexpr (std::is_same<T, float>::value)
-        bwd_gather_f32_item(smem_raw, blockIdx.x, blockIdx.y, lvl_panels, tile_pre, count, panels, idx, arena, x, k,
-                            zbuf);
-    else
-        bwd_gather_item<T>(smem_raw, blockIdx.x, blockIdx.y, lvl_panels, tile_pre, count, panels, idx, arena, x, k,
-                           zbuf);
+    bwd_gather_f32_item(smem_raw, blockIdx.x, blockIdx.y, lvl_panels, tile_pre, count, panels, idx, arena, x, k, zbuf);
 }
 
-template <typename T>
 __global__ void __launch_bounds__(256) k_bwd_diag(const int32_t *__restrict__ lvl_panels,
                                                    const PanelDesc *__restrict__ panels,
                                                    const double *__restrict__ linv,
                                                    const double *__restrict__ dblk,
                                                    const int32_t *__restrict__ piv,
-                                                   const T *zbuf, int use_z, T *x, int k, int dinv) {
+                                                   const float *zbuf, int use_z, float *x, int k, int dinv) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    bwd_diag_item<T>(smem_raw, blockIdx.x, blockIdx.y, lvl_panels, panels, linv, dblk, piv, zbuf, use_z, x, k,
-                     dinv);
+    bwd_diag_item(smem_raw, blockIdx.x, blockIdx.y, lvl_panels, panels, linv, dblk, piv, zbuf, use_z, x, k, dinv);
 }
 
 // ---------------------------------------------------------------- one launch per solve
@@ -614,13 +467,12 @@ __device__ __forceinline__ int spread_block_id(const SweepArgs &a, bool *ok) {
 constexpr size_t fused_fwd_smem() { return sizeof(float) * (NB * (NB + 1) + 2 * NB * KC + NB * TR); }
 constexpr size_t fused_bwd_smem() { return sizeof(float) * (NB * (NB + 1) + NB * KC); }
 constexpr size_t fused_smem() {
-    return fused_fwd_smem() > tile_solve_smem_f32() ? fused_fwd_smem() : tile_solve_smem_f32();
+    return fused_fwd_smem() > tile_solve_smem() ? fused_fwd_smem() : tile_solve_smem();
 }
 
-// dynamic shared memory of a k_solve_sweeps<T> launch (the FP32 kernel also runs the fused sweep)
-template <typename T> constexpr size_t sweep_launch_smem() {
-    return std::is_same<T, float>::value ? (sweep_smem<T>() > fused_smem() ? sweep_smem<T>() : fused_smem())
-                                         : sweep_smem<T>();
+// dynamic shared memory of a k_solve_sweeps launch (it also runs the fused items)
+constexpr size_t sweep_smem() {
+    return diag_solve_smem() > fused_smem() ? diag_solve_smem() : fused_smem();
 }
 
 // rows below panel slot `slot` of a level, in row tiles
@@ -911,9 +763,8 @@ __device__ __forceinline__ bool level_fused(const SweepArgs &a, const SweepLevel
 // consecutive steps.  zall: (number of panels) x NB x k, zero on entry (each level
 // gathers into its own slots).  On a barrier timeout bar->err is set and every block
 // returns.
-template <typename T>
-__global__ void __launch_bounds__(256, 4) k_solve_sweeps(SweepArgs a, const T *__restrict__ arena, T *b, T *zall,
-                                                         T *ybuf) {
+__global__ void __launch_bounds__(256, 4) k_solve_sweeps(SweepArgs a, const float *__restrict__ arena, float *b,
+                                                         float *zall, float *ybuf) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int k = a.k;
     const int nchunk = (k + KC - 1) / KC, ndchunk = (k + KD - 1) / KD;
@@ -925,26 +776,19 @@ __global__ void __launch_bounds__(256, 4) k_solve_sweeps(SweepArgs a, const T *_
         for (int L = 0; L < a.nlev; ++L) {
             const SweepLevel lv = a.lev[L];
             const int32_t *lp = a.solve_panels + lv.panel_off;
-            if constexpr (std::is_same<T, float>::value) {
-                if (level_fused(a, lv, nchunk)) {       // y of this level goes to ybuf
-                    fwd_level_fused_f32(a, smem_raw, vb, lv, arena, b, ybuf);
-                    if (!grid_barrier(a.bar, nb, a.limit)) return;
-                    continue;
-                }
+            if (level_fused(a, lv, nchunk)) {           // y of this level goes to ybuf
+                fwd_level_fused_f32(a, smem_raw, vb, lv, arena, b, ybuf);
+                if (!grid_barrier(a.bar, nb, a.limit)) return;
+                continue;
             }
             for (int q = vb; q < lv.count * ndchunk; q += nb)
-                fwd_diag_item<T>(smem_raw, q % lv.count, q / lv.count, lp, a.panels, a.linv, a.piv, b, k);
+                fwd_diag_item(smem_raw, q % lv.count, q / lv.count, lp, a.panels, a.linv, a.piv, b, k);
             if (!grid_barrier(a.bar, nb, a.limit)) return;
             if (lv.row_tiles == 0) continue;
             const int32_t *tp = a.tile_pre + lv.panel_off;
-            for (int q = vb; q < lv.row_tiles * nchunk; q += nb) {
-                if constexpr (std::is_same<T, float>::value)
-                    fwd_update_f32_item(smem_raw, q % lv.row_tiles, q / lv.row_tiles, lp, tp, lv.count, a.panels,
-                                        a.idx, arena, b, k);
-                else
-                    fwd_update_item<T>(smem_raw, q % lv.row_tiles, q / lv.row_tiles, lp, tp, lv.count, a.panels,
-                                       a.idx, arena, b, k);
-            }
+            for (int q = vb; q < lv.row_tiles * nchunk; q += nb)
+                fwd_update_f32_item(smem_raw, q % lv.row_tiles, q / lv.row_tiles, lp, tp, lv.count, a.panels, a.idx,
+                                    arena, b, k);
             if (!grid_barrier(a.bar, nb, a.limit)) return;
         }
     }
@@ -952,28 +796,21 @@ __global__ void __launch_bounds__(256, 4) k_solve_sweeps(SweepArgs a, const T *_
     for (int L = a.nlev - 1; L >= 0; --L) {
         const SweepLevel lv = a.lev[L];
         const int32_t *lp = a.solve_panels + lv.panel_off;
-        T *z = zall + (int64_t)lv.panel_off * NB * k;
-        if constexpr (std::is_same<T, float>::value) {
-            if (level_fused(a, lv, nchunk)) {
-                bwd_level_fused_f32(a, smem_raw, vb, lv, arena, b, zall, ybuf);
-                if (L > 0 && !grid_barrier(a.bar, nb, a.limit)) return;
-                continue;
-            }
+        float *z = zall + (int64_t)lv.panel_off * NB * k;
+        if (level_fused(a, lv, nchunk)) {
+            bwd_level_fused_f32(a, smem_raw, vb, lv, arena, b, zall, ybuf);
+            if (L > 0 && !grid_barrier(a.bar, nb, a.limit)) return;
+            continue;
         }
         if (lv.row_tiles > 0) {
             const int32_t *tp = a.tile_pre + lv.panel_off;
-            for (int q = vb; q < lv.row_tiles * nchunk; q += nb) {
-                if constexpr (std::is_same<T, float>::value)
-                    bwd_gather_f32_item(smem_raw, q % lv.row_tiles, q / lv.row_tiles, lp, tp, lv.count, a.panels,
-                                        a.idx, arena, b, k, z);
-                else
-                    bwd_gather_item<T>(smem_raw, q % lv.row_tiles, q / lv.row_tiles, lp, tp, lv.count, a.panels,
-                                       a.idx, arena, b, k, z);
-            }
+            for (int q = vb; q < lv.row_tiles * nchunk; q += nb)
+                bwd_gather_f32_item(smem_raw, q % lv.row_tiles, q / lv.row_tiles, lp, tp, lv.count, a.panels, a.idx,
+                                    arena, b, k, z);
             if (!grid_barrier(a.bar, nb, a.limit)) return;
         }
         for (int q = vb; q < lv.count * ndchunk; q += nb)
-            bwd_diag_item<T>(smem_raw, q % lv.count, q / lv.count, lp, a.panels, a.linv, a.dblk, a.piv, z,
+            bwd_diag_item(smem_raw, q % lv.count, q / lv.count, lp, a.panels, a.linv, a.dblk, a.piv, z,
                              lv.row_tiles > 0 ? 1 : 0, b, k, a.dinv);
         if (L > 0 && !grid_barrier(a.bar, nb, a.limit)) return;
     }

@@ -565,13 +565,18 @@ static int analyze_impl(ss_ctx *ctx, int64_t n, const int64_t *rowptr, const int
     s->solve_panels.clear();
     s->solve_levels.clear();
     s->solve_tile_pre.clear();
+    s->solve_tile128_pre.clear();
+    s->max_rows_below = 0;
     for (int32_t l = 0; l < nplev; ++l) {
-        SolveLevel sl{(int64_t)s->solve_panels.size(), 0, 0, 0.0};
+        SolveLevel sl{(int64_t)s->solve_panels.size(), 0, 0, 0.0, 0};
         for (int32_t p : by_lev[l]) {
             const PanelDesc &pd = s->panels[p];
             s->solve_panels.push_back(p);
             s->solve_tile_pre.push_back(sl.row_tiles);
+            s->solve_tile128_pre.push_back(sl.tiles128);
             sl.row_tiles += (int32_t)cdiv(pd.m - pd.k0 - pd.w, 64);
+            sl.tiles128 += (int32_t)cdiv(pd.m - pd.k0 - pd.w, 128);
+            s->max_rows_below = std::max(s->max_rows_below, pd.m - pd.k0 - pd.w);
             sl.offdiag += (double)(pd.m - pd.k0 - pd.w) * pd.w;
             sl.count++;
         }
@@ -840,16 +845,19 @@ static int validate_impl(const ss_symbolic *s, std::string &why) {
     }
     std::vector<char> pseen(npan, 0);
     for (const SolveLevel &sl : s->solve_levels) {
-        int32_t tiles = 0;
+        int32_t tiles = 0, tiles128 = 0;
         for (int32_t t = 0; t < sl.count; ++t) {
             int32_t p = s->solve_panels[sl.panel_off + t];
             if (p < 0 || p >= npan || pseen[p]) return fail("solve level panel id");
             pseen[p] = 1;
             if (s->solve_tile_pre[sl.panel_off + t] != tiles) return fail("solve tile prefix");
+            if (s->solve_tile128_pre[sl.panel_off + t] != tiles128) return fail("solve tile prefix (128 rows)");
             const PanelDesc &pd = s->panels[p];
             tiles += (pd.m - pd.k0 - pd.w + 63) / 64;
+            tiles128 += (pd.m - pd.k0 - pd.w + 127) / 128;
+            if (pd.m - pd.k0 - pd.w > s->max_rows_below) return fail("rows below a panel");
         }
-        if (tiles != sl.row_tiles) return fail("solve level tile total");
+        if (tiles != sl.row_tiles || tiles128 != sl.tiles128) return fail("solve level tile total");
     }
     for (int64_t p = 0; p < npan; ++p)
         if (!pseen[p]) return fail("panel missing from the solve schedule");
