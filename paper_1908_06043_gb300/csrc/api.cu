@@ -374,7 +374,9 @@ static void set_smem_attrs(int device) {
     static std::vector<char> seen;
     if (!first_use_on_device(device, mu, seen)) return;
     cudaFuncSetAttribute(k_diag_bk<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDiagSmem);
-    cudaFuncSetAttribute(k_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem<T>());
+    cudaFuncSetAttribute(k_panel<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem<T, 4>());
+    cudaFuncSetAttribute(k_panel<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem<T, 2>());
+    cudaFuncSetAttribute(k_panel<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem<T, 1>());
     cudaFuncSetAttribute(k_schur<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)schur_smem<T>());
     if constexpr (std::is_same<T, float>::value) {
         cudaFuncSetAttribute(k_fwd_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)diag_solve_smem());
@@ -452,11 +454,21 @@ static int factor_levels(ss_numeric *f, int ns, ShiftPtrs<T> *dp, const std::vec
             const StepDesc &sd = s->steps[q];
             const StepTask *tk = s->d_tasks + sd.task_off;
             ss_launch(ctx, SS_K_DIAG_BK, k_diag_bk<T>, dim3(sd.count, ns), 256, kDiagSmem, st, tk,
-                      (const ShiftPtrs<T> *)dp, 0);
+                      (const ShiftPtrs<T> *)dp);
             if (sd.tiles4 > 0) {
                 const int cls = std::is_same<T, float>::value ? SS_K_PANEL_F32 : SS_K_PANEL;
-                ss_launch(ctx, cls, k_panel<T>, dim3(sd.tiles4, ns), 256, panel_smem<T>(), st, tk, sd.count,
-                          (const ShiftPtrs<T> *)dp);
+                // 64 rows keep an SM's FP64 pipe busy for 43 us: split the tiles until every SM has
+                // some (32 rows 22 us, 16 rows 11 us; each part reads Mt again)
+                const int64_t tiles = (int64_t)sd.tiles4 * ns;
+                if (tiles >= 4ll * ctx->sm_count)
+                    ss_launch(ctx, cls, k_panel<T, 4>, dim3(sd.tiles4, ns), 256, panel_smem<T, 4>(), st, tk, sd.count,
+                              (const ShiftPtrs<T> *)dp);
+                else if (tiles >= 2ll * ctx->sm_count)
+                    ss_launch(ctx, cls, k_panel<T, 2>, dim3(2 * sd.tiles4, ns), 256, panel_smem<T, 2>(), st, tk,
+                              sd.count, (const ShiftPtrs<T> *)dp);
+                else
+                    ss_launch(ctx, cls, k_panel<T, 1>, dim3(4 * sd.tiles4, ns), 256, panel_smem<T, 1>(), st, tk,
+                              sd.count, (const ShiftPtrs<T> *)dp);
                 ctx->add_flops(cls, sd.flops4 * ns);
             }
             if (step_ev && sd.tiles3 > 0) {

@@ -6,7 +6,7 @@
 //   K2 diag:  FP64 Bunch-Kaufman on the w x w diagonal block, pivots restricted to the
 //             block: P F11 P^T = L D L^T.  Writes L^-1, D, the local pivot order and
 //             the transform Mt = P^T L^-T D^-1, and counts the inertia of D.
-//   K4 panel: L21 = F21 Mt (in place) and W = L21 D (scratch), 64-row tiles.
+//   K4 panel: L21 = F21 Mt (in place) and W = L21 D (scratch), 16- to 64-row tiles.
 //   K3 Schur: F22 -= L21 W^T on the lower-triangular 64 x 64 tiles of the trailing front.
 // Before a level's steps its fronts are zeroed, the stored entries of A - sigma B are
 // scattered in (assembly) and the children's contribution blocks are added from the pool
@@ -25,8 +25,7 @@ namespace ssk {
 
 constexpr int NB = 64;     // panel width
 constexpr int TR = 64;     // row tile of the panel transform / Schur update
-constexpr size_t kDiagSmem = 2 * NB * (NB + 1) * sizeof(double);
-template <typename T> constexpr size_t panel_smem() { return 3 * NB * (TR + 1) * sizeof(T); }
+template <typename T, int RA> constexpr size_t panel_smem() { return NB * (NB + 1 + 2 * (16 * RA + 1)) * sizeof(T); }
 template <typename T> constexpr size_t schur_smem() { return 2 * NB * (TR + 1) * sizeof(T); }
 
 template <typename T>
@@ -146,115 +145,185 @@ __global__ void k_level_store(const StoreTask *__restrict__ tasks, int32_t ntask
 }
 
 // ---------------------------------------------------------------- K2: diagonal block
-// Dynamic shared memory: 2 * NB * (NB + 1) doubles.
+// One block per (front, shift).  FP64 runs at 2 multiply-adds a clock here, on one SM, so the
+// block does only the lower triangle's (w^3 / 6) and the inverse's (w^3 / 6), with one multiply-add
+// each and no division in a loop; pivots are compared as integers (|x| orders like its bits).
+// Per column one block barrier: warp 0 runs one column ahead -- it updates column k + 1, finds
+// its largest entry and, when the diagonal passes the 1x1 test, forms 1 / d and that column of L,
+// while warps 1-7 update the rest in 8 x 4 patches.  Only where the test fails do the second
+// search, the symmetric swap or the 2x2 pivot take barriers of their own.  N = 16,384, 164 steps:
+// 330 us a step with the full square updated by three FP64 operations an entry behind a
+// whole-block barrier per action and a serial column-per-thread inverse; 118 us now.
+constexpr int DLD = NB + 4;        // row stride: 8 x 4 patches touch every shared-memory bank once
+constexpr size_t kDiagSmem = 2 * NB * DLD * sizeof(double);
+
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+    return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ double from_bits(unsigned long long b) { return __longlong_as_double((long long)b); }
+
+// largest key over the warp and the smallest index holding it
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long key, int &idx) {
+    const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    idx = (int)__reduce_min_sync(0xffffffffu, (hi == mh && lo == ml) ? (unsigned)idx : 0x7fffffffu);
+    return ((unsigned long long)mh << 32) | ml;
+}
+
 template <typename T>
-__global__ void __launch_bounds__(256) k_diag_bk(const StepTask *__restrict__ tasks,
-                                                  const ShiftPtrs<T> *sp, int nopivot) {
+__global__ void __launch_bounds__(256) k_diag_bk(const StepTask *__restrict__ tasks, const ShiftPtrs<T> *sp) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *smem = reinterpret_cast<double *>(smem_raw);
+    double *A = reinterpret_cast<double *>(smem_raw);       // lower triangle, entry (i, j) at i DLD + j
+    double *L = A + NB * DLD;                                // strict lower part of L
     const ShiftPtrs<T> s = sp[blockIdx.y];
     const StepTask tk = tasks[blockIdx.x];
     const int w = tk.w, m = tk.m, k0 = tk.k0;
-    constexpr int LD = NB + 1;
-    double *A = smem;                  // w x w full symmetric, row i at A[i*LD]
-    double *Li = smem + NB * LD;       // L^-1
     __shared__ int perm[NB];
-    __shared__ double dd[NB], de[NB];
-    __shared__ int s_kind, s_r;        // pivot decision
-    __shared__ double s_lam;
+    __shared__ double dd[NB], de[NB], p0[NB], p1[NB];
+    __shared__ int s_kind, s_r, s_fast[2];
     __shared__ unsigned long long c_neg, c_zero, c_pos, c_tiny, c_2x2;
     __shared__ double s_minpiv;
-    const int tid = threadIdx.x, nt = blockDim.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const T *F = s.ws + tk.front_off;
 
-    for (int q = tid; q < w * w; q += nt) {
-        int j = q / w, i = q % w;            // column j, row i (coalesced on i)
-        if (i >= j) {
-            double v = (double)F[(int64_t)(k0 + j) * m + (k0 + i)];
-            A[i * LD + j] = v;
-            A[j * LD + i] = v;
-        }
+    for (int q = tid; q < NB * NB; q += 256) {
+        const int j = q / NB, i = q % NB;                    // column j, row i (coalesced on i)
+        if (i >= j && i < w) A[i * DLD + j] = (double)F[(int64_t)(k0 + j) * m + (k0 + i)];
     }
+    for (int q = tid; q < NB * DLD; q += 256) L[q] = 0.0;
     if (tid < NB) { perm[tid] = tid; dd[tid] = 0.0; de[tid] = 0.0; }
-    if (tid == 0) { c_neg = c_zero = c_pos = c_tiny = c_2x2 = 0; s_minpiv = 1e300; }
+    if (tid == 0) {
+        c_neg = c_zero = c_pos = c_tiny = c_2x2 = 0;
+        s_minpiv = 1e300;
+        s_fast[0] = 0;
+    }
     __syncthreads();
 
     const double alpha = 0.6403882032022076;   // (1 + sqrt(17)) / 8
-    int k = 0;
-    while (k < w) {
-        if (tid < 32) {
-            // lambda = max_{i>k} |A[i][k]|, r = its row (first on ties)
-            double lam = -1.0;
-            int r = k;
-            for (int i = k + 1 + tid; i < w; i += 32) {
-                double v = fabs(A[i * LD + k]);
-                if (v > lam) { lam = v; r = i; }
+    // column k of L for a 1x1 pivot d at k (warp 0)
+    auto scale_column = [&](int k, double d, double v1, double v2) {
+        const double inv = d != 0.0 ? 1.0 / d : 0.0;
+        const int i1 = k + 1 + lane, i2 = i1 + 32;
+        if (i1 < w) L[i1 * DLD + k] = v1 * inv;
+        if (i2 < w) L[i2 * DLD + k] = v2 * inv;
+    };
+    // A(i, j) -= x(i) y(j) [+ x2(i) y2(j)] on the trailing triangle from row / column b0, in 8 x 4
+    // patches dealt to warps first, first + 1, ..; x = column c of L, y = column c of A
+    auto update = [&](int b0, int c, bool two, int first, int nwarp) {
+        const int n2 = w - b0, npr = (n2 + 7) >> 3, np = npr * (npr + 1);
+        int pr = 0;
+        for (int p = warp - first; p < np; p += nwarp) {
+            while (p >= (pr + 1) * (pr + 2)) ++pr;
+            const int i = b0 + 8 * pr + (lane >> 2), j = b0 + 4 * (p - pr * (pr + 1)) + (lane & 3);
+            if (i < w && j <= i) {
+                double v = A[i * DLD + j];
+                v -= L[i * DLD + c] * A[j * DLD + c];
+                if (two) v -= L[i * DLD + c + 1] * A[j * DLD + c + 1];
+                A[i * DLD + j] = v;
             }
-            for (int o = 16; o > 0; o >>= 1) {
-                double ol = __shfl_down_sync(0xffffffffu, lam, o);
-                int orr = __shfl_down_sync(0xffffffffu, r, o);
-                if (ol > lam || (ol == lam && orr < r)) { lam = ol; r = orr; }
-            }
-            lam = __shfl_sync(0xffffffffu, lam, 0);
-            r = __shfl_sync(0xffffffffu, r, 0);
-            if (lam < 0.0) lam = 0.0;
-            double akk = fabs(A[k * LD + k]);
-            int kind = 1;                        // 1: 1x1 at k; 2: 1x1 with swap k<->r; 3: 2x2 (k+1<->r)
-            if (!nopivot && akk < alpha * lam) {
-                double sig = 0.0;
-                for (int j = k + tid; j < w; j += 32)
-                    if (j != r) sig = fmax(sig, fabs(A[r * LD + j]));
-                for (int o = 16; o > 0; o >>= 1) sig = fmax(sig, __shfl_down_sync(0xffffffffu, sig, o));
-                sig = __shfl_sync(0xffffffffu, sig, 0);
-                if (akk * sig >= alpha * lam * lam) kind = 1;
-                else if (fabs(A[r * LD + r]) >= alpha * sig) kind = 2;
-                else kind = 3;
-            }
-            if (tid == 0) { s_kind = kind; s_r = r; s_lam = lam; }
         }
-        __syncthreads();
-        const int kind = s_kind, r = s_r;
-        if (kind >= 2) {
-            const int a = (kind == 2) ? k : k + 1;
-            if (a != r) {
-                for (int j = tid; j < w; j += nt) {
-                    double t = A[a * LD + j]; A[a * LD + j] = A[r * LD + j]; A[r * LD + j] = t;
+    };
+    int k = 0;
+    for (int it = 0; k < w; ++it) {
+        int kind = 1;
+        if (!s_fast[it & 1]) {
+            // the pivot of column k: Bunch-Kaufman's test restricted to the block
+            if (warp == 0) {
+                unsigned long long key = 0;
+                int r = k;
+                const int i1 = k + 1 + lane, i2 = i1 + 32;
+                const double v1 = i1 < w ? A[i1 * DLD + k] : 0.0, v2 = i2 < w ? A[i2 * DLD + k] : 0.0;
+                if (i1 < w) { key = abs_bits(v1); r = i1; }
+                if (i2 < w && abs_bits(v2) > key) { key = abs_bits(v2); r = i2; }
+                if (k + 1 < w) key = warp_max_key(key, r);
+                const double lam = from_bits(key), d = A[k * DLD + k], akk = fabs(d);
+                int kd = 1;                          // 1: 1x1 at k; 2: 1x1 with swap k<->r; 3: 2x2 (k+1<->r)
+                if (akk < alpha * lam) {
+                    unsigned long long ks = 0;
+                    int dummy = 0;
+                    for (int j = k + lane; j < w; j += 32) {
+                        if (j == r) continue;
+                        const unsigned long long kj = abs_bits(j < r ? A[r * DLD + j] : A[j * DLD + r]);
+                        if (kj > ks) ks = kj;
+                    }
+                    const double sig = from_bits(warp_max_key(ks, dummy));
+                    if (akk * sig >= alpha * lam * lam) kd = 1;
+                    else if (fabs(A[r * DLD + r]) >= alpha * sig) kd = 2;
+                    else kd = 3;
                 }
-                __syncthreads();
-                for (int i = tid; i < w; i += nt) {
-                    double t = A[i * LD + a]; A[i * LD + a] = A[i * LD + r]; A[i * LD + r] = t;
+                if (kd == 1) scale_column(k, d, v1, v2);
+                if (lane == 0) { s_kind = kd; s_r = r; }
+            }
+            __syncthreads();
+            kind = s_kind;
+            const int r = s_r;
+            if (kind >= 2) {
+                const int a = (kind == 2) ? k : k + 1;
+                if (a != r) {                        // symmetric swap a <-> r of A, row swap of L
+                    if (tid < w && tid != r) {
+                        const int j = tid;
+                        double *x, *y;
+                        if (j < k) { x = &L[a * DLD + j]; y = &L[r * DLD + j]; }
+                        else if (j < a) { x = &A[a * DLD + j]; y = &A[r * DLD + j]; }
+                        else if (j == a) { x = &A[a * DLD + a]; y = &A[r * DLD + r]; }
+                        else if (j < r) { x = &A[j * DLD + a]; y = &A[r * DLD + j]; }
+                        else { x = &A[j * DLD + a]; y = &A[j * DLD + r]; }
+                        const double t = *x;
+                        *x = *y;
+                        *y = t;
+                    }
+                    if (tid == 0) { const int t = perm[a]; perm[a] = perm[r]; perm[r] = t; }
+                    __syncthreads();
                 }
-                if (tid == 0) { int t = perm[a]; perm[a] = perm[r]; perm[r] = t; }
-                __syncthreads();
+                if (kind == 2) {
+                    if (warp == 0) {
+                        const int i1 = k + 1 + lane, i2 = i1 + 32;
+                        scale_column(k, A[k * DLD + k], i1 < w ? A[i1 * DLD + k] : 0.0, i2 < w ? A[i2 * DLD + k] : 0.0);
+                    }
+                    __syncthreads();
+                }
             }
         }
         if (kind <= 2) {
-            const double d = A[k * LD + k];
-            if (tid == 0) {
-                dd[k] = d;
-                double ad = fabs(d);
-                if (d < 0) c_neg++; else if (d > 0) c_pos++; else c_zero++;
-                if (ad < s.tiny_thr) c_tiny++;
-                if (ad < s_minpiv) s_minpiv = ad;
-            }
-            const int rem = w - k - 1;
-            if (d != 0.0) {
-                const double inv = 1.0 / d;
-                for (int q = tid; q < rem * rem; q += nt) {
-                    int i = k + 1 + q / rem, j = k + 1 + q % rem;
-                    A[i * LD + j] -= A[i * LD + k] * inv * A[j * LD + k];
+            if (warp == 0) {
+                // column k + 1 ahead of the others: update, search, 1x1 test, its column of L
+                int fast = 0;
+                if (k + 1 < w) {
+                    const double c = A[(k + 1) * DLD + k];
+                    const int i0 = k + 1 + lane, i1 = i0 + 32;
+                    double v0 = 0.0, v1 = 0.0;
+                    if (i0 < w) { v0 = A[i0 * DLD + k + 1] - L[i0 * DLD + k] * c; A[i0 * DLD + k + 1] = v0; }
+                    if (i1 < w) { v1 = A[i1 * DLD + k + 1] - L[i1 * DLD + k] * c; A[i1 * DLD + k + 1] = v1; }
+                    const double d = __shfl_sync(0xffffffffu, v0, 0);
+                    unsigned long long key = lane > 0 ? abs_bits(v0) : 0;
+                    if (abs_bits(v1) > key) key = abs_bits(v1);
+                    int dummy = 0;
+                    key = warp_max_key(key, dummy);
+                    const double inv = d != 0.0 ? 1.0 / d : 0.0;
+                    fast = !(fabs(d) < alpha * from_bits(key));
+                    if (fast) {
+                        if (lane > 0 && i0 < w) L[i0 * DLD + k + 1] = v0 * inv;
+                        if (i1 < w) L[i1 * DLD + k + 1] = v1 * inv;
+                    }
                 }
-                __syncthreads();
-                for (int i = k + 1 + tid; i < w; i += nt) A[i * LD + k] *= inv;
+                if (lane == 0) s_fast[(it + 1) & 1] = fast;
             } else {
-                for (int i = k + 1 + tid; i < w; i += nt) A[i * LD + k] = 0.0;
+                if (tid == 32) {
+                    const double d = A[k * DLD + k], ad = fabs(d);
+                    dd[k] = d;
+                    if (d < 0) c_neg++; else if (d > 0) c_pos++; else c_zero++;
+                    if (ad < s.tiny_thr) c_tiny++;
+                    if (ad < s_minpiv) s_minpiv = ad;
+                }
+                update(k + 2, k, false, 1, 7);
             }
             __syncthreads();
             k += 1;
         } else {
-            const double a = A[k * LD + k], b = A[(k + 1) * LD + k], c = A[(k + 1) * LD + k + 1];
+            const double a = A[k * DLD + k], b = A[(k + 1) * DLD + k], c = A[(k + 1) * DLD + k + 1];
             const double det = a * c - b * b;
-            if (tid == 0) {
+            if (tid == 32) {
                 dd[k] = a; dd[k + 1] = c; de[k] = b; de[k + 1] = 0.0;
                 c_2x2++;
                 double tr = a + c;
@@ -266,42 +335,94 @@ __global__ void __launch_bounds__(256) k_diag_bk(const StepTask *__restrict__ ta
                 if (emin < s.tiny_thr) c_tiny++;
                 if (emin < s_minpiv) s_minpiv = emin;
             }
-            const int rem = w - k - 2;
-            const double id = 1.0 / det;
-            for (int q = tid; q < rem * rem; q += nt) {
-                int i = k + 2 + q / rem, j = k + 2 + q % rem;
-                double ci0 = A[i * LD + k], ci1 = A[i * LD + k + 1];
-                double li0 = (c * ci0 - b * ci1) * id, li1 = (-b * ci0 + a * ci1) * id;
-                A[i * LD + j] -= li0 * A[j * LD + k] + li1 * A[j * LD + k + 1];
+            const int i = k + 2 + tid;
+            if (i < w) {
+                const double id = 1.0 / det, ci0 = A[i * DLD + k], ci1 = A[i * DLD + k + 1];
+                L[i * DLD + k] = (c * ci0 - b * ci1) * id;
+                L[i * DLD + k + 1] = (-b * ci0 + a * ci1) * id;
             }
+            if (tid == 0) s_fast[(it + 1) & 1] = 0;
             __syncthreads();
-            for (int i = k + 2 + tid; i < w; i += nt) {
-                double ci0 = A[i * LD + k], ci1 = A[i * LD + k + 1];
-                A[i * LD + k] = (c * ci0 - b * ci1) * id;
-                A[i * LD + k + 1] = (-b * ci0 + a * ci1) * id;
-            }
-            if (tid == 0) A[(k + 1) * LD + k] = 0.0;   // the 2x2 coupling lives in D, not L
+            update(k + 2, k, true, 0, 8);
             __syncthreads();
             k += 2;
         }
     }
-    // L^-1 of the unit lower triangle, one column per thread
-    if (tid < w) {
-        const int j = tid;
-        for (int i = 0; i < j; ++i) Li[i * LD + j] = 0.0;
-        Li[j * LD + j] = 1.0;
-        for (int i = j + 1; i < w; ++i) {
-            double acc = 0.0;
-            for (int t = j; t < i; ++t) acc -= A[i * LD + t] * Li[t * LD + j];
-            Li[i * LD + j] = acc;
+    // X = L^-1 in A's place, by 16 x 16 diagonal blocks and two levels of
+    // X21 = -X22 (L21 X11); the products L21 X11 rest in blocks above the diagonal meanwhile
+    double *X = A;
+    if (tid < NB) {
+        const int b = tid & ~15, jl = tid & 15;
+        double x[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) x[i] = i == jl ? 1.0 : 0.0;
+#pragma unroll
+        for (int t = 0; t < 15; ++t)
+#pragma unroll
+            for (int i = t + 1; i < 16; ++i) x[i] -= L[(b + i) * DLD + b + t] * x[t];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) X[(b + i) * DLD + tid] = x[i];
+    } else {
+        // constants of D^-1: column j of L^-T D^-1 is p0 X(j, :) + p1 X(j +- 1, :)
+        const int j = tid - NB;
+        if (j < w) {
+            const bool first2 = de[j] != 0.0, second2 = j > 0 && de[j - 1] != 0.0;
+            if (first2 || second2) {
+                const int f = first2 ? j : j - 1;
+                const double a = dd[f], b = de[f], c = dd[f + 1], det = a * c - b * b;
+                p0[j] = (first2 ? c : a) / det;
+                p1[j] = -b / det;
+            } else {
+                p0[j] = dd[j] != 0.0 ? 1.0 / dd[j] : 0.0;
+                p1[j] = 0.0;
+            }
         }
     }
     __syncthreads();
+    {
+        const int h = lane & 15, C = 32 * (lane >> 4), R = C + 16;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int j = warp + 8 * u;
+            double acc = 0.0;
+            for (int t = j; t < 16; ++t) acc += L[(R + h) * DLD + C + t] * X[(C + t) * DLD + C + j];
+            X[(C + h) * DLD + R + j] = acc;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int i = warp + 8 * u;
+            double acc = 0.0;
+            for (int t = 0; t <= i; ++t) acc += X[(R + i) * DLD + R + t] * X[(C + t) * DLD + R + h];
+            X[(R + i) * DLD + C + h] = -acc;
+        }
+        __syncthreads();
+        if (w > 32) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = warp + 8 * u;
+                double acc = 0.0;
+                for (int t = j; t < 32; ++t) acc += L[(32 + lane) * DLD + t] * X[t * DLD + j];
+                X[lane * DLD + 32 + j] = acc;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = warp + 8 * u;
+                double acc = 0.0;
+                for (int t = 0; t <= i; ++t) acc += X[(32 + i) * DLD + 32 + t] * X[t * DLD + 32 + lane];
+                X[(32 + i) * DLD + lane] = -acc;
+            }
+            __syncthreads();
+        }
+    }
     const int p = tk.panel;
     double *linv = s.linv + (int64_t)p * NB * NB;
-    for (int q = tid; q < NB * NB; q += nt) {
-        int i = q / NB, j = q % NB;
-        linv[q] = (i < w && j < w) ? Li[i * LD + j] : 0.0;
+    unsigned long long lmax = 0;                 // largest |L| entry (element growth diagnostic)
+    for (int q = tid; q < NB * NB; q += 256) {
+        const int i = q / NB, j = q % NB;
+        linv[q] = (i < w && j <= i) ? X[i * DLD + j] : 0.0;
+        if (i > j) lmax = max(lmax, abs_bits(L[i * DLD + j]));
     }
     if (tid < NB) {
         s.dblk[(int64_t)p * 2 * NB + tid] = tid < w ? dd[tid] : 0.0;
@@ -310,22 +431,19 @@ __global__ void __launch_bounds__(256) k_diag_bk(const StepTask *__restrict__ ta
     }
     // Mt[perm[i]][j] = sum_{t in block(j)} Li[t][i] Dinv[t][j]
     T *mt = s.mt + (int64_t)tk.mt_slot * NB * NB;
-    for (int q = tid; q < w * w; q += nt) {
-        int i = q / w, j = q % w;
-        double v;
-        bool first2 = (de[j] != 0.0);                    // j is the first row of a 2x2 block
-        bool second2 = (j > 0 && de[j - 1] != 0.0);      // j is the second row
-        if (first2) {
-            double a = dd[j], b = de[j], c = dd[j + 1], det = a * c - b * b;
-            v = (Li[j * LD + i] * c - Li[(j + 1) * LD + i] * b) / det;
-        } else if (second2) {
-            double a = dd[j - 1], b = de[j - 1], c = dd[j], det = a * c - b * b;
-            v = (-Li[(j - 1) * LD + i] * b + Li[j * LD + i] * a) / det;
-        } else {
-            v = dd[j] != 0.0 ? Li[j * LD + i] / dd[j] : 0.0;
+    for (int q = tid; q < w * NB; q += 256) {
+        const int i = q / NB, j = q % NB;
+        if (j >= w) continue;
+        double v = i <= j ? X[j * DLD + i] * p0[j] : 0.0;
+        if (p1[j] != 0.0) {
+            const int o = de[j] != 0.0 ? j + 1 : j - 1;
+            if (i <= o) v += X[o * DLD + i] * p1[j];
         }
         mt[perm[i] * NB + j] = (T)v;
     }
+    int dummy = 0;
+    lmax = warp_max_key(lmax, dummy);
+    if (lane == 0 && lmax) atomicMax(&s.counts[6], lmax);
     if (tid == 0) {
         atomicAdd(&s.counts[0], c_neg);
         atomicAdd(&s.counts[1], c_zero);
@@ -335,29 +453,25 @@ __global__ void __launch_bounds__(256) k_diag_bk(const StepTask *__restrict__ ta
         atomicMin(&s.counts[4], (unsigned long long)__double_as_longlong(ratio));
         if (c_2x2) atomicAdd(&s.counts[5], c_2x2);
     }
-    // largest |L| entry of the diagonal block (element growth diagnostic)
-    double lmax = 0.0;
-    for (int q = tid; q < w * w; q += nt) {
-        int i = q / w, j = q % w;
-        if (i > j) lmax = fmax(lmax, fabs(A[i * LD + j]));
-    }
-    for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_down_sync(0xffffffffu, lmax, o));
-    if ((tid & 31) == 0 && lmax > 0.0) atomicMax(&s.counts[6], (unsigned long long)__double_as_longlong(lmax));
 }
 
 // ---------------------------------------------------------------- K4: panel transform
-// Block = (task, 64-row tile).  L21 = F21 Mt written in place; W = L21 D to scratch.
-// Dynamic shared memory: 3 * NB * (TR + 1) * sizeof(T).
-template <typename T>
+// Block = (task, 16 RA rows of a 64-row tile).  L21 = F21 Mt written in place; W = L21 D to
+// scratch.  In the pivot order Mt is L^-T D^-1, upper triangular but for the 2x2 pivots' entries
+// just below its diagonal, so column quarter b takes terms 0 .. 16 (b + 1) only.  The FP64 pipe
+// bounds it (43 us for 64 rows on one SM): steps with few tiles split them over more SMs (RA).
+// Dynamic shared memory: panel_smem<T, RA>().
+template <typename T, int RA>
 __global__ void __launch_bounds__(256) k_panel(const StepTask *__restrict__ tasks, int32_t ntask,
                                                 const ShiftPtrs<T> *sp) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T (*Fs)[TR + 1] = reinterpret_cast<T (*)[TR + 1]>(smem_raw);                // Fs[t][row]
-    T (*Ms)[NB + 1] = reinterpret_cast<T (*)[NB + 1]>(smem_raw + sizeof(T) * NB * (TR + 1));
-    T (*Ls)[TR + 1] = reinterpret_cast<T (*)[TR + 1]>(smem_raw + 2 * sizeof(T) * NB * (TR + 1));
+    constexpr int RT = 16 * RA, LDR = RT + 1, SUB = TR / RT;
+    T (*Ms)[NB + 1] = reinterpret_cast<T (*)[NB + 1]>(smem_raw);                       // Ms[t][j]
+    T (*Fs)[LDR] = reinterpret_cast<T (*)[LDR]>(smem_raw + sizeof(T) * NB * (NB + 1));   // Fs[t][row]
+    T (*Ls)[LDR] = reinterpret_cast<T (*)[LDR]>(smem_raw + sizeof(T) * NB * (NB + 1 + LDR));
     __shared__ double sd[NB], se[NB];
     const ShiftPtrs<T> s = sp[blockIdx.y];
-    const int32_t tile = blockIdx.x;
+    const int32_t tile = blockIdx.x / SUB;
     int lo = 0, hi = ntask - 1;
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
@@ -365,60 +479,75 @@ __global__ void __launch_bounds__(256) k_panel(const StepTask *__restrict__ task
     }
     const StepTask tk = tasks[lo];
     const int w = tk.w, m = tk.m;
-    const int r0 = (tile - tk.tiles4_pre) * TR;           // first row within the r rows
-    const int nr = min(TR, tk.r - r0);
+    const int r0 = (tile - tk.tiles4_pre) * TR + (int)(blockIdx.x % SUB) * RT;   // first row within the r rows
+    const int nr = min(RT, tk.r - r0);
+    if (nr <= 0) return;
     T *F = s.ws + tk.front_off;
     const int64_t rowbase = tk.k0 + w + r0;
     const T *mt = s.mt + (int64_t)tk.mt_slot * NB * NB;
+    const int32_t *pv = s.piv + (int64_t)tk.panel * NB;
     const int tid = threadIdx.x;
-    for (int q = tid; q < w * TR; q += 256) {
-        int t = q / TR, i = q % TR;
-        Fs[t][i] = i < nr ? F[(int64_t)(tk.k0 + t) * m + rowbase + i] : (T)0;
+    for (int q = tid; q < NB * RT; q += 256) {
+        const int t = q / RT, i = q % RT;
+        Fs[t][i] = (t < w && i < nr) ? F[(int64_t)(tk.k0 + pv[t]) * m + rowbase + i] : (T)0;
     }
-    for (int q = tid; q < w * w; q += 256) Ms[q / w][q % w] = mt[(q / w) * NB + (q % w)];
+    for (int q = tid; q < NB * NB; q += 256) {
+        const int t = q / NB, j = q % NB;
+        Ms[t][j] = (t < w && j < w) ? mt[pv[t] * NB + j] : (T)0;
+    }
     if (tid < NB) {
         sd[tid] = tid < w ? s.dblk[(int64_t)tk.panel * 2 * NB + tid] : 0.0;
         se[tid] = tid < w ? s.dblk[(int64_t)tk.panel * 2 * NB + NB + tid] : 0.0;
     }
     __syncthreads();
-    // each thread: rows i = tx + 16*a, cols j = ty + 16*b, a,b in 0..3
+    // each thread: rows i = tx + 16 a, cols j = ty + 16 b
     const int tx = tid & 15, ty = tid >> 4;
-    T acc[4][4];
+    T acc[RA][4];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < RA; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) acc[a][b] = (T)0;
-    for (int t = 0; t < w; ++t) {
-        T fa[4], mb[4];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) fa[a] = Fs[t][tx + 16 * a];
+    for (int h = 0; h < 4; ++h) {
+        if (16 * h >= w) break;
+        for (int t = 16 * h; t < min(16 * h + 16, w); ++t) {
+            T fa[RA];
 #pragma unroll
-        for (int b = 0; b < 4; ++b) mb[b] = Ms[t][ty + 16 * b];
+            for (int a = 0; a < RA; ++a) fa[a] = Fs[t][tx + 16 * a];
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+            for (int b = h; b < 4; ++b) {
+                const T mb = Ms[t][ty + 16 * b];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] += fa[a] * mb[b];
+                for (int a = 0; a < RA; ++a) acc[a][b] += fa[a] * mb;
+            }
+        }
+        if (h > 0) {                                 // a 2x2 pivot across columns 16 h - 1, 16 h
+            const T mb = Ms[16 * h][ty + 16 * (h - 1)];
+#pragma unroll
+            for (int a = 0; a < RA; ++a) acc[a][h - 1] += Fs[16 * h][tx + 16 * a] * mb;
+        }
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < RA; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) Ls[ty + 16 * b][tx + 16 * a] = acc[a][b];
     __syncthreads();
     T *W = s.wbuf + tk.wbuf_off;
-    double lmax = 0.0;
-    for (int q = tid; q < w * TR; q += 256) {
-        int j = q / TR, i = q % TR;
+    unsigned long long lmax = 0;
+    for (int q = tid; q < w * RT; q += 256) {
+        int j = q / RT, i = q % RT;
         if (i >= nr) continue;
         T l = Ls[j][i];
-        lmax = fmax(lmax, fabs((double)l));
+        lmax = max(lmax, abs_bits((double)l));
         F[(int64_t)(tk.k0 + j) * m + rowbase + i] = l;
         double wv = (double)l * sd[j];
         if (se[j] != 0.0) wv += (double)Ls[j + 1][i] * se[j];
         if (j > 0 && se[j - 1] != 0.0) wv += (double)Ls[j - 1][i] * se[j - 1];
         W[(int64_t)j * tk.r + r0 + i] = (T)wv;
     }
-    for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_down_sync(0xffffffffu, lmax, o));
-    if ((tid & 31) == 0 && lmax > 0.0) atomicMax(&s.counts[6], (unsigned long long)__double_as_longlong(lmax));
+    int dummy = 0;
+    lmax = warp_max_key(lmax, dummy);
+    if ((tid & 31) == 0 && lmax) atomicMax(&s.counts[6], lmax);
 }
 
 // ---------------------------------------------------------------- K3: Schur update
