@@ -12,6 +12,7 @@
 
 #include "factor_kernels.cuh"
 #include "fold_kernels.cuh"
+#include "fold_tc.cuh"
 #include "internal.h"
 #include "solve_kernels.cuh"
 #include "sparse_kernels.cuh"
@@ -290,11 +291,29 @@ int ss_symbolic_upload(ss_symbolic *s) {
     SweepLevel *dl = nullptr;
     UP(lev, dl);
     s->d_sweep_lev = dl;
-    UP(s->solve_tile128_pre, s->d_solve_tile128_pre);
-    std::vector<FoldLevel> flev(s->solve_levels.size());
-    for (size_t L = 0; L < flev.size(); ++L)
-        flev[L] = FoldLevel{(int32_t)s->solve_levels[L].panel_off, s->solve_levels[L].count,
-                            s->solve_levels[L].tiles128, 0};
+    // FP64 solves: every level's tiles of 64 and of 128 rows
+    std::vector<FoldLevel> flev;
+    std::vector<FoldTile> t64, t128;
+    for (const SolveLevel &sl : s->solve_levels) {
+        FoldLevel fl{(int32_t)t128.size(), 0, (int32_t)t64.size(), 0};
+        for (int32_t q = 0; q < sl.count; ++q) {
+            const PanelDesc &pd = s->panels[s->solve_panels[sl.panel_off + q]];
+            const int32_t below = pd.k0 + pd.w, r = pd.m - below;
+            const int64_t off = pd.front_off + (int64_t)pd.k0 * pd.m + below, ix = pd.idx_off + below;
+            for (int32_t r0 = 0; r0 < r; r0 += 64)
+                t64.push_back(FoldTile{off + r0, ix + r0, pd.m, pd.w, std::min(64, r - r0), pd.g0});
+            for (int32_t r0 = 0; r0 < r; r0 += kFoldRows)
+                t128.push_back(FoldTile{off + r0, ix + r0, pd.m, pd.w, std::min(kFoldRows, r - r0), pd.g0});
+        }
+        fl.tiles = (int32_t)t128.size() - fl.tile0;
+        fl.tiles_64 = (int32_t)t64.size() - fl.tile0_64;
+        flev.push_back(fl);
+    }
+    FoldTile *dt64 = nullptr, *dt128 = nullptr;
+    UP(t64, dt64);
+    s->d_fold_tiles64 = dt64;
+    UP(t128, dt128);
+    s->d_fold_tiles128 = dt128;
     FoldLevel *df = nullptr;
     UP(flev, df);
     s->d_fold_lev = df;
@@ -305,15 +324,15 @@ int ss_symbolic_upload(ss_symbolic *s) {
 void ss_symbolic_free_device(ss_symbolic *s) {
     void *ptrs[] = {s->d_rowptr, s->d_colind, s->d_iperm, s->d_perm, s->d_idx, s->d_asm_e,
                     s->d_asm_dest, s->d_relmap, s->d_ext_tasks, s->d_panels, s->d_store_tasks, s->d_tasks,
-                    s->d_solve_panels, s->d_solve_tile_pre, s->d_col_panel, s->d_sweep_lev, s->d_solve_tile128_pre,
-                    s->d_fold_lev};
+                    s->d_solve_panels, s->d_solve_tile_pre, s->d_col_panel, s->d_sweep_lev, s->d_fold_tiles64,
+                    s->d_fold_tiles128, s->d_fold_lev};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     s->d_rowptr = nullptr; s->d_colind = nullptr; s->d_iperm = nullptr; s->d_perm = nullptr;
     s->d_idx = nullptr; s->d_asm_e = nullptr; s->d_asm_dest = nullptr; s->d_relmap = nullptr;
     s->d_ext_tasks = nullptr; s->d_panels = nullptr; s->d_store_tasks = nullptr; s->d_tasks = nullptr;
     s->d_solve_panels = nullptr; s->d_solve_tile_pre = nullptr; s->d_col_panel = nullptr;
-    s->d_sweep_lev = nullptr; s->d_solve_tile128_pre = nullptr; s->d_fold_lev = nullptr;
+    s->d_sweep_lev = nullptr; s->d_fold_tiles64 = nullptr; s->d_fold_tiles128 = nullptr; s->d_fold_lev = nullptr;
 }
 
 // ------------------------------------------------------------------ norms
@@ -389,6 +408,7 @@ static void set_smem_attrs(int device) {
         cudaFuncSetAttribute(k_fold_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFoldMidSmem);
         for (int nc = 1; nc <= kFoldMaxNc; ++nc)
             cudaFuncSetAttribute(fold_sweeps_kernel(nc), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFoldSmem);
+        cudaFuncSetAttribute(sstc::k_fold_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sstc::kFtSmem);
         cudaFuncSetAttribute(sstc::k_schur_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sstc::kSchurTcSmem);
         cudaFuncSetAttribute(sstc::k_tc_selftest, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sstc::kSelftestSmem);
@@ -1075,8 +1095,8 @@ static FoldArgs fold_args(const ss_numeric *f, int j, int k, bool full) {
     a.npan = (int32_t)s->panels.size();
     a.k = k;
     a.full = full ? 1 : 0;
-    a.solve_panels = s->d_solve_panels;
-    a.tile_pre = s->d_solve_tile128_pre;
+    a.tiles = (const FoldTile *)s->d_fold_tiles128;
+    a.tiles_64 = (const FoldTile *)s->d_fold_tiles64;
     a.panels = s->d_panels;
     a.idx = s->d_idx;
     a.linv = f->linv[j];
@@ -1143,6 +1163,16 @@ static int fold_per_step(ss_numeric *f, int j, double *b, int k, bool full) {
     return SS_OK;
 }
 
+// Whether a solve of k columns runs on the tensor cores (fold_tc.cuh): where the FP64 work it takes
+// off the CUDA cores, 4.4 ps per entry of L and column, outweighs its longer items, 16 us more per
+// level.  Measured (ms a solve, CUDA cores / tensor cores): N = 864 (13 levels) k = 129 0.48 / 0.50,
+// k = 304 0.78 / 0.54; N = 5,280 (55) k = 17 1.48 / 1.85, k = 48 2.58 / 1.93, k = 304 11.7 / 2.94;
+// N = 16,384 (129) k = 304 61.8 / 10.3.
+static bool fold_uses_tc(const ss_symbolic *s, int k) {
+    return s->ctx->gemm_mode == SS_GEMM_TENSOR && k > kFoldMaxNc &&
+           (double)s->info.l_offdiag_entries * k >= 3.6e6 * (double)s->solve_levels.size();
+}
+
 // both sweeps in one cooperative launch of k_fold_sweeps (every block resident, a bounded grid
 // barrier between levels).  Returns SS_ERR_TIMEOUT if a barrier gave up.
 static int fold_sweeps(ss_numeric *f, int j, double *b, int k, bool full) {
@@ -1164,13 +1194,16 @@ static int fold_sweeps(ss_numeric *f, int j, double *b, int k, bool full) {
     FoldArgs a = fold_args(f, j, k, full);
     a.bar = ctx->d_bar;
     a.limit = 20000000;        // polls of about 64 ns: ~1 s per barrier
+    const bool tc = fold_uses_tc(s, k);
     void *args[] = {(void *)&a, (void *)&b};
+    void *kern = tc ? (void *)sstc::k_fold_tc : (void *)fold_sweeps_kernel(nc);
     g_ss_launches.fetch_add(1, std::memory_order_relaxed);
     size_t slot = 0;
     const bool prof = ctx->prof_mask & (1u << SS_K_SOLVE);
     if (prof) slot = ss_prof_begin(ctx, SS_K_SOLVE);
-    SS_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((void *)fold_sweeps_kernel(nc), dim3(nb), dim3(kFoldThreads), args,
-                                                 kFoldSmem, st));
+    static_assert(kFoldThreads == sstc::kFtThreads, "the middle step runs in blocks of this size");
+    SS_CUDA_TRY(ctx, cudaLaunchCooperativeKernel(kern, dim3(nb), dim3(kFoldThreads), args,
+                                                 tc ? sstc::kFtSmem : kFoldSmem, st));
     if (prof) ss_prof_end(ctx, SS_K_SOLVE, slot);
     ctx->add_flops(SS_K_SOLVE, flops);
     int herr = 0;

@@ -95,11 +95,16 @@ __global__ void __launch_bounds__(256) k_fold_panels(const PanelDesc *__restrict
     }
 }
 
-struct FoldLevel {          // device copy of a solve level
-    int32_t panel_off;      // into the level-ordered panel list
-    int32_t count;          // panels
-    int32_t tiles;          // 128-row tiles of their below-diagonal rows
-    int32_t pad;
+// A tile of a panel's rows below its diagonal block, so that a block needs one load to find its
+// work: entry (i, t) of G is arena[off + t m + i], its global row idx[idx + i], its global column
+// g0 + t; nr rows, w columns.
+struct FoldTile {
+    int64_t off, idx;
+    int32_t m, w, nr, g0;
+};
+struct FoldLevel {          // a solve level's tiles
+    int32_t tile0, tiles;   // 128-row tiles (fold_kernels.cuh)
+    int32_t tile0_64, tiles_64;   // 64-row tiles (fold_tc.cuh)
 };
 
 struct FoldArgs {
@@ -107,8 +112,7 @@ struct FoldArgs {
     int32_t nlev, npan;
     int32_t k;
     int32_t full;           // 1: forward, D^-1 and backward; 0: L^-T only
-    const int32_t *solve_panels;
-    const int32_t *tile_pre;        // per level-ordered panel: exclusive prefix of its tiles in the level
+    const FoldTile *tiles, *tiles_64;
     const PanelDesc *panels;
     const int32_t *idx;
     const double *linv;
@@ -128,51 +132,37 @@ struct FoldItem {
     int32_t nt;             // panel columns of the item
 };
 
-__device__ __forceinline__ PanelDesc fold_panel(const FoldArgs &a, const FoldLevel &lv, int tile, int &r0) {
-    const int32_t *tp = a.tile_pre + lv.panel_off;
-    int lo = 0, hi = lv.count - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (tp[mid] <= tile) lo = mid; else hi = mid - 1;
-    }
-    r0 = (tile - tp[lo]) * kFoldRows;
-    return a.panels[a.solve_panels[lv.panel_off + lo]];
-}
-
 // forward item `sub` of a tile: rows 32 (sub / 4) .. + 31 (one a lane), columns 16 (sub % 4) .. + 15
-__device__ __forceinline__ void fold_load_fwd(const FoldArgs &a, const FoldLevel &lv, int tile, int sub, FoldItem &it) {
-    int r0;
-    const PanelDesc pd = fold_panel(a, lv, tile, r0);
-    const int t0 = 16 * (sub & 3), i = r0 + 32 * (sub >> 2) + (threadIdx.x & 31), r = pd.m - pd.k0 - pd.w;
-    it.nt = min(16, pd.w - t0);
-    if (r0 + 32 * (sub >> 2) >= r) it.nt = 0;
-    it.live = i < r ? 1 : 0;
-    it.g0 = pd.g0 + t0;
+__device__ __forceinline__ void fold_load_fwd(const FoldArgs &a, const FoldLevel &lv, int e, FoldItem &it) {
+    const FoldTile tl = a.tiles[lv.tile0 + (e >> 4)];
+    const int sub = e & 15, t0 = 16 * (sub & 3), i0 = 32 * (sub >> 2), i = i0 + (threadIdx.x & 31);
+    it.nt = i0 < tl.nr ? min(16, tl.w - t0) : 0;
+    it.live = i < tl.nr ? 1 : 0;
+    it.g0 = tl.g0 + t0;
     if (it.nt <= 0) return;
-    it.row[0] = it.live ? a.idx[pd.idx_off + pd.k0 + pd.w + i] : 0;
-    const double *F = a.arena + pd.front_off + (int64_t)(pd.k0 + t0) * pd.m + pd.k0 + pd.w + i;
+    it.row[0] = it.live ? a.idx[tl.idx + i] : 0;
+    const double *F = a.arena + tl.off + (int64_t)t0 * tl.m + i;
 #pragma unroll
-    for (int u = 0; u < 16; ++u) it.g[u] = (it.live && u < it.nt) ? __ldg(F + (int64_t)u * pd.m) : 0.0;
+    for (int u = 0; u < 16; ++u) it.g[u] = (it.live && u < it.nt) ? __ldg(F + (int64_t)u * tl.m) : 0.0;
 }
 
 // backward item `sub` of a tile: its 128 rows (lane + 32 j), columns 4 sub .. + 3
-__device__ __forceinline__ void fold_load_bwd(const FoldArgs &a, const FoldLevel &lv, int tile, int sub, FoldItem &it) {
-    int r0;
-    const PanelDesc pd = fold_panel(a, lv, tile, r0);
-    const int t0 = 4 * sub, r = pd.m - pd.k0 - pd.w;
-    it.nt = min(4, pd.w - t0);
+__device__ __forceinline__ void fold_load_bwd(const FoldArgs &a, const FoldLevel &lv, int e, FoldItem &it) {
+    const FoldTile tl = a.tiles[lv.tile0 + (e >> 4)];
+    const int t0 = 4 * (e & 15);
+    it.nt = min(4, tl.w - t0);
     it.live = 0;
-    it.g0 = pd.g0 + t0;
+    it.g0 = tl.g0 + t0;
     if (it.nt <= 0) return;
-    const double *F = a.arena + pd.front_off + (int64_t)(pd.k0 + t0) * pd.m + pd.k0 + pd.w;
+    const double *F = a.arena + tl.off + (int64_t)t0 * tl.m;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const int i = r0 + (int)(threadIdx.x & 31) + 32 * j;
-        const bool in = i < r;
+        const int i = (int)(threadIdx.x & 31) + 32 * j;
+        const bool in = i < tl.nr;
         it.live |= (in ? 1 : 0) << j;
-        it.row[j] = in ? a.idx[pd.idx_off + pd.k0 + pd.w + i] : 0;
+        it.row[j] = in ? a.idx[tl.idx + i] : 0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) it.g[4 * j + u] = (in && u < it.nt) ? __ldg(F + (int64_t)u * pd.m + i) : 0.0;
+        for (int u = 0; u < 4; ++u) it.g[4 * j + u] = (in && u < it.nt) ? __ldg(F + (int64_t)u * tl.m + i) : 0.0;
     }
 }
 
@@ -267,16 +257,15 @@ __device__ __forceinline__ void fold_bwd(const FoldItem &it, double *b, int k, i
 // item `sub` of a tile is rows 16 (sub / 2) .. + 15 and columns 32 (sub % 2) .. + 31, one column a
 // lane, so nothing is summed across lanes (a lane's 16 entries are one 128-byte line of its
 // column).  N = 16,384, k = 304: 63.1 ms a solve with fold_bwd's items, 61.8 ms with these.
-__device__ __forceinline__ void fold_load_bwd_wide(const FoldArgs &a, const FoldLevel &lv, int tile, int sub, FoldItem &it) {
-    int r0;
-    const PanelDesc pd = fold_panel(a, lv, tile, r0);
-    const int lane = threadIdx.x & 31, t0 = 32 * (sub & 1), i0 = r0 + 16 * (sub >> 1), r = pd.m - pd.k0 - pd.w;
-    it.nt = i0 < r ? min(32, pd.w - t0) : 0;
-    it.g0 = pd.g0 + t0;
+__device__ __forceinline__ void fold_load_bwd_wide(const FoldArgs &a, const FoldLevel &lv, int e, FoldItem &it) {
+    const FoldTile tl = a.tiles[lv.tile0 + (e >> 4)];
+    const int sub = e & 15, lane = threadIdx.x & 31, t0 = 32 * (sub & 1), i0 = 16 * (sub >> 1);
+    it.nt = i0 < tl.nr ? min(32, tl.w - t0) : 0;
+    it.g0 = tl.g0 + t0;
     if (it.nt <= 0) return;
-    it.live = min(16, r - i0);
-    it.row[0] = lane < it.live ? a.idx[pd.idx_off + pd.k0 + pd.w + i0 + lane] : 0;
-    const double *F = a.arena + pd.front_off + (int64_t)(pd.k0 + t0 + lane) * pd.m + pd.k0 + pd.w + i0;
+    it.live = min(16, tl.nr - i0);
+    it.row[0] = lane < it.live ? a.idx[tl.idx + i0 + lane] : 0;
+    const double *F = a.arena + tl.off + (int64_t)(t0 + lane) * tl.m + i0;
 #pragma unroll
     for (int u = 0; u < 16; ++u) it.g[u] = (u < it.live && lane < it.nt) ? __ldg(F + u) : 0.0;
 }
@@ -396,16 +385,16 @@ __global__ void __launch_bounds__(kFoldThreads, 1) k_fold_sweeps(const FoldArgs 
     FoldItem it;
     if (a.full) {
         FoldLevel lv = a.lev[0];
-        if (q0 < lv.tiles * 16 * nch) fold_load_fwd(a, lv, (q0 % (lv.tiles * 16)) >> 4, q0 & 15, it);
+        if (q0 < lv.tiles * 16 * nch) fold_load_fwd(a, lv, q0 % (lv.tiles * 16), it);
         for (int L = 0; L < a.nlev; ++L) {
             const int per = lv.tiles * 16;
+            const FoldLevel nx = L + 1 < a.nlev ? a.lev[L + 1] : FoldLevel{0, 0, 0, 0};
             for (int q = q0; q < per * nch; q += nw) {
-                if (q != q0) fold_load_fwd(a, lv, (q % per) >> 4, q & 15, it);
+                if (q != q0) fold_load_fwd(a, lv, q % per, it);
                 fold_fwd<NC>(it, ws, b, k, (q / per) * NC);
             }
             // the next level's entries, before the barrier
-            const FoldLevel nx = L + 1 < a.nlev ? a.lev[L + 1] : FoldLevel{0, 0, 0, 0};
-            if (q0 < nx.tiles * 16 * nch) fold_load_fwd(a, nx, (q0 % (nx.tiles * 16)) >> 4, q0 & 15, it);
+            if (q0 < nx.tiles * 16 * nch) fold_load_fwd(a, nx, q0 % (nx.tiles * 16), it);
             if (lv.tiles > 0 && !grid_barrier(a.bar, nb, a.limit)) return;
             lv = nx;
         }
@@ -420,21 +409,21 @@ __global__ void __launch_bounds__(kFoldThreads, 1) k_fold_sweeps(const FoldArgs 
     const bool wide = nch > 1;
     auto load_bwd = [&](const FoldLevel &l, int q) {
         const int e = q % (l.tiles * 16);
-        if (wide) fold_load_bwd_wide(a, l, e >> 4, e & 15, it);
-        else fold_load_bwd(a, l, e >> 4, e & 15, it);
+        if (wide) fold_load_bwd_wide(a, l, e, it);
+        else fold_load_bwd(a, l, e, it);
     };
     FoldLevel lv = a.lev[a.nlev - 1];
     if (q0 < lv.tiles * 16 * nch) load_bwd(lv, q0);
     if (!grid_barrier(a.bar, nb, a.limit)) return;
     for (int L = a.nlev - 1; L >= 0; --L) {
         const int per = lv.tiles * 16;
+        const FoldLevel nx = L > 0 ? a.lev[L - 1] : FoldLevel{0, 0, 0, 0};
         for (int q = q0; q < per * nch; q += nw) {
             if (q != q0) load_bwd(lv, q);
             if (wide) fold_bwd_wide<NC>(it, ws, b, k, (q / per) * NC);
             else fold_bwd<NC>(it, b, k, 0);
         }
         if (L == 0) break;
-        const FoldLevel nx = a.lev[L - 1];
         if (q0 < nx.tiles * 16 * nch) load_bwd(nx, q0);
         if (lv.tiles > 0 && !grid_barrier(a.bar, nb, a.limit)) return;
         lv = nx;
@@ -452,13 +441,13 @@ __global__ void __launch_bounds__(kFoldThreads) k_fold_level(const FoldArgs a, i
     FoldItem it;
     const int c0 = (int)(q / per) * NC, e = (int)(q % per);
     if (backward && nch > 1) {
-        fold_load_bwd_wide(a, lv, e >> 4, e & 15, it);
+        fold_load_bwd_wide(a, lv, e, it);
         fold_bwd_wide<NC>(it, s_ws + (threadIdx.x >> 5) * 16 * kFoldMaxNc, b, a.k, c0);
     } else if (backward) {
-        fold_load_bwd(a, lv, e >> 4, e & 15, it);
+        fold_load_bwd(a, lv, e, it);
         fold_bwd<NC>(it, b, a.k, c0);
     } else {
-        fold_load_fwd(a, lv, e >> 4, e & 15, it);
+        fold_load_fwd(a, lv, e, it);
         fold_fwd<NC>(it, s_ws + (threadIdx.x >> 5) * 16 * kFoldMaxNc, b, a.k, c0);
     }
 }

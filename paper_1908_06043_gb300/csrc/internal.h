@@ -219,7 +219,6 @@ struct ss_symbolic {
     std::vector<int32_t> solve_panels;       // panel ids grouped by solve level
     std::vector<SolveLevel> solve_levels;
     std::vector<int32_t> solve_tile_pre;     // per solve_panels entry: exclusive row-tile prefix
-    std::vector<int32_t> solve_tile128_pre;  // the same for 128-row tiles
     int32_t max_rows_below = 0;              // most rows below a panel's diagonal block
 
     ss_symbolic_info info{};
@@ -241,8 +240,8 @@ struct ss_symbolic {
     int32_t *d_solve_tile_pre = nullptr;
     int32_t *d_col_panel = nullptr;          // permuted column -> panel
     void *d_sweep_lev = nullptr;             // solve levels for the FP32 sweep kernel (SweepLevel)
-    int32_t *d_solve_tile128_pre = nullptr;
-    void *d_fold_lev = nullptr;              // solve levels for the FP64 sweep kernel (FoldLevel)
+    void *d_fold_lev = nullptr;              // solve levels for the FP64 sweep kernels (FoldLevel)
+    void *d_fold_tiles64 = nullptr, *d_fold_tiles128 = nullptr;   // their tiles (FoldTile)
 };
 
 struct ss_numeric {

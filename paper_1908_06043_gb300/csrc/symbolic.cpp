@@ -565,7 +565,6 @@ static int analyze_impl(ss_ctx *ctx, int64_t n, const int64_t *rowptr, const int
     s->solve_panels.clear();
     s->solve_levels.clear();
     s->solve_tile_pre.clear();
-    s->solve_tile128_pre.clear();
     s->max_rows_below = 0;
     for (int32_t l = 0; l < nplev; ++l) {
         SolveLevel sl{(int64_t)s->solve_panels.size(), 0, 0, 0.0, 0};
@@ -573,7 +572,6 @@ static int analyze_impl(ss_ctx *ctx, int64_t n, const int64_t *rowptr, const int
             const PanelDesc &pd = s->panels[p];
             s->solve_panels.push_back(p);
             s->solve_tile_pre.push_back(sl.row_tiles);
-            s->solve_tile128_pre.push_back(sl.tiles128);
             sl.row_tiles += (int32_t)cdiv(pd.m - pd.k0 - pd.w, 64);
             sl.tiles128 += (int32_t)cdiv(pd.m - pd.k0 - pd.w, 128);
             s->max_rows_below = std::max(s->max_rows_below, pd.m - pd.k0 - pd.w);
@@ -851,7 +849,6 @@ static int validate_impl(const ss_symbolic *s, std::string &why) {
             if (p < 0 || p >= npan || pseen[p]) return fail("solve level panel id");
             pseen[p] = 1;
             if (s->solve_tile_pre[sl.panel_off + t] != tiles) return fail("solve tile prefix");
-            if (s->solve_tile128_pre[sl.panel_off + t] != tiles128) return fail("solve tile prefix (128 rows)");
             const PanelDesc &pd = s->panels[p];
             tiles += (pd.m - pd.k0 - pd.w + 63) / 64;
             tiles128 += (pd.m - pd.k0 - pd.w + 127) / 128;
