@@ -1380,12 +1380,31 @@ int spmm_launch_ld(ss_symbolic *s, const double *a, const double *b, const doubl
 #define SS_SPMM_ROWS(NC)                                                                                     \
     ss_launch(ctx, SS_K_SPMM, sss::k_spmm_rows<NC>, grid, 256, 0, ctx->stream, s->n, s->d_rowptr, s->d_colind, a, b, \
               alpha, beta, X, ldx, k, Y, ldy)
-    if (k <= 4)
-        ss_launch(ctx, SS_K_SPMM, sss::k_spmm_nnz<4>, grid, 256, 0, ctx->stream, s->n, s->d_rowptr, s->d_colind, a, b,
-                  alpha, beta, X, ldx, k, Y, ldy);
-    else if (k < 16)
-        ss_launch(ctx, SS_K_SPMM, sss::k_spmm_nnz<16>, grid, 256, 0, ctx->stream, s->n, s->d_rowptr, s->d_colind, a,
-                  b, alpha, beta, X, ldx, k, Y, ldy);
+#define SS_SPMM_NNZ(KW)                                                                                        \
+    do {                                                                                                       \
+        const dim3 g(grid, (unsigned)nch);                                                                     \
+        if (beta)                                                                                              \
+            ss_launch(ctx, SS_K_SPMM, sss::k_spmm_nnz<KW, true>, g, 256, 0, ctx->stream, s->n, s->d_rowptr,    \
+                      s->d_colind, a, b, alpha, beta, X, ldx, k, Y, ldy);                                      \
+        else                                                                                                   \
+            ss_launch(ctx, SS_K_SPMM, sss::k_spmm_nnz<KW, false>, g, 256, 0, ctx->stream, s->n, s->d_rowptr,   \
+                      s->d_colind, a, b, alpha, beta, X, ldx, k, Y, ldy);                                      \
+    } while (0)
+    // lanes over nonzeros below 16 columns, and up to 48 where the rows are long enough to fill the
+    // lanes (columns over lanes leave k mod 32 of them idle)
+    if (k < 16 || (k < 48 && s->nnz >= 64 * s->n)) {
+        const int nch = (k + 7) / 8;
+        switch ((k + nch - 1) / nch) {
+            case 1: SS_SPMM_NNZ(1); break;
+            case 2: SS_SPMM_NNZ(2); break;
+            case 3: SS_SPMM_NNZ(3); break;
+            case 4: SS_SPMM_NNZ(4); break;
+            case 5: SS_SPMM_NNZ(5); break;
+            case 6: SS_SPMM_NNZ(6); break;
+            case 7: SS_SPMM_NNZ(7); break;
+            default: SS_SPMM_NNZ(8); break;
+        }
+    }
     else if (k <= 512) {
         switch ((k + 31) / 32) {     // exactly as many accumulators as the columns need
             case 1: SS_SPMM_ROWS(1); break;
@@ -1410,6 +1429,7 @@ int spmm_launch_ld(ss_symbolic *s, const double *a, const double *b, const doubl
         ss_launch(ctx, SS_K_SPMM, sss::k_spmm_cols, grid, 256, 0, ctx->stream, s->n, s->d_rowptr, s->d_colind, a, b,
                   alpha, beta, X, ldx, k, Y, ldy);
 #undef SS_SPMM_ROWS
+#undef SS_SPMM_NNZ
     ctx->add_flops(SS_K_SPMM, (beta ? 4.0 : 2.0) * (double)s->nnz * k);
     SS_CUDA_TRY(ctx, cudaGetLastError());
     return SS_OK;
