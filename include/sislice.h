@@ -171,13 +171,14 @@ ss_status ss_set_schur_mode(ss_ctx *ctx, int32_t mode, double min_flops);
  * Rayleigh-Ritz, steps 4-5; an implementation choice with no paper counterpart).
  * SS_GEMM_TENSOR (default): products with at least 2,048 rows and small dimensions >= 48 run on the
  * FP16 tensor cores: every operand row (a row of A or B, a column of X) is split exactly
- * into 7 digit slices of 8 bits under one power-of-two scale, the 28 leading digit
+ * into 8 digit slices of 7 bits under one power-of-two scale, the 36 leading digit
  * products are summed exactly (FP32 accumulators in tensor memory, read out as integers
- * every 128 terms of the reduction) and the sum rounded once to FP64; the error is a few
- * units of 2^-53 of K max|a_row| max|b_row| (K the reduction length).  A factor keeps the
- * slices of its A and B (7 x 16 KB per 128-row tile and 64-column piece holding entries)
- * from its first product until ss_factor_destroy; where they do not fit the factor falls
- * back to the CUDA cores.  SS_GEMM_SIMT: CUDA-core FP64.  Errors: SS_ERR_ARG. */
+ * every 512 terms of the reduction) and the sum rounded once to FP64; the error is a few
+ * units of 2^-53 of K max|a_row| max|b_row| (K the reduction length).  The analysis keeps a list of
+ * its pattern's entries (6 bytes each, made by the first sparse product); where that or the digits
+ * of X do not fit the factor falls back to the CUDA cores.  FP64 solves of many right-hand sides
+ * run on the tensor cores in this mode too (7 digits of 8 bits, exact sums).
+ * SS_GEMM_SIMT: CUDA-core FP64.  Errors: SS_ERR_ARG. */
 enum { SS_GEMM_TENSOR = 0, SS_GEMM_SIMT = 1 };
 ss_status ss_set_gemm_mode(ss_ctx *ctx, int32_t mode);
 
@@ -438,9 +439,7 @@ ss_status ss_band_energy_grad(ss_symbolic *sym, const double *X, const double *l
  * Y[i, j] = sum_e (alpha[j] a_vals[e] + beta[j] b_vals[e]) X[col(e), j] over row i,
  * X, Y DEVICE float64 N x k row-major; alpha, beta DEVICE float64[k] (NULL alpha = 1,
  * NULL beta = no B term).  With ss_set_gemm_mode(SS_GEMM_TENSOR), N >= 2,048 and k >= 48
- * the products run on the tensor cores (digit slices of the values made for this call:
- * 7 x 16 KB per 128-row tile and 64-column piece holding entries), A X and B X each
- * rounded once to FP64.  Errors: SS_ERR_ARG, SS_ERR_CUDA, SS_ERR_OOM, SS_ERR_TIMEOUT. */
+ * the products run on the tensor cores, A X and B X each rounded once to FP64.  Errors: SS_ERR_ARG, SS_ERR_CUDA, SS_ERR_OOM, SS_ERR_TIMEOUT. */
 ss_status ss_spmm(ss_symbolic *sym, const double *a_vals, const double *b_vals,
                   const double *alpha, const double *beta, const double *X, int32_t k,
                   double *Y);

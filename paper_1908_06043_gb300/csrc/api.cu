@@ -504,7 +504,7 @@ static int factor_levels(ss_numeric *f, int ns, ShiftPtrs<T> *dp, const std::vec
                 ss_launch(ctx, SS_K_SCHUR_TC, sstc::k_schur_tc, dim3(sd.tc_tiles, ns), sstc::kSchurTcThreads,
                           sstc::kSchurTcSmem, st, tk, sd.count, (const ShiftPtrs<double> *)(void *)dp);
                 ctx->add_flops(SS_K_SCHUR_TC, sd.flops3 * ns);
-                // 112 MMAs of 128 x 64 x 16 per tile
+                // 112 digit products of 128 x 64 x 16 per tile
                 ctx->add_tensor_flops(SS_K_SCHUR_TC, 112.0 * 2.0 * 128 * 64 * 16 * sd.tc_tiles * ns);
             } else if (sd.tiles3 > 0) {
                 const int cls = std::is_same<T, float>::value ? SS_K_SCHUR_F32 : SS_K_SCHUR;
@@ -1167,7 +1167,7 @@ static int fold_per_step(ss_numeric *f, int j, double *b, int k, bool full) {
 // off the CUDA cores, 4.4 ps per entry of L and column, outweighs its longer items, 16 us more per
 // level.  Measured (ms a solve, CUDA cores / tensor cores): N = 864 (13 levels) k = 129 0.48 / 0.50,
 // k = 304 0.78 / 0.54; N = 5,280 (55) k = 17 1.48 / 1.85, k = 48 2.58 / 1.93, k = 304 11.7 / 2.94;
-// N = 16,384 (129) k = 304 61.8 / 10.3.
+// N = 16,384 (129) k = 304 61.8 / 9.2.
 static bool fold_uses_tc(const ss_symbolic *s, int k) {
     return s->ctx->gemm_mode == SS_GEMM_TENSOR && k > kFoldMaxNc &&
            (double)s->info.l_offdiag_entries * k >= 3.6e6 * (double)s->solve_levels.size();

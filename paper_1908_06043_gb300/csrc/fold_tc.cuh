@@ -22,12 +22,12 @@
 // of the product NaN.
 //
 // What bounds it: the chain of one item a level.  Measured per item (cycles): right-hand sides'
-// load and digits 6,000, 112 MMAs 7,100 (48 each, limited by the operands' shared-memory reads at
-// N = 64), read-out 8,100 (7 x 32 KB out of tensor memory), the next tile's digits 3,100, barrier
-// 4,000-7,000; G's tile of the next level is loaded during the MMAs and cut before the barrier.
-// One solve at N = 16,384, k = 304: 61.8 ms on the CUDA cores (0.87 of their FP64 peak), 10.3 ms
-// here; N = 5,280, k = 112: 4.4 -> 2.3 ms.  Tried and left out: an accumulator's read-out under the
-// MMAs of the next ones (each slows the other: 9,000 + 8,400 cycles instead of 7,100 + 8,100).
+// load and digits 6,000, 40 MMAs 4,250 (7,100 as 112 MMAs of N = 64), read-out 8,100 (7 x 32 KB out
+// of tensor memory), the next tile's digits 3,100, barrier 4,000-7,000; G's tile of the next level
+// is loaded during the MMAs and cut before the barrier.  One solve at N = 16,384, k = 304: 61.8 ms
+// on the CUDA cores (0.87 of their FP64 peak), 9.2 ms here; N = 5,280, k = 112: 4.4 -> 1.6 ms.
+// Tried and left out: an accumulator's read-out under the MMAs of the next ones (each slows the
+// other: 9,000 + 8,400 cycles where one after the other takes 7,100 + 8,100).
 #pragma once
 
 #include <cuda_fp16.h>
@@ -97,20 +97,15 @@ __device__ __forceinline__ void ft_store8(const unsigned long long (&z)[8], unsi
     }
 }
 
-// the MMAs of one item: accumulator d (columns 64 d ..) = sum_{p + q = d} A_p B_q^T.  Per K step of 16
+// The MMAs of one item: accumulator d (columns 64 d ..) = sum_{p + q = d} A_p B_q^T.  Per K step of 16
 // the right-hand sides advance 32 bytes inside their 128-byte rows; G does the same when K is its
-// column (forward), or 16 rows = 2,048 bytes when K is its row (backward, MN-major).
+// column (forward), or 16 rows = 2,048 bytes when K is its row (backward, MN-major: the next 64 of
+// a merged N, the next digit, lie a leading byte offset of 8 KB further).
 __device__ __forceinline__ void ft_issue(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t bstep) {
 #pragma unroll 1
-    for (int d = 0; d < kFtSlices; ++d)
-#pragma unroll 1
-        for (int p = 0; p <= d; ++p) {
-            const uint64_t a = da + (uint64_t)(p * (kFtSliceA >> 4)), b = db + (uint64_t)((d - p) * (kFtSliceB >> 4));
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                mma_f16(tmem + (uint32_t)d * 64, a + (uint64_t)(kk * (kKStepBytes >> 4)), b + (uint64_t)(kk * (bstep >> 4)),
-                        idesc, (kk == 0 && p == 0) ? 0u : 1u);
-        }
+    for (int kk = 0; kk < 4; ++kk)
+        issue_digit_step<kFtSlices>(tmem, da + (uint64_t)(kk * (kKStepBytes >> 4)), db + (uint64_t)(kk * (bstep >> 4)),
+                                    kFtSliceA, kFtSliceB, idesc, kk == 0);
 }
 
 // 16 columns of one accumulator; the values are there after ft_tmem_wait on the same registers
@@ -179,7 +174,8 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
-    const uint32_t idesc_f = idesc_f16_f32(kFtCols, kFtRows), idesc_b = idesc_f | (1u << 16);   // bit 16: B is MN-major
+    const uint32_t idesc_f = idesc_f16_f32(kFtCols, 0), idesc_b = idesc_f | (1u << 16);   // bit 16: B is MN-major
+    const uint64_t lbo_b = (uint64_t)((kFtSliceB >> 4) - 1) << 16;   // added to the forward form's field of 1
     uint32_t phase = 0;
 
     // ---- the item in hand, and the one whose entries are being fetched
@@ -261,8 +257,8 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
         __syncthreads();
         if (tid == 0) {
             tc_fence_after();
-            ft_issue(tmem, smem_desc(smem_u32(sa)), smem_desc(smem_u32(sb)), backward ? idesc_b : idesc_f,
-                     backward ? 16u * 128u : kKStepBytes);
+            ft_issue(tmem, smem_desc(smem_u32(sa)), smem_desc(smem_u32(sb)) + (backward ? lbo_b : 0),
+                     backward ? idesc_b : idesc_f, backward ? 16u * 128u : kKStepBytes);
             mma_commit(&bar);
             if (!mbar_wait_bounded(&bar, phase, kFtWaitLimit)) {
                 s_ok = 0;

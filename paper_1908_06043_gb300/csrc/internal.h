@@ -168,7 +168,7 @@ struct FactorPlan {
 };
 
 struct OzPlan;   // tensor-core products: (tile, piece) pairs of the pattern (oz.cu)
-struct OzVals;   // tensor-core products: digit slices of one value array (oz.cu)
+struct OzVals;   // tensor-core products: row exponents of one value array (oz.cu)
 
 struct ss_symbolic {
     ss_ctx *ctx = nullptr;
@@ -267,8 +267,8 @@ struct ss_numeric {
     unsigned long long *d_counts = nullptr;   // per shift: neg, zero, pos, tiny
     std::vector<unsigned long long> h_counts;
     bool counts_valid = false;
-    OzVals *oz[2] = {nullptr, nullptr};  // digit slices of A and B for tensor-core products, or null
-    bool oz_failed = false;               // those slices did not fit: products on the CUDA cores
+    OzVals *oz[2] = {nullptr, nullptr};  // row exponents of A and B for tensor-core products, or null
+    bool oz_failed = false;               // those products' scratch did not fit: CUDA cores
     // several pencils in one block-diagonal pattern (ss_factor_segments): a shift per pencil
     int32_t n_seg = 0;
     int32_t *d_eseg = nullptr;            // pencil of each stored entry (nnz)
@@ -321,7 +321,7 @@ int oz_gemm(ss_ctx *ctx, const double *X, int64_t ldx, int64_t n, int k1, const 
 // or B (which 1) of f; the first pass overwrites Y
 int oz_spmm(ss_numeric *f, int npass, const int *which, const double *const *colscale, const double *alpha,
             const double *X, int64_t ldx, int k, double *Y, int64_t ldy);
-// the same for any value arrays, sliced for this call only
+// the same for any value arrays
 int oz_spmm_vals(ss_symbolic *s, const double *a, const double *b, const double *alpha, const double *beta,
                  const double *X, int64_t ldx, int k, double *Y, int64_t ldy);
 // Y = diag(alpha) A X + diag(beta) B X for value arrays a, b (tensor cores where possible)

@@ -1,6 +1,5 @@
 // Host side of the FP64-accurate tensor-core products (tc_gemm.cuh): operand slicing, the
-// (tile, piece) plan of the sparse pattern, the digit slices of a factor's A and B kept for
-// the factor's lifetime, and the launches.
+// (tile, piece) plan of the sparse pattern, and the launches.
 #include <algorithm>
 #include <mutex>
 #include <vector>
@@ -11,14 +10,15 @@
 struct OzPlan {
     int32_t nrt = 0;
     int64_t npairs = 0;
-    int32_t *d_tile_ptr = nullptr, *d_pair_tile = nullptr, *d_pair_piece = nullptr;
-    int64_t *d_seg = nullptr;
+    int32_t *d_tile_ptr = nullptr, *d_pair_piece = nullptr;
+    int64_t *d_ent_ptr = nullptr;      // npairs + 1
+    uint32_t *d_ent_e = nullptr;       // nnz, sorted by pair
+    uint16_t *d_ent_off = nullptr;
 };
 
 struct OzVals {
     const double *vals = nullptr;
-    unsigned char *sl = nullptr;   // npairs x 7 slice blocks
-    int *em = nullptr;             // per row: largest biased exponent
+    int *em = nullptr;                 // per row: largest biased exponent
 };
 
 namespace {
@@ -65,7 +65,6 @@ void oz_attrs(int device) {
     if (seen[device]) return;
     seen[device] = 1;
     cudaFuncSetAttribute(sstc::k_oz_mm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sstc::kOzGemmSmem);
-    cudaFuncSetAttribute(sstc::k_oz_slice_csr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sstc::kOzCsrSmem);
 }
 
 // exponents and digit slices of a dense operand (blocks kc * nrt + rt)
@@ -124,110 +123,112 @@ int dense_mm(ss_ctx *ctx, const OzOperand &A, const OzOperand &B, int mode, doub
     return run_mm(ctx, g, dim3(nct, nrtA, nsplit), SS_K_GEMM_TC);
 }
 
-// (tile, piece) pairs of the pattern: for each 128-row tile the 32-column pieces that hold
-// entries, and per pair and row the CSR position of the row's first entry in the piece
+// (tile, piece) pairs of the pattern -- for each 128-row tile the 32-column pieces that hold
+// entries -- and the entries of every pair: CSR position (from the tile's first) and place in the
+// pair's digit block
 int plan_build(ss_symbolic *s) {
     ss_ctx *ctx = s->ctx;
-    const int64_t n = s->n;
+    const int64_t n = s->n, npieces = (n + sstc::kOzK - 1) / sstc::kOzK;
     const int32_t nrt = (int32_t)cdivu(n, 128);
-    const int64_t npieces = (n + sstc::kOzK - 1) / sstc::kOzK;
-    std::vector<int32_t> tile_ptr(nrt + 1, 0), pair_tile, pair_piece, mark(npieces, -1), list;
-    std::vector<int64_t> seg;
+    std::vector<std::vector<int32_t>> pieces(nrt), counts(nrt);     // of a tile: pieces ascending, entries of each
+#pragma omp parallel
+    {
+        std::vector<int32_t> cnt(npieces, 0);
+#pragma omp for schedule(dynamic, 16)
+        for (int32_t rt = 0; rt < nrt; ++rt) {
+            const int64_t r1 = std::min<int64_t>(n, (rt + 1ll) * 128);
+            std::vector<int32_t> &list = pieces[rt];
+            for (int64_t p = s->rowptr[rt * 128ll]; p < s->rowptr[r1]; ++p)
+                if (cnt[s->colind[p] / sstc::kOzK]++ == 0) list.push_back(s->colind[p] / sstc::kOzK);
+            std::sort(list.begin(), list.end());
+            for (int32_t pc : list) {
+                counts[rt].push_back(cnt[pc]);
+                cnt[pc] = 0;
+            }
+        }
+    }
+    std::vector<int32_t> tile_ptr(nrt + 1, 0), pair_piece;
+    std::vector<int64_t> ent_ptr(1, 0);
     for (int32_t rt = 0; rt < nrt; ++rt) {
-        list.clear();
-        const int64_t r0 = (int64_t)rt * 128, r1 = std::min<int64_t>(n, r0 + 128);
-        for (int64_t p = s->rowptr[r0]; p < s->rowptr[r1]; ++p) {
-            const int32_t pc = s->colind[p] / sstc::kOzK;
-            if (mark[pc] != rt) {
-                mark[pc] = rt;
-                list.push_back(pc);
-            }
+        for (size_t u = 0; u < pieces[rt].size(); ++u) {
+            pair_piece.push_back(pieces[rt][u]);
+            ent_ptr.push_back(ent_ptr.back() + counts[rt][u]);
         }
-        std::sort(list.begin(), list.end());
-        const size_t base = pair_tile.size();
-        for (int32_t pc : list) {
-            pair_tile.push_back(rt);
-            pair_piece.push_back(pc);
+        tile_ptr[rt + 1] = (int32_t)pair_piece.size();
+    }
+    std::vector<uint32_t> ent_e(std::max<int64_t>(1, s->nnz));
+    std::vector<uint16_t> ent_off(std::max<int64_t>(1, s->nnz));
+#pragma omp parallel
+    {
+        std::vector<int64_t> at(npieces, 0);
+#pragma omp for schedule(dynamic, 16)
+        for (int32_t rt = 0; rt < nrt; ++rt) {
+            const int64_t r0 = rt * 128ll, r1 = std::min<int64_t>(n, r0 + 128), e0 = s->rowptr[r0];
+            for (int32_t q = tile_ptr[rt]; q < tile_ptr[rt + 1]; ++q) at[pair_piece[q]] = ent_ptr[q];
+            for (int64_t r = r0; r < r1; ++r)
+                for (int64_t p = s->rowptr[r]; p < s->rowptr[r + 1]; ++p) {
+                    const int64_t o = at[s->colind[p] / sstc::kOzK]++;
+                    ent_e[o] = (uint32_t)(p - e0);
+                    ent_off[o] = (uint16_t)sstc::oz_offset((int)(r - r0), (int)(s->colind[p] % sstc::kOzK));
+                }
         }
-        seg.resize(pair_tile.size() * 128, 0);
-        for (int r = 0; r < 128; ++r) {
-            const int64_t row = r0 + r;
-            int64_t ptr = row < n ? s->rowptr[row] : 0;
-            const int64_t end = row < n ? s->rowptr[row + 1] : 0;
-            for (size_t u = 0; u < list.size(); ++u) {
-                while (ptr < end && s->colind[ptr] < (int64_t)list[u] * sstc::kOzK) ++ptr;
-                seg[(base + u) * 128 + r] = ptr;
-            }
-        }
-        tile_ptr[rt + 1] = (int32_t)pair_tile.size();
     }
     OzPlan *pl = new OzPlan();
     pl->nrt = nrt;
-    pl->npairs = (int64_t)pair_tile.size();
-    cudaError_t e = cudaMalloc(&pl->d_tile_ptr, sizeof(int32_t) * tile_ptr.size());
-    if (e == cudaSuccess) e = cudaMalloc(&pl->d_pair_tile, sizeof(int32_t) * std::max<size_t>(1, pair_tile.size()));
-    if (e == cudaSuccess) e = cudaMalloc(&pl->d_pair_piece, sizeof(int32_t) * std::max<size_t>(1, pair_piece.size()));
-    if (e == cudaSuccess) e = cudaMalloc(&pl->d_seg, sizeof(int64_t) * std::max<size_t>(1, seg.size()));
+    pl->npairs = (int64_t)pair_piece.size();
     s->oz_plan = pl;
+    auto up = [&](auto **d, const auto &h) {
+        cudaError_t e = cudaMalloc((void **)d, sizeof(h[0]) * std::max<size_t>(1, h.size()));
+        if (e == cudaSuccess && !h.empty()) e = cudaMemcpy(*d, h.data(), sizeof(h[0]) * h.size(), cudaMemcpyHostToDevice);
+        return e;
+    };
+    cudaError_t e = up(&pl->d_tile_ptr, tile_ptr);
+    if (e == cudaSuccess) e = up(&pl->d_pair_piece, pair_piece);
+    if (e == cudaSuccess) e = up(&pl->d_ent_ptr, ent_ptr);
+    if (e == cudaSuccess) e = up(&pl->d_ent_e, ent_e);
+    if (e == cudaSuccess) e = up(&pl->d_ent_off, ent_off);
     if (e != cudaSuccess) {
         cudaGetLastError();
+        oz_free_symbolic(s);
         return ctx->set_error(SS_ERR_OOM, "tensor-core product plan: device allocation failed");
-    }
-    SS_CUDA_TRY(ctx, cudaMemcpy(pl->d_tile_ptr, tile_ptr.data(), sizeof(int32_t) * tile_ptr.size(),
-                                cudaMemcpyHostToDevice));
-    if (!pair_tile.empty()) {
-        SS_CUDA_TRY(ctx, cudaMemcpy(pl->d_pair_tile, pair_tile.data(), sizeof(int32_t) * pair_tile.size(),
-                                    cudaMemcpyHostToDevice));
-        SS_CUDA_TRY(ctx, cudaMemcpy(pl->d_pair_piece, pair_piece.data(), sizeof(int32_t) * pair_piece.size(),
-                                    cudaMemcpyHostToDevice));
-        SS_CUDA_TRY(ctx, cudaMemcpy(pl->d_seg, seg.data(), sizeof(int64_t) * seg.size(), cudaMemcpyHostToDevice));
     }
     return SS_OK;
 }
 
-// exponents and digit slices of one value array on the pattern, into v (device memory from
-// buf, or owned by v when buf is null)
+// row exponents of one value array on the pattern, into v (device memory from buf, or owned by v
+// when buf is null)
 int vals_make(ss_symbolic *s, const double *vals, OzVals *v, Scratch *buf) {
     ss_ctx *ctx = s->ctx;
     int rc;
     if (!s->oz_plan && (rc = plan_build(s)) != SS_OK) return rc;
-    const OzPlan *pl = s->oz_plan;
-    const size_t bytes = (size_t)std::max<int64_t>(1, pl->npairs) * sstc::kOzStageA;
     v->vals = vals;
     if (buf) {
-        OZ_ALLOC(ctx, buf->get(&v->sl, bytes));
         OZ_ALLOC(ctx, buf->get(&v->em, (size_t)s->n));
     } else {
-        cudaError_t e = cudaMalloc(&v->sl, bytes);
-        if (e == cudaSuccess) e = cudaMalloc(&v->em, sizeof(int) * s->n);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return ctx->set_error(SS_ERR_OOM, "tensor-core product: slices of the pencil do not fit");
-        }
+        OZ_ALLOC(ctx, cudaMalloc(&v->em, sizeof(int) * s->n));
     }
     oz_attrs(ctx->device);
-    ss_launch(ctx, SS_K_SPMM_TC, sstc::k_oz_csr_expmax, cdivu(s->n, 256), 256, 0, ctx->stream, s->n,
+    ss_launch(ctx, SS_K_SPMM_TC, sstc::k_oz_csr_expmax, cdivu(s->n * 32, 256), 256, 0, ctx->stream, s->n,
               (const int64_t *)s->d_rowptr, vals, v->em);
-    if (pl->npairs > 0)
-        ss_launch(ctx, SS_K_SPMM_TC, sstc::k_oz_slice_csr, (unsigned)pl->npairs, 128, sstc::kOzCsrSmem, ctx->stream,
-                  s->n, (const int64_t *)s->d_rowptr, (const int32_t *)s->d_colind, vals, (const int64_t *)pl->d_seg,
-                  (const int32_t *)pl->d_pair_tile, (const int32_t *)pl->d_pair_piece, (const int *)v->em, v->sl);
     SS_CUDA_TRY(ctx, cudaGetLastError());
     return SS_OK;
 }
 
-// digit slices of value array `which` (0: A, 1: B) of f, made on first use
+// row exponents of value array `which` (0: A, 1: B) of f, made on first use
 int vals_get(ss_numeric *f, int which, OzVals **out) {
     *out = f->oz[which];
     if (*out) return SS_OK;
     OzVals *v = new OzVals();
-    f->oz[which] = v;        // freed with the factor, also after a failure here
     const int rc = vals_make(f->sym, which == 0 ? f->a_vals : f->b_vals, v, nullptr);
-    if (rc == SS_OK) *out = v;
-    return rc;
+    if (rc != SS_OK) {
+        delete v;
+        return rc;
+    }
+    f->oz[which] = *out = v;   // freed with the factor
+    return SS_OK;
 }
 
-// pass p adds alpha[p] diag(colscale[p]) M_p X, M_p the array sliced in v[p]; the first
+// pass p adds alpha[p] diag(colscale[p]) M_p X, M_p the array of v[p]; the first
 // pass overwrites Y
 int spmm_core(ss_symbolic *s, int npass, OzVals *const *v, const double *const *colscale, const double *alpha,
               const double *X, int64_t ldx, int k, double *Y, int64_t ldy) {
@@ -242,8 +243,10 @@ int spmm_core(ss_symbolic *s, int npass, OzVals *const *v, const double *const *
     const OzPlan *pl = s->oz_plan;
     for (int p = 0; p < npass; ++p) {
         sstc::OzMM g{};
-        g.slA = v[p]->sl; g.emA = v[p]->em; g.nrtA = pl->nrt; g.rowsA = s->n;
+        g.emA = v[p]->em; g.nrtA = pl->nrt; g.rowsA = s->n;
         g.tile_ptr = pl->d_tile_ptr; g.pair_piece = pl->d_pair_piece;
+        g.ent_ptr = pl->d_ent_ptr; g.ent_e = pl->d_ent_e; g.ent_off = pl->d_ent_off;
+        g.rowptr = s->d_rowptr; g.vals = v[p]->vals;
         g.slB = sx; g.emB = ex; g.nrtB = (int)cdivu(k, 128); g.rowsB = k;
         g.mode = 1; g.alpha = alpha[p]; g.beta = p == 0 ? 0.0 : 1.0; g.colscale = colscale[p];
         g.out = Y; g.ldo = ldy;
@@ -315,7 +318,7 @@ int spmm_f(ss_numeric *f, const double *a, const double *b, const double *alpha,
         const double al[2] = {1.0, 1.0};
         const int rc = oz_spmm(f, beta ? 2 : 1, which, cs, al, X, ldx, k, Y, ldy);
         if (rc != SS_ERR_OOM) return rc;
-        // the pencil's slices do not fit beside the factor: CUDA cores from now on
+        // the plan or the digits of X do not fit beside the factor: CUDA cores from now on
         f->oz_failed = true;
         s->ctx->err.clear();
     }
@@ -325,7 +328,6 @@ int spmm_f(ss_numeric *f, const double *a, const double *b, const double *alpha,
 void oz_free_numeric(ss_numeric *f) {
     auto drop = [](OzVals *&v) {
         if (!v) return;
-        if (v->sl) cudaFree(v->sl);
         if (v->em) cudaFree(v->em);
         delete v;
         v = nullptr;
@@ -336,7 +338,7 @@ void oz_free_numeric(ss_numeric *f) {
 void oz_free_symbolic(ss_symbolic *s) {
     OzPlan *pl = s->oz_plan;
     if (!pl) return;
-    void *ptrs[] = {pl->d_tile_ptr, pl->d_pair_tile, pl->d_pair_piece, pl->d_seg};
+    void *ptrs[] = {pl->d_tile_ptr, pl->d_pair_piece, pl->d_ent_ptr, pl->d_ent_e, pl->d_ent_off};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     delete pl;

@@ -13,10 +13,11 @@
 // Y = round(x 2^(55 - E)) is a 56-bit integer whose 8 balanced base-128 digits q_0 .. q_7
 // (|q_p| <= 64, exact in FP16) are the slices: x = 2^(E - 6) sum_p q_p 2^(-7p) up to
 // 2^(E - 56).  The digits are cut from the FP64 bit pattern with integer arithmetic.
-// Slice layout.  The reduction is cut into pieces of 32.  For 128-row tile rt and piece kc,
-// eight 8 KB blocks of digits in the MMA's core-matrix layout (oz_offset below) at block
-// index kc * nrt + rt (dense) or at the index of the (tile, piece) pair (sparse A: only
-// pieces that hold entries).
+// Slice layout.  The reduction is cut into pieces of 32.  For 128-row tile rt and piece kc of a
+// dense operand, eight 8 KB blocks of digits in the MMA's core-matrix layout (oz_offset below) at
+// block index kc * nrt + rt.  A sparse operand has no slices in memory: its tiles hold a few per
+// cent of entries, so the kernel clears a stage and places the digits of the (tile, piece) pair's
+// entries itself, from a list of the pattern's entries sorted by pair (6 bytes an entry).
 // Products.  An output tile of 128 x 64 entries takes, per piece, the 36 digit products with
 // p + q <= 7 on the tensor cores into 8 FP32 accumulators D_d = sum_{p+q=d} (8 x 64 = 512
 // tensor-memory columns), exact over 16 pieces: |D_d| <= 8 * 512 * 64^2 = 2^24.  Every 16
@@ -25,14 +26,21 @@
 // so the result, (hi 2^28 + lo) 2^(E_a + E_b - 61), is the exact sum of the truncated digit
 // expansion rounded once to FP64: its error is a few units of 2^-53 of
 // K max|a_row| max|b_row| (K the reduction length).
-// Pipeline.  Two shared-memory stages of one piece each (64 KB of A, 32 KB of B): the loads
-// of piece i + 1 run while the tensor cores work on piece i.
+// Pipeline.  Two shared-memory stages of one piece each (64 KB of A, 32 KB of B).  One warp issues
+// bulk copies, one the MMAs, sixteen place sparse digits and read the accumulators out; mbarriers
+// between them, so a stage refills as soon as its MMAs have read it and the MMAs of the next piece
+// wait for nothing else.  What bounds it: the 24 merged MMAs of a piece (2,304 cycles of tensor
+// pipe), the read-outs between groups (8 x 32 KB of tensor memory every 16 pieces) and, for dense
+// operands, 96 KB a piece and SM out of L2.  A X at N = 16,384, k = 304 (17,312 pairs x 5 column
+// tiles): 2.18 ms with one thread issuing copies and 72 MMAs a piece in turn and 1.1 GB of digit
+// slices of A in memory, 1.45 ms now.
 #pragma once
 
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "grid_sync.cuh"
 #include "tc_ptx.cuh"
 
 namespace sstc {
@@ -43,11 +51,11 @@ constexpr uint32_t kOzBlock = 128 * kOzK * 2;         // one slice block: 128 ro
 constexpr uint32_t kOzHalf = 64 * kOzK * 2;           // its 64-row half
 constexpr uint32_t kOzStageA = kOzSlices * kOzBlock;  // 64 KB
 constexpr uint32_t kOzStageB = kOzSlices * kOzHalf;   // 32 KB
-constexpr int kOzThreads = 256;
+constexpr int kOzWorkers = 512;                       // threads that place sparse digits and read out
+constexpr int kOzThreads = kOzWorkers + 64;           // and the copy and MMA warps
 constexpr int kOzReadEvery = 16;                      // pieces per exact FP32 accumulation
 constexpr size_t kOzGemmSmem = 1024 + 2 * (size_t)(kOzStageA + kOzStageB);
-constexpr size_t kOzCsrSmem = (size_t)kOzStageA;
-constexpr long long kOzWaitLimit = 1ll << 24;
+constexpr unsigned long long kOzWaitNs = 1000000000ull;   // a wait gives up after this long
 constexpr uint32_t kTmemColsOz = 512;                 // 8 accumulators x 64 columns
 
 // Byte offset of element (row, k) of an R x 32 FP16 tile: 8 x 8 core matrices of 16-byte
@@ -107,14 +115,15 @@ __global__ void __launch_bounds__(128) k_oz_expmax(OzOperand op, int64_t per_k, 
     if (m > 0) atomicMax(&em[row], m);
 }
 
-// em[row] = largest biased exponent of CSR row `row` (0 for an empty or zero row)
-__global__ void k_oz_csr_expmax(int64_t n, const int64_t *__restrict__ rowptr, const double *__restrict__ vals,
-                                int *__restrict__ em) {
-    const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// em[row] = largest biased exponent of CSR row `row` (0 for an empty or zero row); one warp per row
+__global__ void __launch_bounds__(256) k_oz_csr_expmax(int64_t n, const int64_t *__restrict__ rowptr,
+                                                       const double *__restrict__ vals, int *__restrict__ em) {
+    const int64_t row = (blockIdx.x * 256ll + threadIdx.x) >> 5;
     if (row >= n) return;
     int m = 0;
-    for (int64_t p = rowptr[row]; p < rowptr[row + 1]; ++p) m = max(m, biased_exp(vals[p]));
-    em[row] = m;
+    for (int64_t p = rowptr[row] + (threadIdx.x & 31); p < rowptr[row + 1]; p += 32) m = max(m, biased_exp(vals[p]));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) em[row] = m;
 }
 
 // Block (rt, kc), thread = row of the tile.  Zero rows / columns pad the operand.
@@ -146,62 +155,18 @@ __global__ void __launch_bounds__(128) k_oz_slice(OzOperand op, const int *__res
     }
 }
 
-// Sparse operand: block = (tile, piece) pair q, thread = row of the tile.  seg[q * 128 + r]
-// is the CSR position of row r's first entry in the piece (columns 32 piece ..).  The
-// digits are placed in shared memory (zero elsewhere) and the 8 blocks copied out whole.
-__global__ void __launch_bounds__(128) k_oz_slice_csr(int64_t n, const int64_t *__restrict__ rowptr,
-                                                      const int32_t *__restrict__ colind,
-                                                      const double *__restrict__ vals,
-                                                      const int64_t *__restrict__ seg,
-                                                      const int32_t *__restrict__ pair_tile,
-                                                      const int32_t *__restrict__ pair_piece,
-                                                      const int *__restrict__ em, unsigned char *__restrict__ sl) {
-    extern __shared__ __align__(16) unsigned char sm[];
-    const int q = blockIdx.x;
-    const int rho = threadIdx.x;
-    for (uint32_t o = rho * 16; o < kOzCsrSmem; o += 128 * 16)
-        *reinterpret_cast<uint4 *>(sm + o) = make_uint4(0, 0, 0, 0);
-    __syncthreads();
-    const int64_t row = (int64_t)pair_tile[q] * 128 + rho;
-    if (row < n) {
-        const int E = em[row] - 1022;
-        const int64_t c0 = (int64_t)pair_piece[q] * kOzK;
-        const int64_t end = rowptr[row + 1];
-        for (int64_t p = seg[(int64_t)q * 128 + rho]; p < end && colind[p] < c0 + kOzK; ++p) {
-            int d[kOzSlices];
-            oz_digits(vals[p], E, d);
-            const uint32_t off = oz_offset(rho, (int)(colind[p] - c0));
-#pragma unroll
-            for (int s = 0; s < kOzSlices; ++s)
-                *reinterpret_cast<__half *>(sm + (uint32_t)s * kOzBlock + off) = __int2half_rn(d[s]);
-        }
-    }
-    __syncthreads();
-    uint4 *dst = reinterpret_cast<uint4 *>(sl + (uint64_t)q * kOzStageA);
-    for (uint32_t o = rho; o < kOzCsrSmem / 16; o += 128) dst[o] = reinterpret_cast<const uint4 *>(sm)[o];
-}
-
-// 32 lanes x 32 bits, 32 consecutive columns per thread, load and wait in one statement
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-}
-
 struct OzMM {
-    const unsigned char *slA;
+    const unsigned char *slA;    // dense A: slices (null: sparse A)
     const int *emA;
     int nrtA;
     int64_t rowsA;
     const int32_t *tile_ptr;     // sparse A: pairs of row tile rt are [tile_ptr[rt], tile_ptr[rt + 1])
-    const int32_t *pair_piece;   // sparse A: reduction piece of pair q (slice block q)
+    const int32_t *pair_piece;   // reduction piece of pair q
+    const int64_t *ent_ptr;      // entries of pair q are [ent_ptr[q], ent_ptr[q + 1])
+    const uint32_t *ent_e;       // CSR position minus rowptr[128 rt]
+    const uint16_t *ent_off;     // oz_offset of the entry in its block
+    const int64_t *rowptr;
+    const double *vals;
     const unsigned char *slB;
     const int *emB;
     int nrtB;
@@ -215,40 +180,42 @@ struct OzMM {
     int *status;                 // raised when a bounded wait runs out
 };
 
-// The 144 MMAs of one 32-wide piece: accumulator d (tensor-memory columns 64 d ..) gets
-// sum_{p + q = d} A_p B_q^T, p, q < 8, d <= 7.  da, db: descriptors of slice 0 of the
-// stage's A and B.  fresh: the first MMA into each accumulator overwrites it.
-__device__ __forceinline__ void oz_issue_piece(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, bool fresh) {
-    const uint32_t keep_first = fresh ? 0u : 1u;
-#pragma unroll
-    for (int d = 0; d < kOzSlices; ++d) {
-#pragma unroll
-        for (int p = 0; p <= d; ++p) {
-            const uint64_t a = da + (uint64_t)(p * (kOzBlock >> 4));
-            const uint64_t b = db + (uint64_t)((d - p) * (kOzHalf >> 4));
-            mma_f16(tmem + (uint32_t)d * 64, a, b, idesc, p == 0 ? keep_first : 1u);
-            mma_f16(tmem + (uint32_t)d * 64, a + (256 >> 4), b + (256 >> 4), idesc, 1u);   // second K step
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// wait for a phase; false (and *ok cleared) after kOzWaitNs, or when another role has given up
+__device__ __forceinline__ bool oz_wait(uint64_t *bar, uint32_t parity, volatile int *ok) {
+    unsigned long long t0 = 0;
+    for (unsigned it = 1;; ++it) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if ((it & 63u) == 0u) {
+            if (!*ok) return false;
+            const unsigned long long t = gb_clock_ns();
+            if (t0 == 0) t0 = t;
+            else if (t - t0 > kOzWaitNs) {
+                *ok = 0;
+                return false;
+            }
         }
     }
 }
 
 // Output tile (rt, bj) = rows 128 rt .., columns 64 bj ..  (beta = 0 does not read out).
-// blockIdx.x = bj varies fastest, so the CTAs that share one A tile run together and read
-// its slices from L2 after the first.  Thread 0 stages the pieces (two stages) and issues the
-// MMAs; all 8 warps read the accumulators out every 16 pieces (warp w: tensor-memory lanes
-// 32 (w mod 4) .., columns 32 (w / 4) ..).
+// blockIdx.x = bj varies fastest, so the CTAs that share one A tile run together.  Worker warp w
+// reads tensor-memory lanes 32 (w mod 4) .. + 31 and columns 16 (w / 4) .. + 15.
 __global__ void __launch_bounds__(kOzThreads, 1) k_oz_mm(const OzMM g) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char *stage_a[2], *stage_b[2];
-    stage_a[0] = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
-    stage_b[0] = stage_a[0] + kOzStageA;
-    stage_a[1] = stage_b[0] + kOzStageB;
-    stage_b[1] = stage_a[1] + kOzStageA;
-    __shared__ __align__(8) uint64_t full[2], empty[2], accfull, drain;
+    unsigned char *stage[2];         // A digits, then B digits
+    stage[0] = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
+    stage[1] = stage[0] + kOzStageA + kOzStageB;
+    // full: copies landed; placed: sparse digits written (half of the worker warps); empty: MMAs of the stage
+    // done; accfull: accumulators complete; accfree: read out (worker warps)
+    __shared__ __align__(8) uint64_t full[2], placed[2], empty[2], accfull, accfree, drain;
     __shared__ uint32_t s_tmem;
-    __shared__ int s_ok;
+    __shared__ int s_ok, s_em[128];
     const int bj = blockIdx.x, rt = blockIdx.y;
-    const bool sparse = g.tile_ptr != nullptr;
+    const bool sparse = g.slA == nullptr;
     int q0, q1;
     if (sparse) {
         q0 = g.tile_ptr[rt];
@@ -257,13 +224,13 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_mm(const OzMM g) {
         q0 = blockIdx.z * g.per;
         q1 = min(g.nkc, q0 + g.per);
     }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int quarter = warp & 3, half = warp >> 2;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+    const int quarter = warp & 3, grp = (warp >> 2) & 3;
     const int64_t row = (int64_t)rt * 128 + 32 * quarter + lane;
-    const int64_t col0 = (int64_t)bj * 64 + 32 * half;
+    const int64_t col0 = (int64_t)bj * 64 + 16 * grp;
     if (q0 >= q1) {                  // no entries in this tile's rows: the product is zero
-        if (g.mode == 1 && row < g.rowsA)
-            for (int c = 0; c < 32; ++c) {
+        if (g.mode == 1 && row < g.rowsA && warp < kOzWorkers / 32)
+            for (int c = 0; c < 16; ++c) {
                 const int64_t col = col0 + c;
                 if (col >= g.rowsB) break;
                 double *o = g.out + row * g.ldo + col;
@@ -275,120 +242,172 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_mm(const OzMM g) {
         tmem_alloc(&s_tmem, kTmemColsOz);
         tmem_relinquish();
     }
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         for (int b = 0; b < 2; ++b) {
             mbar_init(&full[b], 1);
+            mbar_init(&placed[b], kOzWorkers / 64);
             mbar_init(&empty[b], 1);
         }
         mbar_init(&accfull, 1);
+        mbar_init(&accfree, kOzWorkers / 32);
         mbar_init(&drain, 1);
         fence_mbar_init();
         s_ok = 1;
     }
+    if (sparse && tid < 128) s_em[tid] = (int64_t)rt * 128 + tid < g.rowsA ? g.emA[(int64_t)rt * 128 + tid] : 0;
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
-    const uint32_t idesc = idesc_f16_f32(128, 64);
-    auto issue_loads = [&](int q, int b) {
-        const int kc = sparse ? g.pair_piece[q] : q;
-        const unsigned char *ga = g.slA + (uint64_t)(sparse ? q : kc * g.nrtA + rt) * kOzStageA;
-        const unsigned char *gb = g.slB + ((uint64_t)kc * g.nrtB + (bj >> 1)) * kOzStageA + (uint64_t)(bj & 1) * kOzHalf;
-        mbar_arrive_expect_tx(&full[b], kOzStageA + kOzStageB);
-        bulk_g2s(stage_a[b], ga, kOzStageA, &full[b]);
-        for (int p = 0; p < kOzSlices; ++p)
-            bulk_g2s(stage_b[b] + p * kOzHalf, gb + (uint64_t)p * kOzBlock, kOzHalf, &full[b]);
-    };
-    long long hi[32], lo[32];
-#pragma unroll
-    for (int c = 0; c < 32; ++c) {
-        hi[c] = 0;
-        lo[c] = 0;
-    }
-    int n_loaded = 0, n_landed = 0;                  // pieces whose loads were issued / waited for
-    if (threadIdx.x == 0) {
-        issue_loads(q0, 0);
-        n_loaded = 1;
-    }
-    int n_read = 0;                                  // read-outs done (phase of accfull)
-    for (int q = q0; q < q1; ++q) {
-        const int i = q - q0, b = i & 1;
-        const bool readout = (i % kOzReadEvery) == kOzReadEvery - 1 || q + 1 == q1;
-        if (threadIdx.x == 0 && s_ok) {
-            // piece i: wait for its stage, issue its MMAs, release the stage on completion
-            if (!mbar_wait_bounded(&full[b], (uint32_t)((i >> 1) & 1), kOzWaitLimit)) {
-                s_ok = 0;
-                mbar_wait_bounded(&full[b], (uint32_t)((i >> 1) & 1), kOzWaitLimit);   // copies in flight land
-            } else {
-                n_landed = i + 1;
-                uint32_t sa_addr = smem_u32(stage_a[b]), sb_addr = smem_u32(stage_b[b]);
-                asm volatile("" : "+r"(sa_addr), "+r"(sb_addr));   // keep the descriptors per piece
-                oz_issue_piece(tmem, oz_desc(sa_addr), oz_desc(sb_addr), idesc, (i % kOzReadEvery) == 0);
-                mma_commit(&empty[b]);
-                if (readout) mma_commit(&accfull);
-                // piece i + 1 goes to the other stage once piece i - 1's MMAs have read it
-                if (q + 1 < q1) {
-                    if (i >= 1 && !mbar_wait_bounded(&empty[b ^ 1], (uint32_t)(((i - 1) >> 1) & 1), kOzWaitLimit)) {
-                        s_ok = 0;
-                    } else {
-                        issue_loads(q + 1, b ^ 1);
-                        n_loaded = i + 2;
-                    }
-                }
+    const int np = q1 - q0;
+    volatile int *ok = &s_ok;
+    if (warp == kOzWorkers / 32) {                                   // ---- copies
+        if (lane == 0) {
+            int sent = 0;
+            for (int i = 0; i < np; ++i) {
+                const int b = i & 1, q = q0 + i;
+                if (i >= 2 && !oz_wait(&empty[b], (uint32_t)(((i >> 1) - 1) & 1), ok)) break;
+                const int kc = sparse ? g.pair_piece[q] : q;
+                const unsigned char *gb =
+                    g.slB + ((uint64_t)kc * g.nrtB + (bj >> 1)) * kOzStageA + (uint64_t)(bj & 1) * kOzHalf;
+                mbar_arrive_expect_tx(&full[b], sparse ? kOzStageB : kOzStageA + kOzStageB);
+                if (!sparse) bulk_g2s(stage[b], g.slA + ((uint64_t)kc * g.nrtA + rt) * kOzStageA, kOzStageA, &full[b]);
+                for (int p = 0; p < kOzSlices; ++p)
+                    bulk_g2s(stage[b] + kOzStageA + p * kOzHalf, gb + (uint64_t)p * kOzBlock, kOzHalf, &full[b]);
+                sent = i + 1;
             }
+            // copies in flight land before the CTA may leave
+            for (int i = max(0, sent - 2); i < sent; ++i)
+                mbar_wait_bounded(&full[i & 1], (uint32_t)((i >> 1) & 1), 1ll << 24);
         }
-        if (!readout) continue;
-        if (threadIdx.x == 0 && s_ok && !mbar_wait_bounded(&accfull, (uint32_t)(n_read & 1), kOzWaitLimit)) s_ok = 0;
-        ++n_read;
-        __syncthreads();                               // accumulators complete (or a wait ran out)
-        if (!s_ok) break;
-        tc_fence_after();
-        const uint32_t lane_base = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(32 * half);
+    } else if (warp == kOzWorkers / 32 + 1) {                            // ---- MMAs
+        if (lane == 0) {
+            const uint32_t idesc = idesc_f16_f32(128, 0);
+            bool fine = true;
+            for (int i = 0; i < np && fine; ++i) {
+                const int b = i & 1;
+                fine = oz_wait(&full[b], (uint32_t)((i >> 1) & 1), ok) &&
+                       (!sparse || oz_wait(&placed[b], (uint32_t)((i >> 1) & 1), ok));
+                if (fine && i > 0 && i % kOzReadEvery == 0)     // the accumulators have been read out
+                    fine = oz_wait(&accfree, (uint32_t)((i / kOzReadEvery - 1) & 1), ok);
+                if (!fine) break;
+                tc_fence_after();
+                uint32_t sa_addr = smem_u32(stage[b]), sb_addr = sa_addr + kOzStageA;
+                asm volatile("" : "+r"(sa_addr), "+r"(sb_addr));   // keep the descriptors per piece
+                const uint64_t da = oz_desc(sa_addr), db = oz_desc(sb_addr);
+#pragma unroll 1
+                for (int kk = 0; kk < 2; ++kk)         // K steps of 16: two core matrices, 256 bytes
+                    issue_digit_step<kOzSlices>(tmem, da + (uint64_t)(kk * (256 >> 4)), db + (uint64_t)(kk * (256 >> 4)),
+                                                kOzBlock, kOzHalf, idesc, kk == 0 && i % kOzReadEvery == 0);
+                mma_commit(&empty[b]);
+                if (i % kOzReadEvery == kOzReadEvery - 1 || i + 1 == np) mma_commit(&accfull);
+            }
+            mma_commit(&drain);                        // no MMA in flight when the CTA leaves
+            mbar_wait_bounded(&drain, 0, 1ll << 24);
+        }
+    } else {                                           // ---- sparse digits, read-out
+        long long hi[16], lo[16];
 #pragma unroll
-        for (int d = 0; d < kOzSlices; ++d) {
-            const int sh = 7 * (3 - (d & 3));
+        for (int c = 0; c < 16; ++c) {
+            hi[c] = 0;
+            lo[c] = 0;
+        }
+        auto wait = [&](uint64_t *bar, uint32_t parity) { return __all_sync(0xffffffffu, oz_wait(bar, parity, ok)) != 0; };
+        auto read_out = [&](int group) -> bool {
+            if (!wait(&accfull, (uint32_t)(group & 1))) return false;
+            tc_fence_after();
+            const uint32_t lane_base = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(16 * grp);
 #pragma unroll
-            for (int h16 = 0; h16 < 2; ++h16) {
+            for (int d = 0; d < kOzSlices; ++d) {
                 float r[16];
-                tmem_ld16(lane_base + (uint32_t)(d * 64 + 16 * h16), r);
+                tmem_ld16(lane_base + (uint32_t)(d * 64), r);
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
-                    const long long v = (long long)__float2int_rn(r[c]) << sh;
-                    if (d < 4) hi[16 * h16 + c] += v;
-                    else lo[16 * h16 + c] += v;
+                    const long long x = (long long)__float2int_rn(r[c]) << (7 * (3 - (d & 3)));
+                    if (d < 4) hi[c] += x;
+                    else lo[c] += x;
                 }
             }
-        }
-        tc_fence_before();
-        __syncthreads();                               // accumulators read: the next MMAs may overwrite
-    }
-    if (threadIdx.x == 0 && !s_ok) {
-        // let MMAs and copies in flight finish before the CTA frees its memory (bounded)
-        mma_commit(&drain);
-        mbar_wait_bounded(&drain, 0, kOzWaitLimit);
-        for (int j = n_landed; j < n_loaded; ++j) mbar_wait_bounded(&full[j & 1], (uint32_t)((j >> 1) & 1), kOzWaitLimit);
-        atomicExch(g.status, 1);
-    }
-    if (s_ok && row < g.rowsA) {
-        const int Ea = g.emA[row] - 1022;
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&accfree);
+            return true;
+        };
+        bool fine = true;
+        int done = 0;                                  // accumulation groups read out
+        if (sparse) {
+            // Half of the workers fill stage 0, half stage 1, so a fill may take the time of two
+            // pieces' MMAs.
+            constexpr int kHalfW = kOzWorkers / 2;
+            const double *vals = g.vals + g.rowptr[(int64_t)rt * 128];
+            const int b = tid / kHalfW, wt = tid % kHalfW;
+            unsigned char *sa = stage[b];
+            auto place = [&](uint32_t o, double x) {
+                int d[kOzSlices];
+                oz_digits(x, s_em[(o >> 9) * 8 + ((o >> 4) & 7)] - 1022, d);
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
-            const int64_t col = col0 + c;
-            if (col >= g.rowsB) continue;
-            const int E = Ea + g.emB[col] - 1022 - 61;
-            const double sc = (E >= -1022 && E <= 1023) ? __longlong_as_double((long long)(E + 1023) << 52)
-                                                        : ldexp(1.0, E);
-            const double r = fma(__ll2double_rn(hi[c]), 268435456.0, __ll2double_rn(lo[c])) * sc;
-            double *o = g.out + row * g.ldo + col;
-            if (g.mode == 0) {
-                atomicAdd(o, g.alpha * r);
-            } else {
-                const double s = g.colscale ? g.colscale[col] : 1.0;
-                *o = g.alpha * s * r + (g.beta != 0.0 ? g.beta * *o : 0.0);
+                for (int p = 0; p < kOzSlices; ++p)
+                    *reinterpret_cast<__half *>(sa + (uint32_t)p * kOzBlock + o) = __int2half_rn(d[p]);
+            };
+            // this thread's first two entries of its next pair are loaded a fill ahead
+            uint32_t off[2] = {0, 0};
+            double v[2] = {0.0, 0.0};
+            int64_t p1 = 0, pn = 0;
+            auto ahead = [&](int q) {
+                pn = g.ent_ptr[q] + wt;
+                p1 = g.ent_ptr[q + 1];
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    if (pn + kHalfW * u < p1) {
+                        off[u] = g.ent_off[pn + kHalfW * u];
+                        v[u] = vals[g.ent_e[pn + kHalfW * u]];
+                    }
+            };
+            if (b < np) ahead(q0 + b);
+            for (int i = b; i < np; i += 2) {          // every worker comes to its barriers, whatever happens
+                if (i >= 2 && fine) fine = wait(&empty[b], (uint32_t)(((i >> 1) - 1) & 1));
+                // a group that ended with this stage's last piece is read out first: the MMAs wait
+                if (fine && (done + 1) * kOzReadEvery <= i - 1) fine = read_out(done++);
+                uint4 *z = reinterpret_cast<uint4 *>(sa);
+#pragma unroll
+                for (uint32_t o = 0; o < kOzStageA / 16; o += kHalfW) z[o + wt] = make_uint4(0, 0, 0, 0);
+                asm volatile("bar.sync %0, %1;" ::"r"(1 + b), "n"(kHalfW) : "memory");
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    if (pn + kHalfW * u < p1) place(off[u], v[u]);
+                for (int64_t p = pn + 2 * kHalfW; p < p1; p += kHalfW) place(g.ent_off[p], vals[g.ent_e[p]]);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&placed[b]);
+                if (i + 2 < np) ahead(q0 + i + 2);
+                // one that ended with the other stage's last piece: this piece is ready behind it
+                if (fine && (done + 1) * kOzReadEvery <= i) fine = read_out(done++);
+            }
+        }
+        while (fine && (done + 1) * kOzReadEvery < np) fine = read_out(done++);
+        if (fine) fine = read_out((np - 1) / kOzReadEvery);
+        if (fine && row < g.rowsA) {
+            const int Ea = g.emA[row] - 1022;
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {
+                const int64_t col = col0 + c;
+                if (col >= g.rowsB) continue;
+                const int E = Ea + g.emB[col] - 1022 - 61;
+                const double sc = (E >= -1022 && E <= 1023) ? __longlong_as_double((long long)(E + 1023) << 52)
+                                                            : ldexp(1.0, E);
+                const double r = fma(__ll2double_rn(hi[c]), 268435456.0, __ll2double_rn(lo[c])) * sc;
+                double *o = g.out + row * g.ldo + col;
+                if (g.mode == 0) {
+                    atomicAdd(o, g.alpha * r);
+                } else {
+                    const double s = g.colscale ? g.colscale[col] : 1.0;
+                    *o = g.alpha * s * r + (g.beta != 0.0 ? g.beta * *o : 0.0);
+                }
             }
         }
     }
     tc_fence_before();
     __syncthreads();
+    if (tid == 0 && !s_ok) atomicExch(g.status, 1);
     if (warp == 0) tmem_dealloc(tmem, kTmemColsOz);
 }
 

@@ -27,7 +27,7 @@
 // tc_ptx.cuh), as one 16 KB block per (operand, 128-row tile, slice), and the row
 // exponents; k_schur_tc computes one 128 x 64 output tile per CTA: one bulk copy brings
 // the 7 A-slices of its row tile, seven bring the B-slices of its column half-tile, one
-// thread issues the 28 x 4 MMAs, and four warps read the 7 accumulators back and update
+// thread issues the 28 x 4 digit products (40 MMAs), and eight warps read the 7 accumulators back and update
 // the FP64 front.  Every wait is bounded; a wait that runs out records a timeout in the
 // shift's counters, and the CTA still releases its tensor memory.
 #pragma once
@@ -218,10 +218,13 @@ __global__ void __launch_bounds__(kSchurTcThreads, 1) k_schur_tc(const StepTask 
         if (!mbar_wait_bounded(&bar[0], 0, kWaitLimit)) {
             s_ok = 0;
         } else {
-            const uint32_t idesc = idesc_f16_f32(kTileM, kTileN);
-            static_assert(kSlices == 7 && kAccum == 7, "the issue loop covers 7 slices and 7 accumulators");
-            issue_digit_mmas<kSliceBytes, kHalfSliceBytes, kTileN>(tmem, smem_desc(smem_u32(sa)),
-                                                                    smem_desc(smem_u32(sb)), idesc, true);
+            const uint32_t idesc = idesc_f16_f32(kTileM, 0);
+            static_assert(kAccum == kSlices && kTileN == 64, "accumulator d holds the products p + q = d");
+#pragma unroll 1
+            for (int kk = 0; kk < 4; ++kk)
+                issue_digit_step<kSlices>(tmem, smem_desc(smem_u32(sa)) + (uint64_t)(kk * (kKStepBytes >> 4)),
+                                          smem_desc(smem_u32(sb)) + (uint64_t)(kk * (kKStepBytes >> 4)), kSliceBytes,
+                                          kHalfSliceBytes, idesc, kk == 0);
             mma_commit(&bar[1]);
             if (!mbar_wait_bounded(&bar[1], 0, kWaitLimit)) {
                 s_ok = 0;

@@ -116,28 +116,24 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar) {
                  : "memory");
 }
 
-// The 112 MMAs of one 64-wide piece of a digit-sliced product (7 slices per operand):
-// accumulator d (tensor-memory columns d * kNCols ..) gets sum_{p + q = d} A_p B_q^T.  da, db
-// are the descriptors of slice 0 of A and B, the slices kAStride / kBStride bytes apart.  The
-// descriptors advance by additions to the start-address field (16-byte units), a few
-// instructions per MMA, so one thread keeps the tensor pipe fed; the (d, p) loops stay
-// rolled so the 224 descriptors are not all held in registers.  fresh: the first MMA into
-// each accumulator overwrites it.
-template <uint32_t kAStride, uint32_t kBStride, uint32_t kNCols>
-__device__ __forceinline__ void issue_digit_mmas(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc,
-                                                 bool fresh) {
-    const uint32_t keep_first = fresh ? 0u : 1u;
-#pragma unroll 1
-    for (int d = 0; d < 7; ++d) {
-        const uint32_t t = tmem + (uint32_t)d * kNCols;
-#pragma unroll 1
-        for (int p = 0; p <= d; ++p) {
-            const uint64_t a = da + (uint64_t)(p * (kAStride >> 4));
-            const uint64_t b = db + (uint64_t)((d - p) * (kBStride >> 4));
+// The MMAs of one K step of a digit-sliced product: accumulator d (tensor-memory columns 64 d ..,
+// d < S) gets sum_{p + q = d} A_p B_q^T, N = 64 rows to a digit of B.  The digits of B lie one after
+// another, and so do the accumulators, so A_p times digits q .. q + 3 of B is ONE MMA of N = 256 into
+// accumulators p + q .. p + q + 3: S (S + 1) / 2 products in 10 (S = 7) or 12 (S = 8) MMAs.  At
+// N = 64 an MMA reads 6 KB of operands for 32 cycles of work and took about 60; merged, A is read
+// once for four products and the tensor pipe is the limit.  a, b: descriptors of digit 0 at this K
+// step, digits astride / bstride bytes apart.  fresh: the accumulators are overwritten (p = 0
+// reaches all of them).
+template <int S>
+__device__ __forceinline__ void issue_digit_step(uint32_t tmem, uint64_t a, uint64_t b, uint32_t astride,
+                                                 uint32_t bstride, uint32_t idesc_n0, bool fresh) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                mma_f16(t, a + (uint64_t)(kk * (kKStepBytes >> 4)), b + (uint64_t)(kk * (kKStepBytes >> 4)), idesc,
-                        (kk == 0 && p == 0) ? keep_first : 1u);
+    for (int p = 0; p < S; ++p) {
+#pragma unroll
+        for (int q = 0; q < S - p; q += 4) {
+            const int n = (S - p - q < 4 ? S - p - q : 4) * 64;
+            mma_f16(tmem + (uint32_t)(p + q) * 64, a + (uint64_t)(p * (astride >> 4)), b + (uint64_t)(q * (bstride >> 4)),
+                    idesc_n0 | ((uint32_t)(n >> 3) << 17), (fresh && p == 0) ? 0u : 1u);
         }
     }
 }
