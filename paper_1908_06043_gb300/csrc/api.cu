@@ -102,8 +102,45 @@ extern "C" ss_status ss_create(ss_ctx **ctx, int32_t device, void *cuda_stream) 
         delete c;
         return SS_ERR_CUDA;
     }
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    uint64_t keep = kPoolKeepBytes;
+    if (cudaMemPoolCreate(&c->pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        if (c->pool) cudaMemPoolDestroy(c->pool);
+        c->pool = nullptr;                     // the device's default pool then
+    }
     *ctx = c;
     return SS_OK;
+}
+
+static void pool_trim(ss_ctx *ctx) {
+    cudaGetLastError();
+    if (!ctx->pool) return;
+    cudaStreamSynchronize(ctx->stream);        // blocks freed on the stream can go only then
+    cudaMemPoolTrimTo(ctx->pool, 0);
+}
+
+cudaError_t ss_malloc_async(ss_ctx *ctx, void **p, size_t bytes, cudaStream_t st) {
+    if (!ctx->pool) return cudaMallocAsync(p, bytes, st);
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
+    if (e == cudaErrorMemoryAllocation) {
+        pool_trim(ctx);
+        e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
+    }
+    return e;
+}
+
+cudaError_t ss_malloc(ss_ctx *ctx, void **p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && ctx->pool) {
+        pool_trim(ctx);
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
 }
 
 extern "C" ss_status ss_destroy(ss_ctx *ctx) {
@@ -125,7 +162,7 @@ extern "C" ss_status ss_selftest_barrier(ss_ctx *ctx, int32_t extra_arrivals, in
     SS_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
     cudaStream_t st = ctx->stream;
     GridBar *bar = nullptr;
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&bar, sizeof(GridBar), st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&bar, sizeof(GridBar), st));
     SS_CUDA_TRY(ctx, cudaMemsetAsync(bar, 0, sizeof(GridBar), st));
     const unsigned int nb = (unsigned int)ctx->sm_count;          // one block per SM: resident
     unsigned int expected = nb + (unsigned int)extra_arrivals;
@@ -213,10 +250,10 @@ extern "C" ss_status ss_selftest_tc(ss_ctx *ctx, uint64_t seed, double *max_abs_
     float *dD = nullptr;
     int *dst = nullptr;
     cudaStream_t st = ctx->stream;
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&dA, sstc::kSliceBytes, st));
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&dB, sstc::kHalfSliceBytes, st));
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&dD, sizeof(float) * M * N, st));
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&dst, sizeof(int), st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&dA, sstc::kSliceBytes, st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&dB, sstc::kHalfSliceBytes, st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&dD, sizeof(float) * M * N, st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&dst, sizeof(int), st));
     SS_CUDA_TRY(ctx, cudaMemcpyAsync(dA, ha.data(), sstc::kSliceBytes, cudaMemcpyHostToDevice, st));
     SS_CUDA_TRY(ctx, cudaMemcpyAsync(dB, hb.data(), sstc::kHalfSliceBytes, cudaMemcpyHostToDevice, st));
     SS_CUDA_TRY(ctx, cudaMemsetAsync(dD, 0, sizeof(float) * M * N, st));
@@ -255,7 +292,7 @@ template <typename V>
 static int upload_vec(ss_ctx *ctx, const std::vector<V> &h, V **d) {
     *d = nullptr;
     if (h.empty()) return SS_OK;
-    SS_CUDA_TRY(ctx, cudaMalloc((void **)d, sizeof(V) * h.size()));
+    SS_CUDA_TRY(ctx, ss_malloc(ctx, (void **)d, sizeof(V) * h.size()));
     SS_CUDA_TRY(ctx, cudaMemcpy(*d, h.data(), sizeof(V) * h.size(), cudaMemcpyHostToDevice));
     return SS_OK;
 }
@@ -349,7 +386,7 @@ __global__ void k_row_abs_max(int64_t n, const int64_t *__restrict__ rowptr, con
 int ss_norm1(ss_symbolic *s, const double *vals, double *out) {
     ss_ctx *ctx = s->ctx;
     unsigned long long *d = nullptr, h = 0;
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&d, sizeof(unsigned long long), ctx->stream));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&d, sizeof(unsigned long long), ctx->stream));
     SS_CUDA_TRY(ctx, cudaMemsetAsync(d, 0, sizeof(unsigned long long), ctx->stream));
     ss_launch(ctx, SS_K_MISC, k_row_abs_max, (unsigned)((s->n + 255) / 256), 256, 0, ctx->stream, s->n, s->d_rowptr, vals, d);
     SS_CUDA_TRY(ctx, cudaMemcpyAsync(&h, d, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
@@ -600,13 +637,13 @@ static int factor_wave_graph(ss_numeric *f, const std::vector<int> &js, bool tc,
         pl->ns = ns;
         pl->fp32 = fp32;
         pl->tc = tc ? 1 : 0;
-        cudaError_t e = cudaMalloc(&pl->mt, sizeof(T) * z.mt_n * ns);
-        if (e == cudaSuccess) e = cudaMalloc(&pl->wb, sizeof(T) * z.wb_n * ns);
-        if (e == cudaSuccess) e = cudaMalloc(&pl->ws, sizeof(T) * z.ws_n * ns);
-        if (e == cudaSuccess) e = cudaMalloc(&pl->cb, sizeof(T) * z.cb_n * ns);
-        if (e == cudaSuccess) e = cudaMalloc(&pl->sl, (size_t)z.sl_n * ns);
-        if (e == cudaSuccess) e = cudaMalloc(&pl->ex, sizeof(int32_t) * z.ex_n * ns);
-        if (e == cudaSuccess) e = cudaMalloc(&pl->dp, sizeof(ShiftPtrs<T>) * ns);
+        cudaError_t e = ss_malloc(ctx, &pl->mt, sizeof(T) * z.mt_n * ns);
+        if (e == cudaSuccess) e = ss_malloc(ctx, &pl->wb, sizeof(T) * z.wb_n * ns);
+        if (e == cudaSuccess) e = ss_malloc(ctx, &pl->ws, sizeof(T) * z.ws_n * ns);
+        if (e == cudaSuccess) e = ss_malloc(ctx, &pl->cb, sizeof(T) * z.cb_n * ns);
+        if (e == cudaSuccess) e = ss_malloc(ctx, &pl->sl, (size_t)z.sl_n * ns);
+        if (e == cudaSuccess) e = ss_malloc(ctx, &pl->ex, sizeof(int32_t) * z.ex_n * ns);
+        if (e == cudaSuccess) e = ss_malloc(ctx, &pl->dp, sizeof(ShiftPtrs<T>) * ns);
         s->plans.push_back(pl);
         if (e != cudaSuccess) {
             cudaGetLastError();
@@ -679,6 +716,12 @@ static int factor_run(ss_numeric *f, const std::vector<int> &which) {
     const double per_shift = wave_bytes<T>(z);
     size_t mem_free = 0, mem_tot = 0;
     SS_CUDA_TRY(ctx, cudaMemGetInfo(&mem_free, &mem_tot));
+    if (ctx->pool) {                             // what the pool holds unused is free too
+        uint64_t held = 0, used = 0;
+        if (cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+            cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && held > used)
+            mem_free += (size_t)(held - used);
+    }
     int wave = (int)std::max(1.0, std::min((double)std::min(ns_all, 65535), std::floor(0.8 * (double)mem_free / per_shift)));
     static const unsigned long long init[SS_NCOUNT] = {0, 0, 0, 0, 0x7ff0000000000000ull /* +inf */, 0, 0, 0};
     for (int q = 0; q < ns_all; ++q)
@@ -698,19 +741,19 @@ static int factor_run(ss_numeric *f, const std::vector<int> &which) {
         T *mt = nullptr, *wb = nullptr, *ws = nullptr, *cb = nullptr;
         unsigned char *sl = nullptr;
         int32_t *ex = nullptr;
-        SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&sl, (size_t)z.sl_n * ns, st));
-        SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&ex, sizeof(int32_t) * z.ex_n * ns, st));
-        SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&mt, sizeof(T) * z.mt_n * ns, st));
-        SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&wb, sizeof(T) * z.wb_n * ns, st));
-        SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&ws, sizeof(T) * z.ws_n * ns, st));
-        SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&cb, sizeof(T) * z.cb_n * ns, st));
+        SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&sl, (size_t)z.sl_n * ns, st));
+        SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&ex, sizeof(int32_t) * z.ex_n * ns, st));
+        SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&mt, sizeof(T) * z.mt_n * ns, st));
+        SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&wb, sizeof(T) * z.wb_n * ns, st));
+        SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&ws, sizeof(T) * z.ws_n * ns, st));
+        SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&cb, sizeof(T) * z.cb_n * ns, st));
         std::vector<ShiftPtrs<T>> hp(ns);
         for (int q = 0; q < ns; ++q) {
             fill_shift<T>(f, js[q], hp[q]);
             point_scratch<T>(hp[q], z, q, mt, wb, ws, cb, sl, ex);
         }
         ShiftPtrs<T> *dp = nullptr;
-        SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&dp, sizeof(ShiftPtrs<T>) * ns, st));
+        SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&dp, sizeof(ShiftPtrs<T>) * ns, st));
         SS_CUDA_TRY(ctx, cudaMemcpyAsync(dp, hp.data(), sizeof(ShiftPtrs<T>) * ns, cudaMemcpyHostToDevice, st));
         int rc = factor_levels<T>(f, ns, dp, hp, tc, ctx->step_times ? &step_ev : nullptr);
         if (rc != SS_OK) return rc;
@@ -791,16 +834,16 @@ int ss_factor_create(ss_symbolic *sym, const double *a_vals, const double *b_val
     f->linv.assign(n_shift, nullptr);
     f->dblk.assign(n_shift, nullptr);
     f->piv.assign(n_shift, nullptr);
-    cudaError_t e = cudaMalloc((void **)&f->d_counts, sizeof(unsigned long long) * SS_NCOUNT * n_shift);
+    cudaError_t e = ss_malloc(ctx, (void **)&f->d_counts, sizeof(unsigned long long) * SS_NCOUNT * n_shift);
     if (seg && e == cudaSuccess) {
         // the pencil of every stored entry (from its row) and the shift table, on the device
         f->n_seg = seg->n_seg;
         std::vector<int32_t> eseg(std::max<int64_t>(1, sym->nnz));
         for (int64_t r = 0; r < sym->n; ++r)
             for (int64_t q = sym->rowptr[r]; q < sym->rowptr[r + 1]; ++q) eseg[q] = seg->row_seg[r];
-        e = cudaMalloc((void **)&f->d_eseg, sizeof(int32_t) * eseg.size());
-        if (e == cudaSuccess) e = cudaMalloc((void **)&f->d_rowseg, sizeof(int32_t) * std::max<int64_t>(1, sym->n));
-        if (e == cudaSuccess) e = cudaMalloc((void **)&f->d_seg_sigma, sizeof(double) * n_shift * seg->n_seg);
+        e = ss_malloc(ctx, (void **)&f->d_eseg, sizeof(int32_t) * eseg.size());
+        if (e == cudaSuccess) e = ss_malloc(ctx, (void **)&f->d_rowseg, sizeof(int32_t) * std::max<int64_t>(1, sym->n));
+        if (e == cudaSuccess) e = ss_malloc(ctx, (void **)&f->d_seg_sigma, sizeof(double) * n_shift * seg->n_seg);
         if (e == cudaSuccess)
             e = cudaMemcpy(f->d_eseg, eseg.data(), sizeof(int32_t) * eseg.size(), cudaMemcpyHostToDevice);
         if (e == cudaSuccess)
@@ -810,10 +853,10 @@ int ss_factor_create(ss_symbolic *sym, const double *a_vals, const double *b_val
                            cudaMemcpyHostToDevice);
     }
     for (int j = 0; j < n_shift && e == cudaSuccess; ++j) {
-        if (!f->inertia_only) e = cudaMalloc(&f->arena[j], esz * std::max<int64_t>(1, sym->l_total));
-        if (e == cudaSuccess) e = cudaMalloc((void **)&f->linv[j], sizeof(double) * NB * NB * npan);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&f->dblk[j], sizeof(double) * 2 * NB * npan);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&f->piv[j], sizeof(int32_t) * NB * npan);
+        if (!f->inertia_only) e = ss_malloc(ctx, &f->arena[j], esz * std::max<int64_t>(1, sym->l_total));
+        if (e == cudaSuccess) e = ss_malloc(ctx, (void **)&f->linv[j], sizeof(double) * NB * NB * npan);
+        if (e == cudaSuccess) e = ss_malloc(ctx, (void **)&f->dblk[j], sizeof(double) * 2 * NB * npan);
+        if (e == cudaSuccess) e = ss_malloc(ctx, (void **)&f->piv[j], sizeof(int32_t) * NB * npan);
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -841,7 +884,7 @@ int ss_factor_create(ss_symbolic *sym, const double *a_vals, const double *b_val
             if (rc != SS_OK) break;
             f->arena_lo[j] = (float *)f->arena[j];
             f->arena[j] = nullptr;
-            cudaError_t e2 = cudaMalloc(&f->arena[j], sizeof(double) * std::max<int64_t>(1, sym->l_total));
+            cudaError_t e2 = ss_malloc(ctx, &f->arena[j], sizeof(double) * std::max<int64_t>(1, sym->l_total));
             if (e2 != cudaSuccess) {
                 cudaGetLastError();
                 rc = ctx->set_error(SS_ERR_OOM, "ss_factor: device allocation for an FP64 refactor failed");
@@ -876,7 +919,7 @@ int ss_factor_create(ss_symbolic *sym, const double *a_vals, const double *b_val
         for (int j = 0; j < n_shift && rc == SS_OK; ++j) {
             f->shift_prec[j] = SS_FP64;
             const int64_t na = std::max<int64_t>(1, sym->l_total);
-            cudaError_t e2 = cudaMalloc((void **)&f->arena_lo[j], sizeof(float) * na);
+            cudaError_t e2 = ss_malloc(ctx, (void **)&f->arena_lo[j], sizeof(float) * na);
             if (e2 != cudaSuccess) {
                 cudaGetLastError();
                 f->arena_lo[j] = nullptr;
@@ -996,7 +1039,7 @@ extern "C" ss_status ss_inertia_segments(const ss_numeric *f, int32_t j, int64_t
     const int32_t npan = (int32_t)s->panels.size();
     cudaStream_t st = ctx->stream;
     unsigned long long *d = nullptr;
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&d, sizeof(unsigned long long) * 4 * f->n_seg, st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&d, sizeof(unsigned long long) * 4 * f->n_seg, st));
     SS_CUDA_TRY(ctx, cudaMemsetAsync(d, 0, sizeof(unsigned long long) * 4 * f->n_seg, st));
     const double tiny = 64.0 * 1.1102230246251565e-16 * (f->norm_a1 + std::fabs(f->sigma[j]) * f->norm_b1);
     if (npan > 0)
@@ -1179,7 +1222,7 @@ static int fold_sweeps(ss_numeric *f, int j, double *b, int k, bool full) {
     ss_symbolic *s = f->sym;
     ss_ctx *ctx = s->ctx;
     cudaStream_t st = ctx->stream;
-    if (!ctx->d_bar) SS_CUDA_TRY(ctx, cudaMalloc((void **)&ctx->d_bar, kBarBytes));
+    if (!ctx->d_bar) SS_CUDA_TRY(ctx, ss_malloc(ctx, (void **)&ctx->d_bar, kBarBytes));
     const int nc = fold_nc(k), nch = (k + nc - 1) / nc, mc = fold_mid_cols(k);
     // enough blocks that the largest step's items lie on as many SMs as there are, no more: a
     // barrier over few blocks is quicker
@@ -1229,7 +1272,7 @@ int solve_half_backward(ss_numeric *f, int j, const double *y, int k, double *x)
     const int64_t tot = s->n * k;
     const unsigned g = (unsigned)((tot + 255) / 256);
     double *w = nullptr;
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&w, sizeof(double) * tot, st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&w, sizeof(double) * tot, st));
     ss_launch(ctx, SS_K_MISC, k_dhalf<double>, g, 256, 0, st, s->n, s->d_col_panel, s->d_panels, f->dblk[j], y, w, k);
     int rc = fold_solve(f, j, w, k, false);
     if (rc != SS_OK) return rc;
@@ -1247,7 +1290,7 @@ static int solve_sweeps(ss_numeric *f, int j, float *b, int k, const float *aren
     ss_ctx *ctx = s->ctx;
     cudaStream_t st = ctx->stream;
     const int cls = SS_K_SOLVE_F32;
-    if (!ctx->d_bar) SS_CUDA_TRY(ctx, cudaMalloc((void **)&ctx->d_bar, kBarBytes));
+    if (!ctx->d_bar) SS_CUDA_TRY(ctx, ss_malloc(ctx, (void **)&ctx->d_bar, kBarBytes));
     int32_t *sm_slots = reinterpret_cast<int32_t *>(ctx->d_bar + 1);
     int &per_sm = ctx->sweep_blocks_per_sm;
     if (per_sm == 0) {
@@ -1273,7 +1316,7 @@ static int solve_sweeps(ss_numeric *f, int j, float *b, int k, const float *aren
     const int64_t yn = fused ? s->n * (int64_t)k : 0;
     float *zall = nullptr, *ybuf = nullptr;
     int32_t *arrive = nullptr;
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&zall, sizeof(float) * (zn + an + yn), st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&zall, sizeof(float) * (zn + an + yn), st));
     SS_CUDA_TRY(ctx, cudaMemsetAsync(zall, 0, sizeof(float) * (zn + an), st));
     if (fused) {
         arrive = reinterpret_cast<int32_t *>(zall + zn);
@@ -1340,7 +1383,7 @@ static int solve_levels(ss_numeric *f, int j, float *b, int k) {
     int32_t maxc = 0;
     for (const SolveLevel &sl : s->solve_levels) maxc = std::max(maxc, sl.count);
     float *z = nullptr;
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&z, sizeof(float) * (int64_t)maxc * NB * k, st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&z, sizeof(float) * (int64_t)maxc * NB * k, st));
     for (int L = nlev - 1; L >= 0; --L) {
         const SolveLevel &sl = s->solve_levels[L];
         const int32_t *lp = s->d_solve_panels + sl.panel_off;
@@ -1471,9 +1514,9 @@ int solve_contraction(ss_numeric *f, int j, double *rho) {
     double *r = nullptr, *x = nullptr, *y = nullptr, *co = nullptr;
     float *w = nullptr;
     unsigned long long *mx = nullptr;
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&r, sizeof(double) * (3 * n + 2), st));
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&w, sizeof(float) * n, st));
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&mx, sizeof(unsigned long long) * 2, st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&r, sizeof(double) * (3 * n + 2), st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&w, sizeof(float) * n, st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&mx, sizeof(unsigned long long) * 2, st));
     x = r + n;
     y = x + n;
     co = y + n;
@@ -1513,7 +1556,7 @@ static int shifted_values(ss_numeric *f, int j, const double **out) {
     ss_ctx *ctx = s->ctx;
     if (!f->mvals[j]) {
         double *m = nullptr;
-        SS_CUDA_TRY(ctx, cudaMalloc((void **)&m, sizeof(double) * std::max<int64_t>(1, s->nnz)));
+        SS_CUDA_TRY(ctx, ss_malloc(ctx, (void **)&m, sizeof(double) * std::max<int64_t>(1, s->nnz)));
         const unsigned g = (unsigned)std::min<int64_t>((s->nnz + 255) / 256, (int64_t)ctx->sm_count * 16);
         ss_launch(ctx, SS_K_MISC, k_shifted_vals, std::max(1u, g), 256, 0, ctx->stream, s->nnz, f->a_vals, f->b_vals,
                   f->sigma[j], m);
@@ -1557,10 +1600,10 @@ int solve_apply(ss_numeric *f, int j, const double *R, int k, double *X, int ref
         // refinement in the factor's own precision removes the effect of element growth
         // on the solve's backward error)
         double *w = nullptr, *x = nullptr, *y = nullptr;
-        SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&w, sizeof(double) * tot, st));
+        SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&w, sizeof(double) * tot, st));
         if (refine > 0) {
-            SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&x, sizeof(double) * tot, st));
-            SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&y, sizeof(double) * tot, st));
+            SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&x, sizeof(double) * tot, st));
+            SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&y, sizeof(double) * tot, st));
         }
         double *out = refine > 0 ? x : X;
         ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, double>, g, 256, 0, st, s->n, k, s->d_perm, R, w, 0);
@@ -1595,13 +1638,13 @@ int solve_apply(ss_numeric *f, int j, const double *R, int k, double *X, int ref
         refine = std::max(refine, std::min(8, (int)std::ceil(std::log(1e-13) / std::log(f->rho[j])) - 1));
     }
     unsigned long long *mx = nullptr;
-    if (target > 0.0) SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&mx, sizeof(unsigned long long) * 2, st));
+    if (target > 0.0) SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&mx, sizeof(unsigned long long) * 2, st));
     float *wf = nullptr;
     double *r = nullptr, *y = nullptr, *x = nullptr;
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&wf, sizeof(float) * tot, st));
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&r, sizeof(double) * tot, st));
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&y, sizeof(double) * tot, st));
-    SS_CUDA_TRY(ctx, cudaMallocAsync((void **)&x, sizeof(double) * tot, st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&wf, sizeof(float) * tot, st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&r, sizeof(double) * tot, st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&y, sizeof(double) * tot, st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&x, sizeof(double) * tot, st));
     SS_CUDA_TRY(ctx, cudaMemsetAsync(x, 0, sizeof(double) * tot, st));
     for (int it = 0; it <= refine; ++it) {
         const double *rhs = R;

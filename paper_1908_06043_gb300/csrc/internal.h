@@ -27,6 +27,7 @@ struct ss_ctx {
     std::vector<double> *step_times = nullptr;   // per factor step Schur time (autotuner), or null
     int64_t plan_gen = 0;                     // bumped when a setting baked into captured graphs changes
     double tc_min_flops = 2.0e7;              // a factor step's Schur flops below which it stays on CUDA cores
+    cudaMemPool_t pool = nullptr;             // this context's scratch (ss_malloc_async)
     GridBar *d_bar = nullptr;                 // grid barrier state of the sweep kernel
     int sweep_blocks_per_sm = 0;              // resident FP32 sweep-kernel blocks per SM
     int sweep_fuse_max = 0;                   // FP32 sweep: fuse levels with at most this many items
@@ -53,9 +54,18 @@ struct ss_ctx {
         for (cudaEvent_t e : ev_pool) cudaEventDestroy(e);
         if (cap_stream) cudaStreamDestroy(cap_stream);
         if (d_bar) cudaFree(d_bar);
+        if (pool) cudaMemPoolDestroy(pool);
     }
 };
 
+// Stream-ordered scratch of the context's calls, freed with cudaFreeAsync.  The context has a pool
+// of its own that keeps up to kPoolKeepBytes between calls (the default pool gives everything back
+// at each synchronisation, and mapping 0.1 - 2 GB again took up to 4 ms a call); what it holds unused
+// goes back when an allocation would fail, and all of it with the context.
+constexpr uint64_t kPoolKeepBytes = 1ull << 30;
+cudaError_t ss_malloc_async(ss_ctx *ctx, void **p, size_t bytes, cudaStream_t st);
+// cudaMalloc that takes the pool's unused memory back before it gives up
+cudaError_t ss_malloc(ss_ctx *ctx, void **p, size_t bytes);
 extern std::atomic<int64_t> g_ss_launches;
 size_t ss_prof_begin(ss_ctx *ctx, int cls);
 void ss_prof_end(ss_ctx *ctx, int cls, size_t slot);

@@ -33,11 +33,12 @@ constexpr double kPieceTensorFlops = 36.0 * 2.0 * 2.0 * 128 * 64 * 16;
 // per-call device scratch from the stream-ordered pool
 struct Scratch {
     std::vector<void *> ptrs;
+    ss_ctx *ctx;
     cudaStream_t st;
-    explicit Scratch(cudaStream_t s) : st(s) {}
+    explicit Scratch(ss_ctx *c) : ctx(c), st(c->stream) {}
     template <typename T>
     cudaError_t get(T **p, size_t count) {
-        cudaError_t e = cudaMallocAsync((void **)p, sizeof(T) * std::max<size_t>(count, 1), st);
+        cudaError_t e = ss_malloc_async(ctx, (void **)p, sizeof(T) * std::max<size_t>(count, 1), st);
         if (e == cudaSuccess) ptrs.push_back(*p);
         return e;
     }
@@ -81,7 +82,7 @@ int slice_dense(ss_ctx *ctx, const OzOperand &op, Scratch &buf, unsigned char **
 }
 
 int run_mm(ss_ctx *ctx, sstc::OzMM g, dim3 grid, int cls) {
-    Scratch buf(ctx->stream);
+    Scratch buf(ctx);
     OZ_ALLOC(ctx, buf.get(&g.status, 1));
     SS_CUDA_TRY(ctx, cudaMemsetAsync(g.status, 0, sizeof(int), ctx->stream));
     ss_launch(ctx, cls, sstc::k_oz_mm, grid, sstc::kOzThreads, sstc::kOzGemmSmem, ctx->stream, g);
@@ -97,7 +98,7 @@ int run_mm(ss_ctx *ctx, sstc::OzMM g, dim3 grid, int cls) {
 int dense_mm(ss_ctx *ctx, const OzOperand &A, const OzOperand &B, int mode, double alpha, double beta, double *out,
              int64_t ldo, double flops) {
     oz_attrs(ctx->device);
-    Scratch buf(ctx->stream);
+    Scratch buf(ctx);
     unsigned char *sa, *sb;
     int *ea, *eb;
     int rc;
@@ -178,7 +179,7 @@ int plan_build(ss_symbolic *s) {
     pl->npairs = (int64_t)pair_piece.size();
     s->oz_plan = pl;
     auto up = [&](auto **d, const auto &h) {
-        cudaError_t e = cudaMalloc((void **)d, sizeof(h[0]) * std::max<size_t>(1, h.size()));
+        cudaError_t e = ss_malloc(ctx, (void **)d, sizeof(h[0]) * std::max<size_t>(1, h.size()));
         if (e == cudaSuccess && !h.empty()) e = cudaMemcpy(*d, h.data(), sizeof(h[0]) * h.size(), cudaMemcpyHostToDevice);
         return e;
     };
@@ -205,7 +206,7 @@ int vals_make(ss_symbolic *s, const double *vals, OzVals *v, Scratch *buf) {
     if (buf) {
         OZ_ALLOC(ctx, buf->get(&v->em, (size_t)s->n));
     } else {
-        OZ_ALLOC(ctx, cudaMalloc(&v->em, sizeof(int) * s->n));
+        OZ_ALLOC(ctx, ss_malloc(ctx, (void **)&v->em, sizeof(int) * s->n));
     }
     oz_attrs(ctx->device);
     ss_launch(ctx, SS_K_SPMM_TC, sstc::k_oz_csr_expmax, cdivu(s->n * 32, 256), 256, 0, ctx->stream, s->n,
@@ -234,7 +235,7 @@ int spmm_core(ss_symbolic *s, int npass, OzVals *const *v, const double *const *
               const double *X, int64_t ldx, int k, double *Y, int64_t ldy) {
     ss_ctx *ctx = s->ctx;
     int rc;
-    Scratch buf(ctx->stream);
+    Scratch buf(ctx);
     unsigned char *sx;
     int *ex;
     // operand rows of X = its k columns, reduction over the n rows
@@ -294,7 +295,7 @@ int oz_spmm(ss_numeric *f, int npass, const int *which, const double *const *col
 
 int oz_spmm_vals(ss_symbolic *s, const double *a, const double *b, const double *alpha, const double *beta,
                  const double *X, int64_t ldx, int k, double *Y, int64_t ldy) {
-    Scratch buf(s->ctx->stream);
+    Scratch buf(s->ctx);
     OzVals va, vb;
     int rc;
     if ((rc = vals_make(s, a, &va, &buf)) != SS_OK) return rc;

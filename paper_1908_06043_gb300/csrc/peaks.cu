@@ -55,7 +55,7 @@ extern "C" ss_status ss_measure_peak(ss_ctx *ctx, int32_t kind, double seconds, 
     SS_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
     const unsigned grid = (unsigned)ctx->sm_count * 4;
     void *sink = nullptr;
-    SS_CUDA_TRY(ctx, cudaMallocAsync(&sink, sizeof(double) * grid, ctx->stream));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&sink, sizeof(double) * grid, ctx->stream));
     long long iters = 1 << 12;
     float ms = 0.f;
     int rc = SS_OK;

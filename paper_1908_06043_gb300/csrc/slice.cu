@@ -21,11 +21,12 @@ namespace {
 
 struct DevBuf {
     std::vector<void *> ptrs;
+    ss_ctx *ctx;
     cudaStream_t st;
-    explicit DevBuf(cudaStream_t s) : st(s) {}
+    explicit DevBuf(ss_ctx *c) : ctx(c), st(c->stream) {}
     template <typename T>
     cudaError_t get(T **p, size_t count) {
-        cudaError_t e = cudaMallocAsync((void **)p, sizeof(T) * std::max<size_t>(count, 1), st);
+        cudaError_t e = ss_malloc_async(ctx, (void **)p, sizeof(T) * std::max<size_t>(count, 1), st);
         if (e == cudaSuccess) ptrs.push_back(*p);
         return e;
     }
@@ -289,7 +290,7 @@ int slice_solve_impl(ss_numeric *f, int j, double lo, double hi, const ss_solve_
     cudaStream_t st = ctx->stream;
     auto t0 = std::chrono::steady_clock::now();
     const int64_t n = s->n;
-    DevBuf buf(st);
+    DevBuf buf(ctx);
     double *V, *BV, *W, *BW, *T1, *T2, *G, *Rinv, *Q, *theta_d, *resid_d, *rr;
     int *info;
     TRY_ALLOC(ctx, buf.get(&V, (size_t)n * k));
@@ -467,7 +468,7 @@ int block_lanczos_impl(ss_numeric *f, int j, double lo, double hi, const ss_solv
     const int refine = o.refine > 0 ? o.refine : 2;
     const double tol = o.tol > 0 ? o.tol : 1e-10;
     const double sigma = f->sigma[j];
-    DevBuf buf(st);
+    DevBuf buf(ctx);
     double *Vb, *AV, *W, *Wk, *T, *Gp, *Rinv, *Hc, *H, *Q, *theta_d, *Qsel, *resid_d, *rr, *be;
     int *info;
     TRY_ALLOC(ctx, buf.get(&Vb, (size_t)n * dmax));
@@ -596,7 +597,7 @@ int lanczos_impl(ss_symbolic *s, ss_numeric *fb, const double *a_vals, const dou
     cudaStream_t st = ctx->stream;
     const int64_t n = s->n;
     int rc;
-    DevBuf buf(st);
+    DevBuf buf(ctx);
     const int64_t blk = n * nv;
     double *X, *BX, *u, *w, *bw, *h, *alpha, *beta, *nrm;
     TRY_ALLOC(ctx, buf.get(&X, (size_t)(steps + 1) * blk));
@@ -735,7 +736,7 @@ extern "C" ss_status ss_dos_estimate(ss_symbolic *s, const double *a_vals, const
         int rc = factor_spd_b(s, b_vals, &fb);
         if (rc != SS_OK) return rc;
         double *x0 = nullptr;
-        rc = cudaMallocAsync((void **)&x0, sizeof(double) * s->n * n_vec, ctx->stream) == cudaSuccess ? SS_OK
+        rc = ss_malloc_async(ctx, (void **)&x0, sizeof(double) * s->n * n_vec, ctx->stream) == cudaSuccess ? SS_OK
              : ctx->set_error(SS_ERR_OOM, "ss_dos_estimate: device allocation failed");
         // start vectors of Lanczos on G^-1 A G^-T (B = G G^T) become x0 = G^-T y0 for the
         // equivalent B-orthonormal Lanczos on B^-1 A
