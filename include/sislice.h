@@ -349,7 +349,8 @@ ss_status ss_factor_stats(const ss_numeric *f, int32_t shift_idx, double *min_pi
  * R and X are DEVICE float64 N x k row-major (may alias).  `refine` FP64 iterative
  * refinement corrections are applied (X += M^-1 (R - (A - sigma_j B) X)); for a shift
  * solved in FP32 at least as many as its contraction factor needs to reach 1e-13 (at
- * most 8).  The residual uses the values of A - sigma_j B, formed on the shift's first
+ * most 8).  Refined solves of many right-hand sides at a shift that has an FP64 factor as well
+ * (SS_FP64_SOLVE32) run in FP64 on the tensor cores, with `refine` corrections.  The residual uses the values of A - sigma_j B, formed on the shift's first
  * refined solve and kept with the factor (nnz doubles per shift).
  * Errors: SS_ERR_ARG, SS_ERR_CUDA, SS_ERR_OOM, SS_ERR_TIMEOUT (sweep kernel barrier). */
 ss_status ss_solve(ss_numeric *f, int32_t shift_idx, const double *R, int32_t k, double *X,

@@ -1631,17 +1631,22 @@ int solve_apply(ss_numeric *f, int j, const double *R, int k, double *X, int ref
     }
     // mixed: FP32 solves inside FP64 iterative refinement, X_0 = 0.  With a target the
     // residual decides when to stop; otherwise a requested refinement gets at least the
-    // number of steps the shift's contraction factor needs to reach 1e-13
+    // number of steps the shift's contraction factor needs to reach 1e-13.  A refined block
+    // solve of a shift whose FP64 factor is there too runs its solves in FP64 on the tensor cores:
+    // one contracts the residual by 1e-10 where an FP32 one gives 1e-1 .. 1e-2 (N = 16,384, k = 304:
+    // 9.2 ms a solve against 6.4 ms, and 3 instead of 8 or 9 for two requested refinements)
+    const bool in_f64 = refine > 0 && f->shift_prec[j] == SS_FP64 && ctx->solve_mode == SS_SOLVE_SWEEP_KERNEL &&
+                        fold_uses_tc(s, k);
     if (target > 0.0) {
         refine = std::max(refine, 12);
-    } else if (refine > 0 && f->rho[j] > 0.0 && f->rho[j] < 1.0) {
+    } else if (!in_f64 && refine > 0 && f->rho[j] > 0.0 && f->rho[j] < 1.0) {
         refine = std::max(refine, std::min(8, (int)std::ceil(std::log(1e-13) / std::log(f->rho[j])) - 1));
     }
     unsigned long long *mx = nullptr;
     if (target > 0.0) SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&mx, sizeof(unsigned long long) * 2, st));
-    float *wf = nullptr;
+    void *w = nullptr;
     double *r = nullptr, *y = nullptr, *x = nullptr;
-    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&wf, sizeof(float) * tot, st));
+    SS_CUDA_TRY(ctx, ss_malloc_async(ctx, &w, (in_f64 ? sizeof(double) : sizeof(float)) * tot, st));
     SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&r, sizeof(double) * tot, st));
     SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&y, sizeof(double) * tot, st));
     SS_CUDA_TRY(ctx, ss_malloc_async(ctx, (void **)&x, sizeof(double) * tot, st));
@@ -1664,13 +1669,23 @@ int solve_apply(ss_numeric *f, int j, const double *R, int k, double *X, int ref
             ss_launch(ctx, SS_K_MISC, k_axpy_sub, g, 256, 0, st, tot, R, y, r);
             rhs = r;
         }
-        ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<float, double>, g, 256, 0, st, s->n, k, s->d_perm, rhs, wf, 0);
-        if ((rc = solve_permuted(f, j, wf, k)) != SS_OK) return rc;
-        ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, float>, g, 256, 0, st, s->n, k, s->d_perm, wf, x, 2);
+        if (in_f64) {
+            double *wd = (double *)w;
+            ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, double>, g, 256, 0, st, s->n, k, s->d_perm, rhs, wd, 0);
+            if ((rc = solve_permuted(f, j, wd, k)) != SS_OK) return rc;
+            ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, double>, g, 256, 0, st, s->n, k, s->d_perm,
+                      (const double *)wd, x, 2);
+        } else {
+            float *wf = (float *)w;
+            ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<float, double>, g, 256, 0, st, s->n, k, s->d_perm, rhs, wf, 0);
+            if ((rc = solve_permuted(f, j, wf, k)) != SS_OK) return rc;
+            ss_launch(ctx, SS_K_PERMUTE, k_permute_rows<double, float>, g, 256, 0, st, s->n, k, s->d_perm,
+                      (const float *)wf, x, 2);
+        }
         if (steps_done && it > 0) (*steps_done)++;
     }
     SS_CUDA_TRY(ctx, cudaMemcpyAsync(X, x, sizeof(double) * tot, cudaMemcpyDeviceToDevice, st));
-    cudaFreeAsync(wf, st);
+    cudaFreeAsync(w, st);
     cudaFreeAsync(r, st);
     cudaFreeAsync(y, st);
     cudaFreeAsync(x, st);
