@@ -177,12 +177,14 @@ struct FactorPlan {
     int64_t gen = 0;       // ss_ctx::plan_gen at capture
 };
 
+struct OzSamples; // tensor-core products: the pattern by output tiles (oz.cu)
 struct OzPlan;   // tensor-core products: (tile, piece) pairs of the pattern (oz.cu)
 struct OzVals;   // tensor-core products: row exponents of one value array (oz.cu)
 
 struct ss_symbolic {
     ss_ctx *ctx = nullptr;
     OzPlan *oz_plan = nullptr;
+    OzSamples *oz_samples = nullptr;
     std::vector<FactorPlan *> plans;         // captured factorisations (freed with the analysis)
     std::vector<int8_t> step_mode;           // per factor step: -1 rule of ss_set_schur_mode,
                                              // 0 CUDA cores, 1 tensor cores (autotuner)
@@ -337,6 +339,9 @@ int oz_spmm_vals(ss_symbolic *s, const double *a, const double *b, const double 
 // Y = diag(alpha) A X + diag(beta) B X for value arrays a, b (tensor cores where possible)
 int spmm_f(ss_numeric *f, const double *a, const double *b, const double *alpha, const double *beta, const double *X,
            int64_t ldx, int k, double *Y, int64_t ldy);
+// grad_a = X X^T, grad_b = -X diag(lambda) X^T on the stored pattern (X n x ne)
+bool oz_sddmm_ok(const ss_symbolic *s, int ne);
+int oz_sddmm(ss_symbolic *s, const double *X, const double *lambda, int ne, double *grad_a, double *grad_b);
 void oz_free_numeric(ss_numeric *f);
 void oz_free_symbolic(ss_symbolic *s);
 // x = P L^-T D^-1/2 y (y permuted order, x original order), SPD factors only

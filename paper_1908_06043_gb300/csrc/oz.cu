@@ -16,6 +16,15 @@ struct OzPlan {
     uint16_t *d_ent_off = nullptr;
 };
 
+// entries at or below the diagonal by (128-row tile, 64-column tile), for the sampled product X Y^T
+struct OzSamples {
+    int64_t ntiles = 0;
+    int32_t *d_rt = nullptr, *d_ct = nullptr;
+    int64_t *d_ptr = nullptr;          // ntiles + 1
+    uint32_t *d_e = nullptr, *d_t = nullptr;   // CSR positions of the entry and its mirror image
+    uint16_t *d_off = nullptr;
+};
+
 struct OzVals {
     const double *vals = nullptr;
     int *em = nullptr;                 // per row: largest biased exponent
@@ -196,6 +205,79 @@ int plan_build(ss_symbolic *s) {
     return SS_OK;
 }
 
+int samples_build(ss_symbolic *s) {
+    ss_ctx *ctx = s->ctx;
+    const int64_t n = s->n, nct = (n + 63) / 64;
+    const int32_t nrt = (int32_t)cdivu(n, 128);
+    std::vector<std::vector<int32_t>> cts(nrt), counts(nrt);
+#pragma omp parallel
+    {
+        std::vector<int32_t> cnt(nct, 0);
+#pragma omp for schedule(dynamic, 16)
+        for (int32_t rt = 0; rt < nrt; ++rt) {
+            const int64_t r0 = rt * 128ll, r1 = std::min<int64_t>(n, r0 + 128);
+            for (int64_t r = r0; r < r1; ++r)
+                for (int64_t p = s->rowptr[r]; p < s->rowptr[r + 1] && s->colind[p] <= r; ++p)
+                    if (cnt[s->colind[p] / 64]++ == 0) cts[rt].push_back(s->colind[p] / 64);
+            std::sort(cts[rt].begin(), cts[rt].end());
+            for (int32_t ct : cts[rt]) {
+                counts[rt].push_back(cnt[ct]);
+                cnt[ct] = 0;
+            }
+        }
+    }
+    std::vector<int32_t> rts, ctl;
+    std::vector<int64_t> ptr(1, 0), first(nrt, 0);
+    for (int32_t rt = 0; rt < nrt; ++rt) {
+        first[rt] = (int64_t)rts.size();
+        for (size_t u = 0; u < cts[rt].size(); ++u) {
+            rts.push_back(rt);
+            ctl.push_back(cts[rt][u]);
+            ptr.push_back(ptr.back() + counts[rt][u]);
+        }
+    }
+    const size_t m = (size_t)std::max<int64_t>(1, ptr.back());
+    std::vector<uint32_t> e(m), t(m);
+    std::vector<uint16_t> off(m);
+#pragma omp parallel
+    {
+        std::vector<int64_t> at(nct, 0);
+#pragma omp for schedule(dynamic, 16)
+        for (int32_t rt = 0; rt < nrt; ++rt) {
+            const int64_t r0 = rt * 128ll, r1 = std::min<int64_t>(n, r0 + 128);
+            for (size_t u = 0; u < cts[rt].size(); ++u) at[cts[rt][u]] = ptr[first[rt] + u];
+            for (int64_t r = r0; r < r1; ++r)
+                for (int64_t p = s->rowptr[r]; p < s->rowptr[r + 1] && s->colind[p] <= r; ++p) {
+                    const int64_t c = s->colind[p], o = at[c / 64]++;
+                    const int32_t *b = s->colind.data() + s->rowptr[c], *z = s->colind.data() + s->rowptr[c + 1];
+                    e[o] = (uint32_t)p;
+                    t[o] = (uint32_t)(std::lower_bound(b, z, (int32_t)r) - s->colind.data());   // (c, r): the pattern is symmetric
+                    off[o] = (uint16_t)((r - r0) * 64 + c % 64);
+                }
+        }
+    }
+    OzSamples *pl = new OzSamples();
+    pl->ntiles = (int64_t)rts.size();
+    s->oz_samples = pl;
+    auto up = [&](auto **d, const auto &h) {
+        cudaError_t er = ss_malloc(ctx, (void **)d, sizeof(h[0]) * std::max<size_t>(1, h.size()));
+        if (er == cudaSuccess && !h.empty()) er = cudaMemcpy(*d, h.data(), sizeof(h[0]) * h.size(), cudaMemcpyHostToDevice);
+        return er;
+    };
+    cudaError_t er = up(&pl->d_rt, rts);
+    if (er == cudaSuccess) er = up(&pl->d_ct, ctl);
+    if (er == cudaSuccess) er = up(&pl->d_ptr, ptr);
+    if (er == cudaSuccess) er = up(&pl->d_e, e);
+    if (er == cudaSuccess) er = up(&pl->d_t, t);
+    if (er == cudaSuccess) er = up(&pl->d_off, off);
+    if (er != cudaSuccess) {
+        cudaGetLastError();
+        oz_free_symbolic(s);
+        return ctx->set_error(SS_ERR_OOM, "sampled product plan: device allocation failed");
+    }
+    return SS_OK;
+}
+
 // row exponents of one value array on the pattern, into v (device memory from buf, or owned by v
 // when buf is null)
 int vals_make(ss_symbolic *s, const double *vals, OzVals *v, Scratch *buf) {
@@ -336,7 +418,52 @@ void oz_free_numeric(ss_numeric *f) {
     for (OzVals *&v : f->oz) drop(v);
 }
 
+// X Y^T sampled on the pattern needs 32-bit CSR positions and enough columns to fill a piece
+bool oz_sddmm_ok(const ss_symbolic *s, int ne) {
+    return s->ctx->gemm_mode == SS_GEMM_TENSOR && s->n >= 2048 && ne >= 48 && s->nnz < (1ll << 32);
+}
+
+int oz_sddmm(ss_symbolic *s, const double *X, const double *lambda, int ne, double *grad_a, double *grad_b) {
+    ss_ctx *ctx = s->ctx;
+    int rc;
+    if (!s->oz_samples && (rc = samples_build(s)) != SS_OK) return rc;
+    const OzSamples *sp = s->oz_samples;
+    oz_attrs(ctx->device);
+    Scratch buf(ctx);
+    unsigned char *sx, *sl;
+    int *ex, *el;
+    // operand rows = rows of X (and of X diag(lambda)), reduction over the ne columns
+    OzOperand x{X, ne, 1, s->n, ne};
+    if ((rc = slice_dense(ctx, x, buf, &sx, &ex)) != SS_OK) return rc;
+    const int nkc = (int)cdivu(ne, sstc::kOzK), nrt = (int)cdivu(s->n, 128);
+    for (int pass = 0; pass < 2; ++pass) {
+        double *out = pass == 0 ? grad_a : grad_b;
+        if (!out || sp->ntiles == 0) continue;
+        sstc::OzMM g{};
+        g.slA = sx; g.emA = ex; g.nrtA = nrt; g.rowsA = s->n;
+        g.slB = sx; g.emB = ex; g.nrtB = nrt; g.rowsB = s->n;
+        if (pass == 1) {
+            x.kscale = lambda;
+            if ((rc = slice_dense(ctx, x, buf, &sl, &el)) != SS_OK) return rc;
+            g.slB = sl; g.emB = el;
+        }
+        g.nkc = nkc; g.per = nkc; g.mode = 2; g.alpha = pass == 0 ? 1.0 : -1.0; g.out = out;
+        g.samp_rt = sp->d_rt; g.samp_ct = sp->d_ct; g.samp_ptr = sp->d_ptr;
+        g.samp_e = sp->d_e; g.samp_t = sp->d_t; g.samp_off = sp->d_off;
+        ctx->add_tensor_flops(SS_K_SDDMM, kPieceTensorFlops * (double)sp->ntiles * nkc);
+        if ((rc = run_mm(ctx, g, dim3((unsigned)sp->ntiles, 1, 1), SS_K_SDDMM)) != SS_OK) return rc;
+    }
+    return SS_OK;
+}
+
 void oz_free_symbolic(ss_symbolic *s) {
+    if (OzSamples *sp = s->oz_samples) {
+        void *q[] = {sp->d_rt, sp->d_ct, sp->d_ptr, sp->d_e, sp->d_t, sp->d_off};
+        for (void *p : q)
+            if (p) cudaFree(p);
+        delete sp;
+        s->oz_samples = nullptr;
+    }
     OzPlan *pl = s->oz_plan;
     if (!pl) return;
     void *ptrs[] = {pl->d_tile_ptr, pl->d_pair_piece, pl->d_ent_ptr, pl->d_ent_e, pl->d_ent_off};

@@ -78,6 +78,11 @@ struct OzOperand {
     const double *M;
     int64_t ld_row, ld_k;
     int64_t rows, kdim;
+    const double *kscale = nullptr;                   // element (row, t) times kscale[t] (null: 1)
+    __device__ __forceinline__ double at(int64_t row, int64_t t) const {
+        const double v = M[row * ld_row + t * ld_k];
+        return kscale ? v * kscale[t] : v;
+    }
 };
 
 // the 8 balanced base-128 digits (top first) of round(x 2^(55 - E)), |x| < 2^E
@@ -111,7 +116,7 @@ __global__ void __launch_bounds__(128) k_oz_expmax(OzOperand op, int64_t per_k, 
     if (row >= op.rows) return;
     const int64_t t0 = (int64_t)blockIdx.y * per_k, t1 = min(op.kdim, t0 + per_k);
     int m = 0;
-    for (int64_t t = t0; t < t1; ++t) m = max(m, biased_exp(op.M[row * op.ld_row + t * op.ld_k]));
+    for (int64_t t = t0; t < t1; ++t) m = max(m, biased_exp(op.at(row, t)));
     if (m > 0) atomicMax(&em[row], m);
 }
 
@@ -142,7 +147,7 @@ __global__ void __launch_bounds__(128) k_oz_slice(OzOperand op, const int *__res
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int64_t t = t0 + 8 * c + u;
-            const double v = (live && t < op.kdim) ? op.M[row * op.ld_row + t * op.ld_k] : 0.0;
+            const double v = (live && t < op.kdim) ? op.at(row, t) : 0.0;
             int q[kOzSlices];
             oz_digits(v, E, q);
 #pragma unroll
@@ -172,7 +177,13 @@ struct OzMM {
     int nrtB;
     int64_t rowsB;
     int nkc, per;                // dense A: pieces [z per, min(nkc, (z + 1) per)), block kc * nrtA + rt
-    int mode;                    // 0: out += alpha r (atomic); 1: out = alpha s_col r + beta out
+    int mode;                    // 0: out += alpha r (atomic); 1: out = alpha s_col r + beta out;
+                                 // 2: sampled (dense A): CTA x is output tile (samp_rt[x], samp_ct[x]) and
+                                 // writes alpha r of its entries to out
+    const int32_t *samp_rt, *samp_ct;
+    const int64_t *samp_ptr;     // entries of tile x are [samp_ptr[x], samp_ptr[x + 1])
+    const uint32_t *samp_e, *samp_t;   // CSR position of the entry and of its mirror image
+    const uint16_t *samp_off;    // 64 (row in the tile) + column in the tile
     double alpha, beta;
     const double *colscale;      // mode 1: per-column factor s_col (null: 1)
     double *out;
@@ -214,7 +225,8 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_mm(const OzMM g) {
     __shared__ __align__(8) uint64_t full[2], placed[2], empty[2], accfull, accfree, drain;
     __shared__ uint32_t s_tmem;
     __shared__ int s_ok, s_em[128];
-    const int bj = blockIdx.x, rt = blockIdx.y;
+    const bool sampled = g.mode == 2;
+    const int bj = sampled ? g.samp_ct[blockIdx.x] : blockIdx.x, rt = sampled ? g.samp_rt[blockIdx.x] : blockIdx.y;
     const bool sparse = g.slA == nullptr;
     int q0, q1;
     if (sparse) {
@@ -385,16 +397,34 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_mm(const OzMM g) {
         }
         while (fine && (done + 1) * kOzReadEvery < np) fine = read_out(done++);
         if (fine) fine = read_out((np - 1) / kOzReadEvery);
-        if (fine && row < g.rowsA) {
-            const int Ea = g.emA[row] - 1022;
+        // the product rounded once; a non-finite operand row makes it NaN
+        const int emA = row < g.rowsA ? g.emA[row] : 0;
+        auto result = [&](int c, int64_t col) -> double {
+            const int emB = g.emB[col], E = emA + emB - 2044 - 61;
+            const double sc = (E >= -1022 && E <= 1023) ? __longlong_as_double((long long)(E + 1023) << 52)
+                                                        : ldexp(1.0, E);
+            const double r = fma(__ll2double_rn(hi[c]), 268435456.0, __ll2double_rn(lo[c])) * sc;
+            return (emA == 0x7ff || emB == 0x7ff) ? __longlong_as_double(0x7ff8000000000000ll) : r;
+        };
+        if (sampled) {
+            // the tile goes through shared memory (the stages are free: every MMA is done)
+            double (*tile)[65] = reinterpret_cast<double (*)[65]>(stage[0]);
+#pragma unroll
+            for (int c = 0; c < 16; ++c)
+                if (fine && row < g.rowsA && col0 + c < g.rowsB) tile[32 * quarter + lane][16 * grp + c] = result(c, col0 + c);
+            asm volatile("bar.sync 3, %0;" ::"n"(kOzWorkers) : "memory");
+            if (fine)
+                for (int64_t p = g.samp_ptr[blockIdx.x] + tid; p < g.samp_ptr[blockIdx.x + 1]; p += kOzWorkers) {
+                    const double v = g.alpha * tile[g.samp_off[p] >> 6][g.samp_off[p] & 63];
+                    g.out[g.samp_e[p]] = v;
+                    g.out[g.samp_t[p]] = v;
+                }
+        } else if (fine && row < g.rowsA) {
 #pragma unroll
             for (int c = 0; c < 16; ++c) {
                 const int64_t col = col0 + c;
                 if (col >= g.rowsB) continue;
-                const int E = Ea + g.emB[col] - 1022 - 61;
-                const double sc = (E >= -1022 && E <= 1023) ? __longlong_as_double((long long)(E + 1023) << 52)
-                                                            : ldexp(1.0, E);
-                const double r = fma(__ll2double_rn(hi[c]), 268435456.0, __ll2double_rn(lo[c])) * sc;
+                const double r = result(c, col);
                 double *o = g.out + row * g.ldo + col;
                 if (g.mode == 0) {
                     atomicAdd(o, g.alpha * r);
