@@ -447,6 +447,7 @@ static void set_smem_attrs(int device) {
             cudaFuncSetAttribute(fold_sweeps_kernel(nc), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFoldSmem);
         cudaFuncSetAttribute(sstc::k_fold_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sstc::kFtSmem);
         cudaFuncSetAttribute(sstc::k_schur_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sstc::kSchurTcSmem);
+        cudaFuncSetAttribute(sstc::k_tc_slice, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sstc::kTcSliceSmem);
         cudaFuncSetAttribute(sstc::k_tc_selftest, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sstc::kSelftestSmem);
     }
@@ -536,10 +537,12 @@ static int factor_levels(ss_numeric *f, int ns, ShiftPtrs<T> *dp, const std::vec
                 (*step_ev)[q] = {e0, e1};
             }
             if (step_uses_tc(s, ctx, q, tc)) {
-                ss_launch(ctx, SS_K_SCHUR_TC, sstc::k_tc_slice, dim3(sd.sl_tiles, ns), 128, 0, st, tk, sd.count,
-                          (const ShiftPtrs<double> *)(void *)dp);
-                ss_launch(ctx, SS_K_SCHUR_TC, sstc::k_schur_tc, dim3(sd.tc_tiles, ns), sstc::kSchurTcThreads,
-                          sstc::kSchurTcSmem, st, tk, sd.count, (const ShiftPtrs<double> *)(void *)dp);
+                ss_launch(ctx, SS_K_SCHUR_TC, sstc::k_tc_slice, dim3(sd.sl_tiles, ns), sstc::kTcSliceThreads,
+                          sstc::kTcSliceSmem, st, tk, sd.count, (const ShiftPtrs<double> *)(void *)dp);
+                const int32_t total = sd.tc_tiles * ns;
+                ss_launch(ctx, SS_K_SCHUR_TC, sstc::k_schur_tc, (unsigned)std::min(total, ctx->sm_count),
+                          sstc::kSchurTcThreads, sstc::kSchurTcSmem, st, tk, sd.count,
+                          (const ShiftPtrs<double> *)(void *)dp, sd.tc_tiles, total);
                 ctx->add_flops(SS_K_SCHUR_TC, sd.flops3 * ns);
                 // 112 digit products of 128 x 64 x 16 per tile
                 ctx->add_tensor_flops(SS_K_SCHUR_TC, 112.0 * 2.0 * 128 * 64 * 16 * sd.tc_tiles * ns);

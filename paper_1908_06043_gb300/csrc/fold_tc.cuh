@@ -13,13 +13,8 @@
 // scales 2^e_i are moved into x2 first (an exponent addition).  Each right-hand-side column of an
 // item has its own scale over the item's 64 terms.
 //
-// Digits without conversions: y = round(x 2^(55 - E)) plus the constant 0x80..80 has the digits,
-// biased by 128, as its bytes; a byte u is the FP16 number (0x6400 | u) - 1152 (one byte
-// permutation, one logic operation and one packed subtraction for two digits).  The read-out
-// forms the 7 accumulators' sum as one 64-bit integer (its last bits, 2^-62 of the scales, lie
-// below the dropped digit products) and packs it into an FP64 by shifts: FP64 instructions run at
-// 2 a clock and SM here, and an item uses none.  A non-finite operand makes its whole column (row)
-// of the product NaN.
+// Cutting and summing digits takes integer instructions only (digits8.cuh).  A non-finite operand
+// makes its whole column (row) of the product NaN.
 //
 // What bounds it: the chain of one item a level.  Measured per item (cycles): right-hand sides'
 // load and digits 6,000, 40 MMAs 4,250 (7,100 as 112 MMAs of N = 64), read-out 8,100 (7 x 32 KB out
@@ -37,6 +32,7 @@
 #include <type_traits>
 
 #include "fold_kernels.cuh"
+#include "digits8.cuh"
 #include "tc_ptx.cuh"
 
 namespace sstc {
@@ -46,56 +42,11 @@ using ssk::NB;
 constexpr int kFtThreads = 512;
 constexpr int kFtCols = 128;                        // right-hand sides of an item
 constexpr int kFtRows = 64;                         // rows of G in an item
-constexpr int kFtSlices = 7;
 constexpr uint32_t kFtSliceA = kFtCols * 64 * 2;    // one digit of the right-hand sides: 16 KB
 constexpr uint32_t kFtSliceB = kFtRows * 64 * 2;    // one digit of G: 8 KB
 constexpr size_t kFtSmem = 1024 + (size_t)kFtSlices * (kFtSliceA + kFtSliceB);
 constexpr uint32_t kFtTmemCols = 512;               // 7 accumulators x 64 columns
-constexpr int kFtNan = 1 << 20;                     // "exponent" of a non-finite value
-constexpr int kFtZero = -(1 << 20);                 // "exponent" of zero
 constexpr long long kFtWaitLimit = 1ll << 24;
-
-// biased exponent of v plus sh; kFtZero for zero (and denormals, which count as zero), kFtNan
-__device__ __forceinline__ int ft_exp(double v, int sh) {
-    const int ex = (int)((__double_as_longlong(v) >> 52) & 0x7ff);
-    return ex == 0 ? kFtZero : (ex == 0x7ff ? kFtNan : ex + sh);
-}
-
-// round(x 2^(55 - E)) + 0x80808080808080 for |x| < 2^E; em = E + 1022 >= ex, the exponents as from
-// ft_exp
-__device__ __forceinline__ unsigned long long ft_biased(double v, int ex, int em) {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
-    unsigned long long m = (bits & ((1ull << 52) - 1)) | (1ull << 52);
-    m = (((m << 3) >> min(em - ex, 60)) + 1) >> 1;  // 4 m 2^(ex - em), rounded
-    if (ex == kFtZero) m = 0;
-    const unsigned long long s = (unsigned long long)((long long)bits >> 63);
-    return ((m ^ s) - s) + 0x80808080808080ull;
-}
-
-// the 7 digits of 8 values (biased as above) as FP16, 16 bytes to each slice
-__device__ __forceinline__ void ft_store8(const unsigned long long (&z)[8], unsigned char *dst, uint32_t stride) {
-    const __half2 bias = __half2half2(__ushort_as_half((unsigned short)0x6480));    // 1152
-#pragma unroll
-    for (int p = 0; p < kFtSlices; ++p) {
-        uint32_t o[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const unsigned long long z0 = z[2 * e], z1 = z[2 * e + 1];
-            uint32_t h;
-            if (p == 0) {                           // the top digit is 0 .. 256: both bytes
-                h = __byte_perm((uint32_t)(z0 >> 32), (uint32_t)(z1 >> 32), 0x7632) | 0x64006400u;
-            } else {
-                const int byte = 6 - p;             // of the 8 bytes of z
-                const uint32_t w0 = (uint32_t)(byte >= 4 ? z0 >> 32 : z0), w1 = (uint32_t)(byte >= 4 ? z1 >> 32 : z1);
-                const uint32_t b = byte & 3;
-                h = (__byte_perm(w0, w1, b | (b << 4) | ((4 + b) << 8) | ((4 + b) << 12)) & 0x00ff00ffu) | 0x64006400u;
-            }
-            const __half2 d = __hsub2(*reinterpret_cast<const __half2 *>(&h), bias);
-            o[e] = *reinterpret_cast<const uint32_t *>(&d);
-        }
-        *reinterpret_cast<uint4 *>(dst + p * stride) = make_uint4(o[0], o[1], o[2], o[3]);
-    }
-}
 
 // The MMAs of one item: accumulator d (columns 64 d ..) = sum_{p + q = d} A_p B_q^T.  Per K step of 16
 // the right-hand sides advance 32 bytes inside their 128-byte rows; G does the same when K is its
@@ -106,47 +57,6 @@ __device__ __forceinline__ void ft_issue(uint32_t tmem, uint64_t da, uint64_t db
     for (int kk = 0; kk < 4; ++kk)
         issue_digit_step<kFtSlices>(tmem, da + (uint64_t)(kk * (kKStepBytes >> 4)), db + (uint64_t)(kk * (bstep >> 4)),
                                     kFtSliceA, kFtSliceB, idesc, kk == 0);
-}
-
-// 16 columns of one accumulator; the values are there after ft_tmem_wait on the same registers
-__device__ __forceinline__ void ft_tmem_ld(uint32_t t, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(t)
-        : "memory");
-}
-__device__ __forceinline__ void ft_tmem_wait(uint32_t (&r)[16]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-                 :
-                 : "memory");
-}
-
-// integer-valued |a| <= 2^22 plus 0x4B400000 as an integer: the bits of a + 1.5 2^23
-constexpr long long kFtMagic = 0x4B400000ll;
-__device__ __forceinline__ long long ft_int22(uint32_t a) {
-    return (long long)__float_as_int(__uint_as_float(a) + 12582912.0f);
-}
-// integer-valued |a| < 2^23 as int
-__device__ __forceinline__ int ft_int23(uint32_t a) {
-    const int b = (int)a, s = b >> 31;
-    const int m = __float_as_int(__uint_as_float(a) + __int_as_float((b & (int)0x80000000) | 0x4B000000)) & 0x7fffff;
-    return (m ^ s) - s;
-}
-
-// bits of T 2^E, rounded to nearest (ties away), by shifts and an integer addition: no branch, for
-// |T| < 2^62 and results in the normal range (or T = 0)
-__device__ __forceinline__ unsigned long long ft_pack(long long T, int E) {
-    const unsigned long long s = (unsigned long long)(T >> 63);
-    unsigned long long u = ((unsigned long long)T ^ s) - s;
-    const int lz = __clzll((long long)u);           // 64 for T = 0: u stays 0
-    u <<= (lz & 63);
-    const unsigned long long bits = ((unsigned long long)(uint32_t)(1023 + 62 - lz + E) << 52) + (u >> 11) + ((u >> 10) & 1);
-    return T == 0 ? 0ull : (bits | (s & (1ull << 63)));
 }
 
 __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a, double *b) {
@@ -277,15 +187,10 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
     auto read_out = [&](int c0, int c1, bool backward, const ssk::FoldTile &t) {
         const int c = 32 * (warp & 3) + lane, n0 = 16 * (warp >> 2);
         if (c0 + 32 * (warp & 3) >= c1) return;      // this warp's right-hand sides do not exist
-        const int ec = s_ec[c] - 1022 - 52, lim = backward ? t.w : t.nr;
+        const int ec = s_ec[c] - 1022 - kTUnit, lim = backward ? t.w : t.nr;
         const bool live = c0 + c < c1;
         const uint32_t lane_base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)n0;
-        uint32_t r[16];
         long long T[16];
-        auto load = [&](int d) {
-            ft_tmem_ld(lane_base + (uint32_t)d * 64, r);
-            ft_tmem_wait(r);
-        };
         bool far = false;
         if (!backward) {
 #pragma unroll
@@ -297,37 +202,10 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
             far = ec < -950 || ec > 900;
         }
         far &= live && s_ec[c] > kFtZero / 2;        // a zero column: its products are zero
-        // T = a_0 2^38 + a_1 2^30 + a_2 2^22 + a_3 2^14 + a_4 2^6 + (a_5 2^8 + a_6) 2^-10: the magic
-        // numbers' share is taken off once; the last term is rounded to FP32 (below 0.2) and to an
-        // integer
-        load(6);
-#pragma unroll
-        for (int e = 0; e < 16; ++e) T[e] = r[e];
-        load(5);
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const float x = fmaf(__uint_as_float(r[e]), 256.0f, __uint_as_float((uint32_t)T[e]));
-            T[e] = __float_as_int(fmaf(x, 1.0f / 1024.0f, 12582912.0f));
-        }
-        load(4);
-#pragma unroll
-        for (int e = 0; e < 16; ++e) T[e] += (long long)ft_int23(r[e]) * 64;
-        load(3);
-#pragma unroll
-        for (int e = 0; e < 16; ++e) T[e] += ft_int22(r[e]) * (1 << 14);
-        load(2);
-#pragma unroll
-        for (int e = 0; e < 16; ++e) T[e] += ft_int22(r[e]) * (1 << 22);
-        load(1);
-#pragma unroll
-        for (int e = 0; e < 16; ++e) T[e] += ft_int22(r[e]) * (1 << 30);
-        load(0);
+        ft_sum(lane_base, T);
         tc_fence_before();
-        constexpr long long kAll =
-            (long long)((unsigned long long)kFtMagic * (1ull + (1ull << 14) + (1ull << 22) + (1ull << 30) + (1ull << 38)));
 #pragma unroll
-        for (int e = 0; e < 16; ++e)
-            T[e] = kAll - (long long)((unsigned long long)T[e] + ((unsigned long long)ft_int22(r[e]) << 38));
+        for (int e = 0; e < 16; ++e) T[e] = -T[e];
         if (__any_sync(0xffffffffu, far)) {
 #pragma unroll 1
             for (int e = 0; e < 16; ++e) {
