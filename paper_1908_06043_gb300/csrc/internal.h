@@ -189,6 +189,7 @@ struct ss_symbolic {
     std::vector<int8_t> step_mode;           // per factor step: -1 rule of ss_set_schur_mode,
                                              // 0 CUDA cores, 1 tensor cores (autotuner)
     int64_t n = 0, nnz = 0;
+    int64_t max_row = 0;                     // most entries of a row
     int nb = 64;
     std::vector<int32_t> perm, iperm;        // perm[new] = old, iperm[old] = new
     std::vector<int64_t> rowptr;             // host copy of the pattern

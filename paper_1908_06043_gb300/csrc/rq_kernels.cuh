@@ -29,37 +29,127 @@ __device__ __forceinline__ void dd_add(DD &s, double hi, double lo) {
     s.lo += se + lo;
 }
 
-// Block (bx, by): rows [bx*rows_per, ...) x columns [128 by, 128 by + 128), one thread per
-// column.  For each row i, y = (A x)_i and z = (B x)_i in double-double, then x_i y and
-// x_i z are added to the thread's double-double numerator and denominator.  Partial
-// sums: part[(bx k + c) * 4 + {num hi, num lo, den hi, den lo}].
-__global__ void __launch_bounds__(128) k_rq_dd_partial(int64_t n, const int64_t *__restrict__ rowptr,
-                                                       const int32_t *__restrict__ colind,
-                                                       const double *__restrict__ a, const double *__restrict__ b,
-                                                       const double *__restrict__ X, int k, int64_t rows_per,
-                                                       double *__restrict__ part) {
-    const int c = blockIdx.y * 128 + threadIdx.x;
+// The products run in integers: double-double arithmetic takes some 20 FP64 operations per stored
+// entry and column at 2 a clock and SM, a 64 x 64-bit multiply-add into 128 bits some ten at 64.
+// Column c of X becomes x~ = round(x 2^(xbits - E_c)), |x| < 2^E_c: the quotient of x~ differs from
+// that of x by the residual times the rounding (second order, below 1e-20), as long as numerator and
+// denominator share x~.  A row of A (of B) becomes round(a 2^(61 - E_i)): relative to the row's
+// largest entry, 2^-62, below double-double's use for the dot products that follow.  Sums over a row
+// are exact: 2^(61 + xbits) times its entries stays below 2^127.  The column's scale cancels in the
+// quotient.  N = 16,384, k = 304: 102 ms with double-double products, %%RQ%% ms now.
+
+// round(v 2^(bits - E)) for |v| < 2^E, E = em - 1022, em >= the biased exponent of v
+__device__ __forceinline__ long long rq_fixed(double v, int em, int bits) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int ex = (int)((b >> 52) & 0x7ff);
+    if (ex == 0) return 0;
+    // v = m 2^(ex - 1075), so v 2^(bits - em + 1022) = m 2^9 2^-(em - ex + 62 - bits)
+    unsigned long long m = ((b & ((1ull << 52) - 1)) | (1ull << 52)) << 9;
+    const int rs = min(em - ex + 62 - bits, 63);
+    m = ((m >> (rs - 1)) + 1) >> 1;                 // rs >= 1: bits <= 61
+    return (long long)b < 0 ? -(long long)m : (long long)m;
+}
+__device__ __forceinline__ int rq_exp(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7ff); }
+
+// em[c] = largest biased exponent of column c (zeroed by the caller)
+__global__ void k_rq_colmax(int64_t n, int k, const double *__restrict__ X, int64_t rows_per, int *__restrict__ em) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= k) return;
+    const int64_t r0 = blockIdx.y * rows_per, r1 = min(n, r0 + rows_per);
+    int m = 0;
+    for (int64_t r = r0; r < r1; ++r) m = max(m, rq_exp(X[r * k + c]));
+    if (m) atomicMax(&em[c], m);
+}
+
+__global__ void k_rq_fixed(int64_t n, int k, const double *__restrict__ X, const int *__restrict__ em, int xbits,
+                           long long *__restrict__ xi) {
+    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (q < n * k) xi[q] = rq_fixed(X[q], em[q % k], xbits);
+}
+
+// T 2^-s as double-double (T's low and high 64 bits converted apart)
+__device__ __forceinline__ DD rq_dd(__int128 T) {
+    const double h = (double)(long long)(T >> 64) * 18446744073709551616.0;
+    const double l = (double)(unsigned long long)T;
+    // |h| may be below l: an exact sum either way (TwoSum)
+    const double t = h + l, z = t - h;
+    // l itself may have been rounded: its error goes in with the low part
+    const unsigned long long lo = (unsigned long long)T, back = l >= 18446744073709551616.0 ? 0ull : (unsigned long long)l;
+    const double le = (double)(long long)(lo - back);
+    return DD{t, (h - (t - z)) + (l - z) + le};
+}
+
+// Block (bx, by): rows [bx rows_per, ...) x columns [64 by, 64 by + 64).  Warp w takes rows w, w + 8, ..,
+// a lane columns lane and lane + 32: y = (A x~)_i and z = (B x~)_i in 128-bit integers, then x~_i y
+// and x~_i z are added to the lane's double-double numerators and denominators.  Partial
+// sums: part[(bx k + c) * 4 + {num hi, num lo, den hi, den lo}].
+constexpr int kRqWarps = 8;
+__global__ void __launch_bounds__(32 * kRqWarps) k_rq_partial(int64_t n, const int64_t *__restrict__ rowptr,
+                                                              const int32_t *__restrict__ colind,
+                                                              const double *__restrict__ a, const double *__restrict__ b,
+                                                              const long long *__restrict__ xi,
+                                                              const int *__restrict__ em, int k, int64_t rows_per,
+                                                              double *__restrict__ part) {
+    __shared__ DD s_sum[kRqWarps][2][64];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c0 = blockIdx.y * 64;
     const int64_t r0 = blockIdx.x * rows_per, r1 = min(n, r0 + rows_per);
-    DD num{0.0, 0.0}, den{0.0, 0.0};
-    for (int64_t i = r0; i < r1; ++i) {
-        DD y{0.0, 0.0}, z{0.0, 0.0};
-        for (int64_t p = rowptr[i]; p < rowptr[i + 1]; ++p) {
-            const double xv = X[(int64_t)colind[p] * k + c];
-            dd_add_prod(y, a[p], xv);
-            dd_add_prod(z, b[p], xv);
+    const bool in[2] = {c0 + lane < k, c0 + 32 + lane < k};
+    DD num[2] = {{0.0, 0.0}, {0.0, 0.0}}, den[2] = {{0.0, 0.0}, {0.0, 0.0}};
+    for (int64_t i = r0 + warp; i < r1; i += kRqWarps) {
+        const int64_t p0 = rowptr[i], p1 = rowptr[i + 1];
+        int ea = 0, eb = 0;
+        for (int64_t p = p0 + lane; p < p1; p += 32) {
+            ea = max(ea, rq_exp(a[p]));
+            eb = max(eb, rq_exp(b[p]));
         }
-        const double xi = X[i * k + c];
-        dd_add_prod(num, xi, y.hi);
-        dd_add_prod(num, xi, y.lo);
-        dd_add_prod(den, xi, z.hi);
-        dd_add_prod(den, xi, z.lo);
+        ea = __reduce_max_sync(0xffffffffu, ea);
+        eb = __reduce_max_sync(0xffffffffu, eb);
+        __int128 y[2] = {0, 0}, z[2] = {0, 0};
+        for (int64_t q0 = p0; q0 < p1; q0 += 32) {
+            const int cnt = (int)min((int64_t)32, p1 - q0);
+            const bool live = lane < cnt;
+            const int col = live ? colind[q0 + lane] : 0;
+            const long long av = live ? rq_fixed(a[q0 + lane], ea, 61) : 0, bv = live ? rq_fixed(b[q0 + lane], eb, 61) : 0;
+#pragma unroll 4
+            for (int e = 0; e < cnt; ++e) {
+                const long long *x = xi + (int64_t)__shfl_sync(0xffffffffu, col, e) * k + c0 + lane;
+                const long long ae = __shfl_sync(0xffffffffu, av, e), be = __shfl_sync(0xffffffffu, bv, e);
+                const long long x0 = in[0] ? x[0] : 0, x1 = in[1] ? x[32] : 0;
+                y[0] += (__int128)ae * x0;
+                z[0] += (__int128)be * x0;
+                y[1] += (__int128)ae * x1;
+                z[1] += (__int128)be * x1;
+            }
+        }
+        const double sa = ldexp(1.0, ea - 1022 - 61), sb = ldexp(1.0, eb - 1022 - 61);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            if (in[u]) {
+                const double v = (double)xi[i * k + c0 + lane + 32 * u];
+                const DD ya = rq_dd(y[u]), zb = rq_dd(z[u]);
+                // non-finite entries have no fixed-point form
+                const double bad_a = ea == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : sa;
+                const double bad_b = eb == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : sb;
+                dd_add_prod(num[u], v, ya.hi * bad_a);
+                dd_add_prod(num[u], v, ya.lo * bad_a);
+                dd_add_prod(den[u], v, zb.hi * bad_b);
+                dd_add_prod(den[u], v, zb.lo * bad_b);
+            }
     }
-    double *o = part + ((int64_t)blockIdx.x * k + c) * 4;
-    o[0] = num.hi;
-    o[1] = num.lo;
-    o[2] = den.hi;
-    o[3] = den.lo;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        s_sum[warp][0][lane + 32 * u] = num[u];
+        s_sum[warp][1][lane + 32 * u] = den[u];
+    }
+    __syncthreads();
+    const int c = threadIdx.x & 63, side = threadIdx.x >> 6;
+    if (side < 2 && c0 + c < k) {
+        DD t{0.0, 0.0};
+        for (int w = 0; w < kRqWarps; ++w) dd_add(t, s_sum[w][side][c].hi, s_sum[w][side][c].lo);
+        double *o = part + ((int64_t)blockIdx.x * k + c0 + c) * 4 + 2 * side;
+        o[0] = em[c0 + c] == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : t.hi;
+        o[1] = t.lo;
+    }
 }
 
 // theta[c] = (sum of numerators) / (sum of denominators), summed and divided in

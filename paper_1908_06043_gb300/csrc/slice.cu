@@ -265,14 +265,26 @@ int rq_polish(ss_numeric *f, const double *X, int k, double *theta_d, DevBuf &bu
     ss_symbolic *s = f->sym;
     ss_ctx *ctx = s->ctx;
     const int64_t n = s->n;
-    const int nby = (int)cdiv(k, 128);
-    const int64_t nbx = std::max<int64_t>(1, std::min<int64_t>(cdiv(n, 16), cdiv(32ll * ctx->sm_count, nby)));
+    cudaStream_t st = ctx->stream;
+    const int nby = (int)cdiv(k, 64);
+    const int64_t nbx = std::max<int64_t>(1, std::min<int64_t>(cdiv(n, sss::kRqWarps), cdiv(16ll * ctx->sm_count, nby)));
     const int64_t rows_per = (n + nbx - 1) / nbx;
     const int64_t nparts = (n + rows_per - 1) / rows_per;
+    // 61 + xbits + log2(entries of a row) <= 126
+    int xbits = 52;
+    while (xbits > 30 && ((int64_t)1 << (126 - 61 - xbits)) < s->max_row) --xbits;
     double *part;
+    long long *xi;
+    int *em;
     TRY_ALLOC(ctx, buf.get(&part, (size_t)nparts * k * 4));
-    ss_launch(ctx, SS_K_MISC, sss::k_rq_dd_partial, dim3((unsigned)nparts, nby), 128, 0, ctx->stream, n, s->d_rowptr,
-              s->d_colind, f->a_vals, f->b_vals, X, k, rows_per, part);
+    TRY_ALLOC(ctx, buf.get(&xi, (size_t)n * k));
+    TRY_ALLOC(ctx, buf.get(&em, (size_t)k));
+    SS_CUDA_TRY(ctx, cudaMemsetAsync(em, 0, sizeof(int) * k, st));
+    const int64_t per = std::max<int64_t>(64, n / 256);
+    ss_launch(ctx, SS_K_MISC, sss::k_rq_colmax, dim3(cdiv(k, 128), cdiv(n, per)), 128, 0, st, n, k, X, per, em);
+    ss_launch(ctx, SS_K_MISC, sss::k_rq_fixed, cdiv(n * k, 256), 256, 0, st, n, k, X, (const int *)em, xbits, xi);
+    ss_launch(ctx, SS_K_MISC, sss::k_rq_partial, dim3((unsigned)nparts, nby), 32 * sss::kRqWarps, 0, st, n, s->d_rowptr,
+              s->d_colind, f->a_vals, f->b_vals, (const long long *)xi, (const int *)em, k, rows_per, part);
     ss_launch(ctx, SS_K_MISC, sss::k_rq_dd_finish, cdiv(k, 256), 256, 0, ctx->stream, k, (int)nparts,
               (const double *)part, theta_d);
     SS_CUDA_TRY(ctx, cudaGetLastError());

@@ -199,6 +199,7 @@ static int analyze_impl(ss_ctx *ctx, int64_t n, const int64_t *rowptr, const int
     s->ctx = ctx;
     s->n = n;
     s->nnz = rowptr[n];
+    for (int64_t i = 0; i < n; ++i) s->max_row = std::max<int64_t>(s->max_row, rowptr[i + 1] - rowptr[i]);
     int leaf = (opt && opt->nd_leaf > 0) ? opt->nd_leaf : 64;
     int nb = (opt && opt->panel > 0) ? opt->panel : 64;
     if (nb != 64) return ctx->set_error(SS_ERR_ARG, "panel width must be 64");
