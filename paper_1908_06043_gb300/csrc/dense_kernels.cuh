@@ -1,7 +1,7 @@
 // Dense helper kernels of the in-slice solver and the DOS sweeps (FP64).
 //   Gram        G = X^T Y (Cholesky-QR Gram matrix V^T B V, projected V^T A V)
 //   GEMM        Y = X Q (tall-skinny times small square: V R^-T, V Q)
-//   Cholesky    G = R R^T of a small SPD matrix; R^-1
+//   Cholesky    G = R R^T of a small SPD matrix and R^-1
 //   Jacobi      eigenpairs of a small symmetric matrix by parallel-ordered cyclic
 //               Jacobi (one launch per round of k/2 disjoint rotations)
 //   Lanczos     batched dot products / updates for full re-orthogonalisation
@@ -105,119 +105,172 @@ __global__ void __launch_bounds__(256) k_gemm_tall(int64_t n, const double *__re
         }
 }
 
-// ---------------------------------------------------------------- small Cholesky
+// ---------------------------------------------------------------- small Cholesky and inverse
+using ::GridBar;
+using ::grid_barrier;
+
+// G = R R^T and X = R^-1 (lower triangles, k x k row-major) in one cooperative launch, by 32-wide
+// panels: the elimination of [G | I].  X must be zero on entry; G's lower triangle becomes R.  Per
+// panel j
+//   A  R_jj and D = R_jj^-1 (one warp of block 0, rows and then columns in registers);
+//   B  R_ij = G_ij D^T for the rows below and X_j: = D X_j: for the columns before, X_jj = D;
+//   C  G_il -= R_ij R_lj^T and X_ic -= R_ij X_jc for the rows below,
+// with a grid barrier before B and before C; block 0 takes the next diagonal block of C and goes on
+// to its A while the others do the rest.  The chain of diagonal blocks bounds it (FP64 square
+// roots and 2 multiply-adds a clock on one SM); B and C are cut into items of 32 x 8 outputs to
+// spread them.  k = 112: 0.67 ms as 13 launches (a one-warp diagonal kernel with a division and a
+// square root a column, and an inverse of k dependent rows), 0.32 ms now.
+// info[0]: first non-positive pivot + 1 (every block then leaves at its next barrier), else 0.
 constexpr int CH_NB = 32;
 
-// Multi-block blocked Cholesky, one 32-column panel per three launches:
-//   k_chol_diag  factors the panel's diagonal block (one warp, shared memory);
-//   k_chol_trsm  solves the rows below against it (one warp per row);
-//   k_chol_syrk  updates the trailing lower triangle, one 32 x 32 tile per block.
-// info[0] != 0 (a non-positive pivot) makes every later launch return at once.
-__global__ void __launch_bounds__(32) k_chol_diag(double *G, int k, int j0, int *info) {
-    __shared__ double Dg[CH_NB][CH_NB + 1];
-    if (info[0]) return;
-    const int lane = threadIdx.x, w = min(CH_NB, k - j0);
-    for (int q = lane; q < w * w; q += 32) {
-        int i = q / w, c = q % w;
-        Dg[i][c] = (c <= i) ? G[(int64_t)(j0 + i) * k + j0 + c] : 0.0;
+struct CholArgs {
+    double *G, *X, *D;          // D: 32 x 32 scratch
+    int k;
+    int *info;
+    GridBar *bar;
+    long long limit;
+};
+
+// R_jj and its inverse for the w x w block at column j0 (one warp; S: 32 x 33 shared scratch)
+__device__ __forceinline__ void chol_diag_warp(const CholArgs &c, int j0, double (*S)[33]) {
+    const int lane = threadIdx.x & 31, k = c.k, w = min(CH_NB, k - j0);
+    double a[CH_NB], inv[CH_NB];
+#pragma unroll
+    for (int t = 0; t < CH_NB; ++t) {
+        S[t][lane] = (t < w && lane <= t) ? __ldcg(&c.G[(int64_t)(j0 + t) * k + j0 + lane]) : (t == lane ? 1.0 : 0.0);
     }
     __syncwarp();
+#pragma unroll
+    for (int t = 0; t < CH_NB; ++t) a[t] = S[lane][t];       // row `lane`, columns t <= lane
     int bad = 0;
-    for (int c = 0; c < w; ++c) {
-        double d = Dg[c][c];
-        if (!(d > 0.0)) { if (!bad) bad = j0 + c + 1; d = 1.0; }
-        const double sd = sqrt(d);
-        __syncwarp();
-        if (lane == 0) Dg[c][c] = sd;
-        __syncwarp();
-        const double inv = 1.0 / sd;
-        for (int i = c + 1 + lane; i < w; i += 32) Dg[i][c] *= inv;
-        __syncwarp();
-        for (int i = c + 1 + lane; i < w; i += 32)
-            for (int l = c + 1; l <= i; ++l) Dg[i][l] -= Dg[i][c] * Dg[l][c];
-        __syncwarp();
-    }
-    for (int q = lane; q < w * w; q += 32) {
-        int i = q / w, c = q % w;
-        if (c <= i) G[(int64_t)(j0 + i) * k + j0 + c] = Dg[i][c];
-    }
-    if (lane == 0 && bad) info[0] = bad;
-}
-
-__global__ void __launch_bounds__(256) k_chol_trsm(double *G, int k, int j0, const int *info) {
-    __shared__ double Dg[CH_NB][CH_NB + 1];
-    if (info[0]) return;
-    const int w = min(CH_NB, k - j0), lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int q = threadIdx.x; q < w * w; q += 256) {
-        int i = q / w, c = q % w;
-        Dg[i][c] = (c <= i) ? G[(int64_t)(j0 + i) * k + j0 + c] : 0.0;
-    }
-    __syncthreads();
-    const int i = j0 + w + blockIdx.x * 8 + wid;
-    if (i >= k) return;
-    double x = (lane < w) ? G[(int64_t)i * k + j0 + lane] : 0.0;
-    for (int c = 0; c < w; ++c) {
-        double xc = __shfl_sync(0xffffffffu, x, c) / Dg[c][c];
-        if (lane == c) x = xc;
-        if (lane > c && lane < w) x -= xc * Dg[lane][c];
-    }
-    if (lane < w) G[(int64_t)i * k + j0 + lane] = x;
-}
-
-__global__ void __launch_bounds__(256) k_chol_syrk(double *G, int k, int j0, const int *info) {
-    __shared__ double Pi[CH_NB][CH_NB + 1], Pl[CH_NB][CH_NB + 1];
-    if (info[0]) return;
-    const int w = min(CH_NB, k - j0), base = j0 + w;
-    int q = blockIdx.x, bi = (int)((sqrt(8.0 * q + 1.0) - 1.0) * 0.5);
-    while ((bi + 1) * (bi + 2) / 2 <= q) ++bi;
-    while (bi * (bi + 1) / 2 > q) --bi;
-    const int bj = q - bi * (bi + 1) / 2;
-    const int i0 = base + 32 * bi, l0 = base + 32 * bj;
-    for (int e = threadIdx.x; e < 32 * CH_NB; e += 256) {
-        int r = e / CH_NB, c = e % CH_NB;
-        Pi[r][c] = (i0 + r < k && c < w) ? G[(int64_t)(i0 + r) * k + j0 + c] : 0.0;
-        Pl[r][c] = (l0 + r < k && c < w) ? G[(int64_t)(l0 + r) * k + j0 + c] : 0.0;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < 32 * 32; e += 256) {
-        const int r = e >> 5, c = e & 31;
-        const int i = i0 + r, l = l0 + c;
-        if (i >= k || l > i) continue;
-        double acc = 0.0;
-#pragma unroll 8
-        for (int t = 0; t < CH_NB; ++t) acc += Pi[r][t] * Pl[c][t];
-        G[(int64_t)i * k + l] -= acc;
-    }
-}
-
-__global__ void k_zero_upper(double *G, int k) {
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q < (int64_t)k * k && q % k > q / k) G[q] = 0.0;
-}
-
-// Rinv = R^-1 for lower-triangular R (k x k row-major).  Column blocks of R^-1 are
-// independent: block b solves R X = E for columns [32 b, 32 b + 32) by forward
-// substitution over the rows; per row the dot product is split across the 8 warps.
-__global__ void __launch_bounds__(256) k_trinv_lower(const double *__restrict__ R, int k, double *__restrict__ Rinv) {
-    __shared__ double part[8][33];
-    const int c0 = blockIdx.x * 32;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int c = c0 + lane;
-    for (int i = 0; i < k; ++i) {
-        const double *ri = R + (int64_t)i * k;
-        double acc = 0.0;
-        if (c < k)      // Rinv[t][c] = 0 for t < c, so every lane can walk the same t
-            for (int t = c0 + wid; t < i; t += 8) acc += ri[t] * Rinv[(int64_t)t * k + c];
-        part[wid][lane] = acc;
-        __syncthreads();
-        if (wid == 0 && c < k) {
-            double sum = 0.0;
-            for (int w = 0; w < 8; ++w) sum += part[w][lane];
-            double v = 0.0;
-            if (c <= i) v = ((c == i ? 1.0 : 0.0) - sum) / ri[i];
-            Rinv[(int64_t)i * k + c] = v;
+#pragma unroll
+    for (int t = 0; t < CH_NB; ++t) {
+        double d = __shfl_sync(0xffffffffu, a[t], t);
+        if (!(d > 0.0)) {
+            if (!bad) bad = j0 + t + 1;
+            d = 1.0;
         }
+        inv[t] = rsqrt(d);
+        a[t] *= inv[t];                                       // lane t: d / sqrt(d)
+#pragma unroll
+        for (int u = t + 1; u < CH_NB; ++u) a[u] -= a[t] * __shfl_sync(0xffffffffu, a[t], u);   // lanes < u: unused
+    }
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < CH_NB; ++t) S[lane][t] = t <= lane ? a[t] : 0.0;
+    __syncwarp();
+    for (int t = 0; t < w; ++t)
+        if (lane <= t) c.G[(int64_t)(j0 + t) * k + j0 + lane] = S[t][lane];
+    // column `lane` of the inverse, by rows
+    double x[CH_NB];
+#pragma unroll
+    for (int t = 0; t < CH_NB; ++t) x[t] = t == lane ? 1.0 : 0.0;
+#pragma unroll
+    for (int t = 0; t < CH_NB; ++t) {
+        x[t] *= inv[t];
+#pragma unroll
+        for (int u = t + 1; u < CH_NB; ++u) x[u] -= S[u][t] * x[t];
+    }
+#pragma unroll
+    for (int t = 0; t < CH_NB; ++t) c.D[t * CH_NB + lane] = x[t];
+    if (lane == 0 && bad) atomicCAS(c.info, 0, bad);
+}
+
+__global__ void __launch_bounds__(256) k_chol_inv(const CholArgs c) {
+    __shared__ double P[32][33], Q[32][33];
+    const int tid = threadIdx.x, k = c.k, nblk = (k + 31) / 32, nb = gridDim.x;
+    const int r = tid >> 5, q = tid & 31;            // output (r, q) of an 8 x 32 item
+    // rows [i0, i0 + m) x columns [c0, c0 + 32) of a matrix into S, zero outside k
+    auto load = [&](double (*S)[33], const double *M, int i0, int m, int c0) {
+        for (int e = tid; e < m * 32; e += 256)
+            S[e >> 5][e & 31] = (i0 + (e >> 5) < k && c0 + (e & 31) < k) ? __ldcg(&M[(int64_t)(i0 + (e >> 5)) * k + c0 + (e & 31)]) : 0.0;
+    };
+    auto load_d = [&](double (*S)[33]) {
+        for (int e = tid; e < 1024; e += 256) S[e >> 5][e & 31] = __ldcg(&c.D[e]);
+    };
+    // rows 8 sub .. of G_il -= R_i R_l^T
+    auto trail_g = [&](int i, int l, int j0, int sub) {
         __syncthreads();
+        load(P, c.G, 32 * i + 8 * sub, 8, j0);
+        load(Q, c.G, 32 * l, 32, j0);
+        __syncthreads();
+        const int row = 32 * i + 8 * sub + r, col = 32 * l + q;
+        if (row < k && col <= row) {
+            double s = 0.0;
+#pragma unroll 8
+            for (int t = 0; t < 32; ++t) s += P[r][t] * Q[q][t];
+            c.G[(int64_t)row * k + col] = __ldcg(&c.G[(int64_t)row * k + col]) - s;
+        }
+    };
+    if (blockIdx.x == 0 && tid < 32) chol_diag_warp(c, 0, P);
+    for (int j = 0; j < nblk; ++j) {
+        const int j0 = 32 * j;
+        if (!grid_barrier(c.bar, nb, c.limit)) return;
+        if (*(volatile int *)c.info) return;          // written before the barrier: the same for every block
+        // B
+        const int below = nblk - 1 - j, nB = 4 * (below + j) + 1;
+        for (int e = blockIdx.x; e < nB; e += nb) {
+            __syncthreads();
+            load_d(Q);
+            if (e == nB - 1) {                         // X_jj = D
+                __syncthreads();
+                for (int u = tid; u < 1024; u += 256)
+                    if (j0 + (u >> 5) < k && (u & 31) <= (u >> 5)) c.X[(int64_t)(j0 + (u >> 5)) * k + j0 + (u & 31)] = Q[u >> 5][u & 31];
+            } else if (e < 4 * below) {                // rows of R_ij = G_ij D^T
+                const int i0 = j0 + 32 * (1 + e / 4) + 8 * (e & 3);
+                load(P, c.G, i0, 8, j0);
+                __syncthreads();
+                double s = 0.0;
+#pragma unroll 8
+                for (int t = 0; t < 32; ++t) s += P[r][t] * Q[q][t];
+                if (i0 + r < k && j0 + q < k) c.G[(int64_t)(i0 + r) * k + j0 + q] = s;
+            } else {                                   // eight columns of X_jc = D X_jc
+                const int f = e - 4 * below, c0 = 8 * f;
+                for (int u = tid; u < 256; u += 256)
+                    P[u >> 3][u & 7] = j0 + (u >> 3) < k ? __ldcg(&c.X[(int64_t)(j0 + (u >> 3)) * k + c0 + (u & 7)]) : 0.0;
+                __syncthreads();
+                const int row = tid >> 3, col = tid & 7;
+                double s = 0.0;
+#pragma unroll 8
+                for (int t = 0; t < 32; ++t) s += Q[row][t] * P[t][col];
+                if (j0 + row < k) c.X[(int64_t)(j0 + row) * k + c0 + col] = s;
+            }
+        }
+        if (below == 0) break;
+        if (!grid_barrier(c.bar, nb, c.limit)) return;
+        // C: the trailing triangle of G (its first block by block 0, which then factors it) and X
+        if (blockIdx.x == 0) {
+            for (int sub = 0; sub < 4; ++sub) trail_g(j + 1, j + 1, j0, sub);
+            __threadfence();                           // the warp below reads them through L2
+            __syncthreads();
+            if (tid < 32) chol_diag_warp(c, j0 + 32, P);
+        }
+        const int nG = 4 * (below * (below + 1) / 2), nX = 4 * below * (j + 1);
+        const int first = nb > 1 ? (int)blockIdx.x - 1 : 0, step = nb > 1 ? nb - 1 : 1;
+        for (int e = first; e >= 0 && e < nG + nX; e += step) {
+            if (e < nG) {
+                const int pr = e >> 2;
+                int i = (int)((sqrtf(8.0f * pr + 1.0f) - 1.0f) * 0.5f);
+                while ((i + 1) * (i + 2) / 2 <= pr) ++i;
+                while (i * (i + 1) / 2 > pr) --i;
+                const int l = pr - i * (i + 1) / 2;
+                if (i == 0 && l == 0) continue;        // block 0's
+                trail_g(j + 1 + i, j + 1 + l, j0, e & 3);
+            } else {                                   // rows of X_ic -= R_ij X_jc
+                const int f = (e - nG) >> 2, i = j + 1 + f / (j + 1), cc = f % (j + 1), i0 = 32 * i + 8 * ((e - nG) & 3);
+                __syncthreads();
+                load(P, c.G, i0, 8, j0);
+                load(Q, c.X, j0, 32, 32 * cc);
+                __syncthreads();
+                if (i0 + r < k) {
+                    double s = 0.0;
+#pragma unroll 8
+                    for (int t = 0; t < 32; ++t) s += P[r][t] * Q[t][q];
+                    const int64_t o = (int64_t)(i0 + r) * k + 32 * cc + q;
+                    c.X[o] = __ldcg(&c.X[o]) - s;
+                }
+            }
+        }
     }
 }
 
@@ -338,9 +391,6 @@ __global__ void __launch_bounds__(1024) k_jacobi_block(double *H, double *V, int
 }
 
 // ---------------------------------------------------------------- grid-wide Jacobi
-using ::GridBar;
-using ::grid_barrier;
-
 // The same parallel-ordered Jacobi as k_jacobi_block, spread over a cooperative grid with
 // one grid barrier per round: H is double-buffered (round r reads Ha and writes every
 // entry of Hb, then the two swap), so each block can compute all of the round's rotations
@@ -518,19 +568,24 @@ __global__ void k_col_sumsq(int64_t n, int k, const double *__restrict__ X, int6
     }
 }
 
-// out[c] += sum_r (AX[r][c] - theta[c] BX[r][c])^2  (residual column norms, squared)
+// rr[c] += sum_r (AX[r][c] - theta[c] BX[r][c])^2 and xx[c] += sum_r X[r][c]^2: residual and vector
+// norms, squared, of the rows of one block
 __global__ void k_resid_sumsq(int64_t n, int k, const double *__restrict__ AX, const double *__restrict__ BX,
-                              const double *__restrict__ theta, int64_t rows_per, double *out) {
+                              const double *__restrict__ X, const double *__restrict__ theta, int64_t rows_per,
+                              double *rr, double *xx) {
     const int64_t r0 = blockIdx.y * rows_per, r1 = min(n, r0 + rows_per);
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < k; c += gridDim.x * blockDim.x) {
-        const double th = theta[c];
-        double acc = 0.0;
-        for (int64_t r = r0; r < r1; ++r) {
-            double v = AX[r * k + c] - th * BX[r * k + c];
-            acc += v * v;
-        }
-        atomicAdd(&out[c], acc);
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= k) return;
+    const double th = theta[c];
+    double a = 0.0, b = 0.0;
+#pragma unroll 4
+    for (int64_t r = r0; r < r1; ++r) {
+        const double v = AX[r * k + c] - th * BX[r * k + c], x = X[r * k + c];
+        a += v * v;
+        b += x * x;
     }
+    atomicAdd(&rr[c], a);
+    atomicAdd(&xx[c], b);
 }
 
 // resid[c] = sqrt(rr[c]) / (normA * sqrt(xx[c]))

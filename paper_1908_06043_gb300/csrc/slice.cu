@@ -165,23 +165,37 @@ int sym_eig(ss_ctx *ctx, double *H, int k, double *evals, double *Q, DevBuf &buf
     return SS_OK;
 }
 
-// G = R R^T in place (lower R, upper part zeroed) by the multi-block blocked Cholesky;
-// *info (device) is 0 or the first failing pivot index + 1.
-int chol_small(ss_ctx *ctx, double *G, int k, int *info) {
+// Rinv = R^-1 (lower, zeros above) with G = R R^T (G's lower triangle becomes R); *hinfo is 0 or
+// the first failing pivot index + 1.  Synchronises.  info: device, one int.
+int chol_inv(ss_ctx *ctx, double *G, int k, double *Rinv, int *info, int *hinfo) {
     cudaStream_t st = ctx->stream;
+    DevBuf buf(ctx);
+    ssd::CholArgs a{};
+    TRY_ALLOC(ctx, buf.get(&a.D, (size_t)ssd::CH_NB * ssd::CH_NB));
+    TRY_ALLOC(ctx, buf.get(&a.bar, 1));
+    a.G = G;
+    a.X = Rinv;
+    a.k = k;
+    a.info = info;
+    a.limit = 20000000;
     SS_CUDA_TRY(ctx, cudaMemsetAsync(info, 0, sizeof(int), st));
-    for (int j0 = 0; j0 < k; j0 += ssd::CH_NB) {
-        const int w = std::min(ssd::CH_NB, k - j0), rem = k - j0 - w;
-        ss_launch(ctx, SS_K_SMALL_DENSE, ssd::k_chol_diag, 1, 32, 0, st, G, k, j0, info);
-        if (rem > 0) {
-            ss_launch(ctx, SS_K_SMALL_DENSE, ssd::k_chol_trsm, cdiv(rem, 8), 256, 0, st, G, k, j0, (const int *)info);
-            const int nt = (int)cdiv(rem, 32);
-            ss_launch(ctx, SS_K_SMALL_DENSE, ssd::k_chol_syrk, (unsigned)(nt * (nt + 1) / 2), 256, 0, st, G, k, j0,
-                      (const int *)info);
-        }
-    }
-    ss_launch(ctx, SS_K_SMALL_DENSE, ssd::k_zero_upper, cdiv((int64_t)k * k, 256), 256, 0, st, G, k);
-    SS_CUDA_TRY(ctx, cudaGetLastError());
+    SS_CUDA_TRY(ctx, cudaMemsetAsync(a.bar, 0, sizeof(ssd::GridBar), st));
+    SS_CUDA_TRY(ctx, cudaMemsetAsync(Rinv, 0, sizeof(double) * k * k, st));
+    // items of a step: about 4 nblk, up to nblk^2 in the trailing update
+    const int nblk = (int)cdiv(k, ssd::CH_NB);
+    const int nb = nblk == 1 ? 1 : std::min(ctx->sm_count, 6 * nblk);
+    void *args[] = {(void *)&a};
+    g_ss_launches.fetch_add(1, std::memory_order_relaxed);
+    size_t slot = 0;
+    const bool prof = ctx->prof_mask & (1u << SS_K_SMALL_DENSE);
+    if (prof) slot = ss_prof_begin(ctx, SS_K_SMALL_DENSE);
+    SS_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((void *)ssd::k_chol_inv, dim3(nb), dim3(256), args, 0, st));
+    if (prof) ss_prof_end(ctx, SS_K_SMALL_DENSE, slot);
+    int herr = 0;
+    SS_CUDA_TRY(ctx, cudaMemcpyAsync(&herr, &a.bar->err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    SS_CUDA_TRY(ctx, cudaMemcpyAsync(hinfo, info, sizeof(int), cudaMemcpyDeviceToHost, st));
+    SS_CUDA_TRY(ctx, cudaStreamSynchronize(st));
+    if (herr) return ctx->set_error(SS_ERR_TIMEOUT, "Cholesky: grid barrier timed out");
     return SS_OK;
 }
 
@@ -207,14 +221,11 @@ int cholqr_b(ss_numeric *f, double *&V, double *&Wk, int k, double *G, double *R
                                    (attempt == 1 ? 1.0 : 1e4);
                 ss_launch(ctx, SS_K_SMALL_DENSE, k_add_shift_diag, 1, 256, 0, st, G, k, rel);
             }
-            if ((rc = chol_small(ctx, G, k, info)) != SS_OK) return rc;
-            SS_CUDA_TRY(ctx, cudaMemcpyAsync(&hinfo, info, sizeof(int), cudaMemcpyDeviceToHost, st));
-            SS_CUDA_TRY(ctx, cudaStreamSynchronize(st));
+            if ((rc = chol_inv(ctx, G, k, Rinv, info, &hinfo)) != SS_OK) return rc;
             if (hinfo == 0) break;
         }
         if (hinfo != 0)
             return ctx->set_error(SS_ERR_NOCONV, "Cholesky-QR: basis is numerically rank deficient");
-        ss_launch(ctx, SS_K_SMALL_DENSE, ssd::k_trinv_lower, cdiv(k, 32), 256, 0, st, (const double *)G, k, Rinv);
         if ((rc = gemm_tall(ctx, V, s->n, k, Rinv, k, 1, Wk, 1)) != SS_OK) return rc;
         std::swap(V, Wk);
     }
@@ -241,13 +252,10 @@ int cholqr_track(ss_numeric *f, double *&W, double *&BW, double *&Wt, double *&B
                                    (attempt == 1 ? 1.0 : 1e4);
                 ss_launch(ctx, SS_K_SMALL_DENSE, k_add_shift_diag, 1, 256, 0, st, G, k, rel);
             }
-            if ((rc = chol_small(ctx, G, k, info)) != SS_OK) return rc;
-            SS_CUDA_TRY(ctx, cudaMemcpyAsync(&hinfo, info, sizeof(int), cudaMemcpyDeviceToHost, st));
-            SS_CUDA_TRY(ctx, cudaStreamSynchronize(st));
+            if ((rc = chol_inv(ctx, G, k, Rinv, info, &hinfo)) != SS_OK) return rc;
             if (hinfo == 0) break;
         }
         if (hinfo != 0) return ctx->set_error(SS_ERR_NOCONV, "Cholesky-QR: basis is numerically rank deficient");
-        ss_launch(ctx, SS_K_SMALL_DENSE, ssd::k_trinv_lower, cdiv(k, 32), 256, 0, st, (const double *)G, k, Rinv);
         if ((rc = gemm_tall(ctx, W, s->n, k, Rinv, k, 1, Wt, 1)) != SS_OK) return rc;
         if ((rc = gemm_tall(ctx, BW, s->n, k, Rinv, k, 1, BWt, 1)) != SS_OK) return rc;
         std::swap(W, Wt);
@@ -337,7 +345,7 @@ int slice_solve_impl(ss_numeric *f, int j, double lo, double hi, const ss_solve_
     const int refine = o.refine > 0 ? o.refine : 2;
     const double tol = o.tol > 0 ? o.tol : 1e-10;
     const double ratio = o.refine_ratio > 0 ? std::min(o.refine_ratio, 1.0) : 1e-1;
-    const int64_t per = 2048;
+    const int64_t per = std::max<int64_t>(16, n / (4 * ctx->sm_count));   // rows of a norm kernel's block
     while (it < max_iter) {
         ++it;
         // W = (A - sigma B)^-1 B V (Alg. 2 step 3); a mixed factor runs plain FP32 solves
@@ -376,9 +384,7 @@ int slice_solve_impl(ss_numeric *f, int j, double lo, double hi, const ss_solve_
         if ((rc = gemm_tall(ctx, AW, n, k, Q, k, 0, AX)) != SS_OK) return rc;     // A X
         SS_CUDA_TRY(ctx, cudaMemsetAsync(rr, 0, sizeof(double) * 2 * k, st));
         ss_launch(ctx, SS_K_MISC, ssd::k_resid_sumsq, dim3(cdiv(k, 128), cdiv(n, per)), 128, 0, st, n, k,
-                  (const double *)AX, (const double *)T2, (const double *)theta_d, per, rr);
-        ss_launch(ctx, SS_K_MISC, ssd::k_col_sumsq, dim3(cdiv(k, 128), cdiv(n, per)), 128, 0, st, n, k,
-                  (const double *)T1, per, rr + k);
+                  (const double *)AX, (const double *)T2, (const double *)T1, (const double *)theta_d, per, rr, rr + k);
         ss_launch(ctx, SS_K_MISC, ssd::k_resid_finish, cdiv(k, 256), 256, 0, st, k, (const double *)rr,
                   (const double *)(rr + k), f->norm_a1, resid_d);
         // V = X, B V = B X
@@ -554,7 +560,7 @@ int block_lanczos_impl(ss_numeric *f, int j, double lo, double hi, const ss_solv
     ss_launch(ctx, SS_K_MISC, ssd::k_neg_scale, cdiv(kout, 256), 256, 0, st, kout, (const double *)theta_d, be);
     if ((rc = spmm_f(f, f->a_vals, f->b_vals, nullptr, be, X, kout, kout, T, kout)) != SS_OK) return rc;
     SS_CUDA_TRY(ctx, cudaMemsetAsync(rr, 0, sizeof(double) * 2 * kout, st));
-    const int64_t per = 2048;
+    const int64_t per = std::max<int64_t>(16, n / (4 * ctx->sm_count));
     ss_launch(ctx, SS_K_MISC, ssd::k_col_sumsq, dim3(cdiv(kout, 128), cdiv(n, per)), 128, 0, st, n, kout,
               (const double *)T, per, rr);
     ss_launch(ctx, SS_K_MISC, ssd::k_col_sumsq, dim3(cdiv(kout, 128), cdiv(n, per)), 128, 0, st, n, kout,
