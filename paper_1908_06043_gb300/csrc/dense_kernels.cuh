@@ -2,8 +2,7 @@
 //   Gram        G = X^T Y (Cholesky-QR Gram matrix V^T B V, projected V^T A V)
 //   GEMM        Y = X Q (tall-skinny times small square: V R^-T, V Q)
 //   Cholesky    G = R R^T of a small SPD matrix and R^-1
-//   Jacobi      eigenpairs of a small symmetric matrix by parallel-ordered cyclic
-//               Jacobi (one launch per round of k/2 disjoint rotations)
+//   Jacobi      eigenpairs of small symmetric matrices by parallel-ordered cyclic Jacobi
 //   Lanczos     batched dot products / updates for full re-orthogonalisation
 #pragma once
 
@@ -280,142 +279,108 @@ __global__ void __launch_bounds__(256) k_chol_inv(const CholArgs c) {
 // by the classical Jacobi angle that annihilates H[p][q]:
 //   theta = (H_qq - H_pp) / (2 H_pq), t = sign(theta) / (|theta| + sqrt(theta^2 + 1)),
 //   c = 1 / sqrt(t^2 + 1), s = t c;  H' = J^T H J, V' = V J.
-__device__ __forceinline__ int jac_partner(int i, int r, int kp) {
+// t needs no more than FP32: an angle off by 1e-7 leaves 1e-7 of H[p][q], which the next sweep
+// takes.  c and s are FP64 to the last bits (two Newton steps), so J stays orthogonal.  That makes a
+// rotation some 15 FP64 instructions instead of two divisions and two square roots.
+
+// pair t of round r: (p, q), p < q; q = kp - 1 >= k is the dummy of an odd k
+__device__ __forceinline__ int2 jac_pair(int t, int r, int kp) {
     const int m = kp - 1;
-    if (i == m) return r;
-    if (i == r) return m;
-    int p = (2 * r - i) % m;
-    if (p < 0) p += m;
-    return p;
+    if (t == 0) return make_int2(r, m);
+    int i = r + t, y = r - t;
+    if (i >= m) i -= m;
+    if (y < 0) y += m;
+    return make_int2(min(i, y), max(i, y));
 }
 
-// The whole eigensolve in one block: every round computes the k/2 rotations from the
-// current H, then each thread rotates whole 2 x 2 blocks {p, q} x {p', q'} of H in place
-// (H' = J^T H J touches only the rows/columns of the pairs) and row pairs of V (V' = V J).
-// Sweeps stop once off(H)^2 <= tol^2 ||H||_F^2 or after max_sweeps.  H and V are k x k
-// row-major in global memory (V must hold the identity or a previous rotation on entry).
-// Shared memory: 3 * (kp / 2) values (pair, c, s).
-__global__ void __launch_bounds__(1024) k_jacobi_block(double *H, double *V, int k, double thr, double tol,
-                                                       int max_sweeps, int *sweeps_done) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int kp = k + (k & 1);
-    const int np = kp / 2;
-    int *pp = reinterpret_cast<int *>(smem_raw);             // p of pair t (p < q)
-    int *pq = pp + np;                                        // q of pair t
-    double *pc = reinterpret_cast<double *>(pq + np);        // 2 np ints: 8-byte aligned for every np
-    double *ps = pc + np;
-    __shared__ double red_off[32], red_all[32];
-    __shared__ int s_stop;
-    const int tid = threadIdx.x, nt = blockDim.x;
-    int sweep = 0;
-    for (; sweep < max_sweeps; ++sweep) {
-        // convergence test
-        double off = 0.0, all = 0.0;
-        for (int64_t q = tid; q < (int64_t)k * k; q += nt) {
-            double v = H[q] * H[q];
-            all += v;
-            if (q / k != q % k) off += v;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            off += __shfl_down_sync(0xffffffffu, off, o);
-            all += __shfl_down_sync(0xffffffffu, all, o);
-        }
-        if ((tid & 31) == 0) { red_off[tid >> 5] = off; red_all[tid >> 5] = all; }
-        __syncthreads();
-        if (tid == 0) {
-            double o2 = 0.0, a2 = 0.0;
-            for (int w = 0; w < (nt >> 5); ++w) { o2 += red_off[w]; a2 += red_all[w]; }
-            s_stop = (o2 <= tol * tol * a2) ? 1 : 0;
-        }
-        __syncthreads();
-        if (s_stop) break;
-        for (int r = 0; r < kp - 1; ++r) {
-            // rotations of this round
-            for (int t = tid; t < np; t += nt) {
-                int i = (t == 0) ? kp - 1 : (r + t) % (kp - 1);
-                int y = jac_partner(i, r, kp);
-                int p = min(i, y), q = max(i, y);
-                double c = 1.0, sn = 0.0;
-                if (q < k) {
-                    const double hpq = H[(int64_t)p * k + q];
-                    const double hpp = H[(int64_t)p * k + p], hqq = H[(int64_t)q * k + q];
-                    if (hpq != 0.0 && fabs(hpq) > thr * sqrt(fabs(hpp * hqq))) {
-                        const double th = (hqq - hpp) / (2.0 * hpq);
-                        const double tt = (th >= 0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
-                        c = 1.0 / sqrt(tt * tt + 1.0);
-                        sn = tt * c;
-                    }
-                }
-                pp[t] = p; pq[t] = q; pc[t] = c; ps[t] = sn;
-            }
-            __syncthreads();
-            // H <- J^T H J on 2 x 2 blocks (pair a rows) x (pair b columns)
-            for (int64_t e = tid; e < (int64_t)np * np; e += nt) {
-                const int ta = (int)(e / np), tb = (int)(e % np);
-                const int p1 = pp[ta], q1 = pq[ta], p2 = pp[tb], q2 = pq[tb];
-                const double c1 = pc[ta], s1 = ps[ta], c2 = pc[tb], s2 = ps[tb];
-                if (s1 == 0.0 && s2 == 0.0) continue;
-                const bool rq = q1 < k, cq = q2 < k;
-                double h11 = H[(int64_t)p1 * k + p2];
-                double h12 = cq ? H[(int64_t)p1 * k + q2] : 0.0;
-                double h21 = rq ? H[(int64_t)q1 * k + p2] : 0.0;
-                double h22 = (rq && cq) ? H[(int64_t)q1 * k + q2] : 0.0;
-                // columns: new_p = c h_p - s h_q, new_q = s h_p + c h_q
-                double a11 = c2 * h11 - s2 * h12, a12 = s2 * h11 + c2 * h12;
-                double a21 = c2 * h21 - s2 * h22, a22 = s2 * h21 + c2 * h22;
-                // rows
-                double b11 = c1 * a11 - s1 * a21, b21 = s1 * a11 + c1 * a21;
-                double b12 = c1 * a12 - s1 * a22, b22 = s1 * a12 + c1 * a22;
-                if (ta == tb && s1 != 0.0) { b12 = 0.0; b21 = 0.0; }   // the annihilated pair
-                H[(int64_t)p1 * k + p2] = b11;
-                if (cq) H[(int64_t)p1 * k + q2] = b12;
-                if (rq) H[(int64_t)q1 * k + p2] = b21;
-                if (rq && cq) H[(int64_t)q1 * k + q2] = b22;
-            }
-            // V <- V J on row pairs (column pair tb)
-            for (int64_t e = tid; e < (int64_t)k * np; e += nt) {
-                const int row = (int)(e / np), tb = (int)(e % np);
-                const double s2 = ps[tb];
-                if (s2 == 0.0) continue;
-                const int p2 = pp[tb], q2 = pq[tb];
-                const double c2 = pc[tb];
-                double *vr = V + (int64_t)row * k;
-                const double vp = vr[p2], vq = vr[q2];
-                vr[p2] = c2 * vp - s2 * vq;
-                vr[q2] = s2 * vp + c2 * vq;
-            }
-            __syncthreads();
-        }
-    }
-    if (tid == 0 && sweeps_done) *sweeps_done = sweep;
+// (c, s) of the rotation of (p, q); thr: relative size below which H[p][q] is left alone
+__device__ __forceinline__ double2 jac_rotation(double hpp, double hqq, double hpq, double thr) {
+    if (hpq == 0.0 || hpq * hpq <= thr * thr * fabs(hpp * hqq)) return make_double2(1.0, 0.0);
+    const double a = hqq - hpp, b = 2.0 * hpq;
+    // theta = a / b in FP32, both scaled by the larger one's exponent
+    const int ea = (int)((__double_as_longlong(a) >> 52) & 0x7ff), eb = (int)((__double_as_longlong(b) >> 52) & 0x7ff);
+    const int e = max(1, min(2045, 2046 - max(ea, eb)));
+    const double sc = __longlong_as_double((long long)e << 52);
+    const float af = (float)(a * sc), bf = (float)(b * sc);
+    const float th = af / bf;                               // bf = 0: infinite, t = 0
+    const float tf = copysignf(1.0f / (fabsf(th) + sqrtf(fmaf(th, th, 1.0f))), th);
+    if (!(fabsf(tf) > 0.0f)) return make_double2(1.0, 0.0);
+    const double t = (double)tf, u = fma(t, t, 1.0);
+    double y = (double)rsqrtf((float)u);                    // 1 <= u <= 2
+    y = fma(0.5 * y, fma(-u * y, y, 1.0), y);
+    y = fma(0.5 * y, fma(-u * y, y, 1.0), y);
+    return make_double2(y, t * y);
 }
 
-// ---------------------------------------------------------------- grid-wide Jacobi
-// The same parallel-ordered Jacobi as k_jacobi_block, spread over a cooperative grid with
-// one grid barrier per round: H is double-buffered (round r reads Ha and writes every
-// entry of Hb, then the two swap), so each block can compute all of the round's rotations
-// itself from Ha into shared memory (np x 24 bytes of dynamic shared memory) while other
-// blocks already write Hb.  acc: 2 * max_sweeps doubles (zeroed) for the per-sweep
-// off-diagonal / total norms.  On return the matrix is in H (copied back from the scratch
-// buffer H2 when the last round left it there).
-__global__ void __launch_bounds__(256) k_jacobi_grid(double *H, double *H2, double *V, int k, double thr, double tol,
-                                                     int max_sweeps, double *acc, GridBar *bar, long long limit,
-                                                     int *sweeps_done) {
+// Parallel-ordered Jacobi on a cooperative grid, one grid barrier per round, for one or several
+// matrices of the same order (group g = blockIdx.x / nb of nb blocks takes matrix g, with barrier
+// g).  H is double-buffered (round r reads Ha and writes every entry of Hb, then the two swap), so
+// each block can compute all of the round's rotations itself from Ha into shared memory (np x 16
+// bytes of dynamic shared memory) while other blocks already write Hb; a thread loads the entries
+// of its own items before it computes rotations, so a round costs one memory latency.  H is
+// symmetric: items are the 2 x 2 blocks of pairs ta <= tb, written to both triangles.  acc: 2
+// max_sweeps doubles a matrix (zeroed) for the per-sweep off-diagonal / total norms.  On return the
+// matrix is in H (copied back from the scratch buffer H2 when the last round left it there).
+// What bounds it: k - 1 rounds a sweep of barrier, load, rotation, update, store.  k = 112: 4.15 ms
+// with both triangles, two divisions and two square roots a rotation and 13 blocks, 2.6 ms now;
+// k = 100, four matrices: 25 ms one after the other (a single block below k = 97), 4.1 ms now.
+struct JacArgs {
+    double *H, *H2, *V;          // matrix g at g k^2
+    int k, nb;                   // blocks per matrix
+    double thr, tol;
+    int max_sweeps;
+    double *acc;
+    GridBar *bar;
+    long long limit;
+};
+constexpr int kJacThreads = 128;
+
+__global__ void __launch_bounds__(kJacThreads) k_jacobi_grid(const JacArgs a) {
     extern __shared__ __align__(16) unsigned char jac_smem[];
-    const int kp = k + (k & 1);
-    const int np = kp / 2;
+    const int k = a.k, nb = a.nb, grp = blockIdx.x / nb, blk = blockIdx.x % nb;
+    const int kp = k + (k & 1), np = kp / 2;
     double2 *s_cs = reinterpret_cast<double2 *>(jac_smem);
-    int2 *s_pq = reinterpret_cast<int2 *>(jac_smem + sizeof(double2) * np);
-    const unsigned int nb = gridDim.x;
-    const int64_t gtid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t gthreads = (int64_t)nb * blockDim.x;
-    __shared__ double red_off[8], red_all[8];
-    double *Ha = H, *Hb = H2;
+    const int gtid = blk * kJacThreads + threadIdx.x, gthreads = nb * kJacThreads;
+    __shared__ double red_off[kJacThreads / 32], red_all[kJacThreads / 32];
+    double *H = a.H + (int64_t)grp * k * k, *V = a.V + (int64_t)grp * k * k;
+    double *Ha = H, *Hb = a.H2 + (int64_t)grp * k * k, *acc = a.acc + 2 * a.max_sweeps * grp;
+    GridBar *bar = a.bar + grp;
+    const int nH = np * (np + 1) / 2;
+    auto block_of = [&](int e, int &ta, int &tb) {        // e = tb (tb + 1) / 2 + ta, ta <= tb
+        tb = (int)((sqrtf(8.0f * e + 1.0f) - 1.0f) * 0.5f);
+        while ((tb + 1) * (tb + 2) / 2 <= e) ++tb;
+        while (tb * (tb + 1) / 2 > e) --tb;
+        ta = e - tb * (tb + 1) / 2;
+    };
+    int ta0 = 0, tb0 = 0;
+    if (gtid < nH) block_of(gtid, ta0, tb0);
+    const int row0 = gtid / np, vb0 = gtid % np;          // first row pair of V
+    auto load_h = [&](int2 x, int2 y, double (&h)[4]) {
+        const bool rq = x.y < k, cq = y.y < k;
+        h[0] = __ldcg(&Ha[(int64_t)x.x * k + y.x]);
+        h[1] = cq ? __ldcg(&Ha[(int64_t)x.x * k + y.y]) : 0.0;
+        h[2] = rq ? __ldcg(&Ha[(int64_t)x.y * k + y.x]) : 0.0;
+        h[3] = (rq && cq) ? __ldcg(&Ha[(int64_t)x.y * k + y.y]) : 0.0;
+    };
+    auto turn_h = [&](int2 x, int2 y, double2 r1, double2 r2, const double (&h)[4]) {
+        const bool rq = x.y < k, cq = y.y < k;
+        const double u11 = r2.x * h[0] - r2.y * h[1], u12 = r2.y * h[0] + r2.x * h[1];
+        const double u21 = r2.x * h[2] - r2.y * h[3], u22 = r2.y * h[2] + r2.x * h[3];
+        const double b11 = r1.x * u11 - r1.y * u21, b21 = r1.y * u11 + r1.x * u21;
+        double b12 = r1.x * u12 - r1.y * u22;
+        const double b22 = r1.y * u12 + r1.x * u22;
+        if (x.x == y.x) b12 = b21;                        // a diagonal block stays symmetric
+        Hb[(int64_t)x.x * k + y.x] = b11;
+        Hb[(int64_t)y.x * k + x.x] = b11;
+        if (cq) { Hb[(int64_t)x.x * k + y.y] = b12; Hb[(int64_t)y.y * k + x.x] = b12; }
+        if (rq) { Hb[(int64_t)x.y * k + y.x] = b21; Hb[(int64_t)y.x * k + x.y] = b21; }
+        if (rq && cq) { Hb[(int64_t)x.y * k + y.y] = b22; Hb[(int64_t)y.y * k + x.y] = b22; }
+    };
     int sweep = 0;
-    for (; sweep < max_sweeps; ++sweep) {
+    for (; sweep < a.max_sweeps; ++sweep) {
         double off = 0.0, all = 0.0;
         for (int64_t q = gtid; q < (int64_t)k * k; q += gthreads) {
-            double v = Ha[q] * Ha[q];
+            const double h = __ldcg(&Ha[q]), v = h * h;
             all += v;
             if (q / k != q % k) off += v;
         }
@@ -427,96 +392,89 @@ __global__ void __launch_bounds__(256) k_jacobi_grid(double *H, double *H2, doub
         __syncthreads();
         if (threadIdx.x == 0) {
             double o2 = 0.0, a2 = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { o2 += red_off[w]; a2 += red_all[w]; }
+            for (int w = 0; w < kJacThreads / 32; ++w) { o2 += red_off[w]; a2 += red_all[w]; }
             atomicAdd(&acc[2 * sweep], o2);
             atomicAdd(&acc[2 * sweep + 1], a2);
         }
-        if (!grid_barrier(bar, nb, limit)) return;
+        if (!grid_barrier(bar, nb, a.limit)) return;
         const double o2 = *(volatile double *)&acc[2 * sweep], a2 = *(volatile double *)&acc[2 * sweep + 1];
-        if (o2 <= tol * tol * a2) break;
+        if (o2 <= a.tol * a.tol * a2) break;
         for (int r = 0; r < kp - 1; ++r) {
-            // the round's rotations, from Ha, by every block
-            for (int t = threadIdx.x; t < np; t += blockDim.x) {
-                int i = (t == 0) ? kp - 1 : (int)((r + t) % (kp - 1));
-                int y = jac_partner(i, r, kp);
-                int p = min(i, y), q = max(i, y);
-                double c = 1.0, sn = 0.0;
-                if (q < k) {
-                    const double hpq = Ha[(int64_t)p * k + q];
-                    const double hpp = Ha[(int64_t)p * k + p], hqq = Ha[(int64_t)q * k + q];
-                    if (hpq != 0.0 && fabs(hpq) > thr * sqrt(fabs(hpp * hqq))) {
-                        const double th = (hqq - hpp) / (2.0 * hpq);
-                        const double tt = (th >= 0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
-                        c = 1.0 / sqrt(tt * tt + 1.0);
-                        sn = tt * c;
-                    }
-                }
-                s_pq[t] = make_int2(p, q);
-                s_cs[t] = make_double2(c, sn);
+            // this thread's first items, then the round's rotations
+            double h[4], v0 = 0.0, v1 = 0.0;
+            const int2 x0 = jac_pair(ta0, r, kp), y0 = jac_pair(tb0, r, kp), z0 = jac_pair(vb0, r, kp);
+            if (gtid < nH) load_h(x0, y0, h);
+            if (row0 < k && z0.y < k) {
+                v0 = __ldcg(&V[(int64_t)row0 * k + z0.x]);
+                v1 = __ldcg(&V[(int64_t)row0 * k + z0.y]);
+            }
+            for (int t = threadIdx.x; t < np; t += kJacThreads) {
+                const int2 pq = jac_pair(t, r, kp);
+                s_cs[t] = pq.y < k ? jac_rotation(__ldcg(&Ha[(int64_t)pq.x * k + pq.x]), __ldcg(&Ha[(int64_t)pq.y * k + pq.y]),
+                                                  __ldcg(&Ha[(int64_t)pq.x * k + pq.y]), a.thr)
+                                   : make_double2(1.0, 0.0);
             }
             __syncthreads();
-            // Hb = J^T Ha J, every 2 x 2 block written (copied where both rotations are trivial)
-            for (int64_t e = gtid; e < (int64_t)np * np; e += gthreads) {
-                const int ta = (int)(e / np), tb = (int)(e % np);
-                const double2 r1 = s_cs[ta], r2 = s_cs[tb];
-                const double c1 = r1.x, s1 = r1.y, c2 = r2.x, s2 = r2.y;
-                const int2 a1 = s_pq[ta], a2p = s_pq[tb];
-                const int p1 = a1.x, q1 = a1.y, p2 = a2p.x, q2 = a2p.y;
-                const bool rq = q1 < k, cq = q2 < k;
-                const double h11 = Ha[(int64_t)p1 * k + p2];
-                const double h12 = cq ? Ha[(int64_t)p1 * k + q2] : 0.0;
-                const double h21 = rq ? Ha[(int64_t)q1 * k + p2] : 0.0;
-                const double h22 = (rq && cq) ? Ha[(int64_t)q1 * k + q2] : 0.0;
-                double b11 = h11, b12 = h12, b21 = h21, b22 = h22;
-                if (s1 != 0.0 || s2 != 0.0) {
-                    const double x11 = c2 * h11 - s2 * h12, x12 = s2 * h11 + c2 * h12;
-                    const double x21 = c2 * h21 - s2 * h22, x22 = s2 * h21 + c2 * h22;
-                    b11 = c1 * x11 - s1 * x21;
-                    b21 = s1 * x11 + c1 * x21;
-                    b12 = c1 * x12 - s1 * x22;
-                    b22 = s1 * x12 + c1 * x22;
-                    if (ta == tb && s1 != 0.0) { b12 = 0.0; b21 = 0.0; }
-                }
-                Hb[(int64_t)p1 * k + p2] = b11;
-                if (cq) Hb[(int64_t)p1 * k + q2] = b12;
-                if (rq) Hb[(int64_t)q1 * k + p2] = b21;
-                if (rq && cq) Hb[(int64_t)q1 * k + q2] = b22;
+            // Hb = J^T Ha J, every 2 x 2 block written
+            if (gtid < nH) turn_h(x0, y0, s_cs[ta0], s_cs[tb0], h);
+            for (int e = gtid + gthreads; e < nH; e += gthreads) {
+                int ta, tb;
+                block_of(e, ta, tb);
+                const int2 x = jac_pair(ta, r, kp), y = jac_pair(tb, r, kp);
+                load_h(x, y, h);
+                turn_h(x, y, s_cs[ta], s_cs[tb], h);
             }
             // V = V J (each entry updated by exactly one thread per round)
-            for (int64_t e = gtid; e < (int64_t)k * np; e += gthreads) {
-                const int row = (int)(e / np), tb = (int)(e % np);
-                const double2 r2 = s_cs[tb];
-                if (r2.y == 0.0) continue;
-                const int2 a2p = s_pq[tb];
-                double *vr = V + (int64_t)row * k;
-                const double vp = vr[a2p.x], vq = vr[a2p.y];
-                vr[a2p.x] = r2.x * vp - r2.y * vq;
-                vr[a2p.y] = r2.y * vp + r2.x * vq;
+            if (row0 < k && z0.y < k) {
+                const double2 c = s_cs[vb0];
+                V[(int64_t)row0 * k + z0.x] = c.x * v0 - c.y * v1;
+                V[(int64_t)row0 * k + z0.y] = c.y * v0 + c.x * v1;
             }
-            if (!grid_barrier(bar, nb, limit)) return;
+            for (int e = gtid + gthreads; e < k * np; e += gthreads) {
+                const int row = e / np, tb = e - row * np;
+                const int2 z = jac_pair(tb, r, kp);
+                const double2 c = s_cs[tb];
+                if (z.y >= k || c.y == 0.0) continue;
+                double *vr = V + (int64_t)row * k;
+                const double vp = __ldcg(&vr[z.x]), vq = __ldcg(&vr[z.y]);
+                vr[z.x] = c.x * vp - c.y * vq;
+                vr[z.y] = c.y * vp + c.x * vq;
+            }
+            if (!grid_barrier(bar, nb, a.limit)) return;
             double *t = Ha;
             Ha = Hb;
             Hb = t;
         }
     }
     if (Ha != H)
-        for (int64_t q = gtid; q < (int64_t)k * k; q += gthreads) H[q] = Ha[q];
-    if (gtid == 0 && sweeps_done) *sweeps_done = sweep;
+        for (int64_t q = gtid; q < (int64_t)k * k; q += gthreads) H[q] = __ldcg(&Ha[q]);
 }
 
-// ascending eigenvalues with their eigenvector columns: rank by (value, index)
-__global__ void k_eig_sort(const double *__restrict__ H, const double *__restrict__ V, int k,
-                           double *__restrict__ evals, double *__restrict__ Q) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= k) return;
-    const double li = H[(int64_t)i * k + i];
-    int rank = 0;
-    for (int j = 0; j < k; ++j) {
-        double lj = H[(int64_t)j * k + j];
-        if (lj < li || (lj == li && j < i)) ++rank;
+// ascending eigenvalues with their eigenvector columns: rank by (value, index).  Block (bx, g): matrix
+// g, rows 32 bx .. + 31 of Q; every block ranks all values itself.
+__global__ void __launch_bounds__(256) k_eig_sort(const double *__restrict__ H, const double *__restrict__ V, int k,
+                                                  double *__restrict__ evals, double *__restrict__ Q) {
+    extern __shared__ __align__(16) double s_val[];            // k values, then their ranks
+    int *rank = reinterpret_cast<int *>(s_val + k);
+    const int64_t off = (int64_t)blockIdx.y * k * k;
+    for (int i = threadIdx.x; i < k; i += 256) s_val[i] = H[off + (int64_t)i * k + i];
+    __syncthreads();
+    for (int i = threadIdx.x; i < k; i += 256) {
+        const double li = s_val[i];
+        int r = 0;
+        for (int j = 0; j < k; ++j) {
+            const double lj = s_val[j];
+            if (lj < li || (lj == li && j < i)) ++r;
+        }
+        rank[i] = r;
+        if (blockIdx.x == 0) evals[(int64_t)blockIdx.y * k + r] = li;
     }
-    evals[rank] = li;
-    for (int r = 0; r < k; ++r) Q[(int64_t)r * k + rank] = V[(int64_t)r * k + i];
+    __syncthreads();
+    const int r0 = blockIdx.x * 32, r1 = min(k, r0 + 32);
+    for (int e = threadIdx.x; e < (r1 - r0) * k; e += 256) {
+        const int row = r0 + e / k, i = e % k;
+        Q[off + (int64_t)row * k + rank[i]] = V[off + (int64_t)row * k + i];
+    }
 }
 
 // copy an n x k block between leading dimensions
@@ -531,7 +489,7 @@ __global__ void k_copy_cols(int64_t n, int k, const double *__restrict__ X, int6
 
 __global__ void k_set_identity(double *V, int k) {
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q < (int64_t)k * k) V[q] = (q / k == q % k) ? 1.0 : 0.0;
+    if (q < (int64_t)k * k) V[(int64_t)blockIdx.y * k * k + q] = (q / k == q % k) ? 1.0 : 0.0;
 }
 
 // ---------------------------------------------------------------- column reductions

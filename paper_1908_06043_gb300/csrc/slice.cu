@@ -109,58 +109,63 @@ __global__ void k_add_shift_diag(double *G, int k, double rel) {
     for (int i = threadIdx.x; i < k; i += blockDim.x) G[(int64_t)i * k + i] += rel * s_tr;
 }
 
-// Symmetric eigenproblem of H (k x k, destroyed): ascending evals (device) and Q.
-// eigenpairs of the symmetric k x k H by parallel-ordered Jacobi, stopped once the
-// off-diagonal Frobenius norm is below tol times the whole norm
-int sym_eig(ss_ctx *ctx, double *H, int k, double *evals, double *Q, DevBuf &buf, double tol = 1e-14) {
+// Symmetric eigenproblems of `count` matrices H (k x k each, one after another, destroyed): ascending
+// evals (device) and Q, by parallel-ordered Jacobi, stopped once the off-diagonal Frobenius norm is
+// below tol times the whole norm.
+int sym_eig(ss_ctx *ctx, double *H, int k, double *evals, double *Q, DevBuf &buf, double tol = 1e-14, int count = 1) {
     cudaStream_t st = ctx->stream;
     double *V;
-    TRY_ALLOC(ctx, buf.get(&V, (size_t)k * k));
+    TRY_ALLOC(ctx, buf.get(&V, (size_t)k * k * count));
     const unsigned g = cdiv((int64_t)k * k, 256);
-    ss_launch(ctx, SS_K_SMALL_DENSE, k_symmetrize, g, 256, 0, st, H, k);
-    ss_launch(ctx, SS_K_JACOBI, ssd::k_set_identity, g, 256, 0, st, V, k);
-    if (k > 1 && k <= 96) {
-        const int np = (k + (k & 1)) / 2;
-        const size_t smem = sizeof(int) * (2 * np + 2) + sizeof(double) * 2 * np;
-        ss_launch(ctx, SS_K_JACOBI, ssd::k_jacobi_block, 1, 1024, smem, st, H, V, k, 1e-18, tol, 40,
-                  (int *)nullptr);
-    } else if (k > 96) {
+    for (int m = 0; m < count; ++m)
+        ss_launch(ctx, SS_K_SMALL_DENSE, k_symmetrize, g, 256, 0, st, H + (int64_t)m * k * k, k);
+    ss_launch(ctx, SS_K_JACOBI, ssd::k_set_identity, dim3(g, count), 256, 0, st, V, k);
+    if (k > 1) {
         // cooperative grid: every block resident, rounds separated by a bounded barrier
         const int np = (k + (k & 1)) / 2, max_sweeps = 40;
-        const size_t smem = (sizeof(double2) + sizeof(int2)) * (size_t)np;
-        double *acc, *H2;
-        ssd::GridBar *bar;
-        int *status;
-        TRY_ALLOC(ctx, buf.get(&H2, (size_t)k * k));
-        TRY_ALLOC(ctx, buf.get(&acc, (size_t)2 * max_sweeps));
-        TRY_ALLOC(ctx, buf.get(&bar, 1));
-        TRY_ALLOC(ctx, buf.get(&status, 1));
-        SS_CUDA_TRY(ctx, cudaMemsetAsync(acc, 0, sizeof(double) * 2 * max_sweeps, st));
-        SS_CUDA_TRY(ctx, cudaMemsetAsync(bar, 0, sizeof(ssd::GridBar), st));
-        SS_CUDA_TRY(ctx, cudaFuncSetAttribute(ssd::k_jacobi_grid, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)std::max<size_t>(smem, 1)));
+        const size_t smem = sizeof(double2) * (size_t)np;
+        ssd::JacArgs a{};
+        TRY_ALLOC(ctx, buf.get(&a.H2, (size_t)k * k * count));
+        TRY_ALLOC(ctx, buf.get(&a.acc, (size_t)2 * max_sweeps * count));
+        TRY_ALLOC(ctx, buf.get(&a.bar, (size_t)count));
+        SS_CUDA_TRY(ctx, cudaMemsetAsync(a.acc, 0, sizeof(double) * 2 * max_sweeps * count, st));
+        SS_CUDA_TRY(ctx, cudaMemsetAsync(a.bar, 0, sizeof(ssd::GridBar) * count, st));
+        if (smem > 48 * 1024)
+            SS_CUDA_TRY(ctx, cudaFuncSetAttribute(ssd::k_jacobi_grid, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)smem));
         int per_sm = 0;
-        SS_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ssd::k_jacobi_grid, 256, smem));
-        const int64_t want = ((int64_t)np * np + 255) / 256;
-        int nb = (int)std::min<int64_t>(std::max(1, std::min(per_sm, 2)) * (int64_t)ctx->sm_count, std::max<int64_t>(1, want));
-        const double thr = 1e-18;
-        const long long limit = 20000000;      // units of 64 ns: ~1.3 s
-        int *sw = status;
-        void *args[] = {(void *)&H, (void *)&H2, (void *)&V, (void *)&k, (void *)&thr, (void *)&tol,
-                        (void *)&max_sweeps, (void *)&acc, (void *)&bar, (void *)&limit, (void *)&sw};
+        SS_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ssd::k_jacobi_grid, ssd::kJacThreads, smem));
+        if (per_sm <= 0) return ctx->set_error(SS_ERR_CUDA, "Jacobi eigensolver cannot be resident");
+        // a thread per row pair of V, at most one block an SM
+        const int64_t want = ((int64_t)k * np + ssd::kJacThreads - 1) / ssd::kJacThreads;
+        const int room = std::max(1, ctx->sm_count / count);
+        a.nb = (int)std::min<int64_t>(room, std::max<int64_t>(1, want));
+        a.H = H;
+        a.V = V;
+        a.k = k;
+        a.thr = 1e-18;
+        a.tol = tol;
+        a.max_sweeps = max_sweeps;
+        a.limit = 20000000;                    // units of 64 ns: ~1.3 s
+        void *args[] = {(void *)&a};
         g_ss_launches.fetch_add(1, std::memory_order_relaxed);
         size_t slot = 0;
         const bool prof = ctx->prof_mask & (1u << SS_K_JACOBI);
         if (prof) slot = ss_prof_begin(ctx, SS_K_JACOBI);
-        SS_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((void *)ssd::k_jacobi_grid, dim3(nb), dim3(256), args, smem, st));
+        SS_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((void *)ssd::k_jacobi_grid, dim3(a.nb * count), dim3(ssd::kJacThreads),
+                                                     args, smem, st));
         if (prof) ss_prof_end(ctx, SS_K_JACOBI, slot);
-        int herr = 0;
-        SS_CUDA_TRY(ctx, cudaMemcpyAsync(&herr, &bar->err, sizeof(int), cudaMemcpyDeviceToHost, st));
+        std::vector<ssd::GridBar> hb(count);
+        SS_CUDA_TRY(ctx, cudaMemcpyAsync(hb.data(), a.bar, sizeof(ssd::GridBar) * count, cudaMemcpyDeviceToHost, st));
         SS_CUDA_TRY(ctx, cudaStreamSynchronize(st));
-        if (herr) return ctx->set_error(SS_ERR_TIMEOUT, "Jacobi eigensolver: grid barrier timed out");
+        for (const ssd::GridBar &b : hb)
+            if (b.err) return ctx->set_error(SS_ERR_TIMEOUT, "Jacobi eigensolver: grid barrier timed out");
     }
-    ss_launch(ctx, SS_K_JACOBI, ssd::k_eig_sort, cdiv(k, 256), 256, 0, st, (const double *)H, (const double *)V, k,
-              evals, Q);
+    const size_t ssm = (sizeof(double) + sizeof(int)) * (size_t)k;
+    if (ssm > 48 * 1024)
+        SS_CUDA_TRY(ctx, cudaFuncSetAttribute(ssd::k_eig_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
+    ss_launch(ctx, SS_K_JACOBI, ssd::k_eig_sort, dim3(cdiv(k, 32), count), 256, ssm, st, (const double *)H,
+              (const double *)V, k, evals, Q);
     SS_CUDA_TRY(ctx, cudaGetLastError());
     return SS_OK;
 }
@@ -668,22 +673,37 @@ int lanczos_impl(ss_symbolic *s, ss_numeric *fb, const double *a_vals, const dou
     SS_CUDA_TRY(ctx, cudaStreamSynchronize(st));
     std::memset(theta, 0, sizeof(double) * steps * nv);
     std::memset(zeta2, 0, sizeof(double) * steps * nv);
+    // the runs' tridiagonal eigenproblems, neighbours of the same length together
     double *T, *Q, *ev;
-    TRY_ALLOC(ctx, buf.get(&T, (size_t)steps * steps));
-    TRY_ALLOC(ctx, buf.get(&Q, (size_t)steps * steps));
-    TRY_ALLOC(ctx, buf.get(&ev, (size_t)steps));
-    std::vector<double> hq(steps);
+    TRY_ALLOC(ctx, buf.get(&T, (size_t)steps * steps * nv));
+    TRY_ALLOC(ctx, buf.get(&Q, (size_t)steps * steps * nv));
+    TRY_ALLOC(ctx, buf.get(&ev, (size_t)steps * nv));
     for (int c = 0; c < nv; ++c) {
         int m = steps;
         for (int j = 0; j + 1 < steps; ++j)
             if (hb[(size_t)j * nv + c] <= 1e-13 * std::max(1.0, std::fabs(ha[(size_t)j * nv + c]))) { m = j + 1; break; }
         m_run[c] = m;
-        ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_tridiag, cdiv((int64_t)m * m, 256), 256, 0, st, alpha, beta, nv, c, m, T);
-        if ((rc = sym_eig(ctx, T, m, ev, Q, buf)) != SS_OK) return rc;
-        SS_CUDA_TRY(ctx, cudaMemcpyAsync(theta + (size_t)c * steps, ev, sizeof(double) * m, cudaMemcpyDeviceToHost, st));
-        SS_CUDA_TRY(ctx, cudaMemcpyAsync(hq.data(), Q, sizeof(double) * m, cudaMemcpyDeviceToHost, st));
+    }
+    for (int c0 = 0; c0 < nv;) {
+        const int m = m_run[c0];
+        int cnt = 1;
+        while (c0 + cnt < nv && cnt < 16 && m_run[c0 + cnt] == m) ++cnt;
+        for (int q = 0; q < cnt; ++q)
+            ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_tridiag, cdiv((int64_t)m * m, 256), 256, 0, st, alpha, beta, nv, c0 + q,
+                      m, T + (int64_t)q * m * m);
+        if ((rc = sym_eig(ctx, T, m, ev, Q, buf, 1e-14, cnt)) != SS_OK) return rc;
+        std::vector<double> he((size_t)m * cnt), hq((size_t)m * cnt);
+        SS_CUDA_TRY(ctx, cudaMemcpyAsync(he.data(), ev, sizeof(double) * m * cnt, cudaMemcpyDeviceToHost, st));
+        for (int q = 0; q < cnt; ++q)
+            SS_CUDA_TRY(ctx, cudaMemcpyAsync(hq.data() + (size_t)q * m, Q + (int64_t)q * m * m, sizeof(double) * m,
+                                             cudaMemcpyDeviceToHost, st));
         SS_CUDA_TRY(ctx, cudaStreamSynchronize(st));
-        for (int i = 0; i < m; ++i) zeta2[(size_t)c * steps + i] = hq[i] * hq[i];
+        for (int q = 0; q < cnt; ++q)
+            for (int i = 0; i < m; ++i) {
+                theta[(size_t)(c0 + q) * steps + i] = he[(size_t)q * m + i];
+                zeta2[(size_t)(c0 + q) * steps + i] = hq[(size_t)q * m + i] * hq[(size_t)q * m + i];
+            }
+        c0 += cnt;
     }
     return SS_OK;
 }
