@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
         __syncthreads();
         sweep(true);
     }
-    if (!ok && tid == 0 && s_ok == 0) atomicExch(&a.bar->err, 1);
+    if (!ok && tid == 0 && s_ok == 0) ::grid_fail(a.bar);
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kFtTmemCols);
