@@ -152,7 +152,8 @@ extern "C" const char *ss_last_error(const ss_ctx *ctx) { return ctx ? ctx->err.
 
 // every block waits at one grid barrier that expects `expected` arrivals
 __global__ void k_barrier_selftest(GridBar *bar, unsigned int expected, long long limit) {
-    grid_barrier(bar, expected, limit);
+    unsigned int at = 0;
+    grid_barrier(bar, expected, limit, at);
 }
 
 extern "C" ss_status ss_selftest_barrier(ss_ctx *ctx, int32_t extra_arrivals, int64_t limit) {
@@ -424,6 +425,20 @@ static void (*fold_sweeps_kernel(int nc))(FoldArgs, double *) {
     }
 }
 
+// the same, one level a launch
+static void (*fold_level_kernel(int nc))(FoldArgs, int, int, int, double *) {
+    switch (nc) {
+        case 1: return k_fold_level<1>;
+        case 2: return k_fold_level<2>;
+        case 3: return k_fold_level<3>;
+        case 4: return k_fold_level<4>;
+        case 5: return k_fold_level<5>;
+        case 6: return k_fold_level<6>;
+        case 7: return k_fold_level<7>;
+        default: return k_fold_level<8>;
+    }
+}
+
 template <typename T>
 static void set_smem_attrs(int device) {
     static std::mutex mu;
@@ -443,8 +458,10 @@ static void set_smem_attrs(int device) {
     } else {
         cudaFuncSetAttribute(k_fold_panels, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFoldPanelsSmem);
         cudaFuncSetAttribute(k_fold_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFoldMidSmem);
-        for (int nc = 1; nc <= kFoldMaxNc; ++nc)
+        for (int nc = 1; nc <= kFoldMaxNc; ++nc) {
+            cudaFuncSetAttribute(fold_level_kernel(nc), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFoldItemSmem);
             cudaFuncSetAttribute(fold_sweeps_kernel(nc), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFoldSmem);
+        }
         cudaFuncSetAttribute(sstc::k_fold_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sstc::kFtSmem);
         cudaFuncSetAttribute(sstc::k_schur_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sstc::kSchurTcSmem);
         cudaFuncSetAttribute(sstc::k_tc_slice, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sstc::kTcSliceSmem);
@@ -1181,39 +1198,29 @@ static int fold_per_step(ss_numeric *f, int j, double *b, int k, bool full) {
     auto level = [&](int L, int backward) {
         const SolveLevel &sl = s->solve_levels[L];
         if (sl.tiles128 == 0) return;
-        const int64_t items = (int64_t)sl.tiles128 * 16 * nch;
+        const int split = fold_split((int64_t)sl.tiles128 * 16 * nch, (int64_t)kFoldWarps / 2 * ctx->sm_count);
+        const int64_t items = ((int64_t)sl.tiles128 * 16 << split) * nch;
         const unsigned grid = (unsigned)((items + kFoldWarps - 1) / kFoldWarps);
         const int cls = backward ? SS_K_BWD_GATHER : SS_K_FWD_UPDATE;
-        switch (nc) {
-#define SS_FOLD_LEVEL(N) case N: ss_launch(ctx, cls, k_fold_level<N>, grid, kFoldThreads, 0, st, a, L, backward, b); break
-            SS_FOLD_LEVEL(1);
-            SS_FOLD_LEVEL(2);
-            SS_FOLD_LEVEL(3);
-            SS_FOLD_LEVEL(4);
-            SS_FOLD_LEVEL(5);
-            SS_FOLD_LEVEL(6);
-            SS_FOLD_LEVEL(7);
-            default: ss_launch(ctx, cls, k_fold_level<8>, grid, kFoldThreads, 0, st, a, L, backward, b);
-#undef SS_FOLD_LEVEL
-        }
+        ss_launch(ctx, cls, fold_level_kernel(nc), grid, kFoldThreads, fold_item_smem(nc), st, a, L, split, backward, b);
         ctx->add_flops(cls, 2.0 * sl.offdiag * k);
     };
     const int nlev = (int)s->solve_levels.size();
     for (int L = 0; full && L < nlev; ++L) level(L, 0);
-    const int mc = fold_mid_cols(k);
+    const int mc = fold_mid_cols(k, a.npan, ctx->sm_count);
     if (a.npan > 0)
         ss_launch(ctx, SS_K_FWD_DIAG, k_fold_mid, dim3((unsigned)a.npan, (unsigned)((k + mc - 1) / mc)), kFoldThreads,
-                  kFoldMidSmem, st, a, b);
+                  kFoldMidSmem, st, a, mc, b);
     for (int L = nlev - 1; L >= 0; --L) level(L, 1);
     SS_CUDA_TRY(ctx, cudaGetLastError());
     return SS_OK;
 }
 
 // Whether a solve of k columns runs on the tensor cores (fold_tc.cuh): where the FP64 work it takes
-// off the CUDA cores, 4.4 ps per entry of L and column, outweighs its longer items, 16 us more per
-// level.  Measured (ms a solve, CUDA cores / tensor cores): N = 864 (13 levels) k = 129 0.48 / 0.50,
-// k = 304 0.78 / 0.54; N = 5,280 (55) k = 17 1.48 / 1.85, k = 48 2.58 / 1.93, k = 304 11.7 / 2.94;
-// N = 16,384 (129) k = 304 61.8 / 9.2.
+// off the CUDA cores, about 4 ps per entry of L and column, outweighs its longer items, 13 - 16 us a
+// level and sweep.  Measured (ms a solve, CUDA cores / tensor cores): N = 864 (13 levels) k = 129
+// 0.36 / 0.36, k = 304 0.69 / 0.39; N = 5,280 (55) k = 32 1.54 / 1.43, k = 48 2.15 / 1.50, k = 304
+// 10.6 / 2.48; N = 16,384 (129) k = 16 4.6 / 4.3, k = 48 11.5 / 4.4, k = 304 61 / 9.3.
 static bool fold_uses_tc(const ss_symbolic *s, int k) {
     return s->ctx->gemm_mode == SS_GEMM_TENSOR && k > kFoldMaxNc &&
            (double)s->info.l_offdiag_entries * k >= 3.6e6 * (double)s->solve_levels.size();
@@ -1226,7 +1233,7 @@ static int fold_sweeps(ss_numeric *f, int j, double *b, int k, bool full) {
     ss_ctx *ctx = s->ctx;
     cudaStream_t st = ctx->stream;
     if (!ctx->d_bar) SS_CUDA_TRY(ctx, ss_malloc(ctx, (void **)&ctx->d_bar, kBarBytes));
-    const int nc = fold_nc(k), nch = (k + nc - 1) / nc, mc = fold_mid_cols(k);
+    const int nc = fold_nc(k), nch = (k + nc - 1) / nc, mc = fold_mid_cols(k, (int)s->panels.size(), ctx->sm_count);
     // enough blocks that the largest step's items lie on as many SMs as there are, no more: a
     // barrier over few blocks is quicker
     int64_t items = (int64_t)s->panels.size() * ((k + mc - 1) / mc);

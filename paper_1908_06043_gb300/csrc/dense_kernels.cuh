@@ -201,10 +201,11 @@ __global__ void __launch_bounds__(256) k_chol_inv(const CholArgs c) {
             c.G[(int64_t)row * k + col] = __ldcg(&c.G[(int64_t)row * k + col]) - s;
         }
     };
+    unsigned int at = 0;
     if (blockIdx.x == 0 && tid < 32) chol_diag_warp(c, 0, P);
     for (int j = 0; j < nblk; ++j) {
         const int j0 = 32 * j;
-        if (!grid_barrier(c.bar, nb, c.limit)) return;
+        if (!grid_barrier(c.bar, nb, c.limit, at)) return;
         if (*(volatile int *)c.info) return;          // written before the barrier: the same for every block
         // B
         const int below = nblk - 1 - j, nB = 4 * (below + j) + 1;
@@ -236,7 +237,7 @@ __global__ void __launch_bounds__(256) k_chol_inv(const CholArgs c) {
             }
         }
         if (below == 0) break;
-        if (!grid_barrier(c.bar, nb, c.limit)) return;
+        if (!grid_barrier(c.bar, nb, c.limit, at)) return;
         // C: the trailing triangle of G (its first block by block 0, which then factors it) and X
         if (blockIdx.x == 0) {
             for (int sub = 0; sub < 4; ++sub) trail_g(j + 1, j + 1, j0, sub);
@@ -345,6 +346,7 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi_grid(const JacArgs a) {
     double *H = a.H + (int64_t)grp * k * k, *V = a.V + (int64_t)grp * k * k;
     double *Ha = H, *Hb = a.H2 + (int64_t)grp * k * k, *acc = a.acc + 2 * a.max_sweeps * grp;
     GridBar *bar = a.bar + grp;
+    unsigned int at = 0;
     const int nH = np * (np + 1) / 2;
     auto block_of = [&](int e, int &ta, int &tb) {        // e = tb (tb + 1) / 2 + ta, ta <= tb
         tb = (int)((sqrtf(8.0f * e + 1.0f) - 1.0f) * 0.5f);
@@ -396,7 +398,7 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi_grid(const JacArgs a) {
             atomicAdd(&acc[2 * sweep], o2);
             atomicAdd(&acc[2 * sweep + 1], a2);
         }
-        if (!grid_barrier(bar, nb, a.limit)) return;
+        if (!grid_barrier(bar, nb, a.limit, at)) return;
         const double o2 = *(volatile double *)&acc[2 * sweep], a2 = *(volatile double *)&acc[2 * sweep + 1];
         if (o2 <= a.tol * a.tol * a2) break;
         for (int r = 0; r < kp - 1; ++r) {
@@ -440,7 +442,7 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi_grid(const JacArgs a) {
                 vr[z.x] = c.x * vp - c.y * vq;
                 vr[z.y] = c.y * vp + c.x * vq;
             }
-            if (!grid_barrier(bar, nb, a.limit)) return;
+            if (!grid_barrier(bar, nb, a.limit, at)) return;
             double *t = Ha;
             Ha = Hb;
             Hb = t;

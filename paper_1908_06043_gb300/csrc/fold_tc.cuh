@@ -242,13 +242,15 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
     };
     auto tile = [&](const ssk::FoldLevel &lv, int q) { return a.tiles_64[lv.tile0_64 + q % lv.tiles_64]; };
     bool ok = true;
+    unsigned int at = 0;
     auto sweep = [&](bool backward) {
         const int first = backward ? a.nlev - 1 : 0, step = backward ? -1 : 1;
         ssk::FoldLevel lv = a.lev[first];
         int qa, qb;
         range(lv, qa, qb);
+        if (backward) ::grid_arrive(a.bar, nb, at);                                     // the middle step is done
         if (qa < qb) { fetch(tile(lv, qa)); cut_g(); }
-        if (backward && !::grid_barrier(a.bar, nb, a.limit)) { ok = false; return; }    // the middle step is done
+        if (backward && !::grid_wait(a.bar, a.limit, at)) { ok = false; return; }
         for (int n = 0; n < a.nlev; ++n) {
             const bool more = n + 1 < a.nlev;
             const ssk::FoldLevel nx = more ? a.lev[first + step * (n + 1)] : ssk::FoldLevel{0, 0, 0, 0};
@@ -274,8 +276,11 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
                 read_out(c0, c1, backward, t);
                 __syncthreads();                     // s_row, s_er, s_ec and the accumulators are free
             }
+            // the next item's digits while the other blocks arrive
+            const bool wait = (more || !backward) && lv.tiles_64 > 0;
+            if (wait) ::grid_arrive(a.bar, nb, at);
             if (na < nbq) cut_g();
-            if ((more || !backward) && lv.tiles_64 > 0 && !::grid_barrier(a.bar, nb, a.limit)) { ok = false; return; }
+            if (wait && !::grid_wait(a.bar, a.limit, at)) { ok = false; return; }
             lv = nx;
             qa = na;
             qb = nbq;
@@ -283,10 +288,12 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
     };
     if (a.full) sweep(false);
     if (ok) {
-        const int mc = ssk::fold_mid_cols(k), nm = (k + mc - 1) / mc;
+        const int mc = ssk::fold_mid_cols(k, a.npan, nb), nm = (k + mc - 1) / mc;
         for (int q = blockIdx.x; q < a.npan * nm; q += nb) {
             __syncthreads();
-            ssk::fold_mid_any(sa, a, q % a.npan, q / a.npan, b);
+            ssk::fold_mid_load(sa, a, q % a.npan);
+            __syncthreads();
+            ssk::fold_mid_any(sa, a, mc, q % a.npan, q / a.npan, b);
         }
         __syncthreads();
         sweep(true);

@@ -431,14 +431,14 @@ struct SweepArgs {
 // of a step land on distinct SMs: a cooperative launch may place consecutive blocks on
 // the same SM, where small steps would then share one SM's FP64 units.  Falls back to
 // blockIdx.x when the SM ids exceed the counter array (the same for every block).
-__device__ __forceinline__ int spread_block_id(const SweepArgs &a, bool *ok) {
+__device__ __forceinline__ int spread_block_id(const SweepArgs &a, unsigned int &at, bool *ok) {
     __shared__ int s_r, s_vb;
     unsigned smid, nsmid;
     asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
     asm volatile("mov.u32 %0, %%nsmid;" : "=r"(nsmid));
     const bool use = a.sm_slots != nullptr && (int)nsmid <= a.nsm_slots;
     if (use && threadIdx.x == 0) s_r = atomicAdd(&a.sm_slots[smid], 1);
-    *ok = grid_barrier(a.bar, gridDim.x, a.limit);
+    *ok = grid_barrier(a.bar, gridDim.x, a.limit, at);
     if (!use || !*ok) return blockIdx.x;
     if (threadIdx.x == 0) {
         const int r = s_r;
@@ -769,8 +769,9 @@ __global__ void __launch_bounds__(256, 4) k_solve_sweeps(SweepArgs a, const floa
     const int k = a.k;
     const int nchunk = (k + KC - 1) / KC, ndchunk = (k + KD - 1) / KD;
     const unsigned nb = gridDim.x;
+    unsigned int at = 0;
     bool ok = true;
-    const int vb = spread_block_id(a, &ok);
+    const int vb = spread_block_id(a, at, &ok);
     if (!ok) return;
     if (a.forward) {
         for (int L = 0; L < a.nlev; ++L) {
@@ -778,18 +779,18 @@ __global__ void __launch_bounds__(256, 4) k_solve_sweeps(SweepArgs a, const floa
             const int32_t *lp = a.solve_panels + lv.panel_off;
             if (level_fused(a, lv, nchunk)) {           // y of this level goes to ybuf
                 fwd_level_fused_f32(a, smem_raw, vb, lv, arena, b, ybuf);
-                if (!grid_barrier(a.bar, nb, a.limit)) return;
+                if (!grid_barrier(a.bar, nb, a.limit, at)) return;
                 continue;
             }
             for (int q = vb; q < lv.count * ndchunk; q += nb)
                 fwd_diag_item(smem_raw, q % lv.count, q / lv.count, lp, a.panels, a.linv, a.piv, b, k);
-            if (!grid_barrier(a.bar, nb, a.limit)) return;
+            if (!grid_barrier(a.bar, nb, a.limit, at)) return;
             if (lv.row_tiles == 0) continue;
             const int32_t *tp = a.tile_pre + lv.panel_off;
             for (int q = vb; q < lv.row_tiles * nchunk; q += nb)
                 fwd_update_f32_item(smem_raw, q % lv.row_tiles, q / lv.row_tiles, lp, tp, lv.count, a.panels, a.idx,
                                     arena, b, k);
-            if (!grid_barrier(a.bar, nb, a.limit)) return;
+            if (!grid_barrier(a.bar, nb, a.limit, at)) return;
         }
     }
     if (!a.backward) return;
@@ -799,7 +800,7 @@ __global__ void __launch_bounds__(256, 4) k_solve_sweeps(SweepArgs a, const floa
         float *z = zall + (int64_t)lv.panel_off * NB * k;
         if (level_fused(a, lv, nchunk)) {
             bwd_level_fused_f32(a, smem_raw, vb, lv, arena, b, zall, ybuf);
-            if (L > 0 && !grid_barrier(a.bar, nb, a.limit)) return;
+            if (L > 0 && !grid_barrier(a.bar, nb, a.limit, at)) return;
             continue;
         }
         if (lv.row_tiles > 0) {
@@ -807,12 +808,12 @@ __global__ void __launch_bounds__(256, 4) k_solve_sweeps(SweepArgs a, const floa
             for (int q = vb; q < lv.row_tiles * nchunk; q += nb)
                 bwd_gather_f32_item(smem_raw, q % lv.row_tiles, q / lv.row_tiles, lp, tp, lv.count, a.panels, a.idx,
                                     arena, b, k, z);
-            if (!grid_barrier(a.bar, nb, a.limit)) return;
+            if (!grid_barrier(a.bar, nb, a.limit, at)) return;
         }
         for (int q = vb; q < lv.count * ndchunk; q += nb)
             bwd_diag_item(smem_raw, q % lv.count, q / lv.count, lp, a.panels, a.linv, a.dblk, a.piv, z,
                              lv.row_tiles > 0 ? 1 : 0, b, k, a.dinv);
-        if (L > 0 && !grid_barrier(a.bar, nb, a.limit)) return;
+        if (L > 0 && !grid_barrier(a.bar, nb, a.limit, at)) return;
     }
 }
 
