@@ -528,7 +528,7 @@ static int factor_levels(ss_numeric *f, int ns, ShiftPtrs<T> *dp, const std::vec
         for (int32_t q = s->lev_step_off[l]; q < s->lev_step_off[l + 1]; ++q) {
             const StepDesc &sd = s->steps[q];
             const StepTask *tk = s->d_tasks + sd.task_off;
-            ss_launch(ctx, SS_K_DIAG_BK, k_diag_bk<T>, dim3(sd.count, ns), 256, kDiagSmem, st, tk,
+            ss_launch(ctx, SS_K_DIAG_BK, k_diag_bk<T>, dim3(sd.count, ns), kDiagThreads, kDiagSmem, st, tk,
                       (const ShiftPtrs<T> *)dp);
             if (sd.tiles4 > 0) {
                 const int cls = std::is_same<T, float>::value ? SS_K_PANEL_F32 : SS_K_PANEL;

@@ -145,16 +145,24 @@ __global__ void k_level_store(const StoreTask *__restrict__ tasks, int32_t ntask
 }
 
 // ---------------------------------------------------------------- K2: diagonal block
-// One block per (front, shift).  FP64 runs at 2 multiply-adds a clock here, on one SM, so the
-// block does only the lower triangle's (w^3 / 6) and the inverse's (w^3 / 6), with one multiply-add
-// each and no division in a loop; pivots are compared as integers (|x| orders like its bits).
-// Per column one block barrier: warp 0 runs one column ahead -- it updates column k + 1, finds
-// its largest entry and, when the diagonal passes the 1x1 test, forms 1 / d and that column of L,
-// while warps 1-7 update the rest in 8 x 4 patches.  Only where the test fails do the second
-// search, the symmetric swap or the 2x2 pivot take barriers of their own.  N = 16,384, 164 steps:
-// 330 us a step with the full square updated by three FP64 operations an entry behind a
-// whole-block barrier per action and a serial column-per-thread inverse; 118 us now.
+// One block per (front, shift).  FP64 runs at 2 multiply-adds a clock and SM here and at one warp
+// instruction per 64 clocks and warp, so the block does only the lower triangle's (w^3 / 6) and the
+// inverse's (w^3 / 6), with one multiply-add each and no division in a loop; pivots are compared as
+// integers (|x| orders like its bits).  The chain of columns is the limit: warp 0 runs one column
+// ahead of the others.  It updates column k + 1, finds its largest entry and, where the diagonal fails
+// the 1x1 test -- every other column of the shifted pencils -- row r of that entry, in registers; it
+// decides on the pivot and forms that column of L while 12 other warps write the trailing triangle
+// from one buffer to the other (6 are too few to cover their shared-memory loads).  A swap of k and r
+// is part of that copy, so a column costs one block barrier whether it swaps or not; only 2x2 pivots
+// move rows in place and take barriers of their own.  The three warps on warp 0's scheduler rest, one
+// keeps the books.  A column takes 1,150 - 1,600 clocks, with a failed test 2,200 - 2,900; the inverse
+// 28,000.  N = 16,384, 164 steps, us a step: 330 with the full square updated by three FP64 operations
+// an entry behind a whole-block barrier per action and a serial column-per-thread inverse; 118 with
+// the triangle updated in place, the column ahead and a failed test resolved behind three more
+// barriers; 91 now.  The tests in FP32 with FP64 for near ties instead: no change.
 constexpr int DLD = NB + 4;        // row stride: 8 x 4 patches touch every shared-memory bank once
+constexpr int kDiagThreads = 512;
+// two copies of the triangle; strict lower L, transposed, in the second one's upper half
 constexpr size_t kDiagSmem = 2 * NB * DLD * sizeof(double);
 
 __device__ __forceinline__ unsigned long long abs_bits(double v) {
@@ -162,7 +170,13 @@ __device__ __forceinline__ unsigned long long abs_bits(double v) {
 }
 __device__ __forceinline__ double from_bits(unsigned long long b) { return __longlong_as_double((long long)b); }
 
-// largest key over the warp and the smallest index holding it
+// largest key over the warp
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long key) {
+    const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    return ((unsigned long long)mh << 32) | __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+}
+// and the smallest index holding it
 __device__ __forceinline__ unsigned long long warp_max_key(unsigned long long key, int &idx) {
     const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
     const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
@@ -171,156 +185,194 @@ __device__ __forceinline__ unsigned long long warp_max_key(unsigned long long ke
     return ((unsigned long long)mh << 32) | ml;
 }
 
+// 1 / d (0 for d = 0) from the hardware's approximation x by one step of third order: with
+// e = 1 - d x, 1 / d = x (1 + e + e^2 + ..), so 20 bits become 60 and what is left is the last
+// rounding.  Three dependent multiply-adds; a division takes some ten, and checks.  Outside
+// 2^+-1000: the division.
+__device__ __forceinline__ double diag_recip(double d) {
+    const unsigned ex = (unsigned)(__double_as_longlong(d) >> 52) & 0x7ffu;
+    if (ex - 23u > 2000u) return d != 0.0 ? 1.0 / d : 0.0;
+    double x;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(d));
+    const double e = fma(-d, x, 1.0);
+    return fma(x, fma(e, e, e), x);
+}
+
 template <typename T>
-__global__ void __launch_bounds__(256) k_diag_bk(const StepTask *__restrict__ tasks, const ShiftPtrs<T> *sp) {
+__global__ void __launch_bounds__(kDiagThreads, 1) k_diag_bk(const StepTask *__restrict__ tasks, const ShiftPtrs<T> *sp) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *A = reinterpret_cast<double *>(smem_raw);       // lower triangle, entry (i, j) at i DLD + j
-    double *L = A + NB * DLD;                                // strict lower part of L
+    double *buf = reinterpret_cast<double *>(smem_raw);     // lower triangle, entry (i, j) at i DLD + j
+    double *L = buf + NB * DLD;                              // L(i, j), i > j, at j DLD + i
     const ShiftPtrs<T> s = sp[blockIdx.y];
     const StepTask tk = tasks[blockIdx.x];
     const int w = tk.w, m = tk.m, k0 = tk.k0;
     __shared__ int perm[NB];
     __shared__ double dd[NB], de[NB], p0[NB], p1[NB];
-    __shared__ int s_kind, s_r, s_fast[2];
-    __shared__ unsigned long long c_neg, c_zero, c_pos, c_tiny, c_2x2;
+    __shared__ double s_y[2][NB], s_l[2][NB], s_d[2];        // the pivot's column of A and of L, the pivot
+    __shared__ int s_kind[2], s_r[2];
+    __shared__ unsigned long long c_neg, c_zero, c_pos, c_tiny, c_2x2, s_ratio;
     __shared__ double s_minpiv;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const T *F = s.ws + tk.front_off;
 
-    for (int q = tid; q < NB * NB; q += 256) {
+    for (int q = tid; q < NB * NB; q += kDiagThreads) {
         const int j = q / NB, i = q % NB;                    // column j, row i (coalesced on i)
-        if (i >= j && i < w) A[i * DLD + j] = (double)F[(int64_t)(k0 + j) * m + (k0 + i)];
+        if (i >= j && i < w) buf[i * DLD + j] = (double)F[(int64_t)(k0 + j) * m + (k0 + i)];
+        if (i > j) L[j * DLD + i] = 0.0;
     }
-    for (int q = tid; q < NB * DLD; q += 256) L[q] = 0.0;
     if (tid < NB) { perm[tid] = tid; dd[tid] = 0.0; de[tid] = 0.0; }
     if (tid == 0) {
         c_neg = c_zero = c_pos = c_tiny = c_2x2 = 0;
         s_minpiv = 1e300;
-        s_fast[0] = 0;
     }
     __syncthreads();
 
     const double alpha = 0.6403882032022076;   // (1 + sqrt(17)) / 8
-    // column k of L for a 1x1 pivot d at k (warp 0)
-    auto scale_column = [&](int k, double d, double v1, double v2) {
-        const double inv = d != 0.0 ? 1.0 / d : 0.0;
-        const int i1 = k + 1 + lane, i2 = i1 + 32;
-        if (i1 < w) L[i1 * DLD + k] = v1 * inv;
-        if (i2 < w) L[i2 * DLD + k] = v2 * inv;
-    };
-    // A(i, j) -= x(i) y(j) [+ x2(i) y2(j)] on the trailing triangle from row / column b0, in 8 x 4
-    // patches dealt to warps first, first + 1, ..; x = column c of L, y = column c of A
-    auto update = [&](int b0, int c, bool two, int first, int nwarp) {
-        const int n2 = w - b0, npr = (n2 + 7) >> 3, np = npr * (npr + 1);
-        int pr = 0;
-        for (int p = warp - first; p < np; p += nwarp) {
-            while (p >= (pr + 1) * (pr + 2)) ++pr;
-            const int i = b0 + 8 * pr + (lane >> 2), j = b0 + 4 * (p - pr * (pr + 1)) + (lane & 3);
-            if (i < w && j <= i) {
-                double v = A[i * DLD + j];
-                v -= L[i * DLD + c] * A[j * DLD + c];
-                if (two) v -= L[i * DLD + c + 1] * A[j * DLD + c + 1];
-                A[i * DLD + j] = v;
-            }
+    // Warp 0: the pivot of column c, by Bunch-Kaufman's test restricted to the block, from the
+    // trailing matrix get(i, j), i >= j >= c, whose column c goes to `out`: kind 1 (1x1 at c), 2 (1x1,
+    // swap c <-> r) or 3 (2x2, swap c + 1 <-> r); for 1 and 2 the column after the swap, in s_y, s_l.
+    auto decide = [&](int c, int slot, double *out, auto get) {
+        const int i0 = c + lane, i1 = i0 + 32;
+        const bool long_col = c + 32 < w;
+        double v0 = i0 < w ? get(i0, c) : 0.0, v1 = 0.0;
+        if (long_col && i1 < w) v1 = get(i1, c);
+        double d = __shfl_sync(0xffffffffu, v0, 0), inv = diag_recip(d);
+        if (out) {
+            if (i0 < w) out[i0 * DLD + c] = v0;
+            if (long_col && i1 < w) out[i1 * DLD + c] = v1;
         }
-    };
-    int k = 0;
-    for (int it = 0; k < w; ++it) {
+        unsigned long long key = lane > 0 ? abs_bits(v0) : 0;
+        int r = i0;
+        if (abs_bits(v1) > key) { key = abs_bits(v1); r = i1; }
+        key = warp_max_key(key, r);
         int kind = 1;
-        if (!s_fast[it & 1]) {
-            // the pivot of column k: Bunch-Kaufman's test restricted to the block
-            if (warp == 0) {
-                unsigned long long key = 0;
-                int r = k;
-                const int i1 = k + 1 + lane, i2 = i1 + 32;
-                const double v1 = i1 < w ? A[i1 * DLD + k] : 0.0, v2 = i2 < w ? A[i2 * DLD + k] : 0.0;
-                if (i1 < w) { key = abs_bits(v1); r = i1; }
-                if (i2 < w && abs_bits(v2) > key) { key = abs_bits(v2); r = i2; }
-                if (k + 1 < w) key = warp_max_key(key, r);
-                const double lam = from_bits(key), d = A[k * DLD + k], akk = fabs(d);
-                int kd = 1;                          // 1: 1x1 at k; 2: 1x1 with swap k<->r; 3: 2x2 (k+1<->r)
-                if (akk < alpha * lam) {
-                    unsigned long long ks = 0;
-                    int dummy = 0;
-                    for (int j = k + lane; j < w; j += 32) {
-                        if (j == r) continue;
-                        const unsigned long long kj = abs_bits(j < r ? A[r * DLD + j] : A[j * DLD + r]);
-                        if (kj > ks) ks = kj;
-                    }
-                    const double sig = from_bits(warp_max_key(ks, dummy));
-                    if (akk * sig >= alpha * lam * lam) kd = 1;
-                    else if (fabs(A[r * DLD + r]) >= alpha * sig) kd = 2;
-                    else kd = 3;
-                }
-                if (kd == 1) scale_column(k, d, v1, v2);
-                if (lane == 0) { s_kind = kd; s_r = r; }
-            }
-            __syncthreads();
-            kind = s_kind;
-            const int r = s_r;
-            if (kind >= 2) {
-                const int a = (kind == 2) ? k : k + 1;
-                if (a != r) {                        // symmetric swap a <-> r of A, row swap of L
-                    if (tid < w && tid != r) {
-                        const int j = tid;
-                        double *x, *y;
-                        if (j < k) { x = &L[a * DLD + j]; y = &L[r * DLD + j]; }
-                        else if (j < a) { x = &A[a * DLD + j]; y = &A[r * DLD + j]; }
-                        else if (j == a) { x = &A[a * DLD + a]; y = &A[r * DLD + r]; }
-                        else if (j < r) { x = &A[j * DLD + a]; y = &A[r * DLD + j]; }
-                        else { x = &A[j * DLD + a]; y = &A[j * DLD + r]; }
-                        const double t = *x;
-                        *x = *y;
-                        *y = t;
-                    }
-                    if (tid == 0) { const int t = perm[a]; perm[a] = perm[r]; perm[r] = t; }
-                    __syncthreads();
-                }
-                if (kind == 2) {
-                    if (warp == 0) {
-                        const int i1 = k + 1 + lane, i2 = i1 + 32;
-                        scale_column(k, A[k * DLD + k], i1 < w ? A[i1 * DLD + k] : 0.0, i2 < w ? A[i2 * DLD + k] : 0.0);
-                    }
-                    __syncthreads();
+        // the test |d| < alpha lam; FP64 arithmetic only for |d| between lam / 2 and lam
+        const unsigned long long kd = abs_bits(d);
+        if (kd < key && key <= 0x7ff0000000000000ull) {
+            const double lam = from_bits(key), akk = fabs(d);
+            if (kd + (1ull << 52) <= key || akk < alpha * lam) {
+                double w0 = 0.0, w1 = 0.0;
+                if (i0 < w) w0 = get(max(r, i0), min(r, i0));
+                if (long_col && i1 < w) w1 = get(max(r, i1), min(r, i1));
+                const double h = __shfl_sync(0xffffffffu, r - c >= 32 ? w1 : w0, (r - c) & 31);
+                unsigned long long ks = i0 != r ? abs_bits(w0) : 0;
+                if (i1 != r && abs_bits(w1) > ks) ks = abs_bits(w1);
+                const double inv_h = diag_recip(h);          // beside the tests, not after them
+                const double sig = from_bits(warp_max_key(ks));
+                if (!(akk * sig >= alpha * lam * lam)) {
+                    kind = fabs(h) >= alpha * sig ? 2 : 3;
+                    d = h;
+                    inv = inv_h;
+                    if (i0 != r) v0 = w0;
+                    if (i1 != r) v1 = w1;
                 }
             }
         }
         if (kind <= 2) {
+            if (lane > 0 && i0 < w) { s_y[slot][i0] = v0; s_l[slot][i0] = v0 * inv; }
+            if (long_col && i1 < w) { s_y[slot][i1] = v1; s_l[slot][i1] = v1 * inv; }
+        }
+        if (lane == 0) { s_kind[slot] = kind; s_r[slot] = kind == 1 ? c : r; s_d[slot] = d; }
+    };
+    // The trailing triangle from row / column b0, put(i, j, get(i, j)): strips of 8 rows, each cut
+    // into 8 x 4 patches dealt to the warps of its strip.  A lane keeps its row in a strip, so a patch
+    // is a few instructions -- with few warps a scheduler, dependent instructions, not the FP64 pipe,
+    // are what an update waits for.  Warp u of n has part `part` of `parts` of strip `strip`, the
+    // lowest (longest) strips have the most warps; that only changes when the first strip does.
+    int strip = 0, part = 0, parts = 0;
+    auto deal = [&](int b0, int u, int n) {
+        const int s0 = b0 >> 3, ns = ((w + 7) >> 3) - s0, per = n / ns, more = n - per * ns;   // ns <= 8 <= n
+        const bool lower = u < more * (per + 1);
+        parts = lower ? per + 1 : per;
+        u -= lower ? 0 : more * (per + 1);
+        strip = u / parts;
+        part = u - strip * parts;
+        strip = s0 + ns - 1 - strip - (lower ? 0 : more);
+    };
+    auto patches = [&](int b0, auto get, auto put) {
+        const int i = 8 * strip + (lane >> 2), step = 4 * parts;
+        if (i >= w) return;
+        for (int j = (b0 & ~3) + 4 * part + (lane & 3); j <= i; j += 4 * step) {
+            double v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int c = j + q * step;
+                v[q] = c >= b0 && c <= i ? get(i, c) : 0.0;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int c = j + q * step;
+                if (c >= b0 && c <= i) put(i, c, v[q]);
+            }
+        }
+    };
+    int half = 0, slot = 0, first = -1;          // first strip of deal()
+    if (warp == 0) decide(0, 0, nullptr, [&](int i, int j) { return buf[i * DLD + j]; });
+    __syncthreads();
+    for (int k = 0; k < w; slot ^= 1) {
+        const int kind = s_kind[slot], r = s_r[slot];
+        double *A = buf + half * NB * DLD;
+        if (kind <= 2) {
+            double *B = buf + (half ^ 1) * NB * DLD;
+            const double *y = s_y[slot], *l = s_l[slot];
+            // entry (i, j), k < j <= i, after the swap k <-> r and the pivot
+            auto get = [&](int i, int j) {
+                const int q = i == r ? (j == r ? k * DLD + k : j * DLD + k) : (j == r ? i * DLD + k : i * DLD + j);
+                return A[q] - l[i] * y[j];
+            };
+            auto get1 = [&](int i, int j) { return A[i * DLD + j] - l[i] * y[j]; };      // without a swap
             if (warp == 0) {
-                // column k + 1 ahead of the others: update, search, 1x1 test, its column of L
-                int fast = 0;
-                if (k + 1 < w) {
-                    const double c = A[(k + 1) * DLD + k];
-                    const int i0 = k + 1 + lane, i1 = i0 + 32;
-                    double v0 = 0.0, v1 = 0.0;
-                    if (i0 < w) { v0 = A[i0 * DLD + k + 1] - L[i0 * DLD + k] * c; A[i0 * DLD + k + 1] = v0; }
-                    if (i1 < w) { v1 = A[i1 * DLD + k + 1] - L[i1 * DLD + k] * c; A[i1 * DLD + k + 1] = v1; }
-                    const double d = __shfl_sync(0xffffffffu, v0, 0);
-                    unsigned long long key = lane > 0 ? abs_bits(v0) : 0;
-                    if (abs_bits(v1) > key) key = abs_bits(v1);
-                    int dummy = 0;
-                    key = warp_max_key(key, dummy);
-                    const double inv = d != 0.0 ? 1.0 / d : 0.0;
-                    fast = !(fabs(d) < alpha * from_bits(key));
-                    if (fast) {
-                        if (lane > 0 && i0 < w) L[i0 * DLD + k + 1] = v0 * inv;
-                        if (i1 < w) L[i1 * DLD + k + 1] = v1 * inv;
+                if (k + 1 >= w) {
+                } else if (kind == 1) decide(k + 1, slot ^ 1, B, get1);
+                else decide(k + 1, slot ^ 1, B, get);
+            } else if (warp == 4) {
+                for (int i = k + 1 + lane; i < w; i += 32) L[k * DLD + i] = l[i];
+                if (kind == 2)
+                    for (int j = lane; j < k; j += 32) {
+                        const double t = L[j * DLD + k];
+                        L[j * DLD + k] = L[j * DLD + r];
+                        L[j * DLD + r] = t;
                     }
-                }
-                if (lane == 0) s_fast[(it + 1) & 1] = fast;
-            } else {
-                if (tid == 32) {
-                    const double d = A[k * DLD + k], ad = fabs(d);
+                if (lane == 0) {
+                    if (kind == 2) { const int t = perm[k]; perm[k] = perm[r]; perm[r] = t; }
+                    const double d = s_d[slot];
+                    const unsigned long long ad = abs_bits(d), inf = 0x7ff0000000000000ull;
                     dd[k] = d;
-                    if (d < 0) c_neg++; else if (d > 0) c_pos++; else c_zero++;
-                    if (ad < s.tiny_thr) c_tiny++;
-                    if (ad < s_minpiv) s_minpiv = ad;
+                    if (ad == 0 || ad > inf) c_zero++; else if (__double_as_longlong(d) < 0) c_neg++; else c_pos++;
+                    if (ad < abs_bits(s.tiny_thr)) c_tiny++;
+                    if (ad < abs_bits(s_minpiv)) s_minpiv = from_bits(ad);
                 }
-                update(k + 2, k, false, 1, 7);
+                __syncwarp();
+            } else if ((warp & 3) && k + 2 < w) {
+                if (first != (k + 2) >> 3) {
+                    first = (k + 2) >> 3;
+                    deal(k + 2, 3 * (warp >> 2) + (warp & 3) - 1, 3 * kDiagThreads / 128);
+                }
+                auto put = [&](int i, int j, double v) { B[i * DLD + j] = v; };
+                if (kind == 1) patches(k + 2, get1, put);
+                else patches(k + 2, get, put);
             }
             __syncthreads();
+            half ^= 1;
             k += 1;
         } else {
+            const int a1 = k + 1;
+            if (a1 != r) {                               // symmetric swap a1 <-> r of A, row swap of L
+                if (tid < w && tid != r) {
+                    const int j = tid;
+                    double *x, *y;
+                    if (j < k) { x = &L[j * DLD + a1]; y = &L[j * DLD + r]; }
+                    else if (j < a1) { x = &A[a1 * DLD + j]; y = &A[r * DLD + j]; }
+                    else if (j == a1) { x = &A[a1 * DLD + a1]; y = &A[r * DLD + r]; }
+                    else if (j < r) { x = &A[j * DLD + a1]; y = &A[r * DLD + j]; }
+                    else { x = &A[j * DLD + a1]; y = &A[j * DLD + r]; }
+                    const double t = *x;
+                    *x = *y;
+                    *y = t;
+                }
+                if (tid == 0) { const int t = perm[a1]; perm[a1] = perm[r]; perm[r] = t; }
+                __syncthreads();
+            }
             const double a = A[k * DLD + k], b = A[(k + 1) * DLD + k], c = A[(k + 1) * DLD + k + 1];
             const double det = a * c - b * b;
             if (tid == 32) {
@@ -338,30 +390,38 @@ __global__ void __launch_bounds__(256) k_diag_bk(const StepTask *__restrict__ ta
             const int i = k + 2 + tid;
             if (i < w) {
                 const double id = 1.0 / det, ci0 = A[i * DLD + k], ci1 = A[i * DLD + k + 1];
-                L[i * DLD + k] = (c * ci0 - b * ci1) * id;
-                L[i * DLD + k + 1] = (-b * ci0 + a * ci1) * id;
+                L[k * DLD + i] = (c * ci0 - b * ci1) * id;
+                L[(k + 1) * DLD + i] = (-b * ci0 + a * ci1) * id;
             }
-            if (tid == 0) s_fast[(it + 1) & 1] = 0;
             __syncthreads();
-            update(k + 2, k, true, 0, 8);
+            if (k + 2 < w) deal(k + 2, warp, kDiagThreads / 32);
+            first = -1;
+            if (k + 2 < w) patches(k + 2, [&](int i, int j) {
+                double v = A[i * DLD + j];
+                v -= L[k * DLD + i] * A[j * DLD + k];
+                v -= L[(k + 1) * DLD + i] * A[j * DLD + k + 1];
+                return v;
+            }, [&](int i, int j, double v) { A[i * DLD + j] = v; });
+            __syncthreads();
+            if (warp == 0 && k + 2 < w) decide(k + 2, slot ^ 1, nullptr, [&](int i, int j) { return A[i * DLD + j]; });
             __syncthreads();
             k += 2;
         }
     }
-    // X = L^-1 in A's place, by 16 x 16 diagonal blocks and two levels of
+    // X = L^-1 in the first copy's place, by 8 x 8 diagonal blocks and three levels of
     // X21 = -X22 (L21 X11); the products L21 X11 rest in blocks above the diagonal meanwhile
-    double *X = A;
+    double *X = buf;
     if (tid < NB) {
-        const int b = tid & ~15, jl = tid & 15;
-        double x[16];
+        const int b = tid & ~7, jl = tid & 7;
+        double x[8];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = i == jl ? 1.0 : 0.0;
+        for (int i = 0; i < 8; ++i) x[i] = i == jl ? 1.0 : 0.0;
 #pragma unroll
-        for (int t = 0; t < 15; ++t)
+        for (int t = 0; t < 7; ++t)
 #pragma unroll
-            for (int i = t + 1; i < 16; ++i) x[i] -= L[(b + i) * DLD + b + t] * x[t];
+            for (int i = t + 1; i < 8; ++i) x[i] -= L[(b + t) * DLD + b + i] * x[t];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) X[(b + i) * DLD + tid] = x[i];
+        for (int i = 0; i < 8; ++i) X[(b + i) * DLD + tid] = x[i];
     } else {
         // constants of D^-1: column j of L^-T D^-1 is p0 X(j, :) + p1 X(j +- 1, :)
         const int j = tid - NB;
@@ -377,21 +437,37 @@ __global__ void __launch_bounds__(256) k_diag_bk(const StepTask *__restrict__ ta
                 p1[j] = 0.0;
             }
         }
+        if (tid == 2 * NB) s_ratio = (unsigned long long)__double_as_longlong(s_minpiv / (s.norm > 0 ? s.norm : 1.0));
     }
     __syncthreads();
     {
+        const int C = 16 * (tid >> 6), R = C + 8, i = (tid >> 3) & 7, j = tid & 7;
+        double acc = 0.0;
+        if (tid < 4 * NB) {
+#pragma unroll
+            for (int t = 0; t < 8; ++t) acc += L[(C + t) * DLD + R + i] * X[(C + t) * DLD + C + j];
+            X[(C + i) * DLD + R + j] = acc;
+        }
+        __syncthreads();
+        if (tid < 4 * NB) {
+            acc = 0.0;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) acc += X[(R + i) * DLD + R + t] * X[(C + t) * DLD + R + j];
+            X[(R + i) * DLD + C + j] = -acc;
+        }
+        __syncthreads();
+    }
+    {
         const int h = lane & 15, C = 32 * (lane >> 4), R = C + 16;
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int j = warp + 8 * u;
+        for (int j = warp; j < 16; j += kDiagThreads / 32) {
             double acc = 0.0;
-            for (int t = j; t < 16; ++t) acc += L[(R + h) * DLD + C + t] * X[(C + t) * DLD + C + j];
+            for (int t = j; t < 16; ++t) acc += L[(C + t) * DLD + R + h] * X[(C + t) * DLD + C + j];
             X[(C + h) * DLD + R + j] = acc;
         }
         __syncthreads();
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int i = warp + 8 * u;
+        for (int i = warp; i < 16; i += kDiagThreads / 32) {
             double acc = 0.0;
             for (int t = 0; t <= i; ++t) acc += X[(R + i) * DLD + R + t] * X[(C + t) * DLD + R + h];
             X[(R + i) * DLD + C + h] = -acc;
@@ -399,16 +475,14 @@ __global__ void __launch_bounds__(256) k_diag_bk(const StepTask *__restrict__ ta
         __syncthreads();
         if (w > 32) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int j = warp + 8 * u;
+            for (int j = warp; j < 32; j += kDiagThreads / 32) {
                 double acc = 0.0;
-                for (int t = j; t < 32; ++t) acc += L[(32 + lane) * DLD + t] * X[t * DLD + j];
+                for (int t = j; t < 32; ++t) acc += L[t * DLD + 32 + lane] * X[t * DLD + j];
                 X[lane * DLD + 32 + j] = acc;
             }
             __syncthreads();
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int i = warp + 8 * u;
+            for (int i = warp; i < 32; i += kDiagThreads / 32) {
                 double acc = 0.0;
                 for (int t = 0; t <= i; ++t) acc += X[(32 + i) * DLD + 32 + t] * X[t * DLD + 32 + lane];
                 X[(32 + i) * DLD + lane] = -acc;
@@ -419,10 +493,10 @@ __global__ void __launch_bounds__(256) k_diag_bk(const StepTask *__restrict__ ta
     const int p = tk.panel;
     double *linv = s.linv + (int64_t)p * NB * NB;
     unsigned long long lmax = 0;                 // largest |L| entry (element growth diagnostic)
-    for (int q = tid; q < NB * NB; q += 256) {
+    for (int q = tid; q < NB * NB; q += kDiagThreads) {
         const int i = q / NB, j = q % NB;
         linv[q] = (i < w && j <= i) ? X[i * DLD + j] : 0.0;
-        if (i > j) lmax = max(lmax, abs_bits(L[i * DLD + j]));
+        if (j > i) lmax = max(lmax, abs_bits(L[i * DLD + j]));
     }
     if (tid < NB) {
         s.dblk[(int64_t)p * 2 * NB + tid] = tid < w ? dd[tid] : 0.0;
@@ -431,7 +505,7 @@ __global__ void __launch_bounds__(256) k_diag_bk(const StepTask *__restrict__ ta
     }
     // Mt[perm[i]][j] = sum_{t in block(j)} Li[t][i] Dinv[t][j]
     T *mt = s.mt + (int64_t)tk.mt_slot * NB * NB;
-    for (int q = tid; q < w * NB; q += 256) {
+    for (int q = tid; q < w * NB; q += kDiagThreads) {
         const int i = q / NB, j = q % NB;
         if (j >= w) continue;
         double v = i <= j ? X[j * DLD + i] * p0[j] : 0.0;
@@ -441,16 +515,14 @@ __global__ void __launch_bounds__(256) k_diag_bk(const StepTask *__restrict__ ta
         }
         mt[perm[i] * NB + j] = (T)v;
     }
-    int dummy = 0;
-    lmax = warp_max_key(lmax, dummy);
+    lmax = warp_max_key(lmax);
     if (lane == 0 && lmax) atomicMax(&s.counts[6], lmax);
     if (tid == 0) {
         atomicAdd(&s.counts[0], c_neg);
         atomicAdd(&s.counts[1], c_zero);
         atomicAdd(&s.counts[2], c_pos);
         if (c_tiny) atomicAdd(&s.counts[3], c_tiny);
-        double ratio = s_minpiv / (s.norm > 0 ? s.norm : 1.0);
-        atomicMin(&s.counts[4], (unsigned long long)__double_as_longlong(ratio));
+        atomicMin(&s.counts[4], s_ratio);
         if (c_2x2) atomicAdd(&s.counts[5], c_2x2);
     }
 }
@@ -545,8 +617,7 @@ __global__ void __launch_bounds__(256) k_panel(const StepTask *__restrict__ task
         if (j > 0 && se[j - 1] != 0.0) wv += (double)Ls[j - 1][i] * se[j - 1];
         W[(int64_t)j * tk.r + r0 + i] = (T)wv;
     }
-    int dummy = 0;
-    lmax = warp_max_key(lmax, dummy);
+    lmax = warp_max_key(lmax);
     if ((tid & 31) == 0 && lmax) atomicMax(&s.counts[6], lmax);
 }
 
