@@ -14,7 +14,26 @@
 namespace ssd {
 
 // ---------------------------------------------------------------- Gram G += X^T Y
-// block = 32 x 32 tile of G over one chunk of rows; 256 threads, 2 x 2 outputs each
+// block = 32 x 32 tile of G over one chunk of rows; 256 threads, 2 x 2 outputs each, fewer where the
+// matrix ends in the tile's first half (A, B outputs a thread).  A chunk of 32 rows is 16,400 clocks of
+// an SM's FP64 pipe, so the rows are dealt to the whole chip, 32 a block if need be (at least 256 a
+// block before: n = 5,000, k = 32 91 us, 24 now); consecutive lanes add to consecutive entries of G.
+template <int A, int B>
+__device__ __forceinline__ void gram_chunk(const double (*Xs)[33], const double (*Ys)[33], int tx, int ty, int rows,
+                                           double (&acc)[2][2]) {
+#pragma unroll 8
+    for (int rr = 0; rr < rows; ++rr) {
+        double x[A], y[B];
+#pragma unroll
+        for (int a = 0; a < A; ++a) x[a] = Xs[rr][ty + 16 * a];
+#pragma unroll
+        for (int b = 0; b < B; ++b) y[b] = Ys[rr][tx + 16 * b];
+#pragma unroll
+        for (int a = 0; a < A; ++a)
+#pragma unroll
+            for (int b = 0; b < B; ++b) acc[a][b] += x[a] * y[b];
+    }
+}
 __global__ void __launch_bounds__(256) k_gram(int64_t n, const double *__restrict__ X, int64_t ldx, int k1,
                                               const double *__restrict__ Y, int64_t ldy, int k2,
                                               int64_t rows_per, int sym, double *G) {
@@ -26,6 +45,7 @@ __global__ void __launch_bounds__(256) k_gram(int64_t n, const double *__restric
     const int64_t r_begin = blockIdx.z * rows_per;
     const int64_t r_end = min(n, r_begin + rows_per);
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const bool a2 = i0 + 16 < k1, b2 = j0 + 16 < k2;
     double acc[2][2] = {{0, 0}, {0, 0}};
     for (int64_t r0 = r_begin; r0 < r_end; r0 += 32) {
         for (int q = tid; q < 32 * 32; q += 256) {
@@ -35,20 +55,18 @@ __global__ void __launch_bounds__(256) k_gram(int64_t n, const double *__restric
             Ys[rr][c] = (r < r_end && j0 + c < k2) ? Y[r * ldy + j0 + c] : 0.0;
         }
         __syncthreads();
-#pragma unroll 8
-        for (int rr = 0; rr < 32; ++rr) {
-            double x0 = Xs[rr][tx], x1 = Xs[rr][tx + 16];
-            double y0 = Ys[rr][ty], y1 = Ys[rr][ty + 16];
-            acc[0][0] += x0 * y0; acc[0][1] += x0 * y1;
-            acc[1][0] += x1 * y0; acc[1][1] += x1 * y1;
-        }
+        const int rows = (int)min((int64_t)32, r_end - r0);
+        if (a2 && b2) gram_chunk<2, 2>(Xs, Ys, tx, ty, rows, acc);
+        else if (a2) gram_chunk<2, 1>(Xs, Ys, tx, ty, rows, acc);
+        else if (b2) gram_chunk<1, 2>(Xs, Ys, tx, ty, rows, acc);
+        else gram_chunk<1, 1>(Xs, Ys, tx, ty, rows, acc);
         __syncthreads();
     }
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
-            int i = i0 + tx + 16 * a, j = j0 + ty + 16 * b;
+            int i = i0 + ty + 16 * a, j = j0 + tx + 16 * b;
             if (i < k1 && j < k2) {
                 atomicAdd(&G[(int64_t)i * k2 + j], acc[a][b]);
                 if (sym && blockIdx.x != blockIdx.y) atomicAdd(&G[(int64_t)j * k2 + i], acc[a][b]);
@@ -57,51 +75,59 @@ __global__ void __launch_bounds__(256) k_gram(int64_t n, const double *__restric
 }
 
 // ---------------------------------------------------------------- Y = beta Y + alpha X Q  (or X Q^T)
-// block = 64 rows x 32 columns of Y; k1 chunks of 32 through shared memory.  Q is k1 x k2
+// block = 16 RA rows x 16 columns of Y; k1 chunks of 32 through shared memory.  Q is k1 x k2
 // (ldq = k2) or, transposed, k2 x k1 (ldq = k1).  beta = 0 does not read Y.  tri: the
 // effective Q (k1 x k2) is upper triangular (a lower-triangular Q used transposed), so
-// chunks below column block j0's diagonal are skipped.
+// chunks below column block j0's diagonal are skipped.  Bound by the FP64 pipe: RA is the largest
+// that gives every SM several blocks, terms end at k1 and columns at a multiple of 16 (64 rows x 32
+// columns a block and 32 terms a chunk before: n = 5,000, k = 47 73 us, 27 now).
+template <int RA>
 __global__ void __launch_bounds__(256) k_gemm_tall(int64_t n, const double *__restrict__ X, int64_t ldx, int k1,
                                                    const double *__restrict__ Q, int k2, int transq,
                                                    double alpha, double beta, double *__restrict__ Y,
                                                    int64_t ldy, int tri) {
-    __shared__ double Xs[64][33], Qs[32][33];
-    const int64_t r0 = blockIdx.x * 64ll;
-    const int j0 = blockIdx.y * 32;
-    const int tid = threadIdx.x, tc = tid & 31, tr = tid >> 5;   // column tc, rows tr + 8 a
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    const int t_end = tri ? min(k1, j0 + 32) : k1;
-    for (int t0 = 0; t0 < t_end; t0 += 32) {
-        for (int q = tid; q < 64 * 32; q += 256) {
-            int rr = q >> 5, c = q & 31;
-            int64_t r = r0 + rr;
-            Xs[rr][c] = (r < n && t0 + c < k1) ? X[r * ldx + t0 + c] : 0.0;
-        }
-        for (int q = tid; q < 32 * 32; q += 256) {
-            int t = q >> 5, c = q & 31;
-            double v = 0.0;
-            if (t0 + t < k1 && j0 + c < k2)
-                v = transq ? Q[(int64_t)(j0 + c) * k1 + t0 + t] : Q[(int64_t)(t0 + t) * k2 + j0 + c];
-            Qs[t][c] = v;
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int t = 0; t < 32; ++t) {
-            double qv = Qs[t][tc];
+    constexpr int R = 16 * RA;
+    __shared__ double Xs[R][33], Qs[32][17];
+    const int64_t r0 = (int64_t)blockIdx.x * R;
+    const int tid = threadIdx.x, tc = tid & 15, tr = tid >> 4;   // column tc, rows tr + 16 a
+    for (int64_t j0 = 16ll * blockIdx.y; j0 < k2; j0 += 16ll * gridDim.y) {
+        double acc[RA];
 #pragma unroll
-            for (int a = 0; a < 8; ++a) acc[a] += Xs[tr + 8 * a][t] * qv;
-        }
-        __syncthreads();
-    }
-    if (j0 + tc < k2)
-#pragma unroll
-        for (int a = 0; a < 8; ++a) {
-            int64_t r = r0 + tr + 8 * a;
-            if (r < n) {
-                double *y = Y + r * ldy + j0 + tc;
-                *y = (beta != 0.0 ? beta * *y : 0.0) + alpha * acc[a];
+        for (int a = 0; a < RA; ++a) acc[a] = 0.0;
+        const int t_end = tri ? (int)min((int64_t)k1, j0 + 16) : k1;
+        for (int t0 = 0; t0 < t_end; t0 += 32) {
+            const int nt = min(32, t_end - t0);
+            for (int q = tid; q < R * 32; q += 256) {
+                int rr = q >> 5, c = q & 31;
+                int64_t r = r0 + rr;
+                Xs[rr][c] = (r < n && c < nt) ? X[r * ldx + t0 + c] : 0.0;
             }
+            for (int q = tid; q < 32 * 16; q += 256) {
+                const int t = transq ? q & 31 : q >> 4, c = transq ? q >> 5 : q & 15;
+                double v = 0.0;
+                if (t < nt && j0 + c < k2)
+                    v = transq ? Q[(j0 + c) * k1 + t0 + t] : Q[(int64_t)(t0 + t) * k2 + j0 + c];
+                Qs[t][c] = v;
+            }
+            __syncthreads();
+#pragma unroll 4
+            for (int t = 0; t < nt; ++t) {
+                double qv = Qs[t][tc];
+#pragma unroll
+                for (int a = 0; a < RA; ++a) acc[a] += Xs[tr + 16 * a][t] * qv;
+            }
+            __syncthreads();
         }
+        if (j0 + tc < k2)
+#pragma unroll
+            for (int a = 0; a < RA; ++a) {
+                int64_t r = r0 + tr + 16 * a;
+                if (r < n) {
+                    double *y = Y + r * ldy + j0 + tc;
+                    *y = (beta != 0.0 ? beta * *y : 0.0) + alpha * acc[a];
+                }
+            }
+    }
 }
 
 // ---------------------------------------------------------------- small Cholesky and inverse

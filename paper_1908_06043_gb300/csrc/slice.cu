@@ -55,8 +55,9 @@ int gram_ld(ss_ctx *ctx, const double *X, int64_t ldx, int64_t n, int k1, const 
     if (oz_dense_ok(ctx, n, k1, k2)) return oz_gram(ctx, X, ldx, n, k1, Y, ldy, k2, G);
     const int64_t t1 = cdiv(k1, 32), t2 = cdiv(k2, 32);
     const int64_t bxy = sym ? t1 * (t1 + 1) / 2 : t1 * t2;     // tiles that do work
-    int64_t nz = std::max<int64_t>(1, (4 * (int64_t)ctx->sm_count + bxy - 1) / bxy);
-    nz = std::min<int64_t>(nz, std::max<int64_t>(1, n / 256));
+    // many blocks an SM: tiles at the matrix's end have a half or a quarter of the work
+    int64_t nz = std::max<int64_t>(1, (16 * (int64_t)ctx->sm_count + bxy - 1) / bxy);
+    nz = std::min<int64_t>(nz, cdiv(n, 32));
     int64_t per = ((n + nz - 1) / nz + 31) / 32 * 32;
     nz = (n + per - 1) / per;
     ss_launch(ctx, SS_K_GRAM, ssd::k_gram, dim3(cdiv(k1, 32), cdiv(k2, 32), (unsigned)std::max<int64_t>(1, nz)), 256,
@@ -74,8 +75,12 @@ int gram(ss_ctx *ctx, const double *X, int64_t n, int k1, const double *Y, int k
 int gemm_ld(ss_ctx *ctx, const double *X, int64_t ldx, int64_t n, int k1, const double *Q, int k2, int transq,
             double alpha, double beta, double *Y, int64_t ldy, int tri = 0) {
     if (oz_dense_ok(ctx, n, k1, k2)) return oz_gemm(ctx, X, ldx, n, k1, Q, k2, transq, alpha, beta, Y, ldy);
-    ss_launch(ctx, SS_K_GEMM, ssd::k_gemm_tall, dim3(cdiv(n, 64), cdiv(k2, 32)), 256, 0, ctx->stream, n, X, ldx, k1,
-              Q, k2, transq, alpha, beta, Y, ldy, tri);
+    // the most rows a block (fewer reads of Q) that still leave four blocks an SM
+    const int64_t cols = cdiv(k2, 16), want = 4 * (int64_t)ctx->sm_count;
+    const int ra = cdiv(n, 64) * cols >= want ? 4 : cdiv(n, 32) * cols >= want ? 2 : 1;
+    ss_launch(ctx, SS_K_GEMM, ra == 4 ? ssd::k_gemm_tall<4> : ra == 2 ? ssd::k_gemm_tall<2> : ssd::k_gemm_tall<1>,
+              dim3(cdiv(n, 16 * ra), (unsigned)std::min<int64_t>(cols, 65535)), 256, 0, ctx->stream, n, X, ldx, k1, Q, k2, transq, alpha, beta, Y,
+              ldy, tri);
     ctx->add_flops(SS_K_GEMM, tri ? (double)n * k2 * (k2 + 1) : 2.0 * (double)n * k1 * k2);
     SS_CUDA_TRY(ctx, cudaGetLastError());
     return SS_OK;
