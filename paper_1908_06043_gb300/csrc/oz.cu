@@ -342,12 +342,8 @@ int spmm_core(ss_symbolic *s, int npass, OzVals *const *v, const double *const *
 
 }  // namespace
 
-// The tensor-core products of dense operands take 95 - 110 us whatever the size (digits of both,
-// exponents, a read-back), the CUDA-core ones 1.8 ps a multiply-add.  Gram / gemm, us, CUDA cores and
-// tensor cores: n = 5,000, k = 96 89 / 93 and 108 / 104; n = 10,000, k = 64 81 / 87 and 115 / 107;
-// n = 16,384, k = 64 122 / 120 and 138 / 104; n = 10,000, k = 96 169 / 179 and 125 / 131.
 bool oz_dense_ok(const ss_ctx *ctx, int64_t n, int k1, int k2) {
-    return ctx->gemm_mode == SS_GEMM_TENSOR && n >= 2048 && k1 >= 48 && k2 >= 48 && (double)n * k1 * k2 >= 5.5e7;
+    return ctx->gemm_mode == SS_GEMM_TENSOR && n >= 2048 && k1 >= 48 && k2 >= 48;
 }
 
 bool oz_spmm_ok(const ss_numeric *f, int k) {
