@@ -1641,12 +1641,18 @@ int solve_apply(ss_numeric *f, int j, const double *R, int k, double *X, int ref
     }
     // mixed: FP32 solves inside FP64 iterative refinement, X_0 = 0.  With a target the
     // residual decides when to stop; otherwise a requested refinement gets at least the
-    // number of steps the shift's contraction factor needs to reach 1e-13.  A refined block
-    // solve of a shift whose FP64 factor is there too runs its solves in FP64 on the tensor cores:
-    // one contracts the residual by 1e-10 where an FP32 one gives 1e-1 .. 1e-2 (N = 16,384, k = 304:
-    // 9.2 ms a solve against 6.4 ms, and 3 instead of 8 or 9 for two requested refinements)
-    const bool in_f64 = refine > 0 && f->shift_prec[j] == SS_FP64 && ctx->solve_mode == SS_SOLVE_SWEEP_KERNEL &&
-                        fold_uses_tc(s, k);
+    // number of steps the shift's contraction factor needs to reach 1e-13.  A refined solve of a
+    // shift whose FP64 factor is there too runs its solves in FP64 where these are the quicker ones:
+    // a solve contracts the residual by 1e-10 where an FP32 one gives 1e-1 .. 1e-2, and the folded
+    // sweeps pass a level in 5 - 10 us where the FP32 ones take 48.  Only many columns without the
+    // tensor cores (4 ps of FP64 per entry of L and column) are left to FP32.  Measured, ms a solve,
+    // FP32 / FP64: N = 16,384, k = 304 6.4 / 9.2 (and 8 or 9 / 3 of them for two requested
+    // refinements); k = 1, 8, 16, 48 3.4 / 0.85, 3.3 / 2.5, 3.4 / 4.2, 3.6 / 4.4 (7 / 2 of them for one
+    // refinement at a contraction of 1.5e-2).
+    const bool in_f64 = (refine > 0 || target > 0.0) && f->shift_prec[j] == SS_FP64 &&
+                        ctx->solve_mode == SS_SOLVE_SWEEP_KERNEL &&
+                        (fold_uses_tc(s, k) ||
+                         (double)s->info.l_offdiag_entries * k <= 2e7 * (double)s->solve_levels.size());
     if (target > 0.0) {
         refine = std::max(refine, 12);
     } else if (!in_f64 && refine > 0 && f->rho[j] > 0.0 && f->rho[j] < 1.0) {
