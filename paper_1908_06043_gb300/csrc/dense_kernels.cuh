@@ -522,6 +522,19 @@ __global__ void k_set_identity(double *V, int k) {
 
 // ---------------------------------------------------------------- column reductions
 // out[c] += sum_r X[r][c] * Y[r][c]
+// out[c] += sum of acc over the block's threads tid = c mod nv; 256 threads, nv a power of two.
+// Within warps by shuffles: as one thread a column over 256 / nv values it was most of such a launch.
+__device__ __forceinline__ void column_sums(double acc, int nv, double *s, double *out) {
+    const int tid = threadIdx.x, step = max(nv, 32);
+    for (int o = 16; o >= nv; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    s[tid] = acc;
+    __syncthreads();
+    if (tid < nv) {
+        double v = 0.0;
+        for (int t = tid; t < 256; t += step) v += s[t];
+        atomicAdd(&out[tid], v);
+    }
+}
 __global__ void k_col_dot(int64_t n, int k, const double *__restrict__ X, const double *__restrict__ Y,
                           double *out) {
     // requires 256 % k == 0 so that each thread keeps one column
@@ -531,13 +544,7 @@ __global__ void k_col_dot(int64_t n, int k, const double *__restrict__ X, const 
     const int64_t tot = n * k;
     for (int64_t q = blockIdx.x * 256ll + tid; q < tot; q += (int64_t)gridDim.x * 256)
         acc += X[q] * Y[q];
-    s[tid] = acc;
-    __syncthreads();
-    if (tid < k) {
-        double v = 0.0;
-        for (int t = tid; t < 256; t += k) v += s[t];
-        atomicAdd(&out[tid], v);
-    }
+    column_sums(acc, k, s, out);
 }
 
 // out[c] += sum_r X[r][c]^2 for any k (block per row chunk)
@@ -588,7 +595,7 @@ __global__ void k_neg_scale(int k, const double *__restrict__ x, double *__restr
 
 // ---------------------------------------------------------------- Lanczos helpers
 // h[i][c] = sum_r Q_i[r][c] w[r][c], i < j; grid (j, chunks); 256 % nv == 0
-__global__ void k_lz_dots(const double *__restrict__ Qb, int64_t n, int nv, int j,
+__global__ void __launch_bounds__(256) k_lz_dots(const double *__restrict__ Qb, int64_t n, int nv, int j,
                           const double *__restrict__ w, int64_t per, double *h) {
     __shared__ double s[256];
     const int i = blockIdx.x;
@@ -597,29 +604,35 @@ __global__ void k_lz_dots(const double *__restrict__ Qb, int64_t n, int nv, int 
     const int64_t e0 = blockIdx.y * per, e1 = min(tot, e0 + per);
     const double *q = Qb + (int64_t)i * tot;
     double acc = 0.0;
+#pragma unroll 8
     for (int64_t e = e0 + tid; e < e1; e += 256) acc += q[e] * w[e];
-    s[tid] = acc;
+    column_sums(acc, nv, s, h + (int64_t)i * nv);
+}
+// Re-orthogonalisation, N = 2,688, 4 vectors, 100 steps: 109 us a step with one block a vector in the
+// dots, one thread an entry over all vectors here and one launch an array; 57 us now, of which most is
+// launches and the L2's latency.
+// w -= sum_i X_i h_i (blockIdx.y = 0) and bw -= sum_i BX_i h_i (1): block = 32 entries, the vectors
+// dealt to 8 warps
+__global__ void __launch_bounds__(256) k_lz_sub(const double *__restrict__ X, const double *__restrict__ BX, int64_t n,
+                                                int nv, int j, const double *__restrict__ h, double *w, double *bw) {
+    __shared__ double s[8][33];
+    const int64_t tot = n * nv, e = blockIdx.x * 32ll + (threadIdx.x & 31);
+    const int part = threadIdx.x >> 5, lane = threadIdx.x & 31, c = (int)(e % nv);
+    const double *Q = blockIdx.y ? BX : X;
+    double acc = 0.0;
+    if (e < tot)
+#pragma unroll 4
+        for (int i = part; i < j; i += 8) acc += Q[(int64_t)i * tot + e] * h[(int64_t)i * nv + c];
+    s[part][lane] = acc;
     __syncthreads();
-    if (tid < nv) {
+    if (part == 0 && e < tot) {
         double v = 0.0;
-        for (int t = tid; t < 256; t += nv) v += s[t];
-        atomicAdd(&h[(int64_t)i * nv + tid], v);
+#pragma unroll
+        for (int p = 0; p < 8; ++p) v += s[p][lane];
+        double *o = blockIdx.y ? bw : w;
+        o[e] -= v;
     }
 }
-
-// w[r][c] -= sum_{i<j} Q_i[r][c] h[i][c]
-__global__ void k_lz_sub(const double *__restrict__ Qb, int64_t n, int nv, int j,
-                         const double *__restrict__ h, double *w) {
-    const int64_t tot = n * nv;
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= tot) return;
-    const int c = (int)(e % nv);
-    double acc = w[e];
-    for (int i = 0; i < j; ++i) acc -= Qb[(int64_t)i * tot + e] * h[(int64_t)i * nv + c];
-    w[e] = acc;
-}
-
-// w -= alpha_c q + beta_c q_prev (beta from the previous step, may be null)
 __global__ void k_lz_three_term(int64_t n, int nv, const double *__restrict__ q,
                                 const double *__restrict__ qp, const double *__restrict__ alpha,
                                 const double *__restrict__ beta_prev, double *w) {
@@ -632,18 +645,28 @@ __global__ void k_lz_three_term(int64_t n, int nv, const double *__restrict__ q,
 }
 
 // q_next = w / beta (0 where beta is tiny)
-__global__ void k_lz_normalize(int64_t n, int nv, const double *__restrict__ w,
-                               const double *__restrict__ nrm2, double *__restrict__ beta,
-                               double *__restrict__ qn) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e < nv) beta[e] = sqrt(nrm2[e]);
+// x = w / beta and bx = bw / beta (blockIdx.y) with beta = sqrt(nrm2), 0 for beta = 0; one root and
+// reciprocal a column, the quotient corrected to about its last bit
+__global__ void __launch_bounds__(256) k_lz_normalize(int64_t n, int nv, const double *__restrict__ w,
+                               const double *__restrict__ bw, const double *__restrict__ nrm2, double *__restrict__ beta,
+                               double *__restrict__ x, double *__restrict__ bx) {
+    __shared__ double s_b[256], s_r[256];
+    const int64_t e = blockIdx.x * 256ll + threadIdx.x;
+    if (threadIdx.x < nv) {
+        const double b = sqrt(nrm2[threadIdx.x]);
+        s_b[threadIdx.x] = b;
+        s_r[threadIdx.x] = 1.0 / b;
+        if (blockIdx.x == 0 && blockIdx.y == 0) beta[threadIdx.x] = b;
+    }
+    __syncthreads();
     if (e >= n * nv) return;
     const int c = (int)(e % nv);
-    const double b = sqrt(nrm2[c]);
-    qn[e] = b > 0.0 ? w[e] / b : 0.0;
+    const double b = s_b[c], r = s_r[c], v = (blockIdx.y ? bw : w)[e];
+    double q = v * r;
+    q += r * fma(-q, b, v);
+    if (!isfinite(q)) q = v / b;
+    (blockIdx.y ? bx : x)[e] = b > 0.0 ? q : 0.0;
 }
-
-// dense tridiagonal matrix of run c from alpha[j*nv+c], beta[j*nv+c]
 __global__ void k_lz_tridiag(const double *__restrict__ alpha, const double *__restrict__ beta,
                              int nv, int c, int m, double *T) {
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;

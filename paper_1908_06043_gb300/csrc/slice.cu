@@ -636,27 +636,26 @@ int lanczos_impl(ss_symbolic *s, ss_numeric *fb, const double *a_vals, const dou
     TRY_ALLOC(ctx, buf.get(&h, (size_t)(steps + 1) * nv));
     TRY_ALLOC(ctx, buf.get(&alpha, (size_t)steps * nv));
     TRY_ALLOC(ctx, buf.get(&beta, (size_t)steps * nv));
-    TRY_ALLOC(ctx, buf.get(&nrm, (size_t)nv));
+    TRY_ALLOC(ctx, buf.get(&nrm, (size_t)(steps + 1) * nv));
+    SS_CUDA_TRY(ctx, cudaMemsetAsync(alpha, 0, sizeof(double) * steps * nv, st));
+    SS_CUDA_TRY(ctx, cudaMemsetAsync(nrm, 0, sizeof(double) * (steps + 1) * nv, st));
     const unsigned g = cdiv(blk, 256);
-    auto coldot = [&](const double *x, const double *y, double *out) -> int {
-        SS_CUDA_TRY(ctx, cudaMemsetAsync(out, 0, sizeof(double) * nv, st));
+    auto coldot = [&](const double *x, const double *y, double *out) {      // out: zero
         unsigned gb = std::min<unsigned>(cdiv(blk, 256), 4 * ctx->sm_count);
         ss_launch(ctx, SS_K_LANCZOS, ssd::k_col_dot, gb, 256, 0, st, n, nv, x, y, out);
-        return SS_OK;
     };
     auto reorth = [&](int j) -> int {   // w, bw -= X h, BX h with h = X^T bw  (j+1 vectors)
         SS_CUDA_TRY(ctx, cudaMemsetAsync(h, 0, sizeof(double) * (j + 1) * nv, st));
-        const int64_t per = 32768;
+        const int64_t per = std::max<int64_t>(2048, (blk + 65534) / 65535 + 255 & ~255ll);      // whole columns of threads
         ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_dots, dim3(j + 1, cdiv(blk, per)), 256, 0, st, X, n, nv, j + 1, bw, per, h);
-        ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_sub, g, 256, 0, st, X, n, nv, j + 1, h, w);
-        ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_sub, g, 256, 0, st, BX, n, nv, j + 1, h, bw);
+        ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_sub, dim3(cdiv(blk, 32), 2), 256, 0, st, X, BX, n, nv, j + 1, h, w, bw);
         return SS_OK;
     };
     // x_1 = start / ||start||_B
     if ((rc = spmm_launch(s, b_vals, b_vals, nullptr, nullptr, start, nv, bw)) != SS_OK) return rc;
-    coldot(start, bw, nrm);
-    ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_normalize, g, 256, 0, st, n, nv, start, nrm, beta /*scratch*/, X);
-    ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_normalize, g, 256, 0, st, n, nv, bw, nrm, beta, BX);
+    coldot(start, bw, nrm + (int64_t)steps * nv);
+    ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_normalize, dim3(g, 2), 256, 0, st, n, nv, start, bw, nrm + (int64_t)steps * nv,
+              beta /*scratch*/, X, BX);
     for (int j = 0; j < steps; ++j) {
         double *xj = X + (int64_t)j * blk;
         if ((rc = spmm_launch(s, a_vals, a_vals, nullptr, nullptr, xj, nv, u)) != SS_OK) return rc;
@@ -665,11 +664,10 @@ int lanczos_impl(ss_symbolic *s, ss_numeric *fb, const double *a_vals, const dou
         ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_three_term, g, 256, 0, st, n, nv, xj, j > 0 ? xj - blk : nullptr, alpha + (int64_t)j * nv,
                                                  j > 0 ? beta + (int64_t)(j - 1) * nv : nullptr, w);
         if ((rc = spmm_launch(s, b_vals, b_vals, nullptr, nullptr, w, nv, bw)) != SS_OK) return rc;
-        reorth(j);
-        reorth(j);
-        coldot(w, bw, nrm);
-        ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_normalize, g, 256, 0, st, n, nv, w, nrm, beta + (int64_t)j * nv, X + (int64_t)(j + 1) * blk);
-        ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_normalize, g, 256, 0, st, n, nv, bw, nrm, beta + (int64_t)j * nv, BX + (int64_t)(j + 1) * blk);
+        if ((rc = reorth(j)) != SS_OK || (rc = reorth(j)) != SS_OK) return rc;
+        coldot(w, bw, nrm + (int64_t)j * nv);
+        ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_normalize, dim3(g, 2), 256, 0, st, n, nv, w, bw, nrm + (int64_t)j * nv,
+                  beta + (int64_t)j * nv, X + (int64_t)(j + 1) * blk, BX + (int64_t)(j + 1) * blk);
     }
     SS_CUDA_TRY(ctx, cudaGetLastError());
     std::vector<double> ha((size_t)steps * nv), hb((size_t)steps * nv);
