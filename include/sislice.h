@@ -148,8 +148,8 @@ ss_status ss_set_solve_mode(ss_ctx *ctx, int32_t mode);
  * with one grid barrier instead of two: every update item solves its panel's diagonal
  * block for its own 32 columns, and the last gather item of a panel runs its backward
  * diagonal step.  0 (default): never; -1: levels whose fused items fit in one pass of the
- * resident blocks.  Measured on GB300 (N = 16,384, k = 304): 6.5 ms per FP32 solve unfused,
- * 7.7 ms with -1 and 13.1 ms with every level fused -- the extra work of the fused items
+ * resident blocks.  Measured on GB300 (N = 16,384, k = 304): 6.3 ms per FP32 solve unfused,
+ * 7.6 ms with -1 and 12.8 ms with every level fused -- the extra work of the fused items
  * costs more than the barriers they save, so the default leaves it off.
  * Errors: SS_ERR_ARG (max_items < -1). */
 ss_status ss_set_sweep_fusion(ss_ctx *ctx, int32_t max_items);
@@ -362,7 +362,8 @@ ss_status ss_solve(ss_numeric *f, int32_t shift_idx, const double *R, int32_t k,
  * allocator must not be called -- so this entry point allocates nothing, not even
  * temporarily.  Its working space is a file-scope device array of 4,194,304 doubles
  * (32 MiB, held by every GPU that loads the library until exit): the permuted N x k
- * right-hand sides followed by (widest solve level) x 64 x k doubles of gather buffer.
+ * right-hand sides (the size limit below still counts the (widest solve level) x 64 x k
+ * doubles of gather buffer that an earlier form of the solve kept behind them).
  * The caller passes R and X (DEVICE float64 N x k row-major, may alias) as for
  * ss_solve.  The first call on a device looks up the array's device address with that
  * device current; make that first call before any stream capture.  The address is kept

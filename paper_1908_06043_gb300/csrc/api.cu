@@ -1646,7 +1646,7 @@ int solve_apply(ss_numeric *f, int j, const double *R, int k, double *X, int ref
     // a solve contracts the residual by 1e-10 where an FP32 one gives 1e-1 .. 1e-2, and the folded
     // sweeps pass a level in 5 - 10 us where the FP32 ones take 48.  Only many columns without the
     // tensor cores (4 ps of FP64 per entry of L and column) are left to FP32.  Measured, ms a solve,
-    // FP32 / FP64: N = 16,384, k = 304 6.4 / 9.2 (and 8 or 9 / 3 of them for two requested
+    // FP32 / FP64: N = 16,384, k = 304 6.3 / 9.2 (and 8 or 9 / 3 of them for two requested
     // refinements); k = 1, 8, 16, 48 3.4 / 0.85, 3.3 / 2.5, 3.4 / 4.2, 3.6 / 4.4 (7 / 2 of them for one
     // refinement at a contraction of 1.5e-2).
     const bool in_f64 = (refine > 0 || target > 0.0) && f->shift_prec[j] == SS_FP64 &&

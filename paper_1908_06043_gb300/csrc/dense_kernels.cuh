@@ -349,8 +349,8 @@ __device__ __forceinline__ double2 jac_rotation(double hpp, double hqq, double h
 // max_sweeps doubles a matrix (zeroed) for the per-sweep off-diagonal / total norms.  On return the
 // matrix is in H (copied back from the scratch buffer H2 when the last round left it there).
 // What bounds it: k - 1 rounds a sweep of barrier, load, rotation, update, store.  k = 112: 4.15 ms
-// with both triangles, two divisions and two square roots a rotation and 13 blocks, 2.6 ms now;
-// k = 100, four matrices: 25 ms one after the other (a single block below k = 97), 4.1 ms now.
+// with both triangles, two divisions and two square roots a rotation and 13 blocks, 2.2 ms now;
+// k = 100, four matrices: 25 ms one after the other (a single block below k = 97), 3.4 ms now.
 struct JacArgs {
     double *H, *H2, *V;          // matrix g at g k^2
     int k, nb;                   // blocks per matrix

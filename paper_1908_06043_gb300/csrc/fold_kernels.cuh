@@ -12,12 +12,12 @@
 // error of an FP64 solve is the factor's own in both forms.  The half solve x = P L^-T y needs
 // only L^-T: x1 = P^T L11^-T y1 - G^T x2.
 //
-// What bounds it.  FP64 runs at 2 multiply-adds a clock and SM here, half a one per SM quarter: one
-// warp instruction holds a quarter's pipe for 64 clocks, so an item of 16 x 7 multiply-adds on one
-// warp takes 7,200 clocks however idle the rest of the chip is.  An item is one warp's 32 rows x 16
-// panel columns (forward) or 128 rows x 4 panel columns (backward) times at most 8 right-hand sides;
-// a level with few of them halves its items (columns, rows) up to three times, until every quarter of
-// every SM has two (one: 2% slower, four: 3%).  Few right-hand sides are bound by the chain of levels:
+// What bounds it.  FP64 runs at 2 multiply-adds a clock and SM here, and a warp issues one FP64
+// instruction per 64 clocks at most: an item of 16 x 7 multiply-adds on one warp takes 7,200 clocks
+// however idle the rest of the chip is.  An item is one warp's 32 rows x 16 panel columns (forward) or
+// 128 rows x 4 panel columns (backward) times at most 8 right-hand sides;
+// a level with few of them halves its items (columns, rows) up to three times, to eight warps an
+// SM (four: 2% slower, sixteen: 3%).  Few right-hand sides are bound by the chain of levels:
 // some 850 clocks for b1 (x2) from the L2, the multiply-adds, 800 until the additions are performed,
 // 650 a poll of the barrier.  The entries of a warp's first item in the next level never change: they
 // are fetched while the other blocks arrive, from records read one and two levels before.  The
@@ -132,8 +132,7 @@ struct FoldArgs {
     long long limit;
 };
 
-// A level's items are halved `split` times over, until there is one for each of the `slots` warps
-// that have an SM quarter's FP64 pipe to themselves.
+// A level's items are halved `split` times over, until there is one for each of `slots` warps.
 __host__ __device__ __forceinline__ int fold_split(int64_t items, int64_t slots) {
     int s = 0;
     while (s < 3 && (items << (s + 1)) <= slots) ++s;
