@@ -83,10 +83,12 @@ int slice_dense(ss_ctx *ctx, const OzOperand &op, Scratch &buf, unsigned char **
     OZ_ALLOC(ctx, buf.get(sl, (size_t)nrt * nkc * sstc::kOzStageA));
     OZ_ALLOC(ctx, buf.get(em, (size_t)op.rows));
     SS_CUDA_TRY(ctx, cudaMemsetAsync(*em, 0, sizeof(int) * op.rows, ctx->stream));
-    const int64_t per_k = std::max<int64_t>(64, (int64_t)cdivu(op.kdim, std::max<unsigned>(1, 4 * ctx->sm_count / nrt)));
+    const int64_t per_k = std::max<int64_t>(16, (int64_t)cdivu(op.kdim, std::max<unsigned>(1, 4 * ctx->sm_count / nrt)));
     ss_launch(ctx, SS_K_GEMM_TC, sstc::k_oz_expmax, dim3(nrt, cdivu(op.kdim, per_k)), 128, 0, ctx->stream, op, per_k,
               *em);
-    ss_launch(ctx, SS_K_GEMM_TC, sstc::k_oz_slice, dim3(nrt, nkc), 128, 0, ctx->stream, op, (const int *)*em, *sl);
+    const bool few = (int64_t)nrt * nkc <= 4ll * ctx->sm_count;
+    ss_launch(ctx, SS_K_GEMM_TC, few ? sstc::k_oz_slice<512> : sstc::k_oz_slice<128>, dim3(nrt, nkc), few ? 512 : 128, 0,
+              ctx->stream, op, (const int *)*em, *sl);
     return SS_OK;
 }
 

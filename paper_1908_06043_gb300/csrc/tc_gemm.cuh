@@ -116,6 +116,7 @@ __global__ void __launch_bounds__(128) k_oz_expmax(OzOperand op, int64_t per_k, 
     if (row >= op.rows) return;
     const int64_t t0 = (int64_t)blockIdx.y * per_k, t1 = min(op.kdim, t0 + per_k);
     int m = 0;
+#pragma unroll 8
     for (int64_t t = t0; t < t1; ++t) m = max(m, biased_exp(op.at(row, t)));
     if (m > 0) atomicMax(&em[row], m);
 }
@@ -131,18 +132,22 @@ __global__ void __launch_bounds__(256) k_oz_csr_expmax(int64_t n, const int64_t 
     if ((threadIdx.x & 31) == 0) em[row] = m;
 }
 
-// Block (rt, kc), thread = row of the tile.  Zero rows / columns pad the operand.
-__global__ void __launch_bounds__(128) k_oz_slice(OzOperand op, const int *__restrict__ em,
-                                                  unsigned char *__restrict__ sl) {
+// Block (rt, kc), thread = row of the tile and every NT / 128-th chunk of 8 columns.  Zero
+// rows / columns pad the operand.  With few blocks a load's latency is the limit: 512 threads (N = 5,280,
+// k = 112: dense products 16.4 -> 13.7 ms a window); with many, 128 threads write the wider runs
+// (N = 16,384, k = 304: both products of a step 0.63 ms, 0.66 with 512).
+template <int NT>
+__global__ void __launch_bounds__(NT) k_oz_slice(OzOperand op, const int *__restrict__ em,
+                                                 unsigned char *__restrict__ sl) {
     const int rt = blockIdx.x, kc = blockIdx.y;
     const int nrt = gridDim.x;
-    const int rho = threadIdx.x;
+    const int rho = threadIdx.x % 128;
     const int64_t row = (int64_t)rt * 128 + rho;
     const int64_t t0 = (int64_t)kc * kOzK;
     const bool live = row < op.rows;
     const int E = (live ? em[row] : 0) - 1022;
     unsigned char *blk = sl + ((uint64_t)kc * nrt + rt) * kOzStageA;
-    for (int c = 0; c < kOzK / 8; ++c) {
+    for (int c = threadIdx.x / 128; c < kOzK / 8; c += NT / 128) {
         __align__(16) __half h[kOzSlices][8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
