@@ -226,6 +226,12 @@ ss_status ss_selftest_tc(ss_ctx *ctx, uint64_t seed, double *max_abs_err);
  * SS_ERR_TIMEOUT. */
 ss_status ss_selftest_barrier(ss_ctx *ctx, int32_t extra_arrivals, int64_t limit);
 
+/* Self-test of what the calls do when device memory runs out (no paper counterpart): from now on
+ * every device allocation of this context above max_bytes bytes fails on the host as an
+ * out-of-memory one would; max_bytes < 0 (the state of a new context): no limit.  Errors:
+ * SS_ERR_ARG. */
+ss_status ss_selftest_alloc_limit(ss_ctx *ctx, int64_t max_bytes);
+
 /* ---- ss_analyze (Section 2.1: the sparse LDL^T of A - sigma B is the major cost;
  * Section 5: the paper's solver orders with nested dissection) --------------------
  * Host CSR pattern in, symbolic analysis out: nested-dissection ordering, supernodes

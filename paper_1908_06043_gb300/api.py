@@ -87,6 +87,10 @@ class Context:
         """Run the bounded grid-barrier self-test (raises SisliceError on a timeout)."""
         self.check(self.lib.ss_selftest_barrier(self.h, extra_arrivals, limit), "ss_selftest_barrier")
 
+    def selftest_alloc_limit(self, max_bytes: int = -1):
+        """Let every later device allocation above max_bytes fail as out of memory (-1: none)."""
+        self.check(self.lib.ss_selftest_alloc_limit(self.h, int(max_bytes)), "ss_selftest_alloc_limit")
+
     def set_schur_mode(self, mode: str, min_flops: float = 2e7):
         """"tensor": FP64 Schur updates of factor steps with >= min_flops flops on the
         tensor cores (sliced FP16 operands, FP64-accurate); "simt": all on CUDA cores."""

@@ -124,7 +124,12 @@ static void pool_trim(ss_ctx *ctx) {
     cudaMemPoolTrimTo(ctx->pool, 0);
 }
 
+static bool alloc_refused(const ss_ctx *ctx, size_t bytes) {
+    return ctx->alloc_limit >= 0 && bytes > (size_t)ctx->alloc_limit;
+}
+
 cudaError_t ss_malloc_async(ss_ctx *ctx, void **p, size_t bytes, cudaStream_t st) {
+    if (alloc_refused(ctx, bytes)) return cudaErrorMemoryAllocation;
     if (!ctx->pool) return cudaMallocAsync(p, bytes, st);
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
     if (e == cudaErrorMemoryAllocation) {
@@ -135,6 +140,7 @@ cudaError_t ss_malloc_async(ss_ctx *ctx, void **p, size_t bytes, cudaStream_t st
 }
 
 cudaError_t ss_malloc(ss_ctx *ctx, void **p, size_t bytes) {
+    if (alloc_refused(ctx, bytes)) return cudaErrorMemoryAllocation;
     cudaError_t e = cudaMalloc(p, bytes);
     if (e == cudaErrorMemoryAllocation && ctx->pool) {
         pool_trim(ctx);
@@ -154,6 +160,12 @@ extern "C" const char *ss_last_error(const ss_ctx *ctx) { return ctx ? ctx->err.
 __global__ void k_barrier_selftest(GridBar *bar, unsigned int expected, long long limit) {
     unsigned int at = 0;
     grid_barrier(bar, expected, limit, at);
+}
+
+extern "C" ss_status ss_selftest_alloc_limit(ss_ctx *ctx, int64_t max_bytes) {
+    if (!ctx) return SS_ERR_ARG;
+    ctx->alloc_limit = max_bytes;
+    return SS_OK;
 }
 
 extern "C" ss_status ss_selftest_barrier(ss_ctx *ctx, int32_t extra_arrivals, int64_t limit) {

@@ -28,6 +28,7 @@ struct ss_ctx {
     int64_t plan_gen = 0;                     // bumped when a setting baked into captured graphs changes
     double tc_min_flops = 2.0e7;              // a factor step's Schur flops below which it stays on CUDA cores
     cudaMemPool_t pool = nullptr;             // this context's scratch (ss_malloc_async)
+    int64_t alloc_limit = -1;                 // allocations above this many bytes fail (self-test; -1: none)
     GridBar *d_bar = nullptr;                 // grid barrier state of the sweep kernel
     int sweep_blocks_per_sm = 0;              // resident FP32 sweep-kernel blocks per SM
     int sweep_fuse_max = 0;                   // FP32 sweep: fuse levels with at most this many items

@@ -135,6 +135,28 @@ int dense_mm(ss_ctx *ctx, const OzOperand &A, const OzOperand &B, int mode, doub
     return run_mm(ctx, g, dim3(nct, nrtA, nsplit), SS_K_GEMM_TC);
 }
 
+// the lists of one analysis are freed apart: a failure to build one leaves the other, and the factors
+// that use it, as they were
+void free_plan(ss_symbolic *s) {
+    OzPlan *pl = s->oz_plan;
+    if (!pl) return;
+    void *ptrs[] = {pl->d_tile_ptr, pl->d_pair_piece, pl->d_ent_ptr, pl->d_ent_e, pl->d_ent_off};
+    for (void *p : ptrs)
+        if (p) cudaFree(p);
+    delete pl;
+    s->oz_plan = nullptr;
+}
+
+void free_samples(ss_symbolic *s) {
+    OzSamples *sp = s->oz_samples;
+    if (!sp) return;
+    void *ptrs[] = {sp->d_rt, sp->d_ct, sp->d_ptr, sp->d_e, sp->d_t, sp->d_off};
+    for (void *p : ptrs)
+        if (p) cudaFree(p);
+    delete sp;
+    s->oz_samples = nullptr;
+}
+
 // (tile, piece) pairs of the pattern -- for each 128-row tile the 32-column pieces that hold
 // entries -- and the entries of every pair: CSR position (from the tile's first) and place in the
 // pair's digit block
@@ -201,7 +223,7 @@ int plan_build(ss_symbolic *s) {
     if (e == cudaSuccess) e = up(&pl->d_ent_off, ent_off);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        oz_free_symbolic(s);
+        free_plan(s);
         return ctx->set_error(SS_ERR_OOM, "tensor-core product plan: device allocation failed");
     }
     return SS_OK;
@@ -274,7 +296,7 @@ int samples_build(ss_symbolic *s) {
     if (er == cudaSuccess) er = up(&pl->d_off, off);
     if (er != cudaSuccess) {
         cudaGetLastError();
-        oz_free_symbolic(s);
+        free_samples(s);
         return ctx->set_error(SS_ERR_OOM, "sampled product plan: device allocation failed");
     }
     return SS_OK;
@@ -284,8 +306,6 @@ int samples_build(ss_symbolic *s) {
 // when buf is null)
 int vals_make(ss_symbolic *s, const double *vals, OzVals *v, Scratch *buf) {
     ss_ctx *ctx = s->ctx;
-    int rc;
-    if (!s->oz_plan && (rc = plan_build(s)) != SS_OK) return rc;
     v->vals = vals;
     if (buf) {
         OZ_ALLOC(ctx, buf->get(&v->em, (size_t)s->n));
@@ -319,6 +339,7 @@ int spmm_core(ss_symbolic *s, int npass, OzVals *const *v, const double *const *
               const double *X, int64_t ldx, int k, double *Y, int64_t ldy) {
     ss_ctx *ctx = s->ctx;
     int rc;
+    if (!s->oz_plan && (rc = plan_build(s)) != SS_OK) return rc;
     Scratch buf(ctx);
     unsigned char *sx;
     int *ex;
@@ -459,18 +480,6 @@ int oz_sddmm(ss_symbolic *s, const double *X, const double *lambda, int ne, doub
 }
 
 void oz_free_symbolic(ss_symbolic *s) {
-    if (OzSamples *sp = s->oz_samples) {
-        void *q[] = {sp->d_rt, sp->d_ct, sp->d_ptr, sp->d_e, sp->d_t, sp->d_off};
-        for (void *p : q)
-            if (p) cudaFree(p);
-        delete sp;
-        s->oz_samples = nullptr;
-    }
-    OzPlan *pl = s->oz_plan;
-    if (!pl) return;
-    void *ptrs[] = {pl->d_tile_ptr, pl->d_pair_piece, pl->d_ent_ptr, pl->d_ent_e, pl->d_ent_off};
-    for (void *p : ptrs)
-        if (p) cudaFree(p);
-    delete pl;
-    s->oz_plan = nullptr;
+    free_samples(s);
+    free_plan(s);
 }

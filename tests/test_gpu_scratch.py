@@ -1,0 +1,36 @@
+"""What the calls do when scratch memory does not fit, with device allocations made to fail on the host."""
+import numpy as np
+import pytest
+import torch
+
+from tests.gpu_util import setup
+from workloads.pencils import gaussian_pencil, normal_block
+
+pytestmark = pytest.mark.gpu
+
+
+def test_gradient_fallback_leaves_the_factors_products(gpu_lib):
+    # the lists of the sampled product do not fit: the gradient runs on the CUDA cores, and a factor that
+    # used the tensor-core products before goes on using them
+    p = gaussian_pencil((8, 8, 9), seed=2)
+    ctx, sym, a, b = setup(gpu_lib, p)
+    f = sym.factor(a, b, [-1.1], "fp64")
+    V0 = torch.tensor(normal_block(p.n, 48, 3), device="cuda")
+    run = lambda: f.slice_solve(0, -1.3, -0.9, V0, max_iter=3, check_every=3, allow_noconv=True)
+    before = run()
+    ctx.profile(["spmm_tc"])
+    X = torch.tensor(normal_block(p.n, 64, 5), device="cuda")
+    lam = torch.linspace(-3.0, -1.0, 64, dtype=torch.float64, device="cuda")
+    ctx.selftest_alloc_limit(0)
+    ga, gb = sym.band_energy_grad(X, lam)
+    ctx.selftest_alloc_limit()
+    after = run()
+    assert ctx.profile_query("spmm_tc")[0] > 0
+    rows = torch.repeat_interleave(torch.arange(p.n, device="cuda"), torch.tensor(np.diff(p.rowptr), device="cuda"))
+    cols = torch.tensor(p.colind, device="cuda").long()
+    # 64 rounded products and sums of entries below 5
+    assert torch.allclose(ga, (X[rows] * X[cols]).sum(1), rtol=0, atol=64 * 25 * 2e-16 * 64)
+    assert torch.allclose(gb, -(X[rows] * lam * X[cols]).sum(1), rtol=0, atol=3 * 64 * 25 * 2e-16 * 64)
+    # three iterations of the same start block: the same subspace up to rounding
+    sel = before.resid < 1e-6
+    assert sel.any() and np.abs(after.theta[sel] - before.theta[sel]).max() <= 1e-10
