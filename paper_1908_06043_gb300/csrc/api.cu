@@ -1752,7 +1752,11 @@ extern "C" ss_status ss_band_energy_grad(ss_symbolic *s, const double *X, const 
     const size_t smem = sizeof(double) * 2 * (size_t)n_e;
     if (smem > 220 * 1024) return ctx->set_error(SS_ERR_ARG, "ss_band_energy_grad: n_e too large (max 14080)");
     SS_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-    if (oz_sddmm_ok(s, n_e)) {
+    // the tensor-core form allocates and reads its status back, which a stream that records a graph
+    // cannot do: the one launch below then
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    SS_CUDA_TRY(ctx, cudaStreamIsCapturing(ctx->stream, &capture));
+    if (capture == cudaStreamCaptureStatusNone && oz_sddmm_ok(s, n_e)) {
         const int rc = oz_sddmm(s, X, lambda, n_e, grad_a, grad_b);
         if (rc != SS_ERR_OOM) return rc;
         ctx->err.clear();                      // the digits of X do not fit: CUDA cores
