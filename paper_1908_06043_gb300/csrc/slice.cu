@@ -684,7 +684,8 @@ int lanczos_impl(ss_symbolic *s, ss_numeric *fb, const double *a_vals, const dou
     for (int c = 0; c < nv; ++c) {
         int m = steps;
         for (int j = 0; j + 1 < steps; ++j)
-            if (hb[(size_t)j * nv + c] <= 1e-13 * std::max(1.0, std::fabs(ha[(size_t)j * nv + c]))) { m = j + 1; break; }
+            // (not a number: the square of a norm of rounding errors came out negative)
+            if (!(hb[(size_t)j * nv + c] > 1e-13 * std::max(1.0, std::fabs(ha[(size_t)j * nv + c])))) { m = j + 1; break; }
         m_run[c] = m;
     }
     for (int c0 = 0; c0 < nv;) {
