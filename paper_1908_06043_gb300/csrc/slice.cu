@@ -116,7 +116,8 @@ __global__ void k_add_shift_diag(double *G, int k, double rel) {
 
 // Symmetric eigenproblems of `count` matrices H (k x k each, one after another, destroyed): ascending
 // evals (device) and Q, by parallel-ordered Jacobi, stopped once the off-diagonal Frobenius norm is
-// below tol times the whole norm.
+// below tol times the whole norm.  One cooperative launch for every order: against one block of 1,024
+// threads, us a problem, k = 4 88 -> 62, 16 390 -> 324, 48 2,740 -> 1,430, 96 16,200 -> 2,970.
 int sym_eig(ss_ctx *ctx, double *H, int k, double *evals, double *Q, DevBuf &buf, double tol = 1e-14, int count = 1) {
     cudaStream_t st = ctx->stream;
     double *V;
@@ -676,11 +677,8 @@ int lanczos_impl(ss_symbolic *s, ss_numeric *fb, const double *a_vals, const dou
     SS_CUDA_TRY(ctx, cudaStreamSynchronize(st));
     std::memset(theta, 0, sizeof(double) * steps * nv);
     std::memset(zeta2, 0, sizeof(double) * steps * nv);
-    // the runs' tridiagonal eigenproblems, neighbours of the same length together
-    double *T, *Q, *ev;
-    TRY_ALLOC(ctx, buf.get(&T, (size_t)steps * steps * nv));
-    TRY_ALLOC(ctx, buf.get(&Q, (size_t)steps * steps * nv));
-    TRY_ALLOC(ctx, buf.get(&ev, (size_t)steps * nv));
+    // the runs' tridiagonal eigenproblems, neighbours of the same length together: up to 16, fewer where
+    // their four matrices each would pass 256 MB
     for (int c = 0; c < nv; ++c) {
         int m = steps;
         for (int j = 0; j + 1 < steps; ++j)
@@ -690,12 +688,18 @@ int lanczos_impl(ss_symbolic *s, ss_numeric *fb, const double *a_vals, const dou
     }
     for (int c0 = 0; c0 < nv;) {
         const int m = m_run[c0];
+        const int most = (int)std::min<int64_t>(16, std::max<int64_t>(1, (256ll << 20) / (32ll * m * m)));
         int cnt = 1;
-        while (c0 + cnt < nv && cnt < 16 && m_run[c0 + cnt] == m) ++cnt;
+        while (c0 + cnt < nv && cnt < most && m_run[c0 + cnt] == m) ++cnt;
+        DevBuf group(ctx);
+        double *T, *Q, *ev;
+        TRY_ALLOC(ctx, group.get(&T, (size_t)m * m * cnt));
+        TRY_ALLOC(ctx, group.get(&Q, (size_t)m * m * cnt));
+        TRY_ALLOC(ctx, group.get(&ev, (size_t)m * cnt));
         for (int q = 0; q < cnt; ++q)
             ss_launch(ctx, SS_K_LANCZOS, ssd::k_lz_tridiag, cdiv((int64_t)m * m, 256), 256, 0, st, alpha, beta, nv, c0 + q,
                       m, T + (int64_t)q * m * m);
-        if ((rc = sym_eig(ctx, T, m, ev, Q, buf, 1e-14, cnt)) != SS_OK) return rc;
+        if ((rc = sym_eig(ctx, T, m, ev, Q, group, 1e-14, cnt)) != SS_OK) return rc;
         std::vector<double> he((size_t)m * cnt), hq((size_t)m * cnt);
         SS_CUDA_TRY(ctx, cudaMemcpyAsync(he.data(), ev, sizeof(double) * m * cnt, cudaMemcpyDeviceToHost, st));
         for (int q = 0; q < cnt; ++q)

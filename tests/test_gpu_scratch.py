@@ -4,7 +4,7 @@ import pytest
 import torch
 
 from tests.gpu_util import setup
-from workloads.pencils import gaussian_pencil, normal_block
+from workloads.pencils import gaussian_pencil, laplacian_1d, normal_block
 
 pytestmark = pytest.mark.gpu
 
@@ -34,3 +34,19 @@ def test_gradient_fallback_leaves_the_factors_products(gpu_lib):
     # three iterations of the same start block: the same subspace up to rounding
     sel = before.resid < 1e-6
     assert sel.any() and np.abs(after.theta[sel] - before.theta[sel]).max() <= 1e-10
+
+
+def test_lanczos_runs_hold_the_matrices_of_one_group(gpu_lib):
+    # 64 runs of up to 256 steps on 64 rows: the vectors take 8.4 MB an array, the tridiagonal matrices of
+    # all runs together would take 33.5 MB, those of 16 runs 8.4 MB
+    p = laplacian_1d(64, mass=True)
+    ctx, sym, a, b = setup(gpu_lib, p)
+    x0 = normal_block(p.n, 64, 4)
+    ctx.selftest_alloc_limit(12 << 20)
+    runs = sym.dos_lanczos(a, b, 256, torch.tensor(x0, device="cuda"))
+    A, B = p.dense("a"), p.dense("b")
+    for c, (th, z2) in enumerate(runs):
+        x = x0[:, c]
+        quotient = (x @ A @ x) / (x @ B @ x)
+        assert abs(z2.sum() - 1.0) <= 1e-10
+        assert abs(z2 @ th - quotient) <= 1e-10 * np.abs(th).max()
