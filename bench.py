@@ -52,7 +52,6 @@ def measured_peaks():
         return None
 
 
-TENSOR_CLASSES = {"schur_tc", "gemm_tc", "spmm_tc"}
 FLOP_CLASSES = {"schur", "panel", "fwd_update", "bwd_gather", "spmm", "gram", "gemm", "solve",
                 "schur_f32", "panel_f32", "fwd_update_f32", "bwd_gather_f32", "solve_f32", "schur_tc", "gemm_tc", "spmm_tc"}
 
@@ -593,7 +592,7 @@ def main():
     # against the FMA peak measured on this GPU at the start of the run
     per_launch = dom_t / max(dom_n, 1)
     fp64_equiv = None
-    if dom in TENSOR_CLASSES and dom_t > 0 and dom_tensor > 0:
+    if dom_t > 0 and dom_tensor > 0:
         # FP64 emulated on the FP16 tensor cores: the roofline is the tensor pipe's, with the
         # MMA work the kernels issued (the digit-product algorithm); the FP64-equivalent rate
         # of the same launches is reported beside it

@@ -1255,11 +1255,17 @@ static int fold_sweeps(ss_numeric *f, int j, double *b, int k, bool full) {
         flops += (full ? 4.0 : 2.0) * sl.offdiag * k;
     }
     const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(ctx->sm_count, items));
+    const bool tc = fold_uses_tc(s, k);
+    double tensor_flops = 0.0;
+    if (tc)
+        for (const SolveLevel &sl : s->solve_levels) {
+            const int cw = sstc::ft_width(sl.row_tiles, k, nb);
+            tensor_flops += (full ? 2.0 : 1.0) * sstc::kFtItemFlops * sl.row_tiles * ((k + cw - 1) / cw);
+        }
     SS_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_bar, 0, sizeof(GridBar), st));
     FoldArgs a = fold_args(f, j, k, full);
     a.bar = ctx->d_bar;
     a.limit = 20000000;        // polls of about 64 ns: ~1 s per barrier
-    const bool tc = fold_uses_tc(s, k);
     void *args[] = {(void *)&a, (void *)&b};
     void *kern = tc ? (void *)sstc::k_fold_tc : (void *)fold_sweeps_kernel(nc);
     g_ss_launches.fetch_add(1, std::memory_order_relaxed);
@@ -1271,6 +1277,7 @@ static int fold_sweeps(ss_numeric *f, int j, double *b, int k, bool full) {
                                                  tc ? sstc::kFtSmem : kFoldSmem, st));
     if (prof) ss_prof_end(ctx, SS_K_SOLVE, slot);
     ctx->add_flops(SS_K_SOLVE, flops);
+    ctx->add_tensor_flops(SS_K_SOLVE, tensor_flops);
     int herr = 0;
     SS_CUDA_TRY(ctx, cudaMemcpyAsync(&herr, &ctx->d_bar->err, sizeof(int), cudaMemcpyDeviceToHost, st));
     SS_CUDA_TRY(ctx, cudaStreamSynchronize(st));

@@ -48,6 +48,14 @@ constexpr size_t kFtSmem = 1024 + (size_t)kFtSlices * (kFtSliceA + kFtSliceB);
 constexpr uint32_t kFtTmemCols = 512;               // 7 accumulators x 64 columns
 constexpr long long kFtWaitLimit = 1ll << 24;
 
+// Right-hand sides of an item of a level of `tiles` row tiles on nb blocks: 64 where items of 128 would
+// leave half of the blocks without one (a thread then cuts 8 terms instead of 16), else 128
+__host__ __device__ __forceinline__ int ft_width(int tiles, int k, int nb) {
+    return 2 * tiles * ((k + kFtCols - 1) / kFtCols) <= nb ? kFtCols / 2 : kFtCols;
+}
+// multiply-adds' flops that the tensor cores do for an item: 28 digit products of 128 x 64 x 64
+constexpr double kFtItemFlops = 28.0 * 2.0 * kFtCols * kFtRows * NB;
+
 // The MMAs of one item: accumulator d (columns 64 d ..) = sum_{p + q = d} A_p B_q^T.  Per K step of 16
 // the right-hand sides advance 32 bytes inside their 128-byte rows; G does the same when K is its
 // column (forward), or 16 rows = 2,048 bytes when K is its row (backward, MN-major: the next 64 of
@@ -229,11 +237,7 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
             if (live && n < lim && T[e] != 0) atomicAdd(&b[row * k + c0 + c], __longlong_as_double(T[e]));
         }
     };
-    // Right-hand sides of an item of a level: 64 where items of 128 would leave half of the blocks
-    // without one (a thread then cuts 8 terms instead of 16), else 128
-    auto width = [&](const ssk::FoldLevel &lv) {
-        return 2 * lv.tiles_64 * ((k + kFtCols - 1) / kFtCols) <= nb ? kFtCols / 2 : kFtCols;
-    };
+    auto width = [&](const ssk::FoldLevel &lv) { return ft_width(lv.tiles_64, k, nb); };
     // this block's items of a level: [qa, qb), tile fastest
     auto range = [&](const ssk::FoldLevel &lv, int &qa, int &qb) {
         const int cw = width(lv), items = lv.tiles_64 * ((k + cw - 1) / cw), per = (items + nb - 1) / nb;
