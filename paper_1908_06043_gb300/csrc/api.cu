@@ -888,7 +888,7 @@ int ss_factor_create(ss_symbolic *sym, const double *a_vals, const double *b_val
         if (!f->inertia_only) e = ss_malloc(ctx, &f->arena[j], esz * std::max<int64_t>(1, sym->l_total));
         if (e == cudaSuccess) e = ss_malloc(ctx, (void **)&f->linv[j], sizeof(double) * NB * NB * npan);
         if (e == cudaSuccess) e = ss_malloc(ctx, (void **)&f->dblk[j], sizeof(double) * 2 * NB * npan);
-        if (e == cudaSuccess) e = ss_malloc(ctx, (void **)&f->piv[j], sizeof(int32_t) * NB * npan);
+        if (e == cudaSuccess) e = ss_malloc(ctx, (void **)&f->piv[j], sizeof(int32_t) * (NB * npan + sym->n));
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -1178,6 +1178,7 @@ static FoldArgs fold_args(const ss_numeric *f, int j, int k, bool full) {
     a.dblk = f->dblk[j];
     a.piv = f->piv[j];
     a.arena = (const double *)f->arena[j];
+    a.sc = f->piv[j] + (int64_t)NB * s->panels.size();
     return a;
 }
 
@@ -1187,7 +1188,7 @@ static int fold_nc(int k) {
     return (k + nch - 1) / nch;
 }
 
-// G = L21 L11^-1 P in the FP64 L storage of shift j (once, when its factorisation is done)
+// G = L21 L11^-1 P in the FP64 L storage of shift j and its scales (once, when its factorisation is done)
 static int fold_shift(ss_numeric *f, int j) {
     ss_symbolic *s = f->sym;
     ss_ctx *ctx = s->ctx;
@@ -1196,6 +1197,9 @@ static int fold_shift(ss_numeric *f, int j) {
     ss_launch(ctx, SS_K_PANEL, k_fold_panels, dim3((unsigned)s->panels.size(), (unsigned)((s->max_rows_below + TR - 1) / TR)),
               256, kFoldPanelsSmem, ctx->stream, (const PanelDesc *)s->d_panels, (const double *)f->linv[j],
               (const int32_t *)f->piv[j], (double *)f->arena[j]);
+    ss_launch(ctx, SS_K_PANEL, k_fold_scales, (unsigned)((s->n + 255) / 256), 256, 0, ctx->stream, s->n,
+              (const int32_t *)s->d_perm, (const int64_t *)s->d_rowptr, (const int32_t *)s->d_colind, f->a_vals,
+              f->b_vals, f->sigma[j], f->piv[j] + (int64_t)NB * s->panels.size());
     SS_CUDA_TRY(ctx, cudaGetLastError());
     return SS_OK;
 }

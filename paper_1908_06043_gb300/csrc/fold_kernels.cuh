@@ -128,9 +128,27 @@ struct FoldArgs {
     const double *dblk;
     const int32_t *piv;
     const double *arena;
+    const int32_t *sc;      // scale exponent of every (permuted) column (fold_tc.cuh)
     GridBar *bar;
     long long limit;
 };
+
+// sc[i] = exponent of about sqrt(|a_ii| + |sigma b_ii|), i in permuted order; 0 where that is zero or
+// not finite.  Scaling row and column i of the pencil by 2^s adds s.  Thread = row.
+__global__ void k_fold_scales(int64_t n, const int32_t *__restrict__ perm, const int64_t *__restrict__ rowptr,
+                              const int32_t *__restrict__ colind, const double *__restrict__ a,
+                              const double *__restrict__ b, double sigma, int32_t *__restrict__ sc) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int32_t r = perm[i];
+    int64_t lo = rowptr[r], hi = rowptr[r + 1] - 1;        // the diagonal is stored, columns ascend
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (colind[mid] < r) lo = mid + 1; else hi = mid;
+    }
+    const double d = fabs(a[lo]) + fabs(sigma * b[lo]);
+    sc[i] = d > 0.0 && isfinite(d) ? (ilogb(d) + 1) >> 1 : 0;
+}
 
 // A level's items are halved `split` times over, until there is one for each of `slots` warps.
 __host__ __device__ __forceinline__ int fold_split(int64_t items, int64_t slots) {

@@ -9,9 +9,14 @@
 //   forward   D(c, i) = sum_t b1(t, c) G(i, t):  A = b1^T (128 x 64, K = t), B = G (64 rows, K-major)
 //   backward  D(c, t) = sum_i x2(i, c) G(i, t):  A = x2^T (128 x 64, K = i), B = the same tile of G,
 //             read along its other axis (the MN-major operand form)
-// G's digits are scaled by row; in the backward product the row index is summed over, so the row
-// scales 2^e_i are moved into x2 first (an exponent addition).  Each right-hand-side column of an
-// item has its own scale over the item's 64 terms.
+// G's digits are scaled by row, after column t has been multiplied by 2^s_t (a.sc: about the square root
+// of the diagonal of A - sigma B's terms).  G = F21 F11^-1 takes the factor S2 G S1^-1 when the pencil is
+// scaled to S A S, S B S, so with s_t the digits do not change with the scale of the basis: badly scaled
+// rows lose none of them.  Forward, b1(t) is multiplied by 2^-s_t, backward the result; in the backward
+// product the row index is summed over, so the row scales 2^e_i are moved into x2 first.  All of these are
+// additions to exponents.  Each right-hand-side column of an item has its own scale over the item's 64
+// terms.  One front of 700 rows scaled by 2^-20 .. 2^20, 300 right-hand sides, relative error of a solve
+// against 64 bits: 2.6e-6 without s_t, 6.0e-16 with it (CUDA cores 6.3e-16; unscaled 6.0e-16).
 //
 // Cutting and summing digits takes integer instructions only (digits8.cuh).  A non-finite operand
 // makes its whole column (row) of the product NaN.
@@ -76,8 +81,9 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
     __shared__ int s_ok;
     __shared__ int s_emax[8][kFtCols], s_gmax[8][kFtRows];
     __shared__ int s_ec[kFtCols];                   // em of every right-hand-side column
-    __shared__ int s_er[kFtRows];                   // E of every row of G (|G row| < 2^E), kFtZero, kFtNan
+    __shared__ __align__(16) int s_er[kFtRows];     // E of every row of G (|G row| < 2^E), kFtZero, kFtNan
     __shared__ int s_row[kFtRows];                  // global row of every row of G
+    __shared__ __align__(16) int s_ce[NB];          // minus the scale exponent of every column of G
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int k = a.k, nb = gridDim.x;
     if (warp == 0) {
@@ -100,11 +106,13 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
     ssk::FoldTile tl{};
     double g[8];                                    // G(row gi, columns 8 gt ..)
     int grow = 0;                                   // its global row
+    int gce = 0;                                    // lane l: scale exponent of column 8 gt + l mod 8
     const int gi = tid & 63, gt = tid >> 6;
     auto fetch = [&](const ssk::FoldTile &t) {
         tl = t;
         const double *F = a.arena + t.off + (int64_t)(8 * gt) * t.m + gi;
         if (gt == 0 && gi < t.nr) grow = a.idx[t.idx + gi];
+        gce = 8 * gt + (lane & 7) < t.w ? __ldg(a.sc + t.g0 + 8 * gt + (lane & 7)) : 0;
 #pragma unroll
         for (int u = 0; u < 8; ++u) g[u] = (gi < t.nr && 8 * gt + u < t.w) ? __ldg(F + (int64_t)u * t.m) : 0.0;
     };
@@ -113,11 +121,12 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
         int ex[8], em = kFtZero;
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            ex[u] = ft_exp(g[u], 0);
+            ex[u] = ft_exp(g[u], __shfl_sync(0xffffffffu, gce, u));
             em = max(em, ex[u]);
         }
         s_gmax[gt][gi] = em;
         if (gt == 0) s_row[gi] = grow;
+        if (gi < 8) s_ce[8 * gt + gi] = -gce;
         __syncthreads();
 #pragma unroll
         for (int o = 0; o < 8; ++o) em = max(em, s_gmax[o][gi]);
@@ -127,8 +136,8 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
         for (int u = 0; u < 8; ++u) z[u] = ft_biased(g[u], ex[u], em);
         ft_store8(z, sb + core_offset(gi, 8 * gt), kFtSliceB);
     };
-    // Digits of the item's right-hand sides [c0, c1) into sa: terms b1(t) (forward) or
-    // x2(row i) 2^e_i (backward); needs s_row, s_er of the item.  A thread cuts V terms of a column:
+    // Digits of the item's right-hand sides [c0, c1) into sa: terms b1(t) 2^-s_t (forward) or
+    // x2(row i) 2^e_i (backward); needs s_row, s_er, s_ce of the item.  A thread cuts V terms of a column:
     // 8 where at most 64 right-hand sides exist, else 16.  Rows of the operand without a
     // right-hand side stay as they are: nothing reads those products.
     auto cut_rhs_v = [&](auto vc, int c0, int c1, bool backward, const ssk::FoldTile &t) {
@@ -145,10 +154,13 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
                 const int64_t row = backward ? s_row[n] : t.g0 + n;
                 v[u] = in ? __ldcg(&b[row * k + c0 + c]) : 0.0;
             }
+            const int4 *sh = reinterpret_cast<const int4 *>((backward ? s_er : s_ce) + V * tg);
 #pragma unroll
-            for (int u = 0; u < V; ++u) {
-                ex[u] = ft_exp(v[u], backward ? s_er[V * tg + u] : 0);
-                em = max(em, ex[u]);
+            for (int u = 0; u < V; u += 4) {
+                const int4 h = sh[u / 4];
+                ex[u] = ft_exp(v[u], h.x), ex[u + 1] = ft_exp(v[u + 1], h.y);
+                ex[u + 2] = ft_exp(v[u + 2], h.z), ex[u + 3] = ft_exp(v[u + 3], h.w);
+                em = max(max(em, max(ex[u], ex[u + 1])), max(ex[u + 2], ex[u + 3]));
             }
             s_emax[tg][c] = em;
         }
@@ -199,17 +211,14 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
         const bool live = c0 + c < c1;
         const uint32_t lane_base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)n0;
         long long T[16];
-        bool far = false;
-        if (!backward) {
-#pragma unroll
-            for (int n = 0; n < 16; ++n) {
-                const int er = s_er[n0 + n];
-                far |= er != kFtZero && (ec + er < -950 || ec + er > 900);
-            }
-        } else {
-            far = ec < -950 || ec > 900;
-        }
-        far &= live && s_ec[c] > kFtZero / 2;        // a zero column: its products are zero
+        // scales of the warp's rows (forward) or columns (backward) of G; every lane needs the ends of their
+        // range only
+        const int *es = (backward ? s_ce : s_er) + n0;
+        const int el = es[lane & 15];
+        const int emax = __reduce_max_sync(0xffffffffu, el == kFtZero ? -(1 << 19) : el);
+        const int emin = __reduce_min_sync(0xffffffffu, el == kFtZero ? 1 << 19 : el);
+        // a zero column: its products are zero
+        const bool far = live && s_ec[c] > kFtZero / 2 && (ec + emin < -950 || ec + emax > 900);
         ft_sum(lane_base, T);
         tc_fence_before();
 #pragma unroll
@@ -217,19 +226,25 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
         if (__any_sync(0xffffffffu, far)) {
 #pragma unroll 1
             for (int e = 0; e < 16; ++e) {
-                const int n = n0 + e, er = backward ? 0 : s_er[n];
+                const int n = n0 + e, ee = es[e];
                 long long Te = T[0];
 #pragma unroll
                 for (int u = 1; u < 16; ++u) Te = u == e ? T[u] : Te;
-                const double v = (ec >= kFtNan - 8192 || er == kFtNan) ? __longlong_as_double(0x7ff8000000000000ll)
-                                                                       : (Te == 0 ? 0.0 : ldexp((double)Te, ec + er));
+                const double v = (ec >= kFtNan - 8192 || ee == kFtNan) ? __longlong_as_double(0x7ff8000000000000ll)
+                                                                       : (Te == 0 ? 0.0 : ldexp((double)Te, ec + ee));
                 const int64_t row = backward ? t.g0 + n : s_row[n];
                 if (live && n < lim && v != 0.0) atomicAdd(&b[row * k + c0 + c], v);
             }
             return;
         }
 #pragma unroll
-        for (int e = 0; e < 16; ++e) T[e] = (long long)ft_pack(T[e], ec + (backward ? 0 : s_er[n0 + e]));
+        for (int q = 0; q < 4; ++q) {
+            const int4 v = reinterpret_cast<const int4 *>(es)[q];
+            T[4 * q] = (long long)ft_pack(T[4 * q], ec + v.x);
+            T[4 * q + 1] = (long long)ft_pack(T[4 * q + 1], ec + v.y);
+            T[4 * q + 2] = (long long)ft_pack(T[4 * q + 2], ec + v.z);
+            T[4 * q + 3] = (long long)ft_pack(T[4 * q + 3], ec + v.w);
+        }
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
             const int n = n0 + e;
@@ -271,14 +286,14 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fold_tc(const ssk::FoldArgs a
                 const bool has = q + 1 < qb || na < nbq;
                 ssk::FoldTile tn{};
                 if (has) tn = q + 1 < qb ? tile(lv, q + 1) : tile(nx, na);
-                __syncthreads();                     // s_row, s_er written
+                __syncthreads();                     // s_row, s_er, s_ce written
                 if (backward || t.g0 != last_panel || c0 != last_c0) cut_rhs(c0, c1, backward, t);
                 last_panel = t.g0;
                 last_c0 = c0;
                 if (has) fetch(tn);
                 if (!multiply(backward)) { ok = false; return; }
                 read_out(c0, c1, backward, t);
-                __syncthreads();                     // s_row, s_er, s_ec and the accumulators are free
+                __syncthreads();                     // s_row, s_er, s_ce, s_ec and the accumulators are free
             }
             // the next item's digits while the other blocks arrive
             const bool wait = (more || !backward) && lv.tiles_64 > 0;

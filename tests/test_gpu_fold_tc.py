@@ -77,3 +77,31 @@ def test_cuda_core_solves_count_no_tensor_work(gpu_lib):
     f, M, _ = factored(gpu_lib, "dense_513")
     assert solved(f, np.ones((M.shape[0], 320)), "simt")[1] == 0.0
     assert solved(f, np.ones((M.shape[0], 8)))[1] == 0.0
+
+
+@pytest.mark.parametrize("mode", ["tensor", "simt"])
+@pytest.mark.parametrize("span", [0, 5, 10, 20])
+def test_scaled_basis_keeps_its_digits(gpu_lib, span, mode):
+    # S M S with S = 2^-span .. 2^span per row has the solution S^-1 M^-1 R of the right-hand sides S R: a
+    # positive definite M, which every pivot order factors stably, solved to its own n u cond(M), not to
+    # that of the scaled matrix
+    p = random_sparse_pencil(700, 0.5, 6)
+    n, k = p.n, 300
+    rng = np.random.default_rng(span)
+    S = 2.0 ** rng.integers(-span, span + 1, n)
+    rows, cols = p.rows(), p.colind
+    lam = np.linalg.eigvals(np.linalg.solve(p.dense("b"), p.dense("a"))).real
+    sigma = lam.min() - np.ptp(lam)
+    ctx = gpu_lib.Context(0)
+    ctx.set_schur_mode("simt")                    # the factor itself in plain FP64
+    sym = ctx.analyze(p.rowptr, p.colind, dense=True)
+    scale = S[rows] * S[cols]
+    # (pivots of 2^-40 of the norm are reported as singular, the factor is there all the same)
+    f = sym.factor(torch.tensor(p.a * scale, device="cuda"), torch.tensor(p.b * scale, device="cuda"), [sigma], "fp64",
+                   allow_singular=True)
+    M = p.dense("a") - sigma * p.dense("b")
+    R = rng.standard_normal((n, k))
+    X, flops = solved(f, S[:, None] * R, mode)
+    assert (flops > 0.0) == (mode == "tensor")
+    ref = np.linalg.solve(M, R)
+    assert np.linalg.norm(S[:, None] * X - ref) <= 16 * n * 1.1e-16 * np.linalg.cond(M) * np.linalg.norm(ref)
