@@ -26,19 +26,22 @@ constexpr int kTUnit = 56;                          // T counts 2^(E_a + E_b - k
 constexpr int kFtNan = 1 << 20;                     // "exponent" of a non-finite value
 constexpr int kFtZero = -(1 << 20);                 // "exponent" of zero
 
-// biased exponent of v plus sh; kFtZero for zero (and denormals, which count as zero), kFtNan
+// biased exponent of v plus sh (1 plus sh for a denormal, whose leading bit is not implicit); kFtZero for
+// zero, kFtNan
 __device__ __forceinline__ int ft_exp(double v, int sh) {
-    const int ex = (int)((__double_as_longlong(v) >> 52) & 0x7ff);
-    return ex == 0 ? kFtZero : (ex == 0x7ff ? kFtNan : ex + sh);
+    const uint32_t lo = (uint32_t)__double2loint(v), hi = (uint32_t)__double2hiint(v) & 0x7fffffffu;
+    const int ex = (int)(hi >> 20), e = (hi | lo) == 0 ? kFtZero : max(ex, 1) + sh;
+    return ex == 0x7ff ? kFtNan : e;
 }
 
 // round(x 2^(55 - E)) + 0x80808080808080 for |x| < 2^E; em = E + 1022 >= ex, the exponents as from
 // ft_exp
 __device__ __forceinline__ unsigned long long ft_biased(double v, int ex, int em) {
     const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
-    unsigned long long m = (bits & ((1ull << 52) - 1)) | (1ull << 52);
+    const uint32_t hi = (uint32_t)(bits >> 32);
+    const uint32_t mh = (hi & 0xfffffu) | ((hi & 0x7ff00000u) != 0 ? 0x100000u : 0u);     // 0 for zero
+    unsigned long long m = ((unsigned long long)mh << 32) | (uint32_t)bits;
     m = (((m << 3) >> min(em - ex, 60)) + 1) >> 1;  // 4 m 2^(ex - em), rounded
-    if (ex == kFtZero) m = 0;
     const unsigned long long s = (unsigned long long)((long long)bits >> 63);
     return ((m ^ s) - s) + 0x80808080808080ull;
 }

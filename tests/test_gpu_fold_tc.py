@@ -105,3 +105,24 @@ def test_scaled_basis_keeps_its_digits(gpu_lib, span, mode):
     assert (flops > 0.0) == (mode == "tensor")
     ref = np.linalg.solve(M, R)
     assert np.linalg.norm(S[:, None] * X - ref) <= 16 * n * 1.1e-16 * np.linalg.cond(M) * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("mode", ["tensor", "simt"])
+def test_denormal_right_hand_sides(gpu_lib, mode):
+    # whole multiples, up to 2^43, of the smallest denormal: every addition rounds to one of those, n of them
+    # to an entry, amplified by cond(M)
+    p = random_sparse_pencil(700, 0.5, 6)
+    lam = np.linalg.eigvals(np.linalg.solve(p.dense("b"), p.dense("a"))).real
+    sigma = lam.min() - np.ptp(lam)
+    ctx = gpu_lib.Context(0)
+    sym = ctx.analyze(p.rowptr, p.colind, dense=True)
+    f = sym.factor(torch.tensor(p.a, device="cuda"), torch.tensor(p.b, device="cuda"), [sigma], "fp64")
+    M = p.dense("a") - sigma * p.dense("b")
+    k = 300
+    N = np.rint(2.0 ** 40 * np.random.default_rng(1).standard_normal((p.n, k)))
+    unit = 2.0 ** -1074
+    X, flops = solved(f, N * unit, mode)
+    assert (flops > 0.0) == (mode == "tensor")
+    ref = np.linalg.solve(M, N)
+    tol = 16 * p.n * np.linalg.cond(M) * max(1.0, np.linalg.norm(np.linalg.inv(M), 2))
+    assert np.abs(X / unit - ref).max() <= tol
