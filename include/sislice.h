@@ -226,6 +226,11 @@ ss_status ss_selftest_tc(ss_ctx *ctx, uint64_t seed, double *max_abs_err);
  * SS_ERR_TIMEOUT. */
 ss_status ss_selftest_barrier(ss_ctx *ctx, int32_t extra_arrivals, int64_t limit);
 
+/* Self-test of the reciprocal that the diagonal blocks' pivots use (no paper counterpart): out[i] =
+ * 1 / d[i] within one unit in the last place, 0 for d[i] = 0; d and out DEVICE float64[n].  Errors:
+ * SS_ERR_ARG, SS_ERR_CUDA. */
+ss_status ss_selftest_recip(ss_ctx *ctx, int64_t n, const double *d, double *out);
+
 /* Self-test of what the calls do when device memory runs out (no paper counterpart): from now on
  * every device allocation of this context above max_bytes bytes fails on the host as an
  * out-of-memory one would; max_bytes < 0 (the state of a new context): no limit.  Errors:

