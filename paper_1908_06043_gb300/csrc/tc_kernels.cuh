@@ -114,8 +114,8 @@ __global__ void __launch_bounds__(128, 1) k_tc_selftest(const unsigned char *__r
 // ---------------------------------------------------------------- slice producer
 // Block = one 128-row tile of L21 (the first nrt tiles of a task) or of W (the next nrt);
 // thread = (row, 16 columns).  The kSlices blocks of 16 KB are put together in shared memory and
-// leave as one bulk copy.
-__global__ void __launch_bounds__(kTcSliceThreads, 2) k_tc_slice(const StepTask *__restrict__ tasks, int32_t ntask,
+// leave as one bulk copy; that staging lets one block be resident on an SM.
+__global__ void __launch_bounds__(kTcSliceThreads) k_tc_slice(const StepTask *__restrict__ tasks, int32_t ntask,
                                                                  const ssk::ShiftPtrs<double> *sp) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *sm = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
