@@ -1377,9 +1377,6 @@ static int solve_sweeps(ss_numeric *f, int j, float *b, int k, const float *aren
     a.linv = f->linv[j];
     a.dblk = f->dblk[j];
     a.piv = f->piv[j];
-    a.forward = 1;
-    a.backward = 1;
-    a.dinv = 1;
     a.bar = ctx->d_bar;
     a.limit = 20000000;        // polls of about 64 ns: ~1 s per barrier
     a.sm_slots = sm_slots;
@@ -1437,7 +1434,7 @@ static int solve_levels(ss_numeric *f, int j, float *b, int k) {
             ctx->add_flops(SS_K_BWD_GATHER_F32, 2.0 * sl.offdiag * k);
         }
         ss_launch(ctx, SS_K_BWD_DIAG, k_bwd_diag, dim3(sl.count, ndchunk), 256, diag_solve_smem(), st,
-                  lp, s->d_panels, f->linv[j], f->dblk[j], f->piv[j], z, sl.row_tiles > 0 ? 1 : 0, b, k, 1);
+                  lp, s->d_panels, f->linv[j], f->dblk[j], f->piv[j], z, sl.row_tiles > 0 ? 1 : 0, b, k);
     }
     SS_CUDA_TRY(ctx, cudaFreeAsync(z, st));
     SS_CUDA_TRY(ctx, cudaGetLastError());

@@ -269,7 +269,7 @@ __device__ __forceinline__ void bwd_diag_item(unsigned char *smem_raw, int slot,
                                               const double *__restrict__ linv,
                                               const double *__restrict__ dblk,
                                               const int32_t *__restrict__ piv,
-                                              const float *zbuf, int use_z, float *x, int k, int dinv) {
+                                              const float *zbuf, int use_z, float *x, int k) {
     float (*U)[KD + 1] = reinterpret_cast<float (*)[KD + 1]>(smem_raw);
     float (*Lm)[NB + 1] = reinterpret_cast<float (*)[NB + 1]>(smem_raw + sizeof(float) * NB * (KD + 1));
     __shared__ double sd[NB], se[NB];
@@ -316,9 +316,7 @@ __device__ __forceinline__ void bwd_diag_item(unsigned char *smem_raw, int slot,
         int i = rr + RS * a;
         double u = 0.0;
         if (i < w && c < kc) {
-            if (!dinv) {                            // half solve: D^-1/2 applied beforehand
-                u = (double)U[i][c];
-            } else if (se[i] != 0.0) {              // first row of a 2x2 block
+            if (se[i] != 0.0) {                     // first row of a 2x2 block
                 double A = sd[i], B = se[i], C = sd[i + 1], det = A * C - B * B;
                 u = (C * (double)U[i][c] - B * (double)U[i + 1][c]) / det;
             } else if (i > 0 && se[i - 1] != 0.0) { // second row of a 2x2 block
@@ -394,9 +392,9 @@ __global__ void __launch_bounds__(256) k_bwd_diag(const int32_t *__restrict__ lv
                                                    const double *__restrict__ linv,
                                                    const double *__restrict__ dblk,
                                                    const int32_t *__restrict__ piv,
-                                                   const float *zbuf, int use_z, float *x, int k, int dinv) {
+                                                   const float *zbuf, int use_z, float *x, int k) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    bwd_diag_item(smem_raw, blockIdx.x, blockIdx.y, lvl_panels, panels, linv, dblk, piv, zbuf, use_z, x, k, dinv);
+    bwd_diag_item(smem_raw, blockIdx.x, blockIdx.y, lvl_panels, panels, linv, dblk, piv, zbuf, use_z, x, k);
 }
 
 // ---------------------------------------------------------------- one launch per solve
@@ -418,7 +416,7 @@ struct SweepArgs {
     const double *linv;
     const double *dblk;
     const int32_t *piv;
-    int32_t forward, backward, dinv, nsm_slots;
+    int32_t nsm_slots;
     GridBar *bar;
     long long limit;
     int32_t *sm_slots;     // nsm_slots zeroed counters (blocks seen per SM id), or null
@@ -758,7 +756,7 @@ __device__ __forceinline__ bool level_fused(const SweepArgs &a, const SweepLevel
     return a.arrive != nullptr && (int64_t)(lv.row_tiles + lv.count) * nchunk <= a.fuse_max;
 }
 
-// Forward and/or backward sweep over every level in one cooperative launch.  The work
+// Forward and backward sweep over every level in one cooperative launch.  The work
 // items of a step are spread over the resident blocks; a grid barrier separates
 // consecutive steps.  zall: (number of panels) x NB x k, zero on entry (each level
 // gathers into its own slots).  On a barrier timeout bar->err is set and every block
@@ -773,27 +771,24 @@ __global__ void __launch_bounds__(256, 4) k_solve_sweeps(SweepArgs a, const floa
     bool ok = true;
     const int vb = spread_block_id(a, at, &ok);
     if (!ok) return;
-    if (a.forward) {
-        for (int L = 0; L < a.nlev; ++L) {
-            const SweepLevel lv = a.lev[L];
-            const int32_t *lp = a.solve_panels + lv.panel_off;
-            if (level_fused(a, lv, nchunk)) {           // y of this level goes to ybuf
-                fwd_level_fused_f32(a, smem_raw, vb, lv, arena, b, ybuf);
-                if (!grid_barrier(a.bar, nb, a.limit, at)) return;
-                continue;
-            }
-            for (int q = vb; q < lv.count * ndchunk; q += nb)
-                fwd_diag_item(smem_raw, q % lv.count, q / lv.count, lp, a.panels, a.linv, a.piv, b, k);
+    for (int L = 0; L < a.nlev; ++L) {
+        const SweepLevel lv = a.lev[L];
+        const int32_t *lp = a.solve_panels + lv.panel_off;
+        if (level_fused(a, lv, nchunk)) {           // y of this level goes to ybuf
+            fwd_level_fused_f32(a, smem_raw, vb, lv, arena, b, ybuf);
             if (!grid_barrier(a.bar, nb, a.limit, at)) return;
-            if (lv.row_tiles == 0) continue;
-            const int32_t *tp = a.tile_pre + lv.panel_off;
-            for (int q = vb; q < lv.row_tiles * nchunk; q += nb)
-                fwd_update_f32_item(smem_raw, q % lv.row_tiles, q / lv.row_tiles, lp, tp, lv.count, a.panels, a.idx,
-                                    arena, b, k);
-            if (!grid_barrier(a.bar, nb, a.limit, at)) return;
+            continue;
         }
+        for (int q = vb; q < lv.count * ndchunk; q += nb)
+            fwd_diag_item(smem_raw, q % lv.count, q / lv.count, lp, a.panels, a.linv, a.piv, b, k);
+        if (!grid_barrier(a.bar, nb, a.limit, at)) return;
+        if (lv.row_tiles == 0) continue;
+        const int32_t *tp = a.tile_pre + lv.panel_off;
+        for (int q = vb; q < lv.row_tiles * nchunk; q += nb)
+            fwd_update_f32_item(smem_raw, q % lv.row_tiles, q / lv.row_tiles, lp, tp, lv.count, a.panels, a.idx,
+                                arena, b, k);
+        if (!grid_barrier(a.bar, nb, a.limit, at)) return;
     }
-    if (!a.backward) return;
     for (int L = a.nlev - 1; L >= 0; --L) {
         const SweepLevel lv = a.lev[L];
         const int32_t *lp = a.solve_panels + lv.panel_off;
@@ -812,7 +807,7 @@ __global__ void __launch_bounds__(256, 4) k_solve_sweeps(SweepArgs a, const floa
         }
         for (int q = vb; q < lv.count * ndchunk; q += nb)
             bwd_diag_item(smem_raw, q % lv.count, q / lv.count, lp, a.panels, a.linv, a.dblk, a.piv, z,
-                             lv.row_tiles > 0 ? 1 : 0, b, k, a.dinv);
+                             lv.row_tiles > 0 ? 1 : 0, b, k);
         if (L > 0 && !grid_barrier(a.bar, nb, a.limit, at)) return;
     }
 }
