@@ -472,6 +472,12 @@ ss_status ss_spmm(ss_symbolic *sym, const double *a_vals, const double *b_vals,
 enum { SS_PEAK_FP64_FMA = 0, SS_PEAK_FP32_FMA = 1 };
 ss_status ss_measure_peak(ss_ctx *ctx, int32_t kind, double seconds, double *tflops);
 
+/* Give the device memory that the context keeps between calls back to the device (no paper
+ * counterpart).  The calls' scratch comes from a pool of the context that holds up to 1 GB of freed
+ * blocks, all of which go with ss_destroy; a program whose other allocator needs them before then calls
+ * this.  Synchronises the stream; the next call maps its scratch anew.  Errors: SS_ERR_ARG, SS_ERR_CUDA. */
+ss_status ss_release_scratch(ss_ctx *ctx);
+
 /* Device synchronisation of the context's stream (convenience for bindings). */
 ss_status ss_sync(ss_ctx *ctx);
 

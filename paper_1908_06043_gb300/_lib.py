@@ -52,7 +52,7 @@ class ss_solve_opts(C.Structure):
 
 EXPORTS = ["ss_create", "ss_destroy", "ss_last_error", "ss_analyze", "ss_symbolic_info_get",
            "ss_symbolic_perm", "ss_symbolic_destroy", "ss_symbolic_validate", "ss_factor", "ss_factor_segments", "ss_factor_destroy", "ss_inertia", "ss_inertia_segments", "ss_factor_stats", "ss_factor_quality",
-           "ss_solve", "ss_solve_noalloc", "ss_slice_solve", "ss_dos_estimate", "ss_dos_lanczos", "ss_band_energy_grad", "ss_spmm", "ss_sync", "ss_launch_count", "ss_profile", "ss_profile_query", "ss_set_solve_mode", "ss_set_sweep_fusion", "ss_selftest_barrier", "ss_selftest_recip", "ss_selftest_alloc_limit", "ss_measure_peak", "ss_set_schur_mode", "ss_selftest_tc", "ss_set_factor_graph", "ss_autotune_schur", "ss_set_gemm_mode", "ss_dense_gram", "ss_dense_gemm", "ss_profile_query_tensor"]
+           "ss_solve", "ss_solve_noalloc", "ss_slice_solve", "ss_dos_estimate", "ss_dos_lanczos", "ss_band_energy_grad", "ss_spmm", "ss_sync", "ss_release_scratch", "ss_launch_count", "ss_profile", "ss_profile_query", "ss_set_solve_mode", "ss_set_sweep_fusion", "ss_selftest_barrier", "ss_selftest_recip", "ss_selftest_alloc_limit", "ss_measure_peak", "ss_set_schur_mode", "ss_selftest_tc", "ss_set_factor_graph", "ss_autotune_schur", "ss_set_gemm_mode", "ss_dense_gram", "ss_dense_gemm", "ss_profile_query_tensor"]
 KERNEL_CLASSES = ["assemble", "extend_add", "diag_bk", "panel", "schur", "fwd_diag", "fwd_update", "bwd_gather",
                   "bwd_diag", "permute", "spmm", "gram", "gemm", "small_dense", "jacobi", "lanczos", "sddmm", "misc",
                   "panel_f32", "schur_f32", "fwd_update_f32", "bwd_gather_f32", "solve", "solve_f32",
@@ -110,6 +110,7 @@ def load():
         "ss_band_energy_grad": ([P, P, P, i32, P, P], i32),
         "ss_spmm": ([P, P, P, P, P, P, i32, P], i32),
         "ss_sync": ([P], i32),
+        "ss_release_scratch": ([P], i32),
         "ss_launch_count": ([], i64),
         "ss_profile": ([P, C.c_uint32], i32),
         "ss_profile_query": ([P, i32, C.POINTER(i64), C.POINTER(dbl), C.POINTER(dbl)], i32),

@@ -68,6 +68,10 @@ class Context:
     def sync(self):
         self.check(self.lib.ss_sync(self.h), "ss_sync")
 
+    def release_scratch(self):
+        """Give the scratch memory kept between calls (up to 1 GB) back to the device."""
+        self.check(self.lib.ss_release_scratch(self.h), "ss_release_scratch")
+
     def analyze(self, rowptr: np.ndarray, colind: np.ndarray, nd_leaf: int = 0, dense: bool = False) -> "Symbolic":
         return analyze(self, rowptr, colind, nd_leaf, dense)
 

@@ -124,6 +124,15 @@ static void pool_trim(ss_ctx *ctx) {
     cudaMemPoolTrimTo(ctx->pool, 0);
 }
 
+extern "C" ss_status ss_release_scratch(ss_ctx *ctx) {
+    if (!ctx) return SS_ERR_ARG;
+    if (ctx->device < 0 || !ctx->pool) return SS_OK;
+    SS_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
+    SS_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
+    SS_CUDA_TRY(ctx, cudaMemPoolTrimTo(ctx->pool, 0));
+    return SS_OK;
+}
+
 static bool alloc_refused(const ss_ctx *ctx, size_t bytes) {
     return ctx->alloc_limit >= 0 && bytes > (size_t)ctx->alloc_limit;
 }

@@ -62,7 +62,7 @@ struct ss_ctx {
 // Stream-ordered scratch of the context's calls, freed with cudaFreeAsync.  The context has a pool
 // of its own that keeps up to kPoolKeepBytes between calls (the default pool gives everything back
 // at each synchronisation, and mapping 0.1 - 2 GB again took up to 4 ms a call); what it holds unused
-// goes back when an allocation would fail, and all of it with the context.
+// goes back when an allocation would fail, on ss_release_scratch, and all of it with the context.
 constexpr uint64_t kPoolKeepBytes = 1ull << 30;
 cudaError_t ss_malloc_async(ss_ctx *ctx, void **p, size_t bytes, cudaStream_t st);
 // cudaMalloc that takes the pool's unused memory back before it gives up

@@ -50,3 +50,20 @@ def test_lanczos_runs_hold_the_matrices_of_one_group(gpu_lib):
         quotient = (x @ A @ x) / (x @ B @ x)
         assert abs(z2.sum() - 1.0) <= 1e-10
         assert abs(z2 @ th - quotient) <= 1e-10 * np.abs(th).max()
+
+
+def test_scratch_goes_back_on_request(gpu_lib):
+    p = gaussian_pencil((9, 11, 11), (0.3, 2.0), seed=3)
+    ctx, sym, a, b = setup(gpu_lib, p)
+    X = torch.tensor(normal_block(p.n, 700, 5), device="cuda")
+    lam = torch.linspace(-3.0, -1.0, 700, dtype=torch.float64, device="cuda")
+    sym.band_energy_grad(X, lam)                  # lists of the pattern, modules
+    ctx.release_scratch()
+    free = torch.cuda.mem_get_info()[0]
+    ga, _ = sym.band_energy_grad(X, lam)
+    # 16 bytes an entry of X for each of two operands: 49 MB
+    assert torch.cuda.mem_get_info()[0] <= free - 40e6
+    ctx.release_scratch()
+    assert torch.cuda.mem_get_info()[0] >= free - 4e6
+    again, _ = sym.band_energy_grad(X, lam)
+    assert torch.equal(ga, again)
