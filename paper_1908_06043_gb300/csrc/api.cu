@@ -1207,6 +1207,15 @@ static int fold_nc(int k) {
     return (k + nch - 1) / nch;
 }
 
+int pencil_scales(ss_numeric *f, int j, const int32_t *perm, int32_t *sc) {
+    ss_symbolic *s = f->sym;
+    ss_ctx *ctx = s->ctx;
+    ss_launch(ctx, SS_K_MISC, k_fold_scales, (unsigned)((s->n + 255) / 256), 256, 0, ctx->stream, s->n, perm,
+              (const int64_t *)s->d_rowptr, (const int32_t *)s->d_colind, f->a_vals, f->b_vals, f->sigma[j], sc);
+    SS_CUDA_TRY(ctx, cudaGetLastError());
+    return SS_OK;
+}
+
 // G = L21 L11^-1 P in the FP64 L storage of shift j and its scales (once, when its factorisation is done)
 static int fold_shift(ss_numeric *f, int j) {
     ss_symbolic *s = f->sym;
@@ -1216,11 +1225,7 @@ static int fold_shift(ss_numeric *f, int j) {
     ss_launch(ctx, SS_K_PANEL, k_fold_panels, dim3((unsigned)s->panels.size(), (unsigned)((s->max_rows_below + TR - 1) / TR)),
               256, kFoldPanelsSmem, ctx->stream, (const PanelDesc *)s->d_panels, (const double *)f->linv[j],
               (const int32_t *)f->piv[j], (double *)f->arena[j]);
-    ss_launch(ctx, SS_K_PANEL, k_fold_scales, (unsigned)((s->n + 255) / 256), 256, 0, ctx->stream, s->n,
-              (const int32_t *)s->d_perm, (const int64_t *)s->d_rowptr, (const int32_t *)s->d_colind, f->a_vals,
-              f->b_vals, f->sigma[j], f->piv[j] + (int64_t)NB * s->panels.size());
-    SS_CUDA_TRY(ctx, cudaGetLastError());
-    return SS_OK;
+    return pencil_scales(f, j, s->d_perm, f->piv[j] + (int64_t)NB * s->panels.size());
 }
 
 // one launch per level and sweep: no allocation, no synchronisation

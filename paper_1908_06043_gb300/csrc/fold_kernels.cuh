@@ -133,14 +133,14 @@ struct FoldArgs {
     long long limit;
 };
 
-// sc[i] = exponent of about sqrt(|a_ii| + |sigma b_ii|), i in permuted order; 0 where that is zero or
-// not finite.  Scaling row and column i of the pencil by 2^s adds s.  Thread = row.
+// sc[i] = exponent of about sqrt(|a_rr| + |sigma b_rr|), r = perm[i] (i without perm); 0 where that is
+// zero or not finite.  Scaling row and column i of the pencil by 2^s adds s.  Thread = row.
 __global__ void k_fold_scales(int64_t n, const int32_t *__restrict__ perm, const int64_t *__restrict__ rowptr,
                               const int32_t *__restrict__ colind, const double *__restrict__ a,
                               const double *__restrict__ b, double sigma, int32_t *__restrict__ sc) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const int32_t r = perm[i];
+    const int32_t r = perm ? perm[i] : (int32_t)i;
     int64_t lo = rowptr[r], hi = rowptr[r + 1] - 1;        // the diagonal is stored, columns ascend
     while (lo < hi) {
         const int64_t mid = (lo + hi) >> 1;

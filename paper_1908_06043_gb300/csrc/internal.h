@@ -347,6 +347,8 @@ bool oz_sddmm_ok(const ss_symbolic *s, int ne);
 int oz_sddmm(ss_symbolic *s, const double *X, const double *lambda, int ne, double *grad_a, double *grad_b);
 void oz_free_numeric(ss_numeric *f);
 void oz_free_symbolic(ss_symbolic *s);
+// sc[i] = exponent of the scale of row perm[i] (row i without perm) of the pencil at shift j (k_fold_scales)
+int pencil_scales(ss_numeric *f, int j, const int32_t *perm, int32_t *sc);
 // x = P L^-T D^-1/2 y (y permuted order, x original order), SPD factors only
 int solve_half_backward(ss_numeric *f, int j, const double *y, int k, double *x);
 

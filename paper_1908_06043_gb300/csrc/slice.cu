@@ -280,7 +280,7 @@ int cholqr_track(ss_numeric *f, double *&W, double *&BW, double *&Wt, double *&B
 // carries the rounding of forming W^T A W, about u ||A|| ||x||_2^2 -- up to 2e-9 on the
 // low tail of the Gaussian pencils, whose B-normalised eigenvectors have ||x||_2 of
 // hundreds -- while the quotient of the Ritz vector is second-order in the vector's error.
-int rq_polish(ss_numeric *f, const double *X, int k, double *theta_d, DevBuf &buf) {
+int rq_polish(ss_numeric *f, int j, const double *X, int k, double *theta_d, DevBuf &buf) {
     ss_symbolic *s = f->sym;
     ss_ctx *ctx = s->ctx;
     const int64_t n = s->n;
@@ -289,8 +289,9 @@ int rq_polish(ss_numeric *f, const double *X, int k, double *theta_d, DevBuf &bu
     const int64_t nbx = std::max<int64_t>(1, std::min<int64_t>(cdiv(n, sss::kRqWarps), cdiv(16ll * ctx->sm_count, nby)));
     const int64_t rows_per = (n + nbx - 1) / nbx;
     const int64_t nparts = (n + rows_per - 1) / rows_per;
-    // 61 + xbits + log2(entries of a row) <= 126
-    int xbits = 52;
+    // 61 + xbits + log2(entries of a row) <= 126, as far as that allows 53:
+    // x~ is a whole number that FP64 holds
+    int xbits = 53;
     while (xbits > 30 && ((int64_t)1 << (126 - 61 - xbits)) < s->max_row) --xbits;
     double *part;
     long long *xi;
@@ -298,12 +299,17 @@ int rq_polish(ss_numeric *f, const double *X, int k, double *theta_d, DevBuf &bu
     TRY_ALLOC(ctx, buf.get(&part, (size_t)nparts * k * 4));
     TRY_ALLOC(ctx, buf.get(&xi, (size_t)n * k));
     TRY_ALLOC(ctx, buf.get(&em, (size_t)k));
-    SS_CUDA_TRY(ctx, cudaMemsetAsync(em, 0, sizeof(int) * k, st));
+    SS_CUDA_TRY(ctx, cudaMemsetAsync(em, 0x80, sizeof(int) * k, st));      // below every exponent
+    int32_t *sc;
+    TRY_ALLOC(ctx, buf.get(&sc, (size_t)n));
+    int rc;
+    if ((rc = pencil_scales(f, j, nullptr, sc)) != SS_OK) return rc;
     const int64_t per = std::max<int64_t>(64, n / 256);
-    ss_launch(ctx, SS_K_MISC, sss::k_rq_colmax, dim3(cdiv(k, 128), cdiv(n, per)), 128, 0, st, n, k, X, per, em);
-    ss_launch(ctx, SS_K_MISC, sss::k_rq_fixed, cdiv(n * k, 256), 256, 0, st, n, k, X, (const int *)em, xbits, xi);
+    ss_launch(ctx, SS_K_MISC, sss::k_rq_colmax, dim3(cdiv(k, 128), cdiv(n, per)), 128, 0, st, n, k, X, (const int32_t *)sc, per, em);
+    ss_launch(ctx, SS_K_MISC, sss::k_rq_fixed, cdiv(n * k, 256), 256, 0, st, n, k, X, (const int32_t *)sc, (const int *)em,
+              xbits, xi);
     ss_launch(ctx, SS_K_MISC, sss::k_rq_partial, dim3((unsigned)nparts, nby), 32 * sss::kRqWarps, 0, st, n, s->d_rowptr,
-              s->d_colind, f->a_vals, f->b_vals, (const long long *)xi, (const int *)em, k, rows_per, part);
+              s->d_colind, f->a_vals, f->b_vals, (const int32_t *)sc, (const long long *)xi, (const int *)em, k, rows_per, part);
     ss_launch(ctx, SS_K_MISC, sss::k_rq_dd_finish, cdiv(k, 256), 256, 0, ctx->stream, k, (int)nparts,
               (const double *)part, theta_d);
     SS_CUDA_TRY(ctx, cudaGetLastError());
@@ -459,7 +465,7 @@ int slice_solve_impl(ss_numeric *f, int j, double lo, double hi, const ss_solve_
     (void)maxr_all;
     // the returned eigenvalues: double-double Rayleigh quotients of the Ritz vectors
     if (have_rr) {
-        if ((rc = rq_polish(f, V, k, theta_d, buf)) != SS_OK) return rc;
+        if ((rc = rq_polish(f, j, V, k, theta_d, buf)) != SS_OK) return rc;
         SS_CUDA_TRY(ctx, cudaMemcpyAsync(th.data(), theta_d, sizeof(double) * k, cudaMemcpyDeviceToHost, st));
     }
     SS_CUDA_TRY(ctx, cudaMemcpyAsync(X, V, sizeof(double) * n * k, cudaMemcpyDeviceToDevice, st));
@@ -580,7 +586,7 @@ int block_lanczos_impl(ss_numeric *f, int j, double lo, double hi, const ss_solv
               (const double *)(rr + kout), f->norm_a1, resid_d);
     SS_CUDA_TRY(ctx, cudaMemcpyAsync(resid, resid_d, sizeof(double) * kout, cudaMemcpyDeviceToHost, st));
     // the returned eigenvalues: double-double Rayleigh quotients of the Ritz vectors
-    if ((rc = rq_polish(f, X, kout, theta_d, buf)) != SS_OK) return rc;
+    if ((rc = rq_polish(f, j, X, kout, theta_d, buf)) != SS_OK) return rc;
     SS_CUDA_TRY(ctx, cudaMemcpyAsync(ths.data(), theta_d, sizeof(double) * kout, cudaMemcpyDeviceToHost, st));
     SS_CUDA_TRY(ctx, cudaStreamSynchronize(st));
     std::memcpy(lambda, ths.data(), sizeof(double) * kout);
