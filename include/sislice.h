@@ -445,7 +445,8 @@ ss_status ss_dos_lanczos(ss_symbolic *sym, const double *a_vals, const double *b
  * for every stored entry e = (r, c) of the pattern (DEVICE float64[nnz] each; either
  * may be NULL).  This is the per-stored-entry derivative; a symmetric parameter tying
  * (r, c) and (c, r) gets the sum of both entries.  With ss_set_gemm_mode(SS_GEMM_TENSOR),
- * N >= 2,048 and n_e >= 48 the products run on the tensor cores: every row of X (of X diag(lambda))
+ * N >= 2,048, n_e >= 48 and a pattern that fills 128 x 64 tiles well enough (about 15 entries a row in
+ * a band, 150 scattered ones) the products run on the tensor cores: every row of X (of X diag(lambda))
  * is cut to 55 bits below its largest entry, the products of the digits are summed exactly and the
  * sum is rounded once, so the error of entry (r, c) is a few units of 2^-53 of n_e max|X_r| max|X_c|.
  * That path takes scratch of 32 N n_e bytes (where it does not fit, and on a stream that records a

@@ -343,7 +343,7 @@ int oz_spmm_vals(ss_symbolic *s, const double *a, const double *b, const double 
 int spmm_f(ss_numeric *f, const double *a, const double *b, const double *alpha, const double *beta, const double *X,
            int64_t ldx, int k, double *Y, int64_t ldy);
 // grad_a = X X^T, grad_b = -X diag(lambda) X^T on the stored pattern (X n x ne)
-bool oz_sddmm_ok(const ss_symbolic *s, int ne);
+bool oz_sddmm_ok(ss_symbolic *s, int ne);
 int oz_sddmm(ss_symbolic *s, const double *X, const double *lambda, int ne, double *grad_a, double *grad_b);
 void oz_free_numeric(ss_numeric *f);
 void oz_free_symbolic(ss_symbolic *s);

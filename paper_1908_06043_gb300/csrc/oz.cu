@@ -16,9 +16,12 @@ struct OzPlan {
     uint16_t *d_ent_off = nullptr;
 };
 
-// entries at or below the diagonal by (128-row tile, 64-column tile), for the sampled product X Y^T
+// entries at or below the diagonal by (128-row tile, 64-column tile), for the sampled product X Y^T:
+// the tiles are counted first, the lists made by the first product that takes them
 struct OzSamples {
     int64_t ntiles = 0;
+    std::vector<int32_t> rts, cts;     // row and column tile of every tile (host, until the lists are made)
+    std::vector<int64_t> ptr, first;   // first entry of every tile; first tile of every row tile
     int32_t *d_rt = nullptr, *d_ct = nullptr;
     int64_t *d_ptr = nullptr;          // ntiles + 1
     uint32_t *d_e = nullptr, *d_t = nullptr;   // CSR positions of the entry and its mirror image
@@ -229,8 +232,7 @@ int plan_build(ss_symbolic *s) {
     return SS_OK;
 }
 
-int samples_build(ss_symbolic *s) {
-    ss_ctx *ctx = s->ctx;
+int samples_count(ss_symbolic *s) {
     const int64_t n = s->n, nct = (n + 63) / 64;
     const int32_t nrt = (int32_t)cdivu(n, 128);
     std::vector<std::vector<int32_t>> cts(nrt), counts(nrt);
@@ -250,17 +252,28 @@ int samples_build(ss_symbolic *s) {
             }
         }
     }
-    std::vector<int32_t> rts, ctl;
-    std::vector<int64_t> ptr(1, 0), first(nrt, 0);
+    OzSamples *sp = new OzSamples();
+    s->oz_samples = sp;
+    sp->ptr.assign(1, 0);
+    sp->first.assign(nrt, 0);
     for (int32_t rt = 0; rt < nrt; ++rt) {
-        first[rt] = (int64_t)rts.size();
+        sp->first[rt] = (int64_t)sp->rts.size();
         for (size_t u = 0; u < cts[rt].size(); ++u) {
-            rts.push_back(rt);
-            ctl.push_back(cts[rt][u]);
-            ptr.push_back(ptr.back() + counts[rt][u]);
+            sp->rts.push_back(rt);
+            sp->cts.push_back(cts[rt][u]);
+            sp->ptr.push_back(sp->ptr.back() + counts[rt][u]);
         }
     }
-    const size_t m = (size_t)std::max<int64_t>(1, ptr.back());
+    sp->ntiles = (int64_t)sp->rts.size();
+    return SS_OK;
+}
+
+int samples_build(ss_symbolic *s) {
+    ss_ctx *ctx = s->ctx;
+    OzSamples *sp = s->oz_samples;
+    const int64_t n = s->n, nct = (n + 63) / 64;
+    const int32_t nrt = (int32_t)cdivu(n, 128);
+    const size_t m = (size_t)std::max<int64_t>(1, sp->ptr.back());
     std::vector<uint32_t> e(m), t(m);
     std::vector<uint16_t> off(m);
 #pragma omp parallel
@@ -269,7 +282,8 @@ int samples_build(ss_symbolic *s) {
 #pragma omp for schedule(dynamic, 16)
         for (int32_t rt = 0; rt < nrt; ++rt) {
             const int64_t r0 = rt * 128ll, r1 = std::min<int64_t>(n, r0 + 128);
-            for (size_t u = 0; u < cts[rt].size(); ++u) at[cts[rt][u]] = ptr[first[rt] + u];
+            const int64_t t1 = rt + 1 < nrt ? sp->first[rt + 1] : sp->ntiles;
+            for (int64_t u = sp->first[rt]; u < t1; ++u) at[sp->cts[u]] = sp->ptr[u];
             for (int64_t r = r0; r < r1; ++r)
                 for (int64_t p = s->rowptr[r]; p < s->rowptr[r + 1] && s->colind[p] <= r; ++p) {
                     const int64_t c = s->colind[p], o = at[c / 64]++;
@@ -280,25 +294,26 @@ int samples_build(ss_symbolic *s) {
                 }
         }
     }
-    OzSamples *pl = new OzSamples();
-    pl->ntiles = (int64_t)rts.size();
-    s->oz_samples = pl;
     auto up = [&](auto **d, const auto &h) {
         cudaError_t er = ss_malloc(ctx, (void **)d, sizeof(h[0]) * std::max<size_t>(1, h.size()));
         if (er == cudaSuccess && !h.empty()) er = cudaMemcpy(*d, h.data(), sizeof(h[0]) * h.size(), cudaMemcpyHostToDevice);
         return er;
     };
-    cudaError_t er = up(&pl->d_rt, rts);
-    if (er == cudaSuccess) er = up(&pl->d_ct, ctl);
-    if (er == cudaSuccess) er = up(&pl->d_ptr, ptr);
-    if (er == cudaSuccess) er = up(&pl->d_e, e);
-    if (er == cudaSuccess) er = up(&pl->d_t, t);
-    if (er == cudaSuccess) er = up(&pl->d_off, off);
+    cudaError_t er = up(&sp->d_rt, sp->rts);
+    if (er == cudaSuccess) er = up(&sp->d_ct, sp->cts);
+    if (er == cudaSuccess) er = up(&sp->d_ptr, sp->ptr);
+    if (er == cudaSuccess) er = up(&sp->d_e, e);
+    if (er == cudaSuccess) er = up(&sp->d_t, t);
+    if (er == cudaSuccess) er = up(&sp->d_off, off);
     if (er != cudaSuccess) {
         cudaGetLastError();
         free_samples(s);
         return ctx->set_error(SS_ERR_OOM, "sampled product plan: device allocation failed");
     }
+    sp->rts.clear(), sp->rts.shrink_to_fit();
+    sp->cts.clear(), sp->cts.shrink_to_fit();
+    sp->ptr.clear(), sp->ptr.shrink_to_fit();
+    sp->first.clear(), sp->first.shrink_to_fit();
     return SS_OK;
 }
 
@@ -441,15 +456,25 @@ void oz_free_numeric(ss_numeric *f) {
     for (OzVals *&v : f->oz) drop(v);
 }
 
-// X Y^T sampled on the pattern needs 32-bit CSR positions and enough columns to fill a piece
-bool oz_sddmm_ok(const ss_symbolic *s, int ne) {
-    return s->ctx->gemm_mode == SS_GEMM_TENSOR && s->n >= 2048 && ne >= 48 && s->nnz < (1ll << 32);
+// Whether X Y^T sampled on the pattern runs on the tensor cores: 32-bit CSR positions, enough columns to
+// fill a piece, and the quicker of two estimates in picoseconds.  CUDA cores: two multiply-adds an entry
+// and column and the sums over the lanes, worth 300 columns.  Tensor cores: the launches, every 128 x 64
+// tile that holds an entry in full, and the digits of X and X diag(lambda).  Measured / estimated, us,
+// CUDA cores and tensor cores: N = 20,000, 17 entries a row in 469 tiles, ne = 48 368 / 366 and 286 / 283,
+// ne = 1,640 2,269 / 2,045 and 1,479 / 1,443; 9 a row 209 / 194 and 281 / 283; N = 8,000, 9 scattered
+// entries a row in 4,031 tiles 99 / 78 and 1,136 / 1,281; N = 16,384, 472 a row, ne = 1,640 50,700 and 6,540.
+bool oz_sddmm_ok(ss_symbolic *s, int ne) {
+    if (s->ctx->gemm_mode != SS_GEMM_TENSOR || s->n < 2048 || ne < 48 || s->nnz >= (1ll << 32)) return false;
+    const double cuda = 3.1 * (double)s->nnz * (ne + 300.0), rest = 1.3e8 + 20.0 * (double)s->n * ne;
+    if (cuda <= rest) return false;
+    if (!s->oz_samples && samples_count(s) != SS_OK) return false;
+    return cuda > rest + (double)s->oz_samples->ntiles * (2.5e5 + 700.0 * ne);
 }
 
 int oz_sddmm(ss_symbolic *s, const double *X, const double *lambda, int ne, double *grad_a, double *grad_b) {
     ss_ctx *ctx = s->ctx;
     int rc;
-    if (!s->oz_samples && (rc = samples_build(s)) != SS_OK) return rc;
+    if (!s->oz_samples->d_rt && (rc = samples_build(s)) != SS_OK) return rc;
     const OzSamples *sp = s->oz_samples;
     oz_attrs(ctx->device);
     Scratch buf(ctx);
