@@ -1487,10 +1487,18 @@ int spmm_launch_ld(ss_symbolic *s, const double *a, const double *b, const doubl
             ss_launch(ctx, SS_K_SPMM, sss::k_spmm_nnz<KW, false>, g, 256, 0, ctx->stream, s->n, s->d_rowptr,   \
                       s->d_colind, a, b, alpha, beta, X, ldx, k, Y, ldy);                                      \
     } while (0)
-    // lanes over nonzeros below 16 columns, and up to 48 where the rows are long enough to fill the
-    // lanes (columns over lanes leave k mod 32 of them idle)
-    if (k < 16 || (k < 48 && s->nnz >= 64 * s->n)) {
-        const int nch = (k + 7) / 8;
+    // Lanes over nonzeros below 16 columns; up to 48 the quicker of two estimates in warp instructions, m
+    // entries a row.  Lanes over nonzeros: m / 32 entries a lane times the columns, and the sums over the
+    // lanes of every chunk of 8 columns.  Lanes over columns: the row's entries one after another, the
+    // columns above 32 beside the others where B does not take part, at least 3,000 rows to fill the chip.
+    // Measured, lanes over columns / over nonzeros, us: Gaussian pencils A, k = 31 N = 250 40 / 11,
+    // N = 16,384 (479 a row) 1,123 / 491, A and B 1,049 / 957; bands, N = 16,384, A and B, k = 31 65 a row
+    // 131 / 246, 129 253 / 354, k = 33 65 a row 248 / 277, 129 482 / 397.
+    const int nch = (k + 7) / 8;
+    const double m = (double)s->nnz / (double)s->n, rows = (double)s->n;
+    const double over_nnz = rows * ((beta ? 2.0 : 1.0) * (m / 32.0 + 1.0) * k + (beta ? 22.0 : 9.0) * nch);
+    const double over_cols = std::max(rows, 3000.0) * m * (beta ? 2.4 * ((k + 31) / 32) : 2.2);
+    if (k < 16 || (k < 48 && over_nnz < over_cols)) {
         switch ((k + nch - 1) / nch) {
             case 1: SS_SPMM_NNZ(1); break;
             case 2: SS_SPMM_NNZ(2); break;

@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace sss {
 
 // ---------------------------------------------------------------- SpMM
@@ -90,15 +92,17 @@ __global__ void __launch_bounds__(256) k_spmm_rows(int64_t n, const int64_t *__r
 // One warp per (row, chunk of KW columns), lanes over the row's nonzeros: the FP64 pipe (2
 // multiply-adds a clock and SM) is the limit, and it gets one multiply-add per entry and column (two
 // with B, the sums of A x and B x kept apart) with every lane busy whatever KW is.  Columns
-// c0 = KW blockIdx.y ..; the lanes' sums are folded so that a step adds half as many values as the
-// one before (32 lanes, KW values: about KW additions a lane instead of 5 KW).  N = 16,384 (472
-// entries a row), k = 4, A alone: 216 us with al a + be b formed per entry and column, 86 us now
-// (FP64 floor 53 us).
+// c0 = KW blockIdx.y ..; the lanes' sums, filled up with zeros to a power of two, are folded so that a
+// step adds half as many values as the one before (32 lanes, 5 to 8 values: 9 additions a lane; an odd
+// number of values is added whole at every step, 35 for 7).  N = 16,384 (472 entries a row), A alone:
+// k = 4 216 us with al a + be b formed per entry and column, 76 us now (FP64 floor 53 us); k = 25 587 -> 434
+// with the power of two; a band of 97 entries a row, k = 31 236 -> 153 with the same trips for every lane.
 template <int V, int OFF>
 __device__ __forceinline__ void spmm_fold(double *v, int lane, int &base, int &left, bool &owner) {
+    static_assert((V & (V - 1)) == 0, "a power of two");
     if constexpr (OFF == 0) {
         left = V;
-    } else if constexpr (V % 2 == 0) {
+    } else if constexpr (V > 1) {
         const bool up = (lane & OFF) != 0;
 #pragma unroll
         for (int i = 0; i < V / 2; ++i) {
@@ -108,54 +112,72 @@ __device__ __forceinline__ void spmm_fold(double *v, int lane, int &base, int &l
         base += up ? V / 2 : 0;
         spmm_fold<V / 2, OFF / 2>(v, lane, base, left, owner);
     } else {
-#pragma unroll
-        for (int i = 0; i < V; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], OFF);
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], OFF);
         owner &= (lane & OFF) == 0;
-        spmm_fold<V, OFF / 2>(v, lane, base, left, owner);
+        spmm_fold<1, OFF / 2>(v, lane, base, left, owner);
     }
 }
 
 template <int KW, bool WITH_B>
-__global__ void __launch_bounds__(256) k_spmm_nnz(int64_t n, const int64_t *__restrict__ rowptr,
-                                                  const int32_t *__restrict__ colind, const double *__restrict__ a,
-                                                  const double *__restrict__ b, const double *__restrict__ alpha,
-                                                  const double *__restrict__ beta, const double *__restrict__ X,
-                                                  int64_t ldx, int k, double *__restrict__ Y, int64_t ldy) {
+__global__ void __launch_bounds__(256, WITH_B ? 4 : 5)
+k_spmm_nnz(int64_t n, const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colind,
+           const double *__restrict__ a, const double *__restrict__ b, const double *__restrict__ alpha,
+           const double *__restrict__ beta, const double *__restrict__ X, int64_t ldx, int k, double *__restrict__ Y,
+           int64_t ldy) {
     const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31, c0 = blockIdx.y * KW, kc = min(KW, k - c0);
     if (row >= n) return;
-    constexpr int NV = WITH_B ? 2 * KW : KW;
+    constexpr int KP = KW > 4 ? 8 : KW > 2 ? 4 : KW, NV = WITH_B ? 2 * KP : KP;
     double acc[NV];
 #pragma unroll
     for (int c = 0; c < NV; ++c) acc[c] = 0.0;
     const int64_t p0 = rowptr[row], p1 = rowptr[row + 1];
-#pragma unroll 4
-    for (int64_t p = p0 + lane; p < p1; p += 32) {
-        const double av = a[p];
+    // entry p of the row (zeros for a lane whose `in` is false)
+    auto entry = [&](int64_t p, bool in) {
+        const double av = in ? a[p] : 0.0;
         double bv = 0.0;
-        if constexpr (WITH_B) bv = b[p];
+        if constexpr (WITH_B) bv = in ? b[p] : 0.0;
         const double *x = X + (int64_t)colind[p] * ldx + c0;
 #pragma unroll
         for (int c = 0; c < KW; ++c)
             if (c < kc) {
-                const double xv = x[c];
+                const double xv = in ? x[c] : 0.0;
                 acc[c] += av * xv;
-                if constexpr (WITH_B) acc[KW + c] += bv * xv;
+                if constexpr (WITH_B) acc[KP + c] += bv * xv;
             }
+    };
+    // Four entries a lane at a time while the row fills them for every lane, then what is left in one batch
+    // of the same number for every lane: an unrolled loop over a lane's own entries parts the warp where the
+    // counts differ (97 a row as slow as 193).
+    int64_t q = p0 + lane;
+    for (; q - lane + 128 <= p1; q += 128) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) entry(q + 32 * u, true);
     }
+    auto rest = [&](auto trips) {
+        constexpr int T = decltype(trips)::value;
+#pragma unroll
+        for (int u = 0; u + 1 < T; ++u) entry(q + 32 * u, true);
+        entry(min(q + 32 * (T - 1), p1 - 1), q + 32 * (T - 1) < p1);
+    };
+    const int left_over = (int)(p1 - (q - lane));            // 0 .. 127
+    if (left_over > 96) rest(std::integral_constant<int, 4>{});
+    else if (left_over > 64) rest(std::integral_constant<int, 3>{});
+    else if (left_over > 32) rest(std::integral_constant<int, 2>{});
+    else if (left_over > 0) rest(std::integral_constant<int, 1>{});
     int base = 0, left = 0;
     bool owner = true;
     spmm_fold<NV, 16>(acc, lane, base, left, owner);
-    // value v of the folded sums is A x (v < KW) or B x (v >= KW) of column c0 + v mod KW
+    // value v of the folded sums is A x (v < KP) or B x (v >= KP) of column c0 + v mod KP
     if constexpr (WITH_B) {
-        __shared__ double s_sum[8][2 * KW];
+        __shared__ double s_sum[8][NV];
         double *s = s_sum[threadIdx.x >> 5];
 #pragma unroll
         for (int e = 0; e < NV; ++e)
             if (e < left && owner) s[base + e] = acc[e];
         __syncwarp();
         for (int c = lane; c < kc; c += 32)
-            Y[row * ldy + c0 + c] = (alpha ? alpha[c0 + c] : 1.0) * s[c] + beta[c0 + c] * s[KW + c];
+            Y[row * ldy + c0 + c] = (alpha ? alpha[c0 + c] : 1.0) * s[c] + beta[c0 + c] * s[KP + c];
     } else {
 #pragma unroll
         for (int e = 0; e < NV; ++e)
