@@ -1258,12 +1258,15 @@ static int fold_per_step(ss_numeric *f, int j, double *b, int k, bool full) {
 
 // Whether a solve of k columns runs on the tensor cores (fold_tc.cuh): where the FP64 work it takes
 // off the CUDA cores, about 4 ps per entry of L and column, outweighs its longer items, 13 - 16 us a
-// level and sweep.  Measured (ms a solve, CUDA cores / tensor cores): N = 864 (13 levels) k = 129
-// 0.36 / 0.36, k = 304 0.69 / 0.39; N = 5,280 (55) k = 32 1.54 / 1.43, k = 48 2.15 / 1.50, k = 304
-// 10.6 / 2.48; N = 16,384 (129) k = 16 4.6 / 4.3, k = 48 11.5 / 4.4, k = 304 61 / 9.3.
+// level and sweep.  The CUDA cores take whole items of 32 rows x 16 columns, so entries are counted in
+// these: panels with a row or two below them, as of a path or a narrow band, cost 26 times their entries.
+// Measured (ms a solve, CUDA cores / tensor cores): N = 864 (13 levels) k = 128 0.35 / 0.33, k = 304
+// 0.68 / 0.38; N = 5,280 (55) k = 24 1.26 / 1.38, k = 33 1.68 / 1.42, k = 304 10.6 / 2.38; N = 16,384
+// (129) k = 16 4.6 / 4.3, k = 48 11.5 / 4.4, k = 304 61 / 8.9; a path of 20,000 rows (10) k = 33
+// 0.75 / 0.69, k = 304 4.76 / 3.12 (3.60 with a block a tile in the form before these).
 static bool fold_uses_tc(const ss_symbolic *s, int k) {
     return s->ctx->gemm_mode == SS_GEMM_TENSOR && k > kFoldMaxNc &&
-           (double)s->info.l_offdiag_entries * k >= 3.6e6 * (double)s->solve_levels.size();
+           s->sweep_padded * k >= 3.6e6 * (double)s->solve_levels.size();
 }
 
 // both sweeps in one cooperative launch of k_fold_sweeps (every block resident, a bounded grid

@@ -191,6 +191,8 @@ struct ss_symbolic {
                                              // 0 CUDA cores, 1 tensor cores (autotuner)
     int64_t n = 0, nnz = 0;
     int64_t max_row = 0;                     // most entries of a row
+    double sweep_padded = 0.0;               // entries below the diagonal blocks, in whole items of 32 rows x
+                                             // 16 columns (what an FP64 sweep on the CUDA cores takes)
     int nb = 64;
     std::vector<int32_t> perm, iperm;        // perm[new] = old, iperm[old] = new
     std::vector<int64_t> rowptr;             // host copy of the pattern

@@ -567,6 +567,7 @@ static int analyze_impl(ss_ctx *ctx, int64_t n, const int64_t *rowptr, const int
     s->solve_levels.clear();
     s->solve_tile_pre.clear();
     s->max_rows_below = 0;
+    s->sweep_padded = 0.0;
     for (int32_t l = 0; l < nplev; ++l) {
         SolveLevel sl{(int64_t)s->solve_panels.size(), 0, 0, 0.0, 0};
         for (int32_t p : by_lev[l]) {
@@ -577,6 +578,7 @@ static int analyze_impl(ss_ctx *ctx, int64_t n, const int64_t *rowptr, const int
             sl.tiles128 += (int32_t)cdiv(pd.m - pd.k0 - pd.w, 128);
             s->max_rows_below = std::max(s->max_rows_below, pd.m - pd.k0 - pd.w);
             sl.offdiag += (double)(pd.m - pd.k0 - pd.w) * pd.w;
+            s->sweep_padded += 32.0 * cdiv(pd.m - pd.k0 - pd.w, 32) * 16.0 * cdiv(pd.w, 16);
             sl.count++;
         }
         s->solve_levels.push_back(sl);

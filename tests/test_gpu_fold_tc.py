@@ -5,7 +5,7 @@ import pytest
 import scipy.sparse as sp
 import torch
 
-from workloads.pencils import gaussian_pencil, random_sparse_pencil
+from workloads.pencils import gaussian_pencil, laplacian_1d, random_sparse_pencil
 
 pytestmark = pytest.mark.gpu
 
@@ -69,6 +69,23 @@ def test_few_right_hand_sides(gpu_lib):
         R = np.random.default_rng(k).standard_normal((p.n, k))
         X, flops = solved(f, R)
         assert flops >= 28 * 4.0 * sym.info["l_offdiag_entries"] * k
+        res = np.linalg.norm(R - M @ X, axis=0)
+        assert (res <= tol * (norm * np.linalg.norm(X, axis=0) + np.linalg.norm(R, axis=0))).all()
+
+
+def test_tiles_of_a_row_or_two(gpu_lib):
+    # a path: most panels have one or two rows below them, so whole items of the CUDA cores count, not entries
+    p = laplacian_1d(5000, mass=True)
+    ctx = gpu_lib.Context(0)
+    sym = ctx.analyze(p.rowptr, p.colind)
+    f = sym.factor(torch.tensor(p.a, device="cuda"), torch.tensor(p.b, device="cuda"), [-0.83], "fp64")
+    M = sp.csr_matrix((p.a + 0.83 * p.b, p.colind, p.rowptr), shape=(p.n, p.n))
+    norm = abs(M).sum(axis=1).max()
+    tol = 16 * p.n * 1.1e-16 * max(1.0, f.stats(0)[1])
+    for k in (111, 128, 129, 200):
+        R = np.random.default_rng(k).standard_normal((p.n, k))
+        X, flops = solved(f, R)
+        assert flops > 0.0
         res = np.linalg.norm(R - M @ X, axis=0)
         assert (res <= tol * (norm * np.linalg.norm(X, axis=0) + np.linalg.norm(R, axis=0))).all()
 
