@@ -232,8 +232,9 @@ ss_status ss_selftest_barrier(ss_ctx *ctx, int32_t extra_arrivals, int64_t limit
 ss_status ss_selftest_recip(ss_ctx *ctx, int64_t n, const double *d, double *out);
 
 /* Self-test of what the calls do when device memory runs out (no paper counterpart): from now on
- * every device allocation of this context above max_bytes bytes fails on the host as an
- * out-of-memory one would; max_bytes < 0 (the state of a new context): no limit.  Errors:
+ * every device allocation of this context above max_bytes bytes, and every such host list of the
+ * tensor-core products, fails on the host as an out-of-memory one would; max_bytes < 0 (the state of a new
+ * context): no limit.  Errors:
  * SS_ERR_ARG. */
 ss_status ss_selftest_alloc_limit(ss_ctx *ctx, int64_t max_bytes);
 

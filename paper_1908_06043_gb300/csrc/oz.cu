@@ -1,7 +1,10 @@
 // Host side of the FP64-accurate tensor-core products (tc_gemm.cuh): operand slicing, the
 // (tile, piece) plan of the sparse pattern, and the launches.
 #include <algorithm>
+#include <atomic>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include "internal.h"
@@ -160,6 +163,46 @@ void free_samples(ss_symbolic *s) {
     s->oz_samples = nullptr;
 }
 
+// The lists are built on the host.  Where its memory does not do, the caller gets SS_ERR_OOM as for device
+// memory: nothing may leave a C entry point, or a parallel region, as an exception.
+// `bytes` of host lists are about to be allocated (ss_selftest_alloc_limit)
+void host_room(const ss_ctx *ctx, size_t bytes) {
+    if (ctx->alloc_limit >= 0 && bytes > (size_t)ctx->alloc_limit) throw std::bad_alloc();
+}
+template <typename F>
+int guarded(ss_ctx *ctx, F &&build) {
+    try {
+        return build();
+    } catch (const std::bad_alloc &) {
+        return ctx->set_error(SS_ERR_OOM, "tensor-core product lists: host allocation failed");
+    }
+}
+// body(row tile, counters) for every row tile in parallel, each thread with n counters of zero
+template <typename T, typename F>
+void each_row_tile(const ss_ctx *ctx, int32_t nrt, int64_t n, F &&body) {
+    std::atomic<bool> failed{false};
+#pragma omp parallel
+    {
+        std::vector<T> cnt;
+        try {
+            host_room(ctx, sizeof(T) * n);
+            cnt.assign(n, 0);
+        } catch (const std::bad_alloc &) {
+            failed = true;
+        }
+#pragma omp for schedule(dynamic, 16)
+        for (int32_t rt = 0; rt < nrt; ++rt) {
+            if (failed || cnt.empty()) continue;
+            try {
+                body(rt, cnt);
+            } catch (const std::bad_alloc &) {
+                failed = true;
+            }
+        }
+    }
+    if (failed) throw std::bad_alloc();
+}
+
 // (tile, piece) pairs of the pattern -- for each 128-row tile the 32-column pieces that hold
 // entries -- and the entries of every pair: CSR position (from the tile's first) and place in the
 // pair's digit block
@@ -168,22 +211,17 @@ int plan_build(ss_symbolic *s) {
     const int64_t n = s->n, npieces = (n + sstc::kOzK - 1) / sstc::kOzK;
     const int32_t nrt = (int32_t)cdivu(n, 128);
     std::vector<std::vector<int32_t>> pieces(nrt), counts(nrt);     // of a tile: pieces ascending, entries of each
-#pragma omp parallel
-    {
-        std::vector<int32_t> cnt(npieces, 0);
-#pragma omp for schedule(dynamic, 16)
-        for (int32_t rt = 0; rt < nrt; ++rt) {
-            const int64_t r1 = std::min<int64_t>(n, (rt + 1ll) * 128);
-            std::vector<int32_t> &list = pieces[rt];
-            for (int64_t p = s->rowptr[rt * 128ll]; p < s->rowptr[r1]; ++p)
-                if (cnt[s->colind[p] / sstc::kOzK]++ == 0) list.push_back(s->colind[p] / sstc::kOzK);
-            std::sort(list.begin(), list.end());
-            for (int32_t pc : list) {
-                counts[rt].push_back(cnt[pc]);
-                cnt[pc] = 0;
-            }
+    each_row_tile<int32_t>(ctx, nrt, npieces, [&](int32_t rt, std::vector<int32_t> &cnt) {
+        const int64_t r1 = std::min<int64_t>(n, (rt + 1ll) * 128);
+        std::vector<int32_t> &list = pieces[rt];
+        for (int64_t p = s->rowptr[rt * 128ll]; p < s->rowptr[r1]; ++p)
+            if (cnt[s->colind[p] / sstc::kOzK]++ == 0) list.push_back(s->colind[p] / sstc::kOzK);
+        std::sort(list.begin(), list.end());
+        for (int32_t pc : list) {
+            counts[rt].push_back(cnt[pc]);
+            cnt[pc] = 0;
         }
-    }
+    });
     std::vector<int32_t> tile_ptr(nrt + 1, 0), pair_piece;
     std::vector<int64_t> ent_ptr(1, 0);
     for (int32_t rt = 0; rt < nrt; ++rt) {
@@ -195,21 +233,16 @@ int plan_build(ss_symbolic *s) {
     }
     std::vector<uint32_t> ent_e(std::max<int64_t>(1, s->nnz));
     std::vector<uint16_t> ent_off(std::max<int64_t>(1, s->nnz));
-#pragma omp parallel
-    {
-        std::vector<int64_t> at(npieces, 0);
-#pragma omp for schedule(dynamic, 16)
-        for (int32_t rt = 0; rt < nrt; ++rt) {
-            const int64_t r0 = rt * 128ll, r1 = std::min<int64_t>(n, r0 + 128), e0 = s->rowptr[r0];
-            for (int32_t q = tile_ptr[rt]; q < tile_ptr[rt + 1]; ++q) at[pair_piece[q]] = ent_ptr[q];
-            for (int64_t r = r0; r < r1; ++r)
-                for (int64_t p = s->rowptr[r]; p < s->rowptr[r + 1]; ++p) {
-                    const int64_t o = at[s->colind[p] / sstc::kOzK]++;
-                    ent_e[o] = (uint32_t)(p - e0);
-                    ent_off[o] = (uint16_t)sstc::oz_offset((int)(r - r0), (int)(s->colind[p] % sstc::kOzK));
-                }
-        }
-    }
+    each_row_tile<int64_t>(ctx, nrt, npieces, [&](int32_t rt, std::vector<int64_t> &at) {
+        const int64_t r0 = rt * 128ll, r1 = std::min<int64_t>(n, r0 + 128), e0 = s->rowptr[r0];
+        for (int32_t q = tile_ptr[rt]; q < tile_ptr[rt + 1]; ++q) at[pair_piece[q]] = ent_ptr[q];
+        for (int64_t r = r0; r < r1; ++r)
+            for (int64_t p = s->rowptr[r]; p < s->rowptr[r + 1]; ++p) {
+                const int64_t o = at[s->colind[p] / sstc::kOzK]++;
+                ent_e[o] = (uint32_t)(p - e0);
+                ent_off[o] = (uint16_t)sstc::oz_offset((int)(r - r0), (int)(s->colind[p] % sstc::kOzK));
+            }
+    });
     OzPlan *pl = new OzPlan();
     pl->nrt = nrt;
     pl->npairs = (int64_t)pair_piece.size();
@@ -236,24 +269,18 @@ int samples_count(ss_symbolic *s) {
     const int64_t n = s->n, nct = (n + 63) / 64;
     const int32_t nrt = (int32_t)cdivu(n, 128);
     std::vector<std::vector<int32_t>> cts(nrt), counts(nrt);
-#pragma omp parallel
-    {
-        std::vector<int32_t> cnt(nct, 0);
-#pragma omp for schedule(dynamic, 16)
-        for (int32_t rt = 0; rt < nrt; ++rt) {
-            const int64_t r0 = rt * 128ll, r1 = std::min<int64_t>(n, r0 + 128);
-            for (int64_t r = r0; r < r1; ++r)
-                for (int64_t p = s->rowptr[r]; p < s->rowptr[r + 1] && s->colind[p] <= r; ++p)
-                    if (cnt[s->colind[p] / 64]++ == 0) cts[rt].push_back(s->colind[p] / 64);
-            std::sort(cts[rt].begin(), cts[rt].end());
-            for (int32_t ct : cts[rt]) {
-                counts[rt].push_back(cnt[ct]);
-                cnt[ct] = 0;
-            }
+    each_row_tile<int32_t>(s->ctx, nrt, nct, [&](int32_t rt, std::vector<int32_t> &cnt) {
+        const int64_t r0 = rt * 128ll, r1 = std::min<int64_t>(n, r0 + 128);
+        for (int64_t r = r0; r < r1; ++r)
+            for (int64_t p = s->rowptr[r]; p < s->rowptr[r + 1] && s->colind[p] <= r; ++p)
+                if (cnt[s->colind[p] / 64]++ == 0) cts[rt].push_back(s->colind[p] / 64);
+        std::sort(cts[rt].begin(), cts[rt].end());
+        for (int32_t ct : cts[rt]) {
+            counts[rt].push_back(cnt[ct]);
+            cnt[ct] = 0;
         }
-    }
-    OzSamples *sp = new OzSamples();
-    s->oz_samples = sp;
+    });
+    std::unique_ptr<OzSamples> sp(new OzSamples());
     sp->ptr.assign(1, 0);
     sp->first.assign(nrt, 0);
     for (int32_t rt = 0; rt < nrt; ++rt) {
@@ -265,6 +292,7 @@ int samples_count(ss_symbolic *s) {
         }
     }
     sp->ntiles = (int64_t)sp->rts.size();
+    s->oz_samples = sp.release();
     return SS_OK;
 }
 
@@ -276,24 +304,19 @@ int samples_build(ss_symbolic *s) {
     const size_t m = (size_t)std::max<int64_t>(1, sp->ptr.back());
     std::vector<uint32_t> e(m), t(m);
     std::vector<uint16_t> off(m);
-#pragma omp parallel
-    {
-        std::vector<int64_t> at(nct, 0);
-#pragma omp for schedule(dynamic, 16)
-        for (int32_t rt = 0; rt < nrt; ++rt) {
-            const int64_t r0 = rt * 128ll, r1 = std::min<int64_t>(n, r0 + 128);
-            const int64_t t1 = rt + 1 < nrt ? sp->first[rt + 1] : sp->ntiles;
-            for (int64_t u = sp->first[rt]; u < t1; ++u) at[sp->cts[u]] = sp->ptr[u];
-            for (int64_t r = r0; r < r1; ++r)
-                for (int64_t p = s->rowptr[r]; p < s->rowptr[r + 1] && s->colind[p] <= r; ++p) {
-                    const int64_t c = s->colind[p], o = at[c / 64]++;
-                    const int32_t *b = s->colind.data() + s->rowptr[c], *z = s->colind.data() + s->rowptr[c + 1];
-                    e[o] = (uint32_t)p;
-                    t[o] = (uint32_t)(std::lower_bound(b, z, (int32_t)r) - s->colind.data());   // (c, r): the pattern is symmetric
-                    off[o] = (uint16_t)((r - r0) * 64 + c % 64);
-                }
-        }
-    }
+    each_row_tile<int64_t>(ctx, nrt, nct, [&](int32_t rt, std::vector<int64_t> &at) {
+        const int64_t r0 = rt * 128ll, r1 = std::min<int64_t>(n, r0 + 128);
+        const int64_t t1 = rt + 1 < nrt ? sp->first[rt + 1] : sp->ntiles;
+        for (int64_t u = sp->first[rt]; u < t1; ++u) at[sp->cts[u]] = sp->ptr[u];
+        for (int64_t r = r0; r < r1; ++r)
+            for (int64_t p = s->rowptr[r]; p < s->rowptr[r + 1] && s->colind[p] <= r; ++p) {
+                const int64_t c = s->colind[p], o = at[c / 64]++;
+                const int32_t *b = s->colind.data() + s->rowptr[c], *z = s->colind.data() + s->rowptr[c + 1];
+                e[o] = (uint32_t)p;
+                t[o] = (uint32_t)(std::lower_bound(b, z, (int32_t)r) - s->colind.data());   // (c, r): the pattern is symmetric
+                off[o] = (uint16_t)((r - r0) * 64 + c % 64);
+            }
+    });
     auto up = [&](auto **d, const auto &h) {
         cudaError_t er = ss_malloc(ctx, (void **)d, sizeof(h[0]) * std::max<size_t>(1, h.size()));
         if (er == cudaSuccess && !h.empty()) er = cudaMemcpy(*d, h.data(), sizeof(h[0]) * h.size(), cudaMemcpyHostToDevice);
@@ -338,7 +361,8 @@ int vals_make(ss_symbolic *s, const double *vals, OzVals *v, Scratch *buf) {
 int vals_get(ss_numeric *f, int which, OzVals **out) {
     *out = f->oz[which];
     if (*out) return SS_OK;
-    OzVals *v = new OzVals();
+    OzVals *v = new (std::nothrow) OzVals();
+    if (!v) return f->sym->ctx->set_error(SS_ERR_OOM, "tensor-core product: host allocation failed");
     const int rc = vals_make(f->sym, which == 0 ? f->a_vals : f->b_vals, v, nullptr);
     if (rc != SS_OK) {
         delete v;
@@ -354,7 +378,7 @@ int spmm_core(ss_symbolic *s, int npass, OzVals *const *v, const double *const *
               const double *X, int64_t ldx, int k, double *Y, int64_t ldy) {
     ss_ctx *ctx = s->ctx;
     int rc;
-    if (!s->oz_plan && (rc = plan_build(s)) != SS_OK) return rc;
+    if (!s->oz_plan && (rc = guarded(ctx, [&] { return plan_build(s); })) != SS_OK) return rc;
     Scratch buf(ctx);
     unsigned char *sx;
     int *ex;
@@ -467,14 +491,17 @@ bool oz_sddmm_ok(ss_symbolic *s, int ne) {
     if (s->ctx->gemm_mode != SS_GEMM_TENSOR || s->n < 2048 || ne < 48 || s->nnz >= (1ll << 32)) return false;
     const double cuda = 3.1 * (double)s->nnz * (ne + 300.0), rest = 1.3e8 + 20.0 * (double)s->n * ne;
     if (cuda <= rest) return false;
-    if (!s->oz_samples && samples_count(s) != SS_OK) return false;
+    if (!s->oz_samples && guarded(s->ctx, [&] { return samples_count(s); }) != SS_OK) {
+        s->ctx->err.clear();                   // CUDA cores
+        return false;
+    }
     return cuda > rest + (double)s->oz_samples->ntiles * (2.5e5 + 700.0 * ne);
 }
 
 int oz_sddmm(ss_symbolic *s, const double *X, const double *lambda, int ne, double *grad_a, double *grad_b) {
     ss_ctx *ctx = s->ctx;
     int rc;
-    if (!s->oz_samples->d_rt && (rc = samples_build(s)) != SS_OK) return rc;
+    if (!s->oz_samples->d_rt && (rc = guarded(ctx, [&] { return samples_build(s); })) != SS_OK) return rc;
     const OzSamples *sp = s->oz_samples;
     oz_attrs(ctx->device);
     Scratch buf(ctx);

@@ -21,7 +21,7 @@ def test_gradient_fallback_leaves_the_factors_products(gpu_lib):
     ctx.profile(["spmm_tc"])
     X = torch.tensor(normal_block(p.n, 64, 5), device="cuda")
     lam = torch.linspace(-3.0, -1.0, 64, dtype=torch.float64, device="cuda")
-    ctx.selftest_alloc_limit(0)
+    ctx.selftest_alloc_limit(1 << 16)             # the lists of entries fail on the device, not those on the host
     ga, gb = sym.band_energy_grad(X, lam)
     ctx.selftest_alloc_limit()
     after = run()
@@ -67,3 +67,27 @@ def test_scratch_goes_back_on_request(gpu_lib):
     assert torch.cuda.mem_get_info()[0] >= free - 4e6
     again, _ = sym.band_energy_grad(X, lam)
     assert torch.equal(ga, again)
+
+
+def test_host_lists_that_do_not_fit(gpu_lib):
+    # the lists of a pattern's tiles fail on the host: an out-of-memory status for the product, the CUDA cores
+    # for the gradient, and both work once there is room
+    p = gaussian_pencil((9, 11, 11), (0.3, 2.0), seed=3)
+    ctx, sym, a, b = setup(gpu_lib, p)
+    X = torch.tensor(normal_block(p.n, 64, 5), device="cuda")
+    lam = torch.linspace(-3.0, -1.0, 64, dtype=torch.float64, device="cuda")
+    ctx.selftest_alloc_limit(0)
+    first, _ = sym.band_energy_grad(X, lam)
+    with pytest.raises(gpu_lib.SisliceError, match="SS_ERR_OOM"):
+        sym.spmm(a, b, X)
+    ctx.selftest_alloc_limit()
+    ctx.profile(["sddmm", "spmm_tc"])
+    second, _ = sym.band_energy_grad(X, lam)
+    Y = sym.spmm(a, b, X)
+    ctx.profile_query("sddmm")
+    assert ctx.profile_query_tensor("sddmm") > 0.0 and ctx.profile_query_tensor("spmm_tc") > 0.0
+    xm = X.abs().max().item()
+    assert (first - second).abs().max().item() <= 64 * 64 * 2.0 ** -52 * xm ** 2
+    # n products of entries of A and X, cut 2^-53 below the largest
+    ref = torch.tensor(p.dense("a"), device="cuda") @ X
+    assert (Y - ref).abs().max().item() <= 8 * 2.0 ** -53 * p.n * float(np.abs(p.a).max()) * xm
