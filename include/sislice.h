@@ -361,8 +361,9 @@ ss_status ss_factor_stats(const ss_numeric *f, int32_t shift_idx, double *min_pi
  * R and X are DEVICE float64 N x k row-major (may alias).  `refine` FP64 iterative
  * refinement corrections are applied (X += M^-1 (R - (A - sigma_j B) X)); for a shift
  * solved in FP32 at least as many as its contraction factor needs to reach 1e-13 (at
- * most 8).  Refined solves of many right-hand sides at a shift that has an FP64 factor as well
- * (SS_FP64_SOLVE32) run in FP64 on the tensor cores, with `refine` corrections.  The residual uses the values of A - sigma_j B, formed on the shift's first
+ * most 8).  Refined solves at a shift that has an FP64 factor as well (SS_FP64_SOLVE32) run in FP64 where
+ * its sweeps are the quicker ones -- of few right-hand sides on the CUDA cores, of many on the tensor cores --
+ * with `refine` corrections.  The residual uses the values of A - sigma_j B, formed on the shift's first
  * refined solve and kept with the factor (nnz doubles per shift).
  * Errors: SS_ERR_ARG, SS_ERR_CUDA, SS_ERR_OOM, SS_ERR_TIMEOUT (sweep kernel barrier). */
 ss_status ss_solve(ss_numeric *f, int32_t shift_idx, const double *R, int32_t k, double *X,
@@ -460,7 +461,9 @@ ss_status ss_band_energy_grad(ss_symbolic *sym, const double *X, const double *l
  * Y[i, j] = sum_e (alpha[j] a_vals[e] + beta[j] b_vals[e]) X[col(e), j] over row i,
  * X, Y DEVICE float64 N x k row-major; alpha, beta DEVICE float64[k] (NULL alpha = 1,
  * NULL beta = no B term).  With ss_set_gemm_mode(SS_GEMM_TENSOR), N >= 2,048 and k >= 48
- * the products run on the tensor cores, A X and B X each rounded once to FP64.  Errors: SS_ERR_ARG, SS_ERR_CUDA, SS_ERR_OOM, SS_ERR_TIMEOUT. */
+ * the products run on the tensor cores: the rows of A and B and the columns of X cut to 55 bits below their
+ * largest entry, A X and B X each summed exactly and rounded once to FP64.
+ * Errors: SS_ERR_ARG, SS_ERR_CUDA, SS_ERR_OOM, SS_ERR_TIMEOUT. */
 ss_status ss_spmm(ss_symbolic *sym, const double *a_vals, const double *b_vals,
                   const double *alpha, const double *beta, const double *X, int32_t k,
                   double *Y);
@@ -510,8 +513,9 @@ ss_status ss_profile(ss_ctx *ctx, uint32_t mask);
  * lower triangle only for the Schur update); 0 for the others.  Classes ending in _F32 are the
  * FP32 instantiations of the mixed-precision factor and solves. */
 ss_status ss_profile_query(ss_ctx *ctx, int32_t cls, int64_t *launches, double *seconds, double *flops);
-/* For the tensor-core classes (SS_K_SCHUR_TC, SS_K_GEMM_TC, SS_K_SPMM_TC): the FP16 MMA
- * work (2 M N K per MMA, zero padding of sparse tiles included) their launches issued since
+/* For the classes whose kernels use the tensor cores (SS_K_SCHUR_TC, SS_K_GEMM_TC, SS_K_SPMM_TC,
+ * SS_K_SDDMM, and SS_K_SOLVE for the block solves): the FP16 MMA
+ * work (2 M N K per MMA, zero padding of tiles included) their launches issued since
  * the last ss_profile call; 0 for the other classes.  Call after ss_profile_query (which
  * synchronises).  Errors: SS_ERR_ARG. */
 ss_status ss_profile_query_tensor(ss_ctx *ctx, int32_t cls, double *tensor_flops);

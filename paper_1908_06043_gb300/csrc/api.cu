@@ -1262,7 +1262,7 @@ static int fold_per_step(ss_numeric *f, int j, double *b, int k, bool full) {
 // these: panels with a row or two below them, as of a path or a narrow band, cost 26 times their entries.
 // Measured (ms a solve, CUDA cores / tensor cores): N = 864 (13 levels) k = 128 0.35 / 0.33, k = 304
 // 0.68 / 0.38; N = 5,280 (55) k = 24 1.26 / 1.38, k = 33 1.68 / 1.42, k = 304 10.6 / 2.38; N = 16,384
-// (129) k = 16 4.6 / 4.3, k = 48 11.5 / 4.4, k = 304 61 / 8.9; a path of 20,000 rows (10) k = 33
+// (129) k = 16 4.6 / 4.3, k = 48 11.5 / 4.4, k = 304 61 / 8.8; a path of 20,000 rows (10) k = 33
 // 0.75 / 0.69, k = 304 4.76 / 3.12 (3.60 with a block a tile in the form before these).
 static bool fold_uses_tc(const ss_symbolic *s, int k) {
     return s->ctx->gemm_mode == SS_GEMM_TENSOR && k > kFoldMaxNc &&
@@ -1701,7 +1701,7 @@ int solve_apply(ss_numeric *f, int j, const double *R, int k, double *X, int ref
     // a solve contracts the residual by 1e-10 where an FP32 one gives 1e-1 .. 1e-2, and the folded
     // sweeps pass a level in 5 - 10 us where the FP32 ones take 48.  Only many columns without the
     // tensor cores (4 ps of FP64 per entry of L and column) are left to FP32.  Measured, ms a solve,
-    // FP32 / FP64: N = 16,384, k = 304 6.3 / 9.2 (and 8 or 9 / 3 of them for two requested
+    // FP32 / FP64: N = 16,384, k = 304 6.1 / 8.8 (and 8 or 9 / 3 of them for two requested
     // refinements); k = 1, 8, 16, 48 3.4 / 0.85, 3.3 / 2.5, 3.4 / 4.2, 3.6 / 4.4 (7 / 2 of them for one
     // refinement at a contraction of 1.5e-2).
     const bool in_f64 = (refine > 0 || target > 0.0) && f->shift_prec[j] == SS_FP64 &&

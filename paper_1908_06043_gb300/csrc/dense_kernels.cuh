@@ -521,7 +521,6 @@ __global__ void k_set_identity(double *V, int k) {
 }
 
 // ---------------------------------------------------------------- column reductions
-// out[c] += sum_r X[r][c] * Y[r][c]
 // out[c] += sum of acc over the block's threads tid = c mod nv; 256 threads, nv a power of two.
 // Within warps by shuffles: as one thread a column over 256 / nv values it was most of such a launch.
 __device__ __forceinline__ void column_sums(double acc, int nv, double *s, double *out) {
@@ -535,6 +534,7 @@ __device__ __forceinline__ void column_sums(double acc, int nv, double *s, doubl
         atomicAdd(&out[tid], v);
     }
 }
+// out[c] += sum_r X[r][c] * Y[r][c]
 __global__ void k_col_dot(int64_t n, int k, const double *__restrict__ X, const double *__restrict__ Y,
                           double *out) {
     // requires 256 % k == 0 so that each thread keeps one column
@@ -644,7 +644,6 @@ __global__ void k_lz_three_term(int64_t n, int nv, const double *__restrict__ q,
     w[e] = v;
 }
 
-// q_next = w / beta (0 where beta is tiny)
 // x = w / beta and bx = bw / beta (blockIdx.y) with beta = sqrt(nrm2), 0 for beta = 0; one root and
 // reciprocal a column, the quotient corrected to about its last bit
 __global__ void __launch_bounds__(256) k_lz_normalize(int64_t n, int nv, const double *__restrict__ w,

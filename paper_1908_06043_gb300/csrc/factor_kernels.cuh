@@ -189,8 +189,8 @@ __device__ __forceinline__ unsigned long long warp_max_key(unsigned long long ke
 // iteration (the hyperpower method of order three, Altman 1960): with e = 1 - d x,
 // 1 / d = x (1 + e + e^2 + ..).  The approximation takes and gives 20 bits of mantissa, so |e| < 2^-18 and
 // what is left out, e^3, is below half a unit in the last place; with the last rounding the result is
-// within one unit of 1 / d (3 of 10,000 random d differ from the division).  Three dependent multiply-adds; a division takes some ten, and checks.
-// Outside 2^+-1000: the division.
+// within one unit of 1 / d (3 of 10,000 random d differ from the division).  Three dependent
+// multiply-adds; a division takes some ten, and checks.  Outside 2^+-1000: the division.
 __device__ __forceinline__ double diag_recip(double d) {
     const unsigned ex = (unsigned)(__double_as_longlong(d) >> 52) & 0x7ffu;
     if (ex - 23u > 2000u) return d != 0.0 ? 1.0 / d : 0.0;

@@ -21,11 +21,13 @@
 // Cutting and summing digits takes integer instructions only (digits8.cuh).  A non-finite operand
 // makes its whole column (row) of the product NaN.
 //
-// What bounds it: the chain of one item a level.  Measured per item (cycles): right-hand sides'
-// load and digits 6,000, 40 MMAs 4,250 (7,100 as 112 MMAs of N = 64), read-out 8,100 (7 x 32 KB out
+// What bounds it: an item's load and cut, MMAs and read-out, which take turns.  One item a level over 258
+// level steps would be 2.7 ms at N = 16,384, k = 304; the rest of its 8.8 are items queued in wide levels.
+// Measured per item (cycles): right-hand sides' load and digits 6,000, 40 MMAs 4,250 (7,100 as 112 MMAs of N = 64), read-out 8,100 (7 x 32 KB out
 // of tensor memory), the next tile's digits 3,100, barrier 4,000-7,000; G's tile of the next level
-// is loaded during the MMAs and cut before the barrier.  One solve at N = 16,384, k = 304: 61.8 ms
-// on the CUDA cores (0.87 of their FP64 peak), 9.2 ms here; N = 5,280, k = 112: 4.4 -> 1.6 ms.
+// is loaded during the MMAs and cut before the barrier.  (Measured before the zero test moved into the
+// exponent and scales came four at a time, 4% of a solve.)  One solve at N = 16,384, k = 304: 61.8 ms on the CUDA
+// cores (0.87 of their FP64 peak), 8.8 ms here; N = 5,280, k = 112: 4.4 -> 1.5 ms.
 // Tried and left out: an accumulator's read-out under the MMAs of the next ones (each slows the
 // other: 9,000 + 8,400 cycles where one after the other takes 7,100 + 8,100).
 #pragma once

@@ -31,9 +31,9 @@ __device__ __forceinline__ void dd_add(DD &s, double hi, double lo) {
 
 // The products run in integers: double-double arithmetic takes some 20 FP64 operations per stored
 // entry and column at 2 a clock and SM, a 64 x 64-bit multiply-add into 128 bits some ten at 64.
-// Column c of X becomes x~ = round(x 2^(xbits - E_c)), |x| < 2^E_c: the quotient of x~ differs from
-// that of x by the residual times the rounding (second order, below 1e-20), as long as numerator and
-// denominator share x~.  A row of A (of B) becomes round(a 2^(61 - E_i)): relative to the row's
+// Column c of X becomes x~ = round(x 2^(xbits - E_c)), |x| < 2^E_c, xbits 53 (fewer for rows of more
+// than 4,096 entries): the quotient of x~ differs from that of x by the residual times the rounding
+// (second order, below 1e-20, near convergence), as long as numerator and denominator share x~.  A row of A (of B) becomes round(a 2^(61 - E_i)): relative to the row's
 // largest entry, 2^-62, below double-double's use for the dot products that follow.  Sums over a row
 // are exact: 2^(61 + xbits) times its entries stays below 2^127.  The column's scale cancels in the
 // quotient.  "Largest" is meant after a scaling by powers of two that follows the basis: x_i is
